@@ -748,9 +748,10 @@ mto_status set_design_sync(mto_ctx* c, int n_phase, const double* x_dev, const d
 size_t partials_count(const mto_ctx* c) {
   const Grid& gf = c->lv[c->L].g;
   int maxb = vec_blocks(gf.size(), c->num_sms);
+  if (maxb < c->num_sms) maxb = c->num_sms;  // small launches: up to one block per SM
   for (int mode = 0; mode <= MODE_RESTRICT; ++mode) {
     for (int cols = 1; cols <= 2; ++cols) {
-      const SweepShape s = sweep_shape(gf, mode, MAX_TARGET_WARPS_PER_SM * c->num_sms, cols);
+      const SweepShape s = sweep_shape(gf, mode, MAX_TARGET_WARPS_PER_SM * c->num_sms, cols, c->num_sms);
       if (s.nblocks > maxb) maxb = s.nblocks;
     }
   }

@@ -397,7 +397,7 @@ __device__ __forceinline__ void finish_scalars(DevScalars* sc, int kind, double 
 }
 
 // Deterministic two-stage sum of up to two values per thread.  Every thread
-// of the block must call it.  Block partials go to partials[2*blockIdx.x + k];
+// of the block (any number of warps up to NT / 32) must call it.  Block partials go to partials[2*blockIdx.x + k];
 // the last block to arrive (ticket) adds them in block order, runs the
 // finishing action and re-arms the ticket.  No floating-point atomics.
 template <int NT>
@@ -407,6 +407,7 @@ __device__ __forceinline__ void block_reduce_finish(double v0, double v1, double
   __shared__ double red[2][NT / 32];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int nwarps = (int)(blockDim.x >> 5);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     v0 += __shfl_xor_sync(0xffffffffu, v0, o);
@@ -419,7 +420,7 @@ __device__ __forceinline__ void block_reduce_finish(double v0, double v1, double
   __syncthreads();
   if (threadIdx.x == 0) {
     double a = 0.0, b = 0.0;
-    for (int w = 0; w < NT / 32; ++w) {
+    for (int w = 0; w < nwarps; ++w) {
       a += red[0][w];
       b += red[1][w];
     }
@@ -434,7 +435,7 @@ __device__ __forceinline__ void block_reduce_finish(double v0, double v1, double
   // Last block: sum the partials in block order (fixed for a fixed grid).
   __threadfence();
   double a = 0.0, b = 0.0;
-  for (int k = threadIdx.x; k < (int)gridDim.x; k += NT) {
+  for (int k = threadIdx.x; k < (int)gridDim.x; k += (int)blockDim.x) {
     a += ((volatile double*)partials)[2 * k];
     b += ((volatile double*)partials)[2 * k + 1];
   }
@@ -452,7 +453,7 @@ __device__ __forceinline__ void block_reduce_finish(double v0, double v1, double
   __syncthreads();
   if (threadIdx.x == 0) {
     double s0 = 0.0, s1 = 0.0;
-    for (int w = 0; w < NT / 32; ++w) {
+    for (int w = 0; w < nwarps; ++w) {
       s0 += red[0][w];
       s1 += red[1][w];
     }

@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 1) post2_kernel(const SweepParams<fl
   pdl_wait();
   if (a.sc != nullptr && a.gate && a.sc->done != RUNNING) return;  // uniform over the grid
   const int lane = threadIdx.x & 31;
-  const int wg = blockIdx.x * (SWEEP_NT / 32) + (threadIdx.x >> 5);
+  const int wg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   post2_warp<SRC, PF>(a, wg, lane);
 }
 
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 1) pre2_kernel(const SweepParams<flo
   pdl_wait();
   if (a.sc != nullptr && a.gate && a.sc->done != RUNNING) return;  // uniform over the grid
   const int lane = threadIdx.x & 31;
-  const int wg = blockIdx.x * (SWEEP_NT / 32) + (threadIdx.x >> 5);
+  const int wg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   pre2_warp<SRC, PF>(a, wg, lane);
 }
 

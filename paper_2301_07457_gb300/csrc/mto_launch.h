@@ -39,10 +39,17 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t sme
 // Launch shape of a sweep over grid g (see mto_sweep.cuh and mto_sweep2.cuh).
 // target_warps is the number of warps the launch should expose (a multiple of
 // the SM count); cols is the number of node columns per lane (1 or 2).
+//
+// Warps per block: SWEEP_NT / 32, or with spread > 0 (float64 sweeps: the SM
+// count) as few as give each of `spread` SMs a block.  A warp's float64
+// instruction holds an FP64 pipe for many clocks, so a small grid packed into
+// a few 8-warp blocks ran on a few SMs' pipes while the others idled (one
+// float64 64^2 solve 4.58 -> 3.40 ms).  The float32 sweeps are bound by
+// latency there and lose 1-2% with small blocks, so they keep full ones.
 struct SweepShape {
-  int nstrips, nchunks, H, nblocks;
+  int nstrips, nchunks, H, nblocks, nthreads;
 };
-SweepShape sweep_shape(const Grid& g, int mode, int target_warps, int cols);
+SweepShape sweep_shape(const Grid& g, int mode, int target_warps, int cols, int spread = 0);
 
 // Node columns per lane of the instantiation that launch_sweep uses for a
 // float64 (f64) or float32 sweep of source src in mode `mode`.  Two for every

@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(SWEEP_NT) sweep_kernel(const SweepParams<T> a)
     if (a.replace_gate && (a.sc->rr_every <= 0 || (a.sc->iter % a.sc->rr_every) != 0)) return;
   }
   const int lane = threadIdx.x & 31;
-  const int wg = blockIdx.x * (SWEEP_NT / 32) + (threadIdx.x >> 5);
+  const int wg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int strip = wg % a.nstrips;
   const int chunk = wg / a.nstrips;
   double dot0 = 0.0, dot1 = 0.0;

@@ -770,7 +770,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) sweep2_kernel(const SweepParams<T
     if (a.replace_gate && (a.sc->rr_every <= 0 || (a.sc->iter % a.sc->rr_every) != 0)) return;
   }
   const int lane = threadIdx.x & 31;
-  const int wg = blockIdx.x * (SWEEP_NT / 32) + (threadIdx.x >> 5);
+  const int wg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   double dot0 = 0.0, dot1 = 0.0;
   sweep2_warp<T, SRC, MODE, DOT, ZT, PF>(a, wg, lane, dot0, dot1);
   if constexpr (REDUCE) {

@@ -6,7 +6,7 @@
 
 namespace mto {
 
-SweepShape sweep_shape(const Grid& g, int mode, int target_warps, int cols) {
+SweepShape sweep_shape(const Grid& g, int mode, int target_warps, int cols, int spread) {
   SweepShape sh;
   if (mode == MODE_PRE2) {
     // 29 output coarse columns per warp, coarse rows per task as for the
@@ -50,7 +50,10 @@ SweepShape sweep_shape(const Grid& g, int mode, int target_warps, int cols) {
     sh.nchunks = (g.ny + 1 + h - 1) / h;
   }
   const long long warps = (long long)sh.nstrips * sh.nchunks;
-  sh.nblocks = (int)((warps + SWEEP_NT / 32 - 1) / (SWEEP_NT / 32));
+  long long per_block = SWEEP_NT / 32;
+  if (spread > 0 && (warps + spread - 1) / spread < per_block) per_block = (warps + spread - 1) / spread;
+  sh.nthreads = 32 * (int)per_block;
+  sh.nblocks = (int)((warps + per_block - 1) / per_block);
   return sh;
 }
 
@@ -66,11 +69,11 @@ static cudaError_t go(SweepParams<double> p, int tw, int num_sms, cudaStream_t s
     static const int wave = full_wave_warps(kernel, num_sms);  // same for every device of a run
     tw = wave;
   }
-  const SweepShape sh = sweep_shape(p.g, MODE, tw, COLS);
+  const SweepShape sh = sweep_shape(p.g, MODE, tw, COLS, num_sms);
   p.nstrips = sh.nstrips;
   p.nchunks = sh.nchunks;
   p.H = sh.H;
-  return launch_pdl(kernel, sh.nblocks, SWEEP_NT, 0, s, p);
+  return launch_pdl(kernel, sh.nblocks, sh.nthreads, 0, s, p);
 }
 
 template <>
