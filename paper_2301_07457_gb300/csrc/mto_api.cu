@@ -300,7 +300,7 @@ mto_status fine_cycle(mto_ctx* c, DevScalars* sc, bool with_dot, int* final_idx)
     p.b = b;
     p.out = out;
     p.bc = (T2*)C.b;
-    p.E = MIX ? (const void*)c->Ebf : (const void*)c->Ek4;
+    p.E = MIX ? (const void*)c->Ebf : (const void*)c->Efx;
     p.kf = fine_const<T>(c);
     p.invd1 = c->invd1;
     p.wdiag = T(c->w_over_kdiag);
@@ -372,7 +372,7 @@ mto_status fine_resid(mto_ctx* c, const double2* v, const double2* b, double2* o
   p.v = v;
   p.b = b;
   p.out = out;
-  p.E = c->Ek4;
+  p.E = c->Efx;
   p.finish = finish;
   p.xlag = xlag;
   p.xdir = xdir;
@@ -406,7 +406,7 @@ mto_status enqueue_iteration(mto_ctx* c, int par) {
     p.xvec = c->x;
     p.tag = par ^ 1;
     p.out = c->q;
-    p.E = c->Ek4;
+    p.E = c->Efx;
     p.finish = fuse_update(c) ? FIN_PQ_FUSED : FIN_PQ;
     KL(launch_sweep<double>(SRC_FINE64, MODE_KP, false, c->mixed, p,
                             target_warps64(c), c->num_sms, c->cs));
@@ -635,7 +635,7 @@ void design_params(mto_ctx* c, int n_phase, const double* E_phase, double penal)
 // Finest moduli of element rows [j0, j1) from the design copy c->xdes.
 mto_status enqueue_modulus(mto_ctx* c, int j0, int j1) {
   const Grid& gf = c->lv[c->L].g;
-  KL(launch_modulus(gf, c->n_phase, c->xdes, c->ph, c->penal, c->ipenal, c->E64, c->Ebf, c->Ek4,
+  KL(launch_modulus(gf, c->n_phase, c->xdes, c->ph, c->penal, c->ipenal, c->E64, c->Ebf, c->Efx,
                     c->kf64, c->cs, c->num_sms, j0, j1));
   return MTO_OK;
 }
@@ -801,7 +801,7 @@ mto_status make_slot(mto_ctx* c, mto_ctx** out) {
     s->lv[l].coef64 = c->lv[l].coef64;
   }
   s->E64 = c->E64;
-  s->Ek4 = c->Ek4;
+  s->Efx = c->Efx;
   s->Ebf = c->Ebf;
   s->invd1 = c->invd1;
   s->dof_index = c->dof_index;
@@ -1137,7 +1137,7 @@ static mto_status create_impl(mto_ctx* c, int nelx, int nely, double nu, unsigne
   const Grid& gf = c->lv[c->L].g;
   const size_t nf = (size_t)gf.size();
   ST(dalloc_t(c, &c->E64, nf));
-  ST(dalloc_t(c, &c->Ek4, 4 * nf));
+  ST(dalloc_t(c, &c->Efx, 3 * nf));
   if (c->mixed) {
     ST(dalloc_t(c, &c->Ebf, nf));
     ST(dalloc_t(c, &c->r32, nf));
@@ -1533,7 +1533,7 @@ mto_status mto_apply_operator(mto_ctx* c, int level, int use_vcycle_operator, co
     SweepParams<double> p = base_params<double>(c, B.g);
     p.v = c->tmp;
     p.out = c->q;
-    p.E = c->Ek4;
+    p.E = c->Efx;
     KL(launch_sweep<double>(SRC_FINE64, MODE_APPLY, false, false, p,
                             tw, c->num_sms, c->cs));
     KL(launch_unpack(B.g, c->q, y_dev, c->cs, c->num_sms));

@@ -482,7 +482,7 @@ extern "C" mto_status mto_autotune(mto_ctx* c) {
       p.v = (const double2*)B.z[0];
       p.out = (double2*)B.z[1];
       p.b = fine ? c->r : (const double2*)B.b;
-      p.E = c->Ek4;
+      p.E = c->Efx;
       p.invd1 = c->invd1;
       p.coef = (const double*)B.coef;
       p.invd2 = (const double2*)B.invd2;
@@ -501,7 +501,7 @@ extern "C" mto_status mto_autotune(mto_ctx* c) {
       p.cstride = g.size();
       p.v = c->x;
       p.out = c->tmp;
-      p.E = c->Ek4;
+      p.E = c->Efx;
       return launch_sweep<double>(SRC_FINE64, MODE_APPLY, false, false, p,
                                   tw, c->num_sms, c->stream);
     };

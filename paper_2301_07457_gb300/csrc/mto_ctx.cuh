@@ -74,7 +74,7 @@ struct mto_ctx {
   std::vector<mto::LevelBuf> lv;
   // finest level
   double* E64 = nullptr;
-  double* Ek4 = nullptr;  // E (kA, kB, kC, kG) per element, for the float64 sweeps
+  unsigned long long* Efx = nullptr;  // fixed-point element factors of the float64 sweeps, 3 arrays
   __nv_bfloat16* Ebf = nullptr;
   double* invd1 = nullptr;
   double2 *x = nullptr, *r = nullptr, *q = nullptr, *f = nullptr, *tmp = nullptr;

@@ -1,0 +1,243 @@
+// 96-bit fixed-point arithmetic for the float64 element operator.
+//
+// On GB300 the FP64 pipe issues one add, multiply or FMA for about 38 integer
+// instructions of the same warp, so a float64 stencil is bound by that pipe at
+// a fifth of the memory bandwidth.  Almost all of the element operator is sums
+// and differences, which integers do exactly once the values share a scale.
+// The sweeps therefore convert the marched nodal values to integers with one
+// scale per warp, add and multiply them on the integer pipe, and round once,
+// when K v goes back to float64.
+//
+// Scales.  A nodal value is  F 2^(B - 1113)  with B the largest (biased)
+// float64 exponent met by the warp so far: the value with exponent B has its
+// 53 significant bits at bits 38..90 of F, four bits below the sign bit for the
+// strain coordinates (sums of up to eight values).  A value of exponent e is
+// represented exactly down to e = B - 38 and with an absolute error below
+// 2^-90 of the warp's largest value under that.  Element coefficients are
+// 61-bit integers with one exponent X per element; a product keeps the upper
+// 96 of its 157 bits, so forces are  T 2^(B + Xm - 2132)  with Xm the largest X
+// met so far, with the same relation between the largest force and the last
+// bit.  Every sum of the operator fits: |K v| < 2^95 (bounds at the kernel).
+// The results are more accurate than the float64 evaluation, whose every sum
+// rounds at 2^-53 of its own terms, as long as a node's terms are not more
+// than about 2^30 below the largest of the warp's window (30 columns by the
+// rows of the task).
+//
+// The functions also compile as host code (checked against 128-bit
+// arithmetic there).
+#pragma once
+
+#include "mto_common.cuh"
+
+namespace mto {
+
+struct Fx {
+  unsigned lo, mid;
+  int hi;
+};
+
+__host__ __forceinline__ __int128 fx_wide(const Fx& a) {
+  return ((__int128)a.hi << 64) | ((unsigned long long)a.mid << 32) | a.lo;
+}
+__host__ __forceinline__ Fx fx_narrow(__int128 v) {
+  return Fx{(unsigned)v, (unsigned)(v >> 32), (int)(v >> 64)};
+}
+
+__host__ __device__ __forceinline__ Fx fx_add(const Fx& a, const Fx& b) {
+#ifdef __CUDA_ARCH__
+  Fx r;
+  asm("add.cc.u32 %0, %3, %6;\n\taddc.cc.u32 %1, %4, %7;\n\taddc.u32 %2, %5, %8;"
+      : "=r"(r.lo), "=r"(r.mid), "=r"(r.hi)
+      : "r"(a.lo), "r"(a.mid), "r"(a.hi), "r"(b.lo), "r"(b.mid), "r"(b.hi));
+  return r;
+#else
+  return fx_narrow(fx_wide(a) + fx_wide(b));
+#endif
+}
+__host__ __device__ __forceinline__ Fx fx_sub(const Fx& a, const Fx& b) {
+#ifdef __CUDA_ARCH__
+  Fx r;
+  asm("sub.cc.u32 %0, %3, %6;\n\tsubc.cc.u32 %1, %4, %7;\n\tsubc.u32 %2, %5, %8;"
+      : "=r"(r.lo), "=r"(r.mid), "=r"(r.hi)
+      : "r"(a.lo), "r"(a.mid), "r"(a.hi), "r"(b.lo), "r"(b.mid), "r"(b.hi));
+  return r;
+#else
+  return fx_narrow(fx_wide(a) - fx_wide(b));
+#endif
+}
+__host__ __device__ __forceinline__ Fx fx_zero() { return Fx{0u, 0u, 0}; }
+__host__ __device__ __forceinline__ Fx fx_neg(const Fx& a) { return fx_sub(fx_zero(), a); }
+
+// Low 32 bits of (hi:lo) >> s, 0 <= s < 32.
+__host__ __device__ __forceinline__ unsigned fx_funnel(unsigned lo, unsigned hi, int s) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_r(lo, hi, s);
+#else
+  return (unsigned)((((unsigned long long)hi << 32) | lo) >> s);
+#endif
+}
+
+// High 32 bits of (hi:lo) << s, 0 <= s < 32.
+__host__ __device__ __forceinline__ unsigned fx_funnel_left(unsigned lo, unsigned hi, int s) {
+#ifdef __CUDA_ARCH__
+  return __funnelshift_l(lo, hi, s);
+#else
+  return (unsigned)(((((unsigned long long)hi << 32) | lo) << s) >> 32);
+#endif
+}
+
+// a >> s (floor), 0 <= s < 32.
+__host__ __device__ __forceinline__ Fx fx_sar31(const Fx& a, int s) {
+  return Fx{fx_funnel(a.lo, a.mid, s), fx_funnel(a.mid, (unsigned)a.hi, s), a.hi >> s};
+}
+// a >> s by whole limbs: s - s mod 32 bits, any s >= 0.
+__host__ __device__ __forceinline__ Fx fx_sar_limbs(Fx a, int s) {
+  const int sg = a.hi >> 31;
+  if (s >= 64) {
+    a = Fx{(unsigned)a.hi, (unsigned)sg, sg};
+    if (s >= 96) a = Fx{(unsigned)sg, (unsigned)sg, sg};
+  } else if (s >= 32) {
+    a = Fx{a.mid, (unsigned)a.hi, sg};
+  }
+  return a;
+}
+__host__ __device__ __forceinline__ Fx fx_sar(const Fx& a, int s) {
+  return fx_sar31(fx_sar_limbs(a, s), s & 31);
+}
+
+// Biased exponent of a float64 from its upper word (0: zero or subnormal).
+__host__ __device__ __forceinline__ int fx_exponent(unsigned hi) { return (int)((hi >> 20) & 0x7ffu); }
+
+// The bits of a finite float64 with its exponent B >= 1, before the shift to
+// the common scale: F 2^38, upper two limbs (the lowest is zero), with sign.
+__host__ __device__ __forceinline__ Fx fx_significand(unsigned long long bits) {
+  const unsigned hi = (unsigned)(bits >> 32), lo = (unsigned)bits;
+  const unsigned mh = (hi & 0xfffffu) | (fx_exponent(hi) ? 0x100000u : 0u);
+  const unsigned sg = (unsigned)((int)hi >> 31);
+  unsigned u1 = (lo << 6) ^ sg, u2 = ((mh << 6) | (lo >> 26)) ^ sg;
+#ifdef __CUDA_ARCH__
+  asm("sub.cc.u32 %0, %0, %2;\n\tsubc.u32 %1, %1, %2;" : "+r"(u1), "+r"(u2) : "r"(sg));
+#else
+  const unsigned long long t = (((unsigned long long)u2 << 32) | u1) - (((unsigned long long)sg << 32) | sg);
+  u1 = (unsigned)t;
+  u2 = (unsigned)(t >> 32);
+#endif
+  return Fx{0u, u1, (int)u2};
+}
+
+// (w c) >> 64 for 0 <= c < 2^61, up to 2 units low (the lowest of the six
+// partial products and the lower halves of the next two are left out).
+__host__ __device__ __forceinline__ Fx fx_mul(const Fx& w, unsigned long long c) {
+  const unsigned c0 = (unsigned)c, c1 = (unsigned)(c >> 32);
+#ifdef __CUDA_ARCH__
+  const unsigned h0 = __umulhi(w.lo, c1), h1 = __umulhi(w.mid, c0);
+  const unsigned long long x = (unsigned long long)w.mid * c1 + h0;
+  const unsigned long long y = (unsigned long long)(unsigned)w.hi * c0 + h1;
+  // The middle product takes w.hi as unsigned: 2^32 c0 too much when negative.
+  const unsigned corr = (unsigned)(w.hi >> 31) & c0;
+  const long long z = (long long)w.hi * (int)c1 - (long long)corr;
+  const unsigned xl = (unsigned)x, xh = (unsigned)(x >> 32), yl = (unsigned)y, yh = (unsigned)(y >> 32);
+  const unsigned zl = (unsigned)z, zh = (unsigned)((unsigned long long)z >> 32);
+  Fx r;
+  asm("add.cc.u32 %0, %3, %5;\n\taddc.cc.u32 %1, %4, %6;\n\taddc.u32 %2, %8, 0;\n\t"
+      "add.cc.u32 %1, %1, %7;\n\taddc.u32 %2, %2, 0;"
+      : "=&r"(r.lo), "=&r"(r.mid), "=&r"(r.hi)
+      : "r"(xl), "r"(xh), "r"(yl), "r"(yh), "r"(zl), "r"(zh));
+  return r;
+#else
+  const unsigned long long h0 = ((unsigned long long)w.lo * c1) >> 32, h1 = ((unsigned long long)w.mid * c0) >> 32;
+  return fx_narrow((__int128)((unsigned long long)w.mid * c1 + h0) + (__int128)h1 +
+                   (__int128)w.hi * c0 + (((__int128)w.hi * c1) << 32));
+#endif
+}
+
+// v 2^u rounded to float64 (to nearest but for ties, and for the bits dropped
+// below the 64th significant one); subnormal results and overflow as IEEE
+// (rounded twice at most).
+__host__ __device__ __forceinline__ double fx_to_double(const Fx& v, int u) {
+  const unsigned sg = (unsigned)(v.hi >> 31);
+  unsigned a0 = v.lo ^ sg, a1 = v.mid ^ sg, a2 = (unsigned)v.hi ^ sg;
+#ifdef __CUDA_ARCH__
+  asm("sub.cc.u32 %0, %0, %3;\n\tsubc.cc.u32 %1, %1, %3;\n\tsubc.u32 %2, %2, %3;"
+      : "+r"(a0), "+r"(a1), "+r"(a2)
+      : "r"(sg));
+#else
+  {
+    const Fx m = v.hi < 0 ? fx_neg(v) : v;
+    a0 = m.lo;
+    a1 = m.mid;
+    a2 = (unsigned)m.hi;
+  }
+#endif
+  int ex = u + 63 + 32 + 1022;  // biased exponent less one of a 64-bit significand (a2:a1) with its top bit set
+  if (a2 == 0u) {
+    a2 = a1;
+    a1 = a0;
+    a0 = 0u;
+    ex -= 32;
+  }
+  if (a2 == 0u) {
+    a2 = a1;
+    a1 = a0;
+    a0 = 0u;
+    ex -= 32;
+  }
+#ifdef __CUDA_ARCH__
+  const int lz = __clz((int)a2);
+#else
+  const int lz = a2 ? __builtin_clz(a2) : 32;
+#endif
+  a2 = fx_funnel_left(a1, a2, lz & 31);
+  a1 = fx_funnel_left(a0, a1, lz & 31);
+  ex -= lz;
+  if (a2 == 0u) return 0.0;
+  const unsigned long long m = ((unsigned long long)a2 << 32) | a1;
+  const unsigned long long sign = (unsigned long long)(sg & 0x80000000u) << 32;
+  if (ex < 0 || ex >= 2045) {  // outside the normal range
+#ifdef __CUDA_ARCH__
+    const double r = ldexp(__ull2double_rn(m), ex - 63 - 1022);
+#else
+    const double r = __builtin_ldexp((double)m, ex - 63 - 1022);
+#endif
+    return double_of(bits_of(r) | sign);
+  }
+  return double_of(((m >> 11) + ((m >> 10) & 1u) + ((unsigned long long)ex << 52)) | sign);
+}
+
+// Coefficients of a fine element, as the fixed-point sweeps read them: the
+// three scale factors of its core with a common exponent X (the largest of
+// theirs), c = (61-bit integer) with factor = c 2^(X - 1083).  The low four
+// bits of the three words hold X (bits 0-3, 4-7, 8-10) and the common sign
+// (bit 11): at 2^-57 of the largest factor they are far below float64's
+// rounding and stay in the products.
+struct FxCoef {
+  unsigned long long p, c, g;
+};
+__host__ __device__ __forceinline__ unsigned long long fx_coef_word(double f, int X) {
+  const unsigned long long b = bits_of(f);
+  const int e = fx_exponent((unsigned)(b >> 32));
+  unsigned long long m = b & 0xfffffffffffffull;
+  if (e) m |= 0x10000000000000ull;
+  const int s = X - (e ? e : 1);
+  return s < 64 ? (m << 8) >> s : 0ull;
+}
+__host__ __device__ __forceinline__ FxCoef fx_encode(double p, double c, double g) {
+  const unsigned long long bp = bits_of(p);
+  int X = fx_exponent((unsigned)(bp >> 32));
+  const int ec = fx_exponent((unsigned)(bits_of(c) >> 32)), eg = fx_exponent((unsigned)(bits_of(g) >> 32));
+  if (ec > X) X = ec;
+  if (eg > X) X = eg;
+  if (X == 0 && (p != 0.0 || c != 0.0 || g != 0.0)) X = 1;  // subnormal moduli
+  const unsigned tag = (unsigned)X | ((unsigned)(bp >> 63) << 11);
+  FxCoef r = {0ull, 0ull, 0ull};
+  if (X > 0 && X < 0x7ff) r = {fx_coef_word(p, X), fx_coef_word(c, X), fx_coef_word(g, X)};
+  r.p = (r.p & ~15ull) | (tag & 15u);
+  r.c = (r.c & ~15ull) | ((tag >> 4) & 15u);
+  r.g = (r.g & ~15ull) | (tag >> 8);
+  return r;
+}
+__host__ __device__ __forceinline__ unsigned fx_tag(const FxCoef& k) {
+  return ((unsigned)k.p & 15u) | (((unsigned)k.c & 15u) << 4) | (((unsigned)k.g & 15u) << 8);
+}
+
+}  // namespace mto

@@ -1,0 +1,411 @@
+// Marching sweeps of the float64 finest level with the element operator in
+// 96-bit fixed point (mto_fixed.cuh).
+//
+// Same strips, chunks, modes and edge-force bookkeeping as mto_sweep.cuh, one
+// node column per lane.  The marched vector, its update (p = z + beta p_old,
+// v + P z_c, ...) and the node row's result (q, the smoothed z, the residual)
+// are float64; between them every difference, product and sum of the element
+// operator is an integer.  The core is evaluated on sums and differences of
+// c1 and d2: with A[c1,c1] = A[d2,d2] = kA, A[c1,d2] = kB = nu kA and
+// A[s,s] = kG = (kA - kB) / 2,
+//   t_c1 = P + G, t_d2 = P - G,  P = (kA + kB)/2 E (c1 + d2),  G = kG E (c1 - d2),
+// which takes five products of three factors per element instead of seven of
+// four (24 bytes of element data instead of 32).
+//
+// Measured at 2048^2: K p 0.318 -> 0.125 ms (bound before by the FP64 pipe at
+// 36 operations per node; now the ALU pipe is busy 55-65% of the time, the
+// FP64 pipe 40% with the 6 operations of the CG recurrence, DRAM 3 TB/s: 16
+// warps of 128 registers per SM do not fill any of them), the operator alone
+// 0.323 -> 0.152 ms with its layout conversions, relative error against exact
+// arithmetic 2.3e-16 -> 1.8e-16.  A float64 4096^2 solve takes 196 instead of
+// 373 ms, a mixed 2048^2 solve 14.9 instead of 20.9 ms.
+//
+// Bounds (mto_fixed.cuh; |F| < 2^91): edge differences < 2^92, c1, c3, c2, d1,
+// d2, d3 < 2^93, s and c1 +- d2 < 2^94; factors < 2^61, so every product
+// (>> 64) is < 2^91, a node sums at most 14 of them: |K v| < 2^95.
+//
+// Scales are uniform over the warp.  A row whose largest exponent is above B
+// (or an element above Xm) raises it and shifts the carried state; this
+// happens in the first rows of a task and hardly ever after.  A non-finite
+// nodal value enters as zero and marks its row, and every node next to it gets
+// a NaN; a non-finite modulus makes the task's results NaN.
+#pragma once
+
+#include "mto_fixed.cuh"
+#include "mto_sweep.cuh"
+
+namespace mto {
+
+struct Fx2 {
+  Fx x, y;
+};
+__device__ __forceinline__ Fx2 fadd(const Fx2& a, const Fx2& b) { return {fx_add(a.x, b.x), fx_add(a.y, b.y)}; }
+__device__ __forceinline__ Fx2 fsub(const Fx2& a, const Fx2& b) { return {fx_sub(a.x, b.x), fx_sub(a.y, b.y)}; }
+__device__ __forceinline__ Fx2 fsar(const Fx2& a, int s) { return {fx_sar(a.x, s), fx_sar(a.y, s)}; }
+__device__ __forceinline__ Fx fshfl_down(const Fx& a) {
+  return {__shfl_down_sync(0xffffffffu, a.lo, 1), __shfl_down_sync(0xffffffffu, a.mid, 1),
+          __shfl_down_sync(0xffffffffu, a.hi, 1)};
+}
+__device__ __forceinline__ Fx fshfl_up(const Fx& a) {
+  return {__shfl_up_sync(0xffffffffu, a.lo, 1), __shfl_up_sync(0xffffffffu, a.mid, 1),
+          __shfl_up_sync(0xffffffffu, a.hi, 1)};
+}
+__device__ __forceinline__ Fx2 fshfl_down(const Fx2& a) { return {fshfl_down(a.x), fshfl_down(a.y)}; }
+__device__ __forceinline__ Fx2 fshfl_up(const Fx2& a) { return {fshfl_up(a.x), fshfl_up(a.y)}; }
+
+// A finite pair of nodal values at scale B (all lanes of the warp together).
+__device__ __forceinline__ Fx2 fx2_from(const double2& v, int B) {
+  const int sx = B - max(fx_exponent((unsigned)__double2hiint(v.x)), 1);
+  const int sy = B - max(fx_exponent((unsigned)__double2hiint(v.y)), 1);
+  Fx2 r = {fx_significand(bits_of(v.x)), fx_significand(bits_of(v.y))};
+  if (__any_sync(0xffffffffu, (sx | sy) >= 32)) {
+    r.x = fx_sar_limbs(r.x, sx);
+    r.y = fx_sar_limbs(r.y, sy);
+  }
+  return {fx_sar31(r.x, sx & 31), fx_sar31(r.y, sy & 31)};
+}
+
+template <int MODE, bool DOT, typename ZT> struct FSweep {
+  using S = Sweep<double, SRC_FINE64, MODE, DOT, ZT>;
+  static constexpr bool SMOOTHING = S::SMOOTHING;
+  // SMOOTH0 carries the right-hand side and w/D of its top row to the step
+  // that completes it.
+  static constexpr bool LOADS_B = S::NEEDS_B && MODE != MODE_SMOOTH0;
+  static constexpr bool LOADS_D = SMOOTHING && MODE != MODE_SMOOTH0;
+
+  // Loads of one step: node row je + 1, element row je, node row je.
+  struct Pack {
+    double2 v;
+    ZT z;             // KP: z; RESID: the direction of a pending x step
+    double2 c0, c1;   // PSMOOTH: coarse nodes (I, J), (I, J + 1)
+    double dt;        // SMOOTH0: w/D of the top row
+    FxCoef k;
+    double2 b;        // node row je
+    double d;
+    double2 rd, qd;
+  };
+
+  __device__ __forceinline__ static void load_top(const SweepParams<double>& a, long long k, int i, int jj,
+                                                  bool lag, Pack& r) {
+    if constexpr (MODE == MODE_KP) {
+      r.z = static_cast<const ZT*>(a.zkp)[k];
+      r.v = a.v[k];
+    } else if constexpr (MODE == MODE_PSMOOTH) {
+      r.v = a.v[k];
+      // Column i lies on coarse column I = i / 2 or halfway to I + 1 (the next
+      // lane's), row jj on coarse row jj / 2 or halfway to the next.
+      const long long kc = a.gc.at(max(i, 0) >> 1, max(jj, 0) >> 1);
+      r.c0 = a.zc[kc];
+      r.c1 = a.zc[kc + ((jj & 1) ? a.gc.pitch : 0)];
+    } else if constexpr (MODE == MODE_SMOOTH0) {
+      r.v = a.b[k];
+      r.dt = a.invd1[k];
+    } else if constexpr (MODE == MODE_RESID) {
+      r.v = a.v[k];
+      if (lag) r.z = a.xdir[k];
+    } else {
+      r.v = a.v[k];
+    }
+  }
+  __device__ __forceinline__ static void load(const SweepParams<double>& a, long long k, int i, int je,
+                                              bool lag, Pack& r) {
+    load_top(a, k + a.g.pitch, i, je + 1, lag, r);
+    const unsigned long long* E = static_cast<const unsigned long long*>(a.E) + k;
+    r.k.p = __ldg(E);
+    r.k.c = __ldg(E + a.cstride);
+    r.k.g = __ldg(E + 2 * a.cstride);
+    if constexpr (LOADS_B) r.b = a.b[k];
+    if constexpr (LOADS_D) r.d = a.invd1[k];
+    if constexpr (DOT) {
+      r.rd = a.rdot[k];
+      if (a.qdot != nullptr) r.qd = a.qdot[k];
+    }
+  }
+
+  // Marched value of node (i, jj).
+  __device__ __forceinline__ static double2 value(const SweepParams<double>& a, const Pack& r, int i, int jj,
+                                                  double beta, bool lag, double alag) {
+    if constexpr (MODE == MODE_KP) {
+      return make_double2(fma(beta, r.v.x, to_f64(r.z.x)), fma(beta, r.v.y, to_f64(r.z.y)));
+    } else if constexpr (MODE == MODE_PSMOOTH) {
+      // v + w (t + t of column I + 1 where i is odd, else t again), with
+      // t = c0 or c0 + c1: two or three FP64 operations per component.
+      double2 t = r.c0;
+      double w = 0.5;
+      if (jj & 1) {  // uniform over the warp
+        t = make_double2(r.c0.x + r.c1.x, r.c0.y + r.c1.y);
+        w = 0.25;
+      }
+      const double2 tr = shfl_down2(t);  // lane 31: its own value, used only for halo output
+      const bool odd = i & 1;
+      const double2 s = make_double2(t.x + (odd ? tr.x : t.x), t.y + (odd ? tr.y : t.y));
+      return a.g.valid(i, jj) ? make_double2(fma(w, s.x, r.v.x), fma(w, s.y, r.v.y)) : make_double2(0.0, 0.0);
+    } else if constexpr (MODE == MODE_SMOOTH0) {
+      return make_double2(r.dt * r.v.x, r.dt * r.v.y);  // w/D is zero on clamped and ghost nodes
+    } else if constexpr (MODE == MODE_RESID) {
+      if (lag) return make_double2(fma(alag, r.z.x, r.v.x), fma(alag, r.z.y, r.v.y));
+      return r.v;
+    } else {
+      return r.v;
+    }
+  }
+};
+
+// Two resident blocks per SM, as sweep2_kernel.
+template <int MODE, bool DOT, typename ZT, int PF>
+__global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<double> a) {
+  using F = FSweep<MODE, DOT, ZT>;
+  using Pack = typename F::Pack;
+  constexpr bool REDUCE = DOT || MODE == MODE_RESID || MODE == MODE_KP;
+  pdl_wait();
+  if (a.sc != nullptr && a.gate) {
+    if (a.sc->done != RUNNING) return;  // uniform over the grid
+    if (a.replace_gate && (a.sc->rr_every <= 0 || (a.sc->iter % a.sc->rr_every) != 0)) return;
+  }
+  const Grid g = a.g;
+  const int lane = threadIdx.x & 31;
+  const int wg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  const int strip = wg % a.nstrips;
+  const int chunk = wg / a.nstrips;
+  double dot0 = 0.0, dot1 = 0.0;
+  double beta = 0.0, alag = 0.0;
+  bool vzero = false, lag = false;
+  if constexpr (MODE == MODE_KP) {
+    beta = a.sc->beta;
+    lag = a.sc->x_lag != 0;  // K p advances x by the pending step at its owned nodes
+    alag = a.sc->alpha;
+  }
+  if constexpr (MODE == MODE_RESID) {
+    vzero = a.zero_gate && a.sc->x_nonzero == 0;
+    if (a.xlag && a.sc != nullptr && a.sc->x_lag != 0) {  // works on x + alpha p
+      lag = true;
+      alag = a.sc->alpha;
+    }
+  }
+  const double2 zero2 = make_double2(0.0, 0.0);
+
+  if (vzero) {
+    // Residual of a zero iterate: r = b on the free DOFs, no operator needed.
+    const int i = strip * SWEEP_STRIDE - 1 + lane;
+    if (chunk < a.nchunks && lane >= 1 && lane <= 30 && i >= 0 && i <= g.nx) {
+      const int r0 = chunk * a.H, r1 = min(r0 + a.H - 1, g.ny);
+      for (int j = r0; j <= r1; ++j) {
+        const long long k = g.at(i, j);
+        const double2 r = g.is_fixed(i, j) ? zero2 : a.b[k];
+        a.out[k] = r;
+        if (a.out32 != nullptr) a.out32[k] = make_float2(float(r.x), float(r.y));
+        dot0 = fma(r.x, r.x, fma(r.y, r.y, dot0));
+      }
+    }
+  } else if (chunk < a.nchunks) {
+    constexpr int STRIDE = MODE == MODE_RESTRICT ? SWEEP_RSTRIDE : SWEEP_STRIDE;
+    constexpr int SHIFT = MODE == MODE_RESTRICT ? 2 : 1;
+    const int i = strip * STRIDE - SHIFT + lane;
+    int je0, je1, Jb = 0, Je = 0;
+    if constexpr (MODE == MODE_RESTRICT) {
+      Jb = chunk * (a.H >> 1);
+      Je = min(Jb + (a.H >> 1) - 1, a.gc.ny);
+      je0 = max(2 * Jb - 2, -1);
+      je1 = 2 * Je + 1;
+    } else {
+      const int r0 = chunk * a.H;
+      je0 = r0 - 1;
+      je1 = min(r0 + a.H - 1, g.ny);
+    }
+    const bool own_col = lane >= 1 && lane <= 30 && i >= 0 && i <= g.nx;
+    const bool col_fixed = ((g.fixed & 2u) && i == 0) || ((g.fixed & 4u) && i == g.nx);
+    const long long pitch = g.pitch;
+
+    int B = 1, Xm = 0;             // scales of the nodal values and of the coefficients
+    unsigned bad0 = 0, badp = 0;   // lanes with a non-finite value: node rows je, je - 1
+    Fx2 ac = {fx_zero(), fx_zero()}, gbp = ac, gvp = ac, vb = ac;
+    // Marched values of a row at scale B, which the row raises if it has to;
+    // bad: the lanes whose value is not finite (taken as zero).
+    auto to_fixed = [&](double2 v, unsigned& bad) -> Fx2 {
+      bad = 0;
+      const int e = max(fx_exponent((unsigned)__double2hiint(v.x)), fx_exponent((unsigned)__double2hiint(v.y)));
+      if (__any_sync(0xffffffffu, e > B)) {
+        bad = __ballot_sync(0xffffffffu, e == 0x7ff);
+        if (e == 0x7ff) v = zero2;
+        const int Bn = (int)__reduce_max_sync(0xffffffffu, e == 0x7ff ? 0u : (unsigned)e);
+        if (Bn > B) {
+          ac = fsar(ac, Bn - B);
+          vb = fsar(vb, Bn - B);
+          gbp = fsar(gbp, Bn - B);
+          gvp = fsar(gvp, Bn - B);
+          B = Bn;
+        }
+      }
+      return fx2_from(v, B);
+    };
+
+    const long long k0 = g.at(i, je0);
+    double2 vbd;         // marched values of node row je in float64
+    double2 bc = zero2;  // SMOOTH0: right-hand side and w/D of node row je
+    double dc = 0.0;
+    {
+      Pack r0;
+      F::load_top(a, k0, i, je0, lag, r0);
+      vbd = F::value(a, r0, i, je0, beta, lag, alag);
+      const Fx2 vb0 = to_fixed(vbd, bad0);
+      vb = vb0;
+      ac = fsub(fshfl_down(vb), vb);
+      if constexpr (MODE == MODE_SMOOTH0) {
+        bc = r0.v;
+        dc = r0.dt;
+      }
+    }
+    double2 racc = zero2;  // RESTRICT: partial coarse row of this column
+
+    Pack ring[PF];
+#pragma unroll
+    for (int u = 0; u < PF; ++u)
+      if (je0 + u <= je1) F::load(a, k0 + u * pitch, i, je0 + u, lag, ring[u]);
+
+    long long k = k0;  // offset of node / element (i, je)
+    for (int jb = je0; jb <= je1; jb += PF) {
+#pragma unroll
+      for (int u = 0; u < PF; ++u) {
+        const int je = jb + u;
+        if (je > je1) break;
+        const Pack cur = ring[u];
+        if (je + PF <= je1) F::load(a, k + PF * pitch, i, je + PF, lag, ring[u]);
+        if constexpr (MODE == MODE_KP) {
+          // Pending x step at the top row (owned rows only): x += alpha p_old.
+          if (lag && je + 1 <= je1) {  // uniform over the warp
+            double2 x = a.xvec[k + pitch];
+            x = make_double2(fma(alag, cur.v.x, x.x), fma(alag, cur.v.y, x.y));
+            if (own_col) a.xvec[k + pitch] = x;
+          }
+        }
+        // ---- element (i, je) from rows je (vb) and je + 1 (vt) ----
+        const double2 vtd = F::value(a, cur, i, je + 1, beta, lag, alag);
+        unsigned badt;
+        const Fx2 vt = to_fixed(vtd, badt);
+        const Fx2 bt = fsub(fshfl_down(vt), vt);  // top edge (lane 31: zero, used only for halo output)
+        const Fx2 dl = fsub(vt, vb);              // left edge
+        const Fx2 dr = fshfl_down(dl);            // right edge = next lane's left edge
+        Fx c1 = fx_add(ac.x, bt.x), c3 = fx_sub(bt.x, ac.x);
+        const Fx d1 = fx_add(ac.y, bt.y);
+        Fx d3 = fx_sub(bt.y, ac.y);
+        const Fx d2 = fx_add(dl.y, dr.y);
+        Fx s = fx_add(fx_add(dl.x, dr.x), d1);
+        Fx sp = fx_add(c1, d2), sm = fx_sub(c1, d2);
+        const unsigned tag = fx_tag(cur.k);
+        const int X = (int)(tag & 0x7ffu);
+        if (__any_sync(0xffffffffu, X > Xm)) {
+          const int Xn = (int)__reduce_max_sync(0xffffffffu, (unsigned)X);
+          gbp = fsar(gbp, Xn - Xm);
+          gvp = fsar(gvp, Xn - Xm);
+          Xm = Xn;
+        }
+        if (__any_sync(0xffffffffu, tag >= 0x800u)) {  // a negative modulus somewhere in the row
+          if (tag >= 0x800u) {
+            sp = fx_neg(sp);
+            sm = fx_neg(sm);
+            c3 = fx_neg(c3);
+            d3 = fx_neg(d3);
+            s = fx_neg(s);
+          }
+        }
+        Fx tp = fx_mul(sp, cur.k.p), tg = fx_mul(sm, cur.k.g), tc = fx_mul(c3, cur.k.c), td = fx_mul(d3, cur.k.c),
+           ts = fx_mul(s, cur.k.g);
+        const int sh = Xm - X;
+        if (__any_sync(0xffffffffu, sh >= 32)) {
+          tp = fx_sar_limbs(tp, sh);
+          tg = fx_sar_limbs(tg, sh);
+          tc = fx_sar_limbs(tc, sh);
+          td = fx_sar_limbs(td, sh);
+          ts = fx_sar_limbs(ts, sh);
+        }
+        tp = fx_sar31(tp, sh & 31);
+        tg = fx_sar31(tg, sh & 31);
+        tc = fx_sar31(tc, sh & 31);
+        td = fx_sar31(td, sh & 31);
+        ts = fx_sar31(ts, sh & 31);
+        // ---- edge forces and node row je ----
+        const Fx tc1 = fx_add(tp, tg), td2 = fx_sub(tp, tg);
+        const Fx2 gb = {fx_add(tc1, tc), fx_add(ts, td)};                   // top edge of this element
+        const Fx2 gh = fadd(Fx2{fx_sub(tc1, tc), fx_sub(ts, td)}, gbp);     // edge (i, je) -> (i + 1, je)
+        const Fx2 gsv = {ts, td2};
+        const Fx2 gv = fadd(gsv, fshfl_up(gsv));                            // edge (i, je) -> (i, je + 1)
+        const Fx2 kvf = fadd(fsub(fshfl_up(gh), gh), fsub(gvp, gv));
+        const int unit = B + Xm - 2132;
+        double2 kv = make_double2(fx_to_double(kvf.x, unit), fx_to_double(kvf.y, unit));
+        const unsigned badn = badp | bad0 | badt;
+        if (badn != 0u || Xm == 0x7ff) {  // uniform over the warp; neighbours of non-finite values
+          const bool near = ((badn | (badn << 1) | (badn >> 1)) >> lane) & 1u;
+          if (near || Xm == 0x7ff) kv = make_double2(NAN, NAN);
+        }
+
+        const bool inb = je > je0 && own_col && je >= 0 && je <= g.ny;
+        const bool act = inb && !col_fixed && !(((g.fixed & 1u) && je == 0) || ((g.fixed & 8u) && je == g.ny));
+        if constexpr (MODE == MODE_APPLY) {
+          if (inb) a.out[k] = act ? kv : zero2;
+        } else if constexpr (MODE == MODE_RESID) {
+          double2 r = zero2;
+          if (act) r = sub2(cur.b, kv);
+          if (inb) a.out[k] = r;
+          if (inb && a.out32 != nullptr) a.out32[k] = make_float2(float(r.x), float(r.y));
+          dot0 = fma(r.x, r.x, fma(r.y, r.y, dot0));
+        } else if constexpr (MODE == MODE_KP) {
+          const double2 q = act ? kv : zero2;
+          if (inb) {
+            a.p_out[k] = vbd;
+            a.out[k] = q;
+            dot0 = fma(vbd.x, q.x, fma(vbd.y, q.y, dot0));
+          }
+        } else if constexpr (F::SMOOTHING) {
+          const double2 b = MODE == MODE_SMOOTH0 ? bc : cur.b;
+          const double d = MODE == MODE_SMOOTH0 ? dc : cur.d;
+          double2 zn = zero2;
+          if (act) zn = make_double2(fma(d, b.x - kv.x, vbd.x), fma(d, b.y - kv.y, vbd.y));
+          if (inb) a.out[k] = zn;
+          if constexpr (DOT) {
+            if (act) {
+              dot0 = fma(zn.x, cur.rd.x, fma(zn.y, cur.rd.y, dot0));
+              if (a.qdot != nullptr) dot1 = fma(zn.x, cur.qd.x, fma(zn.y, cur.qd.y, dot1));
+            }
+          }
+        } else if constexpr (MODE == MODE_RESTRICT) {
+          double2 r = zero2;
+          if (act) r = sub2(cur.b, kv);
+          // Full weighting, vertically along the march (1/2, 1, 1/2 over fine
+          // rows 2J - 1, 2J, 2J + 1), then horizontally once per coarse row.
+          if (je > je0) {
+            if (je & 1) {
+              const int Jlo = (je - 1) / 2;
+              const double2 col = make_double2(fma(0.5, r.x, racc.x), fma(0.5, r.y, racc.y));
+              const double2 cu = shfl_up2(col), cd = shfl_down2(col);
+              const double2 val = make_double2(fma(0.5, cu.x + cd.x, col.x), fma(0.5, cu.y + cd.y, col.y));
+              const bool producer = (lane & 1) == 0 && lane >= 2 && lane <= 28;
+              const int I = i >> 1;
+              if (producer && Jlo >= Jb && Jlo <= Je && I >= 0 && I <= a.gc.nx)
+                a.bc[a.gc.at(I, Jlo)] = a.gc.is_fixed(I, Jlo) ? zero2 : val;
+              racc = make_double2(0.5 * r.x, 0.5 * r.y);
+            } else {
+              racc = add2(racc, r);
+            }
+          }
+        }
+        if constexpr (MODE == MODE_SMOOTH0) {
+          bc = cur.v;
+          dc = cur.dt;
+        }
+        ac = bt;
+        gbp = gb;
+        gvp = gv;
+        vb = vt;
+        vbd = vtd;
+        badp = bad0;
+        bad0 = badt;
+        k += pitch;
+      }
+    }
+  }
+  if constexpr (REDUCE) {
+    block_reduce_finish<SWEEP_NT>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
+  }
+}
+
+}  // namespace mto

@@ -4,6 +4,7 @@
 
 #include <utility>
 
+#include "mto_fsweep.cuh"
 #include "mto_fused.cuh"
 #include "mto_gemv.cuh"
 #include "mto_sweep2.cuh"
@@ -53,15 +54,13 @@ SweepShape sweep_shape(const Grid& g, int mode, int target_warps, int cols, int 
 
 // Node columns per lane of the instantiation that launch_sweep uses for a
 // float64 (f64) or float32 sweep of source src in mode `mode`.  Two for every
-// float32 sweep (issue- and latency-bound) and for the float64 outer
-// operator sweeps (K p, residuals: 3% less halo work on the FP64 pipe); one
-// for the float64 V-cycle, where a pair of elements (13 float64 coefficients
-// each on coarse levels) needs too many registers.
+// float32 sweep (issue- and latency-bound), one for the float64 sweeps, where
+// a pair of elements (13 float64 coefficients each on coarse levels, 96-bit
+// values on the finest) needs too many registers.
 constexpr int sweep_cols_of(bool f64, int src, int mode) {
-  if (f64) {
-    return (src == SRC_FINE64 && (mode == MODE_KP || mode == MODE_RESID || mode == MODE_APPLY)) ? 2 : 1;
-  }
-  return 2;
+  (void)src;
+  (void)mode;
+  return f64 ? 1 : 2;
 }
 int sweep_cols(bool f64, int src, int mode);
 
@@ -147,10 +146,11 @@ struct PhaseTable {
   double E[16];
 };
 // E_e = sum_i x_{e,i}^penal E_i (Eq. 5); ipenal >= 0 selects repeated products.
-// Also writes E (kA, kB, kC, kG) per element (Ek4, 4 doubles) for the float64 sweeps.
+// Also writes the fixed-point element factors of the float64 sweeps (Efx: three arrays of g.size()
+// words, mto_fixed.cuh).
 // Element rows [j0, j1) (j1 < 0: to the last row).
 cudaError_t launch_modulus(const Grid& g, int n_phase, const double* x, PhaseTable ph, double penal,
-                           int ipenal, double* E64, __nv_bfloat16* Ebf, double* Ek4,
+                           int ipenal, double* E64, __nv_bfloat16* Ebf, unsigned long long* Efx,
                            FineConst<double> kf, cudaStream_t s, int num_sms, int j0 = 0,
                            int j1 = -1);
 // w / D on the float64 finest level (D = KE_00 * sum of the four moduli).

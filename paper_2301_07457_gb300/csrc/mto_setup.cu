@@ -8,6 +8,7 @@
 //   * the coarsest grid (Alg. 1, l = 0): K_0 on the free DOFs in band
 //     storage, its Cholesky factor (Alg. 3), and the explicit K_0^-1;
 //   * sensitivities dC/dx_{e,i} = -p x^{p-1} E_i u_e^T KE u_e (Eq. 6, Sec. 4).
+#include "mto_fixed.cuh"
 #include "mto_launch.h"
 
 namespace mto {
@@ -24,7 +25,7 @@ __device__ __forceinline__ double xpow(double x, double p, int ip) {
 // Element rows [j0, j1).
 __global__ void modulus_kernel(Grid g, int j0, int j1, int n_phase, const double* __restrict__ x,
                                PhaseTable ph, double penal, int ipenal, double* __restrict__ E64,
-                               __nv_bfloat16* __restrict__ Ebf, double* __restrict__ Ek4,
+                               __nv_bfloat16* __restrict__ Ebf, unsigned long long* __restrict__ Efx,
                                FineConst<double> kf) {
   const long long n = (long long)g.nx * g.ny;
   const long long e1 = (long long)j1 * g.nx;
@@ -36,11 +37,11 @@ __global__ void modulus_kernel(Grid g, int j0, int j1, int n_phase, const double
     const long long k = g.at(i, j);
     E64[k] = E;
     if (Ebf) Ebf[k] = __double2bfloat16(E);
-    // The fine element core's four scale factors, stored so that the float64
-    // sweeps spend no FP64 multiplies on them.
-    double2* q = reinterpret_cast<double2*>(Ek4) + 2 * k;
-    q[0] = make_double2(E * kf.kA, E * kf.kB);
-    q[1] = make_double2(E * kf.kC, E * kf.kG);
+    // The three factors of the fixed-point element core (mto_fsweep.cuh).
+    const FxCoef c = fx_encode(E * (0.5 * (kf.kA + kf.kB)), E * kf.kC, E * kf.kG);
+    Efx[k] = c.p;
+    Efx[k + g.size()] = c.c;
+    Efx[k + 2 * g.size()] = c.g;
   }
 }
 
@@ -484,13 +485,13 @@ static int blocks_for(long long n, int num_sms) {
 }
 
 cudaError_t launch_modulus(const Grid& g, int n_phase, const double* x, PhaseTable ph, double penal,
-                           int ipenal, double* E64, __nv_bfloat16* Ebf, double* Ek4,
+                           int ipenal, double* E64, __nv_bfloat16* Ebf, unsigned long long* Efx,
                            FineConst<double> kf, cudaStream_t s, int num_sms, int j0, int j1) {
   if (j1 < 0) j1 = g.ny;
   if (j0 < 0 || j0 > j1 || j1 > g.ny) return cudaErrorInvalidValue;
   if (j0 == j1) return cudaSuccess;
   modulus_kernel<<<blocks_for((long long)g.nx * (j1 - j0), num_sms), 256, 0, s>>>(
-      g, j0, j1, n_phase, x, ph, penal, ipenal, E64, Ebf, Ek4, kf);
+      g, j0, j1, n_phase, x, ph, penal, ipenal, E64, Ebf, Efx, kf);
   return cudaGetLastError();
 }
 
