@@ -108,11 +108,16 @@ __host__ __device__ __forceinline__ Fx fx_sar(const Fx& a, int s) {
 // Biased exponent of a float64 from its upper word (0: zero or subnormal).
 __host__ __device__ __forceinline__ int fx_exponent(unsigned hi) { return (int)((hi >> 20) & 0x7ffu); }
 
-// The bits of a finite float64 with its exponent B >= 1, before the shift to
-// the common scale: F 2^38, upper two limbs (the lowest is zero), with sign.
-__host__ __device__ __forceinline__ Fx fx_significand(unsigned long long bits) {
-  const unsigned hi = (unsigned)(bits >> 32), lo = (unsigned)bits;
-  const unsigned mh = (hi & 0xfffffu) | (fx_exponent(hi) ? 0x100000u : 0u);
+// The significand of a finite float64 before the shift to the common scale
+// (by B - max(exponent, 1)): times 2^38, upper two limbs (the lowest is zero),
+// with sign.  With FLUSH subnormals give zero: where B > FX_FLUSH_B they lie
+// more than 96 bits below the scale.
+constexpr int FX_FLUSH_B = 97;
+template <bool FLUSH> __host__ __device__ __forceinline__ Fx fx_significand(unsigned long long bits) {
+  const unsigned hi = (unsigned)(bits >> 32);
+  const bool normal = (hi & 0x7ff00000u) != 0u;
+  const unsigned lo = FLUSH && !normal ? 0u : (unsigned)bits;
+  const unsigned mh = normal ? (hi & 0xfffffu) | 0x100000u : (FLUSH ? 0u : hi & 0xfffffu);
   const unsigned sg = (unsigned)((int)hi >> 31);
   unsigned u1 = (lo << 6) ^ sg, u2 = ((mh << 6) | (lo >> 26)) ^ sg;
 #ifdef __CUDA_ARCH__
@@ -154,20 +159,20 @@ __host__ __device__ __forceinline__ Fx fx_mul(const Fx& w, unsigned long long c)
 // v 2^u rounded to float64 (to nearest but for ties, and for the bits dropped
 // below the 64th significant one); subnormal results and overflow as IEEE
 // (rounded twice at most).
-__host__ __device__ __forceinline__ double fx_to_double(const Fx& v, int u) {
+//
+// CHECKED = false leaves the exponent's range to the caller, who knows that u
+// lies in [FX_UNIT_MIN, FX_UNIT_MAX] (the result is normal or zero then).
+constexpr int FX_UNIT_MIN = -1020, FX_UNIT_MAX = 920;
+template <bool CHECKED = true> __host__ __device__ __forceinline__ double fx_to_double(const Fx& v, int u) {
   const unsigned sg = (unsigned)(v.hi >> 31);
-  unsigned a0 = v.lo ^ sg, a1 = v.mid ^ sg, a2 = (unsigned)v.hi ^ sg;
 #ifdef __CUDA_ARCH__
+  unsigned a0 = v.lo ^ sg, a1 = v.mid ^ sg, a2 = (unsigned)v.hi ^ sg;
   asm("sub.cc.u32 %0, %0, %3;\n\tsubc.cc.u32 %1, %1, %3;\n\tsubc.u32 %2, %2, %3;"
       : "+r"(a0), "+r"(a1), "+r"(a2)
       : "r"(sg));
 #else
-  {
-    const Fx m = v.hi < 0 ? fx_neg(v) : v;
-    a0 = m.lo;
-    a1 = m.mid;
-    a2 = (unsigned)m.hi;
-  }
+  const Fx mag = v.hi < 0 ? fx_neg(v) : v;
+  unsigned a0 = mag.lo, a1 = mag.mid, a2 = (unsigned)mag.hi;
 #endif
   int ex = u + 63 + 32 + 1022;  // biased exponent less one of a 64-bit significand (a2:a1) with its top bit set
   if (a2 == 0u) {
@@ -190,10 +195,9 @@ __host__ __device__ __forceinline__ double fx_to_double(const Fx& v, int u) {
   a2 = fx_funnel_left(a1, a2, lz & 31);
   a1 = fx_funnel_left(a0, a1, lz & 31);
   ex -= lz;
-  if (a2 == 0u) return 0.0;
   const unsigned long long m = ((unsigned long long)a2 << 32) | a1;
   const unsigned long long sign = (unsigned long long)(sg & 0x80000000u) << 32;
-  if (ex < 0 || ex >= 2045) {  // outside the normal range
+  if (CHECKED && a2 != 0u && (ex < 0 || ex >= 2045)) {  // outside the normal range
 #ifdef __CUDA_ARCH__
     const double r = ldexp(__ull2double_rn(m), ex - 63 - 1022);
 #else
@@ -201,7 +205,8 @@ __host__ __device__ __forceinline__ double fx_to_double(const Fx& v, int u) {
 #endif
     return double_of(bits_of(r) | sign);
   }
-  return double_of(((m >> 11) + ((m >> 10) & 1u) + ((unsigned long long)ex << 52)) | sign);
+  const double r = double_of(((m >> 11) + ((m >> 10) & 1u) + ((unsigned long long)(unsigned)ex << 52)) | sign);
+  return a2 != 0u ? r : 0.0;
 }
 
 // Coefficients of a fine element, as the fixed-point sweeps read them: the

@@ -54,10 +54,14 @@ __device__ __forceinline__ Fx2 fshfl_down(const Fx2& a) { return {fshfl_down(a.x
 __device__ __forceinline__ Fx2 fshfl_up(const Fx2& a) { return {fshfl_up(a.x), fshfl_up(a.y)}; }
 
 // A finite pair of nodal values at scale B (all lanes of the warp together).
+// Zeros take no shift, so that ghost and clamped nodes cost nothing extra.
 __device__ __forceinline__ Fx2 fx2_from(const double2& v, int B) {
-  const int sx = B - max(fx_exponent((unsigned)__double2hiint(v.x)), 1);
-  const int sy = B - max(fx_exponent((unsigned)__double2hiint(v.y)), 1);
-  Fx2 r = {fx_significand(bits_of(v.x)), fx_significand(bits_of(v.y))};
+  const int ex = fx_exponent((unsigned)__double2hiint(v.x)), ey = fx_exponent((unsigned)__double2hiint(v.y));
+  if (B <= FX_FLUSH_B)  // uniform over the warp: values near the subnormal range
+    return {fx_sar(fx_significand<false>(bits_of(v.x)), B - max(ex, 1)),
+            fx_sar(fx_significand<false>(bits_of(v.y)), B - max(ey, 1))};
+  const int sx = ex ? B - ex : 0, sy = ey ? B - ey : 0;
+  Fx2 r = {fx_significand<true>(bits_of(v.x)), fx_significand<true>(bits_of(v.y))};
   if (__any_sync(0xffffffffu, (sx | sy) >= 32)) {
     r.x = fx_sar_limbs(r.x, sx);
     r.y = fx_sar_limbs(r.y, sy);
@@ -90,6 +94,7 @@ template <int MODE, bool DOT, typename ZT> struct FSweep {
     if constexpr (MODE == MODE_KP) {
       r.z = static_cast<const ZT*>(a.zkp)[k];
       r.v = a.v[k];
+      if (lag) r.b = a.xvec[k];
     } else if constexpr (MODE == MODE_PSMOOTH) {
       r.v = a.v[k];
       // Column i lies on coarse column I = i / 2 or halfway to I + 1 (the next
@@ -218,7 +223,10 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
 
     int B = 1, Xm = 0;             // scales of the nodal values and of the coefficients
     unsigned bad0 = 0, badp = 0;   // lanes with a non-finite value: node rows je, je - 1
-    Fx2 ac = {fx_zero(), fx_zero()}, gbp = ac, gvp = ac, vb = ac;
+    // Carried from the row below: edge differences and sums (i + 1 minus / plus
+    // i) of node row je, and the forces of element row je - 1 on its top and
+    // left edges.
+    Fx2 ac = {fx_zero(), fx_zero()}, sc = ac, gbp = ac, gsp = ac;
     // Marched values of a row at scale B, which the row raises if it has to;
     // bad: the lanes whose value is not finite (taken as zero).
     auto to_fixed = [&](double2 v, unsigned& bad) -> Fx2 {
@@ -230,9 +238,9 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         const int Bn = (int)__reduce_max_sync(0xffffffffu, e == 0x7ff ? 0u : (unsigned)e);
         if (Bn > B) {
           ac = fsar(ac, Bn - B);
-          vb = fsar(vb, Bn - B);
+          sc = fsar(sc, Bn - B);
           gbp = fsar(gbp, Bn - B);
-          gvp = fsar(gvp, Bn - B);
+          gsp = fsar(gsp, Bn - B);
           B = Bn;
         }
       }
@@ -247,9 +255,10 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
       Pack r0;
       F::load_top(a, k0, i, je0, lag, r0);
       vbd = F::value(a, r0, i, je0, beta, lag, alag);
-      const Fx2 vb0 = to_fixed(vbd, bad0);
-      vb = vb0;
-      ac = fsub(fshfl_down(vb), vb);
+      const Fx2 vb = to_fixed(vbd, bad0);
+      const Fx2 vr = fshfl_down(vb);
+      ac = fsub(vr, vb);
+      sc = fadd(vr, vb);
       if constexpr (MODE == MODE_SMOOTH0) {
         bc = r0.v;
         dc = r0.dt;
@@ -273,7 +282,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         if constexpr (MODE == MODE_KP) {
           // Pending x step at the top row (owned rows only): x += alpha p_old.
           if (lag && je + 1 <= je1) {  // uniform over the warp
-            double2 x = a.xvec[k + pitch];
+            double2 x = cur.b;
             x = make_double2(fma(alag, cur.v.x, x.x), fma(alag, cur.v.y, x.y));
             if (own_col) a.xvec[k + pitch] = x;
           }
@@ -282,24 +291,23 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         const double2 vtd = F::value(a, cur, i, je + 1, beta, lag, alag);
         unsigned badt;
         const Fx2 vt = to_fixed(vtd, badt);
-        const Fx2 bt = fsub(fshfl_down(vt), vt);  // top edge (lane 31: zero, used only for halo output)
-        const Fx2 dl = fsub(vt, vb);              // left edge
-        const Fx2 dr = fshfl_down(dl);            // right edge = next lane's left edge
+        const Fx2 vr = fshfl_down(vt);  // lane 31: its own value, used only for halo output
+        const Fx2 bt = fsub(vr, vt), st = fadd(vr, vt);
+        const Fx2 up = fsub(st, sc);  // (c2, d2): left plus right edge
         Fx c1 = fx_add(ac.x, bt.x), c3 = fx_sub(bt.x, ac.x);
-        const Fx d1 = fx_add(ac.y, bt.y);
         Fx d3 = fx_sub(bt.y, ac.y);
-        const Fx d2 = fx_add(dl.y, dr.y);
-        Fx s = fx_add(fx_add(dl.x, dr.x), d1);
-        Fx sp = fx_add(c1, d2), sm = fx_sub(c1, d2);
+        Fx s = fx_add(up.x, fx_add(ac.y, bt.y));  // c2 + d1
+        Fx sp = fx_add(c1, up.y), sm = fx_sub(c1, up.y);
+        // X above Xm, more than 31 below it, or the sign bit of a negative
+        // modulus: one vote for the three rare cases (ghost elements have tag 0).
         const unsigned tag = fx_tag(cur.k);
+        const bool rare = __any_sync(0xffffffffu, tag != 0u && (unsigned)(Xm - (int)tag) >= 32u);
         const int X = (int)(tag & 0x7ffu);
-        if (__any_sync(0xffffffffu, X > Xm)) {
-          const int Xn = (int)__reduce_max_sync(0xffffffffu, (unsigned)X);
+        if (rare) {
+          const int Xn = max(Xm, (int)__reduce_max_sync(0xffffffffu, (unsigned)X));
           gbp = fsar(gbp, Xn - Xm);
-          gvp = fsar(gvp, Xn - Xm);
+          gsp = fsar(gsp, Xn - Xm);
           Xm = Xn;
-        }
-        if (__any_sync(0xffffffffu, tag >= 0x800u)) {  // a negative modulus somewhere in the row
           if (tag >= 0x800u) {
             sp = fx_neg(sp);
             sm = fx_neg(sm);
@@ -311,7 +319,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         Fx tp = fx_mul(sp, cur.k.p), tg = fx_mul(sm, cur.k.g), tc = fx_mul(c3, cur.k.c), td = fx_mul(d3, cur.k.c),
            ts = fx_mul(s, cur.k.g);
         const int sh = Xm - X;
-        if (__any_sync(0xffffffffu, sh >= 32)) {
+        if (rare) {
           tp = fx_sar_limbs(tp, sh);
           tg = fx_sar_limbs(tg, sh);
           tc = fx_sar_limbs(tc, sh);
@@ -324,14 +332,18 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         td = fx_sar31(td, sh & 31);
         ts = fx_sar31(ts, sh & 31);
         // ---- edge forces and node row je ----
-        const Fx tc1 = fx_add(tp, tg), td2 = fx_sub(tp, tg);
-        const Fx2 gb = {fx_add(tc1, tc), fx_add(ts, td)};                   // top edge of this element
+        const Fx tc1 = fx_add(tp, tg);
+        const Fx2 gs = {ts, fx_sub(tp, tg)};                                // left and right edge of this element
+        const Fx2 gb = {fx_add(tc1, tc), fx_add(ts, td)};                   // its top edge
         const Fx2 gh = fadd(Fx2{fx_sub(tc1, tc), fx_sub(ts, td)}, gbp);     // edge (i, je) -> (i + 1, je)
-        const Fx2 gsv = {ts, td2};
-        const Fx2 gv = fadd(gsv, fshfl_up(gsv));                            // edge (i, je) -> (i, je + 1)
-        const Fx2 kvf = fadd(fsub(fshfl_up(gh), gh), fsub(gvp, gv));
+        // A node takes gh and the difference of the vertical forces from the
+        // elements on its left (one shuffle for both) and on its right.
+        const Fx2 gd = fsub(gsp, gs);
+        const Fx2 kvf = fadd(fshfl_up(fadd(gd, gh)), fsub(gd, gh));
         const int unit = B + Xm - 2132;
-        double2 kv = make_double2(fx_to_double(kvf.x, unit), fx_to_double(kvf.y, unit));
+        double2 kv = make_double2(fx_to_double<false>(kvf.x, unit), fx_to_double<false>(kvf.y, unit));
+        if (unit < FX_UNIT_MIN || unit > FX_UNIT_MAX)  // uniform over the warp
+          kv = make_double2(fx_to_double(kvf.x, unit), fx_to_double(kvf.y, unit));
         const unsigned badn = badp | bad0 | badt;
         if (badn != 0u || Xm == 0x7ff) {  // uniform over the warp; neighbours of non-finite values
           const bool near = ((badn | (badn << 1) | (badn >> 1)) >> lane) & 1u;
@@ -394,8 +406,8 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         }
         ac = bt;
         gbp = gb;
-        gvp = gv;
-        vb = vt;
+        gsp = gs;
+        sc = st;
         vbd = vtd;
         badp = bad0;
         bad0 = badt;

@@ -47,7 +47,9 @@ int main() {
     const int e = B - (int)(next_u64() % (t % 2 ? 39 : 120));
     const double v = make(next_u64() & 1, e < 0 ? 0 : e, next_u64());
     const int ev = fx_exponent((unsigned)(bits_of(v) >> 32)), sh = B - (ev ? ev : 1);
-    const Fx f = fx_sar(fx_significand(bits_of(v)), sh);
+    const Fx f = fx_sar(fx_significand<false>(bits_of(v)), sh);
+    if (B > FX_FLUSH_B && fx_wide(fx_sar(fx_significand<true>(bits_of(v)), sh)) != (ev ? fx_wide(f) : 0))
+      return fail("flushed", n);
     i128 m = (i128)(bits_of(v) & 0xfffffffffffffull) | (ev ? (i128)1 << 52 : 0);
     m = (v < 0 ? -m : m) << 38;
     if (fx_wide(f) != (m >> (sh > 127 ? 127 : sh))) return fail("from double", n);
@@ -63,6 +65,9 @@ int main() {
 
     // Back to float64: within half a unit in the last place (ties either way).
     const Fx r = random_fx(96);
+    if (fx_to_double<false>(r, FX_UNIT_MAX) != fx_to_double(r, FX_UNIT_MAX) ||
+        fx_to_double<false>(r, FX_UNIT_MIN) != fx_to_double(r, FX_UNIT_MIN))
+      return fail("unchecked", n);
     const i128 R = fx_wide(r);
     const double got = fx_to_double(r, 0), want = (double)R;
     if (got != want) {
