@@ -127,6 +127,7 @@ template <typename T> SweepParams<T> base_params(const mto_ctx* c, const Grid& g
   std::memset(&p, 0, sizeof(p));
   p.g = g;
   p.cstride = g.size();
+  p.gfix = fix_g(c);
   p.partials = c->partials;
   p.ticket = c->ticket;
   return p;
@@ -180,7 +181,8 @@ mto_status coarse_cycle(mto_ctx* c, int l, DevScalars* sc, int start, int* final
     p.b = (const T2*)L.b;
     p.out = out;
     p.bc = (T2*)C.b;
-    p.coef = (const T*)L.coef;
+    if constexpr (sizeof(T) == 4) p.coef = L.coef;
+    else p.E = L.fx;
     p.invd2 = (const T2*)L.invd2;
     set_cmom(c, p);
     if (cfine) set_cfine(c, p);
@@ -688,16 +690,16 @@ mto_status enqueue_hierarchy(mto_ctx* c) {
     if (c->mixed) {
       // Level L-1 rebuilds its elements from the bf16 fine moduli; deeper
       // levels read scaled moments; level 0 is solved directly.
-      if (l < c->L - 1) KL(launch_kmom(B.g, B.mom, c->nu, (float*)B.coef, c->cs, c->num_sms));
+      if (l < c->L - 1) KL(launch_kmom(B.g, B.mom, c->nu, B.coef, c->cs, c->num_sms));
       KL(launch_coarse_invd<float>(B.g, B.mom, c->nu, c->o.omega, (float2*)B.invd2, c->cs, c->num_sms));
     } else {
-      KL(launch_coefs<double>(B.g, B.mom, c->nu, (double*)B.coef, c->cs, c->num_sms));
+      KL(launch_fx_coefs(B.g, B.mom, c->nu, B.fx, c->cs, c->num_sms));
       KL(launch_coarse_invd<double>(B.g, B.mom, c->nu, c->o.omega, (double2*)B.invd2, c->cs,
                                     c->num_sms));
     }
   }
-  if (!c->mixed)  // the float64 level-0 coefficients of the sweeps (apply_operator)
-    KL(launch_coefs<double>(B0.g, B0.mom, c->nu, (double*)B0.coef, c->cs, c->num_sms));
+  // The coarsest level's factors (apply_operator).
+  KL(launch_fx_coefs(B0.g, B0.mom, c->nu, B0.fx, c->cs, c->num_sms));
   CK(cudaStreamWaitEvent(c->cs, c->ev_join, 0));
   return MTO_OK;
 }
@@ -796,6 +798,7 @@ mto_status make_slot(mto_ctx* c, mto_ctx** out) {
   for (int l = 0; l <= c->L; ++l) {
     s->lv[l].g = c->lv[l].g;
     s->lv[l].coef = c->lv[l].coef;
+    s->lv[l].fx = c->lv[l].fx;
     s->lv[l].invd2 = c->lv[l].invd2;
     s->lv[l].mom = c->lv[l].mom;
     s->lv[l].coef64 = c->lv[l].coef64;
@@ -1120,7 +1123,6 @@ static mto_status create_impl(mto_ctx* c, int nelx, int nely, double nu, unsigne
     c->lv[l].g = make_grid(nelx >> sh, nely >> sh, fixed);
   }
   const size_t vsz = c->mixed ? sizeof(float2) : sizeof(double2);
-  const size_t csz = c->mixed ? sizeof(float) : sizeof(double);
   for (int l = 0; l <= c->L; ++l) {
     LevelBuf& B = c->lv[l];
     const size_t n = (size_t)B.g.size();
@@ -1128,7 +1130,8 @@ static mto_status create_impl(mto_ctx* c, int nelx, int nely, double nu, unsigne
     ST(dalloc(c, &B.z[1], n * vsz));
     if (l < c->L) {
       ST(dalloc(c, &B.b, n * vsz));
-      ST(dalloc(c, &B.coef, n * NCOEF * csz));
+      if (c->mixed && l > 0) ST(dalloc_t(c, &B.coef, n * NMOM));
+      if (!c->mixed || l == 0) ST(dalloc_t(c, &B.fx, n * FX_NCOARSE));
       ST(dalloc(c, &B.invd2, n * vsz));
       ST(dalloc_t(c, &B.mom, n * NMOM));
     }
@@ -1137,7 +1140,7 @@ static mto_status create_impl(mto_ctx* c, int nelx, int nely, double nu, unsigne
   const Grid& gf = c->lv[c->L].g;
   const size_t nf = (size_t)gf.size();
   ST(dalloc_t(c, &c->E64, nf));
-  ST(dalloc_t(c, &c->Efx, 3 * nf));
+  ST(dalloc_t(c, &c->Efx, FX_NFINE * nf));
   if (c->mixed) {
     ST(dalloc_t(c, &c->Ebf, nf));
     ST(dalloc_t(c, &c->r32, nf));
@@ -1544,7 +1547,7 @@ mto_status mto_apply_operator(mto_ctx* c, int level, int use_vcycle_operator, co
     p.out = (float2*)B.z[1];
     p.E = c->Ebf;
     p.kf = c->kf32;
-    p.coef = (const float*)B.coef;
+    p.coef = B.coef;
     set_cmom(c, p);
     const bool cfine = level == c->L - 1;
     if (cfine) set_cfine(c, p);
@@ -1561,7 +1564,7 @@ mto_status mto_apply_operator(mto_ctx* c, int level, int use_vcycle_operator, co
     SweepParams<double> p = base_params<double>(c, B.g);
     p.v = vin;
     p.out = vout;
-    p.coef = c->mixed ? B.coef64 : (const double*)B.coef;
+    p.E = B.fx;
     KL(launch_sweep<double>(SRC_COARSE, MODE_APPLY, false, false, p,
                             tw, c->num_sms, c->cs));
     KL(launch_unpack(B.g, vout, y_dev, c->cs, c->num_sms));

@@ -465,7 +465,7 @@ extern "C" mto_status mto_autotune(mto_ctx* c) {
         p.E = c->Ebf;
         p.kf = c->kf32;
         p.wdiag = (float)c->w_over_kdiag;
-        p.coef = (const float*)B.coef;
+        p.coef = B.coef;
         p.invd2 = (const float2*)B.invd2;
         p.cnu = (float)c->nu;
         p.cg = (float)(0.5 * (1.0 - c->nu));
@@ -482,9 +482,9 @@ extern "C" mto_status mto_autotune(mto_ctx* c) {
       p.v = (const double2*)B.z[0];
       p.out = (double2*)B.z[1];
       p.b = fine ? c->r : (const double2*)B.b;
-      p.E = c->Efx;
+      p.E = fine ? (const void*)c->Efx : (const void*)B.fx;
+      p.gfix = fix_g(c);
       p.invd1 = c->invd1;
-      p.coef = (const double*)B.coef;
       p.invd2 = (const double2*)B.invd2;
       return launch_sweep<double>(src, MODE_SMOOTH, false, false, p, tw, c->num_sms, c->stream);
     };

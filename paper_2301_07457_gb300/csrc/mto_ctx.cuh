@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cstdint>
+#include <cmath>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -17,7 +18,8 @@ struct LevelBuf {
   Grid g{};
   void* z[2] = {nullptr, nullptr};  // V2<T> vectors (ping-pong)
   void* b = nullptr;                // right-hand side of this level
-  void* coef = nullptr;             // T coefficients, NCOEF * g.size()
+  float* coef = nullptr;            // float32 levels: scaled moments, NMOM * g.size()
+  unsigned long long* fx = nullptr;  // float64 levels (always level 0): fixed-point factors, FX_NCOARSE * g.size()
   void* invd2 = nullptr;            // V2<T> w / D
   double* mom = nullptr;            // NMOM * g.size() (coarse levels)
   double* coef64 = nullptr;         // level 0: float64 coefficients for the dense matrix
@@ -223,5 +225,9 @@ void invalidate_graphs(mto_ctx* c);
 mto_status ensure_slots(mto_ctx* c, int want, int* got);
 int target_warps(const mto_ctx* c, int level);
 int target_warps64(const mto_ctx* c);
+// g = (1 - nu) / 2 in units of 2^-64 (0 < g < 1), for the fixed-point coarse elements.
+inline unsigned long long fix_g(const mto_ctx* c) {
+  return (unsigned long long)std::ldexp(0.5 * (1.0 - c->nu), 64);
+}
 
 }  // namespace mto

@@ -17,7 +17,8 @@
 // 61-bit integers with one exponent X per element; a product keeps the upper
 // 96 of its 157 bits, so forces are  T 2^(B + Xm - 2132)  with Xm the largest X
 // met so far, with the same relation between the largest force and the last
-// bit.  Every sum of the operator fits: |K v| < 2^95 (bounds at the kernel).
+// bit (coarse elements: 59-bit integers, T 2^(B + Xm - 2130)).  Every sum of
+// the operator fits: |K v| < 2^95 (bounds at the kernel).
 // The results are more accurate than the float64 evaluation, whose every sum
 // rounds at 2^-53 of its own terms, as long as a node's terms are not more
 // than about 2^30 below the largest of the warp's window (30 columns by the
@@ -130,6 +131,20 @@ template <bool FLUSH> __host__ __device__ __forceinline__ Fx fx_significand(unsi
   return Fx{0u, u1, (int)u2};
 }
 
+// Sign change by a mask (0 or -1).
+__host__ __device__ __forceinline__ Fx fx_flip(const Fx& a, int mask) {
+#ifdef __CUDA_ARCH__
+  Fx r;
+  const unsigned m = (unsigned)mask;
+  asm("sub.cc.u32 %0, %3, %6;\n\tsubc.cc.u32 %1, %4, %6;\n\tsubc.u32 %2, %5, %6;"
+      : "=r"(r.lo), "=r"(r.mid), "=r"(r.hi)
+      : "r"(a.lo ^ m), "r"(a.mid ^ m), "r"((unsigned)a.hi ^ m), "r"(m));
+  return r;
+#else
+  return mask ? fx_neg(a) : a;
+#endif
+}
+
 // (w c) >> 64 for 0 <= c < 2^61, up to 2 units low (the lowest of the six
 // partial products and the lower halves of the next two are left out).
 __host__ __device__ __forceinline__ Fx fx_mul(const Fx& w, unsigned long long c) {
@@ -209,40 +224,57 @@ template <bool CHECKED = true> __host__ __device__ __forceinline__ double fx_to_
   return a2 != 0u ? r : 0.0;
 }
 
-// Coefficients of a fine element, as the fixed-point sweeps read them: the
-// three scale factors of its core with a common exponent X (the largest of
-// theirs), c = (61-bit integer) with factor = c 2^(X - 1083).  The low four
-// bits of the three words hold X (bits 0-3, 4-7, 8-10) and the common sign
-// (bit 11): at 2^-57 of the largest factor they are far below float64's
-// rounding and stay in the products.
-struct FxCoef {
-  unsigned long long p, c, g;
-};
-__host__ __device__ __forceinline__ unsigned long long fx_coef_word(double f, int X) {
+// (m << lift) aligned to exponent X, for a factor f of magnitude m 2^(e - 1075).
+__host__ __device__ __forceinline__ unsigned long long fx_coef_word(double f, int X, int lift) {
   const unsigned long long b = bits_of(f);
   const int e = fx_exponent((unsigned)(b >> 32));
   unsigned long long m = b & 0xfffffffffffffull;
   if (e) m |= 0x10000000000000ull;
   const int s = X - (e ? e : 1);
-  return s < 64 ? (m << 8) >> s : 0ull;
+  return s < 64 ? (m << lift) >> s : 0ull;
 }
-__host__ __device__ __forceinline__ FxCoef fx_encode(double p, double c, double g) {
-  const unsigned long long bp = bits_of(p);
-  int X = fx_exponent((unsigned)(bp >> 32));
-  const int ec = fx_exponent((unsigned)(bits_of(c) >> 32)), eg = fx_exponent((unsigned)(bits_of(g) >> 32));
-  if (ec > X) X = ec;
-  if (eg > X) X = eg;
-  if (X == 0 && (p != 0.0 || c != 0.0 || g != 0.0)) X = 1;  // subnormal moduli
-  const unsigned tag = (unsigned)X | ((unsigned)(bp >> 63) << 11);
-  FxCoef r = {0ull, 0ull, 0ull};
-  if (X > 0 && X < 0x7ff) r = {fx_coef_word(p, X), fx_coef_word(c, X), fx_coef_word(g, X)};
-  r.p = (r.p & ~15ull) | (tag & 15u);
-  r.c = (r.c & ~15ull) | ((tag >> 4) & 15u);
-  r.g = (r.g & ~15ull) | (tag >> 8);
-  return r;
+// Common exponent of n factors: the largest of theirs (0 only if all are zero).
+__host__ __device__ __forceinline__ int fx_common_exponent(const double* f, int n) {
+  int X = 0;
+  for (int i = 0; i < n; ++i) {
+    const unsigned hi = (unsigned)(bits_of(f[i]) >> 32);
+    int e = fx_exponent(hi);
+    if (e == 0 && f[i] != 0.0) e = 1;  // subnormal
+    if (e > X) X = e;
+  }
+  return X;
 }
-__host__ __device__ __forceinline__ unsigned fx_tag(const FxCoef& k) {
-  return ((unsigned)k.p & 15u) | (((unsigned)k.c & 15u) << 4) | (((unsigned)k.g & 15u) << 8);
+// The low four bits of an element's first three words hold a 12-bit tag: the
+// exponent X and, in bit 11, that a factor is negative that no positive
+// modulus makes negative.  They are worth at most 2^-55 of the largest factor,
+// below float64's rounding of it, and stay in the products.
+constexpr unsigned FX_TAG_NEG = 0x800u;
+__host__ __device__ __forceinline__ void fx_put_tag(unsigned long long* w, unsigned tag) {
+  for (int i = 0; i < 3; ++i) w[i] = (w[i] & ~15ull) | ((tag >> (4 * i)) & 15u);
+}
+__host__ __device__ __forceinline__ unsigned fx_tag(const unsigned long long* w) {
+  return ((unsigned)w[0] & 15u) | (((unsigned)w[1] & 15u) << 4) | (((unsigned)w[2] & 15u) << 8);
+}
+
+// A fine element: its three factors (p, c, g of mto_fsweep.cuh) as integers
+// below 2^61, factor = c 2^(X - 1083); all of one sign (that of the modulus).
+constexpr int FX_NFINE = 3;
+__host__ __device__ __forceinline__ void fx_encode_fine(double p, double c, double g, unsigned long long* w) {
+  const double f[FX_NFINE] = {p, c, g};
+  const int X = fx_common_exponent(f, FX_NFINE);
+  for (int i = 0; i < FX_NFINE; ++i) w[i] = X < 0x7ff ? fx_coef_word(f[i], X, 8) : 0ull;
+  fx_put_tag(w, (unsigned)X | (bits_of(p) >> 63 ? FX_TAG_NEG : 0u));
+}
+
+// A coarse element: six factors (FxCoarse below) as magnitudes below 2^59 with
+// the sign in bit 63, factor = c 2^(X - 1081).
+constexpr int FX_NCOARSE = 6;
+enum FxCoarse { FXC_M00 = 0, FXC_M10, FXC_M01, FXC_C3C3, FXC_D3D3, FXC_C3D3 };
+__host__ __device__ __forceinline__ void fx_encode_coarse(const double* f, unsigned long long* w) {
+  const int X = fx_common_exponent(f, FX_NCOARSE);
+  for (int i = 0; i < FX_NCOARSE; ++i)
+    w[i] = X < 0x7ff ? fx_coef_word(f[i], X, 6) | (bits_of(f[i]) & 0x8000000000000000ull) : 0ull;
+  fx_put_tag(w, (unsigned)X | (f[FXC_M00] < 0.0 || f[FXC_C3C3] < 0.0 || f[FXC_D3D3] < 0.0 ? FX_TAG_NEG : 0u));
 }
 
 }  // namespace mto

@@ -69,8 +69,75 @@ __device__ __forceinline__ Fx2 fx2_from(const double2& v, int B) {
   return {fx_sar31(r.x, sx & 31), fx_sar31(r.y, sy & 31)};
 }
 
-template <int MODE, bool DOT, typename ZT> struct FSweep {
-  using S = Sweep<double, SRC_FINE64, MODE, DOT, ZT>;
+// Strain-space forces of an element.
+struct FxStrain {
+  Fx c1, c3, d2, d3, s;
+};
+
+// The element operator of a source.  load(): the element's words.  core(): the
+// forces t of the strains w (same basis), at the element's own scale; neg: a
+// factor may be negative that is positive for every positive modulus.
+template <int SRC> struct FxElem;
+template <> struct FxElem<SRC_FINE64> {
+  static constexpr int N = FX_NFINE, UNIT = -2132;
+  __device__ __forceinline__ static FxStrain core(const SweepParams<double>&, FxStrain w, const unsigned long long* k,
+                                                  bool neg) {
+    if (neg && (fx_tag(k) & FX_TAG_NEG))
+      w = {fx_neg(w.c1), fx_neg(w.c3), fx_neg(w.d2), fx_neg(w.d3), fx_neg(w.s)};
+    const Fx p = fx_mul(fx_add(w.c1, w.d2), k[0]), g = fx_mul(fx_sub(w.c1, w.d2), k[2]);
+    return {fx_add(p, g), fx_mul(w.c3, k[1]), fx_sub(p, g), fx_mul(w.d3, k[1]), fx_mul(w.s, k[2])};
+  }
+};
+template <> struct FxElem<SRC_COARSE> {
+  static constexpr int N = FX_NCOARSE, UNIT = -2130;
+  __device__ __forceinline__ static FxStrain core(const SweepParams<double>& a, FxStrain w,
+                                                  const unsigned long long* k, bool neg) {
+    constexpr unsigned long long MAG = 0x7fffffffffffffffull;
+    const unsigned long long m0 = k[FXC_M00] & MAG, m1 = k[FXC_M10] & MAG, m2 = k[FXC_M01] & MAG,
+                             kc = k[FXC_C3C3] & MAG, kd = k[FXC_D3D3] & MAG, k9 = k[FXC_C3D3] & MAG;
+    // g times the moments (g = (1 - nu) / 2 = gfix 2^-64, nu = 1 - 2 g).
+    const unsigned long long g0 = __umul64hi(m0, a.gfix), g1 = __umul64hi(m1, a.gfix), g2 = __umul64hi(m2, a.gfix);
+    const auto mask = [&](int i) -> int { return (int)(k[i] >> 32) >> 31; };
+    const int s1 = mask(FXC_M10), s2 = mask(FXC_M01), s12 = s1 ^ s2, s9 = mask(FXC_C3D3) ^ s12;
+    const Fx c3 = fx_flip(w.c3, s2), d3 = fx_flip(w.d3, s1), s = fx_flip(w.s, s12);
+    const Fx sum = fx_add(w.c1, w.d2);
+    Fx p = fx_mul(sum, m0 - g0), m = fx_mul(fx_sub(w.c1, w.d2), g0), tc = fx_mul(c3, kc), td = fx_mul(d3, kd),
+       ts = fx_mul(s, g0);
+    if (neg) {
+      const int n0 = mask(FXC_M00);
+      p = fx_flip(p, n0);
+      m = fx_flip(m, n0);
+      ts = fx_flip(ts, n0);
+      tc = fx_flip(tc, mask(FXC_C3C3));
+      td = fx_flip(td, mask(FXC_D3D3));
+    }
+    FxStrain t;
+    {
+      const Fx x2 = fx_mul(c3, m2), x1 = fx_mul(d3, m1), both = fx_add(x1, x2);
+      const Fx y2 = fx_mul(c3, g2), y1 = fx_mul(d3, g1);
+      t.c1 = fx_sub(fx_sub(fx_add(fx_add(p, m), both), y1), y1);
+      t.d2 = fx_sub(fx_sub(fx_add(fx_sub(p, m), both), y2), y2);
+    }
+    {
+      const Fx x = fx_mul(sum, m2), y = fx_mul(w.d2, g2);
+      tc = fx_add(tc, fx_sub(fx_sub(x, y), y));
+      tc = fx_add(tc, fx_mul(s, g1));
+      t.c3 = fx_flip(fx_add(tc, fx_flip(fx_mul(d3, k9), s9)), s2);
+    }
+    {
+      const Fx x = fx_mul(sum, m1), y = fx_mul(w.c1, g1);
+      td = fx_add(td, fx_sub(fx_sub(x, y), y));
+      td = fx_add(td, fx_mul(s, g2));
+      t.d3 = fx_flip(fx_add(td, fx_flip(fx_mul(c3, k9), s9)), s1);
+    }
+    t.s = fx_flip(fx_add(ts, fx_add(fx_mul(c3, g1), fx_mul(d3, g2))), s12);
+    return t;
+  }
+};
+
+template <int SRC, int MODE, bool DOT, typename ZT> struct FSweep {
+  using S = Sweep<double, SRC, MODE, DOT, ZT>;
+  using Elem = FxElem<SRC>;
   static constexpr bool SMOOTHING = S::SMOOTHING;
   // SMOOTH0 carries the right-hand side and w/D of its top row to the step
   // that completes it.
@@ -82,13 +149,21 @@ template <int MODE, bool DOT, typename ZT> struct FSweep {
     double2 v;
     ZT z;             // KP: z; RESID: the direction of a pending x step
     double2 c0, c1;   // PSMOOTH: coarse nodes (I, J), (I, J + 1)
-    double dt;        // SMOOTH0: w/D of the top row
-    FxCoef k;
-    double2 b;        // node row je
-    double d;
+    double2 dt;       // SMOOTH0: w/D of the top row
+    unsigned long long k[Elem::N];
+    double2 b;        // node row je (KP: of the top row, the iterate x to be advanced)
+    double2 d;
     double2 rd, qd;
   };
 
+  __device__ __forceinline__ static double2 load_d(const SweepParams<double>& a, long long k) {
+    if constexpr (SRC == SRC_FINE64) {
+      const double d = a.invd1[k];
+      return make_double2(d, d);
+    } else {
+      return a.invd2[k];
+    }
+  }
   __device__ __forceinline__ static void load_top(const SweepParams<double>& a, long long k, int i, int jj,
                                                   bool lag, Pack& r) {
     if constexpr (MODE == MODE_KP) {
@@ -104,7 +179,7 @@ template <int MODE, bool DOT, typename ZT> struct FSweep {
       r.c1 = a.zc[kc + ((jj & 1) ? a.gc.pitch : 0)];
     } else if constexpr (MODE == MODE_SMOOTH0) {
       r.v = a.b[k];
-      r.dt = a.invd1[k];
+      r.dt = load_d(a, k);
     } else if constexpr (MODE == MODE_RESID) {
       r.v = a.v[k];
       if (lag) r.z = a.xdir[k];
@@ -116,11 +191,10 @@ template <int MODE, bool DOT, typename ZT> struct FSweep {
                                               bool lag, Pack& r) {
     load_top(a, k + a.g.pitch, i, je + 1, lag, r);
     const unsigned long long* E = static_cast<const unsigned long long*>(a.E) + k;
-    r.k.p = __ldg(E);
-    r.k.c = __ldg(E + a.cstride);
-    r.k.g = __ldg(E + 2 * a.cstride);
+#pragma unroll
+    for (int n = 0; n < Elem::N; ++n) r.k[n] = __ldg(E + n * a.cstride);
     if constexpr (LOADS_B) r.b = a.b[k];
-    if constexpr (LOADS_D) r.d = a.invd1[k];
+    if constexpr (LOADS_D) r.d = load_d(a, k);
     if constexpr (DOT) {
       r.rd = a.rdot[k];
       if (a.qdot != nullptr) r.qd = a.qdot[k];
@@ -146,7 +220,7 @@ template <int MODE, bool DOT, typename ZT> struct FSweep {
       const double2 s = make_double2(t.x + (odd ? tr.x : t.x), t.y + (odd ? tr.y : t.y));
       return a.g.valid(i, jj) ? make_double2(fma(w, s.x, r.v.x), fma(w, s.y, r.v.y)) : make_double2(0.0, 0.0);
     } else if constexpr (MODE == MODE_SMOOTH0) {
-      return make_double2(r.dt * r.v.x, r.dt * r.v.y);  // w/D is zero on clamped and ghost nodes
+      return make_double2(r.dt.x * r.v.x, r.dt.y * r.v.y);  // w/D is zero on clamped and ghost nodes
     } else if constexpr (MODE == MODE_RESID) {
       if (lag) return make_double2(fma(alag, r.z.x, r.v.x), fma(alag, r.z.y, r.v.y));
       return r.v;
@@ -157,9 +231,9 @@ template <int MODE, bool DOT, typename ZT> struct FSweep {
 };
 
 // Two resident blocks per SM, as sweep2_kernel.
-template <int MODE, bool DOT, typename ZT, int PF>
+template <int SRC, int MODE, bool DOT, typename ZT, int PF>
 __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<double> a) {
-  using F = FSweep<MODE, DOT, ZT>;
+  using F = FSweep<SRC, MODE, DOT, ZT>;
   using Pack = typename F::Pack;
   constexpr bool REDUCE = DOT || MODE == MODE_RESID || MODE == MODE_KP;
   pdl_wait();
@@ -250,7 +324,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
     const long long k0 = g.at(i, je0);
     double2 vbd;         // marched values of node row je in float64
     double2 bc = zero2;  // SMOOTH0: right-hand side and w/D of node row je
-    double dc = 0.0;
+    double2 dc = zero2;
     {
       Pack r0;
       F::load_top(a, k0, i, je0, lag, r0);
@@ -282,9 +356,8 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         if constexpr (MODE == MODE_KP) {
           // Pending x step at the top row (owned rows only): x += alpha p_old.
           if (lag && je + 1 <= je1) {  // uniform over the warp
-            double2 x = cur.b;
-            x = make_double2(fma(alag, cur.v.x, x.x), fma(alag, cur.v.y, x.y));
-            if (own_col) a.xvec[k + pitch] = x;
+            if (own_col)
+              a.xvec[k + pitch] = make_double2(fma(alag, cur.v.x, cur.b.x), fma(alag, cur.v.y, cur.b.y));
           }
         }
         // ---- element (i, je) from rows je (vb) and je + 1 (vt) ----
@@ -294,12 +367,10 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         const Fx2 vr = fshfl_down(vt);  // lane 31: its own value, used only for halo output
         const Fx2 bt = fsub(vr, vt), st = fadd(vr, vt);
         const Fx2 up = fsub(st, sc);  // (c2, d2): left plus right edge
-        Fx c1 = fx_add(ac.x, bt.x), c3 = fx_sub(bt.x, ac.x);
-        Fx d3 = fx_sub(bt.y, ac.y);
-        Fx s = fx_add(up.x, fx_add(ac.y, bt.y));  // c2 + d1
-        Fx sp = fx_add(c1, up.y), sm = fx_sub(c1, up.y);
-        // X above Xm, more than 31 below it, or the sign bit of a negative
-        // modulus: one vote for the three rare cases (ghost elements have tag 0).
+        const FxStrain w = {fx_add(ac.x, bt.x), fx_sub(bt.x, ac.x), up.y, fx_sub(bt.y, ac.y),
+                            fx_add(up.x, fx_add(ac.y, bt.y))};
+        // X above Xm, more than 31 below it, or an unexpected sign: one vote
+        // for the three rare cases (ghost elements have tag 0).
         const unsigned tag = fx_tag(cur.k);
         const bool rare = __any_sync(0xffffffffu, tag != 0u && (unsigned)(Xm - (int)tag) >= 32u);
         const int X = (int)(tag & 0x7ffu);
@@ -308,39 +379,23 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
           gbp = fsar(gbp, Xn - Xm);
           gsp = fsar(gsp, Xn - Xm);
           Xm = Xn;
-          if (tag >= 0x800u) {
-            sp = fx_neg(sp);
-            sm = fx_neg(sm);
-            c3 = fx_neg(c3);
-            d3 = fx_neg(d3);
-            s = fx_neg(s);
-          }
         }
-        Fx tp = fx_mul(sp, cur.k.p), tg = fx_mul(sm, cur.k.g), tc = fx_mul(c3, cur.k.c), td = fx_mul(d3, cur.k.c),
-           ts = fx_mul(s, cur.k.g);
+        FxStrain t = F::Elem::core(a, w, cur.k, rare);
         const int sh = Xm - X;
-        if (rare) {
-          tp = fx_sar_limbs(tp, sh);
-          tg = fx_sar_limbs(tg, sh);
-          tc = fx_sar_limbs(tc, sh);
-          td = fx_sar_limbs(td, sh);
-          ts = fx_sar_limbs(ts, sh);
-        }
-        tp = fx_sar31(tp, sh & 31);
-        tg = fx_sar31(tg, sh & 31);
-        tc = fx_sar31(tc, sh & 31);
-        td = fx_sar31(td, sh & 31);
-        ts = fx_sar31(ts, sh & 31);
+        if (rare)
+          t = {fx_sar_limbs(t.c1, sh), fx_sar_limbs(t.c3, sh), fx_sar_limbs(t.d2, sh), fx_sar_limbs(t.d3, sh),
+               fx_sar_limbs(t.s, sh)};
+        t = {fx_sar31(t.c1, sh & 31), fx_sar31(t.c3, sh & 31), fx_sar31(t.d2, sh & 31), fx_sar31(t.d3, sh & 31),
+             fx_sar31(t.s, sh & 31)};
         // ---- edge forces and node row je ----
-        const Fx tc1 = fx_add(tp, tg);
-        const Fx2 gs = {ts, fx_sub(tp, tg)};                                // left and right edge of this element
-        const Fx2 gb = {fx_add(tc1, tc), fx_add(ts, td)};                   // its top edge
-        const Fx2 gh = fadd(Fx2{fx_sub(tc1, tc), fx_sub(ts, td)}, gbp);     // edge (i, je) -> (i + 1, je)
+        const Fx2 gs = {t.s, t.d2};                                             // left and right edge of this element
+        const Fx2 gb = {fx_add(t.c1, t.c3), fx_add(t.s, t.d3)};                 // its top edge
+        const Fx2 gh = fadd(Fx2{fx_sub(t.c1, t.c3), fx_sub(t.s, t.d3)}, gbp);   // edge (i, je) -> (i + 1, je)
         // A node takes gh and the difference of the vertical forces from the
         // elements on its left (one shuffle for both) and on its right.
         const Fx2 gd = fsub(gsp, gs);
         const Fx2 kvf = fadd(fshfl_up(fadd(gd, gh)), fsub(gd, gh));
-        const int unit = B + Xm - 2132;
+        const int unit = B + Xm + F::Elem::UNIT;
         double2 kv = make_double2(fx_to_double<false>(kvf.x, unit), fx_to_double<false>(kvf.y, unit));
         if (unit < FX_UNIT_MIN || unit > FX_UNIT_MAX)  // uniform over the warp
           kv = make_double2(fx_to_double(kvf.x, unit), fx_to_double(kvf.y, unit));
@@ -369,9 +424,9 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
           }
         } else if constexpr (F::SMOOTHING) {
           const double2 b = MODE == MODE_SMOOTH0 ? bc : cur.b;
-          const double d = MODE == MODE_SMOOTH0 ? dc : cur.d;
+          const double2 d = MODE == MODE_SMOOTH0 ? dc : cur.d;
           double2 zn = zero2;
-          if (act) zn = make_double2(fma(d, b.x - kv.x, vbd.x), fma(d, b.y - kv.y, vbd.y));
+          if (act) zn = make_double2(fma(d.x, b.x - kv.x, vbd.x), fma(d.y, b.y - kv.y, vbd.y));
           if (inb) a.out[k] = zn;
           if constexpr (DOT) {
             if (act) {

@@ -166,6 +166,9 @@ cudaError_t launch_moments_from_coarse(const Grid& gc, const Grid& gf, const dou
 template <typename T>
 cudaError_t launch_coefs(const Grid& g, const double* mom, double nu, T* coef, cudaStream_t s,
                          int num_sms);
+// Fixed-point factors (FX_NCOARSE arrays of g.size() words) of a float64 coarse level.
+cudaError_t launch_fx_coefs(const Grid& g, const double* mom, double nu, unsigned long long* out,
+                            cudaStream_t s, int num_sms);
 // w / D per DOF of a coarse level from its float64 element moments.
 template <typename T>
 cudaError_t launch_coarse_invd(const Grid& g, const double* mom, double nu, double omega,

@@ -38,10 +38,10 @@ __global__ void modulus_kernel(Grid g, int j0, int j1, int n_phase, const double
     E64[k] = E;
     if (Ebf) Ebf[k] = __double2bfloat16(E);
     // The three factors of the fixed-point element core (mto_fsweep.cuh).
-    const FxCoef c = fx_encode(E * (0.5 * (kf.kA + kf.kB)), E * kf.kC, E * kf.kG);
-    Efx[k] = c.p;
-    Efx[k + g.size()] = c.c;
-    Efx[k + 2 * g.size()] = c.g;
+    unsigned long long w[FX_NFINE];
+    fx_encode_fine(E * (0.5 * (kf.kA + kf.kB)), E * kf.kC, E * kf.kG, w);
+#pragma unroll
+    for (int c = 0; c < FX_NFINE; ++c) Efx[k + c * g.size()] = w[c];
   }
 }
 
@@ -155,6 +155,30 @@ __global__ void coefs_kernel(Grid g, const double* __restrict__ mom, double nu, 
                              kap * gs * M01};
 #pragma unroll
     for (int c = 0; c < NCOEF; ++c) coef[c * s + k] = (T)A[c];
+  }
+}
+
+// Fixed-point factors of a float64 coarse level's elements (mto_fixed.cuh).
+__global__ void fx_coefs_kernel(Grid g, const double* __restrict__ mom, double nu,
+                                unsigned long long* __restrict__ out) {
+  const long long n = (long long)g.nx * g.ny;
+  const long long s = g.size();
+  const double kap = 1.0 / (4.0 * (1.0 - nu * nu)), gs = 0.5 * (1.0 - nu);
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n;
+       t += (long long)gridDim.x * blockDim.x) {
+    const long long k = g.at((int)(t % g.nx), (int)(t / g.nx));
+    const double M20 = mom[3 * s + k], M02 = mom[4 * s + k];
+    double f[FX_NCOARSE];
+    f[FXC_M00] = kap * mom[k];
+    f[FXC_M10] = kap * mom[s + k];
+    f[FXC_M01] = kap * mom[2 * s + k];
+    f[FXC_C3C3] = kap * (M02 + gs * M20);
+    f[FXC_D3D3] = kap * (M20 + gs * M02);
+    f[FXC_C3D3] = kap * (nu + gs) * mom[5 * s + k];
+    unsigned long long w[FX_NCOARSE];
+    fx_encode_coarse(f, w);
+#pragma unroll
+    for (int c = 0; c < FX_NCOARSE; ++c) out[c * s + k] = w[c];
   }
 }
 
@@ -525,6 +549,12 @@ cudaError_t launch_coefs(const Grid& g, const double* mom, double nu, T* coef, c
 }
 template cudaError_t launch_coefs<double>(const Grid&, const double*, double, double*, cudaStream_t, int);
 template cudaError_t launch_coefs<float>(const Grid&, const double*, double, float*, cudaStream_t, int);
+
+cudaError_t launch_fx_coefs(const Grid& g, const double* mom, double nu, unsigned long long* out,
+                            cudaStream_t s, int num_sms) {
+  fx_coefs_kernel<<<blocks_for((long long)g.nx * g.ny, num_sms), 256, 0, s>>>(g, mom, nu, out);
+  return cudaGetLastError();
+}
 
 template <typename T>
 cudaError_t launch_coarse_invd(const Grid& g, const double* mom, double nu, double omega,

@@ -89,6 +89,7 @@ template <typename T> struct SweepParams {
   const T* coef;     // coarse element matrices, NCOEF arrays of g.size() (SRC_CMOM: NMOM moments)
   long long cstride;
   T cnu, cg;         // SRC_CMOM: nu and g = (1 - nu) / 2
+  unsigned long long gfix;  // SRC_COARSE: g in units of 2^-64
   FineConst<T> kf;      // bf16 finest level / SRC_CFINE: scale factors of the element core
   Grid gfine;           // SRC_CFINE: the finer grid whose bf16 moduli E points to
   int redisc;           // SRC_CFINE: rediscretised (mean modulus) instead of Galerkin

@@ -64,8 +64,7 @@ static cudaError_t go(SweepParams<double> p, int tw, int num_sms, cudaStream_t s
   constexpr int COLS = sweep_cols_of(true, SRC, MODE);
   void (*kernel)(SweepParams<double>);
   static_assert(COLS == 1, "one column per lane");
-  if constexpr (SRC == SRC_FINE64) kernel = fsweep_kernel<MODE, DOT, ZT, 1>;
-  else kernel = sweep_kernel<double, SRC, MODE, DOT, ZT, 1>;
+  kernel = fsweep_kernel<SRC, MODE, DOT, ZT, 1>;
   if (tw <= 0) {
     static const int wave = full_wave_warps(kernel, num_sms);  // same for every device of a run
     tw = wave;

@@ -81,24 +81,39 @@ int main() {
     if (!(std::fabs(far - ref) <= std::fabs(ref) * 2.3e-16 + 5e-324) && far != ref) return fail("scaled", n);
     if (fx_to_double(fx_zero(), u) != 0.0) return fail("zero", n);
 
-    // Element factors: the three doubles come back from words and exponent.
+    // Element factors: the doubles come back from words and exponent.
     const int ee = 1 + (int)(next_u64() % 2046);
     const double p = make(t & 1, ee, next_u64());
     const double k[3] = {p, p * 0.45, p * 0.69};
-    const FxCoef q = fx_encode(k[0], k[1], k[2]);
-    const unsigned tag = fx_tag(q);
+    unsigned long long q[FX_NCOARSE];
+    fx_encode_fine(k[0], k[1], k[2], q);
+    unsigned tag = fx_tag(q);
     if ((tag >> 11) != (unsigned)(t & 1)) return fail("factor sign", n);
-    const uint64_t words[3] = {q.p, q.c, q.g};
-    for (int i = 0; i < 3; ++i) {
-      if (words[i] >> 61) return fail("factor range", n);
-      const double back = std::ldexp((double)(words[i] & ~15ull), (int)(tag & 0x7ff) - 1083);
+    for (int i = 0; i < FX_NFINE; ++i) {
+      if (q[i] >> 61) return fail("factor range", n);
+      const double back = std::ldexp((double)(q[i] & ~15ull), (int)(tag & 0x7ff) - 1083);
       if (std::fabs(back - std::fabs(k[i])) > std::fabs(p) * 1.2e-16) return fail("factor", n);
     }
+    const double c6[FX_NCOARSE] = {p, p * 0.01, -p * 0.02, p * 0.3, p * 0.31, (t & 2) ? -p * 1e-3 : p * 1e-3};
+    fx_encode_coarse(c6, q);
+    tag = fx_tag(q);
+    if ((tag >> 11) != (unsigned)(t & 1)) return fail("coarse factor sign", n);
+    for (int i = 0; i < FX_NCOARSE; ++i) {
+      const unsigned long long mag = q[i] & ~(1ull << 63);
+      if (mag >> 59) return fail("coarse factor range", n);
+      double back = std::ldexp((double)(mag & ~15ull), (int)(tag & 0x7ff) - 1081);
+      if (q[i] >> 63) back = -back;
+      if (std::fabs(back - c6[i]) > std::fabs(p) * 1.2e-16) return fail("coarse factor", n);
+    }
+    if (fx_wide(fx_flip(a, -1)) != -fx_wide(a) || fx_wide(fx_flip(a, 0)) != fx_wide(a)) return fail("flip", n);
   }
-  const FxCoef z = fx_encode(0.0, 0.0, 0.0);
-  if (z.p || z.c || z.g) return fail("zero factor", n);
-  if ((fx_tag(fx_encode(NAN, NAN, NAN)) & 0x7ff) != 0x7ff) return fail("nan factor", n);
-  if ((fx_tag(fx_encode(INFINITY, 1.0, 1.0)) & 0x7ff) != 0x7ff) return fail("inf factor", n);
+  unsigned long long z[FX_NCOARSE];
+  fx_encode_fine(0.0, 0.0, 0.0, z);
+  if (z[0] || z[1] || z[2]) return fail("zero factor", n);
+  fx_encode_fine(NAN, NAN, NAN, z);
+  if ((fx_tag(z) & 0x7ff) != 0x7ff) return fail("nan factor", n);
+  fx_encode_fine(INFINITY, 1.0, 1.0, z);
+  if ((fx_tag(z) & 0x7ff) != 0x7ff) return fail("inf factor", n);
   std::printf("ok %lld\n", n);
   return 0;
 }
