@@ -680,9 +680,14 @@ mto_status enqueue_hierarchy(mto_ctx* c) {
   KL(launch_band_assemble(B0.g, B0.coef64, c->dof_index, c->n0, c->bw0, c->Kd, c->cs));
   CK(cudaEventRecord(c->ev_fork, c->cs));
   CK(cudaStreamWaitEvent(c->fac_stream, c->ev_fork, 0));
-  KL(launch_cholesky_inverse(c->n0, c->bw0, c->Kd, c->invL, c->Lsc, c->Kinv, c->err_flag, c->fac_stream,
-                             c->num_sms));
-  c->launches += 1;  // the inverse is a second kernel
+  if (c->m0 > 0) {
+    CK(launch_block_inverse(c->n0, c->m0, c->bw0, c->Kd, c->blk, c->Kinv, c->err_flag, c->fac_stream,
+                            &c->launches));
+  } else {
+    KL(launch_cholesky_inverse(c->n0, c->bw0, c->Kd, c->invL, c->Lsc, c->Kinv, c->err_flag, c->fac_stream,
+                               c->num_sms));
+    c->launches += 1;  // the inverse is a second kernel
+  }
   CK(cudaEventRecord(c->ev_join, c->fac_stream));
   if (!c->mixed) KL(launch_fine_invd(gf, c->E64, c->w_over_kdiag, c->invd1, c->cs, c->num_sms));
   for (int l = c->L - 1; l >= 1; --l) {
@@ -788,6 +793,7 @@ mto_status make_slot(mto_ctx* c, mto_ctx** out) {
   s->w_over_kdiag = c->w_over_kdiag;
   s->n0 = c->n0;
   s->bw0 = c->bw0;
+  s->m0 = c->m0;
   if (cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&s->body_stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&s->ev_slot, cudaEventDisableTiming) != cudaSuccess)
@@ -1195,8 +1201,17 @@ static mto_status create_impl(mto_ctx* c, int nelx, int nely, double nu, unsigne
   ST(dalloc_t(c, &c->dof_index, dof.size()));
   CK(cudaMemcpy(c->dof_index, dof.data(), sizeof(int) * dof.size(), cudaMemcpyHostToDevice));
   ST(dalloc_t(c, &c->Kd, (size_t)c->n0 * (c->bw0 + 1)));
-  ST(dalloc_t(c, &c->invL, (size_t)c->n0));
-  ST(dalloc_t(c, &c->Lsc, 2 * (size_t)c->n0 * (c->bw0 + 1)));
+  // DOFs per free node row (the same for every row: whole edges are clamped).
+  int m0 = 0;
+  for (int i = 0; i <= g0.nx; ++i)
+    if (!(((g0.fixed & 2u) && i == 0) || ((g0.fixed & 4u) && i == g0.nx))) m0 += 2;
+  c->m0 = block_inverse_fits(c->n0, m0) ? m0 : 0;
+  if (c->m0 > 0) {
+    ST(dalloc_t(c, &c->blk, 3 * (size_t)c->n0 * c->m0));
+  } else {
+    ST(dalloc_t(c, &c->invL, (size_t)c->n0));
+    ST(dalloc_t(c, &c->Lsc, 2 * (size_t)c->n0 * (c->bw0 + 1)));
+  }
   ST(dalloc_t(c, &c->Kinv, (size_t)c->n0 * c->n0));
   ST(dalloc_t(c, &c->err_flag, 1));
 
@@ -1206,7 +1221,7 @@ static mto_status create_impl(mto_ctx* c, int nelx, int nely, double nu, unsigne
   ST(dalloc_t(c, &c->rhs_stats, MAX_RHS));
   // Opt-in shared memory of the coarsest factorisation, set once here so that
   // set_design can be captured into graphs.
-  CK(prepare_cholesky_inverse(c->n0, c->bw0));
+  CK(c->m0 > 0 ? prepare_block_inverse(c->m0) : prepare_cholesky_inverse(c->n0, c->bw0));
   CK(prepare_coarsest_gemv(c->n0));
   return MTO_OK;
 }

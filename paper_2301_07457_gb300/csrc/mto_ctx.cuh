@@ -90,6 +90,8 @@ struct mto_ctx {
   int n0 = 0, bw0 = 0;
   int* dof_index = nullptr;
   double *Kd = nullptr, *Kinv = nullptr, *invL = nullptr;  // Kd: band storage of K_0 / its factor
+  int m0 = 0;                  // DOFs per free node row where the block inverse is used, else 0
+  double* blk = nullptr;       // its work space, 3 n0 m0
   double* Lsc = nullptr;  // the factor scaled by its columns' and rows' pivots (inverse)
   int* err_flag = nullptr;
   // reductions

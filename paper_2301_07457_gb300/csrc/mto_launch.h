@@ -191,6 +191,15 @@ cudaError_t prepare_cholesky_inverse(int n, int bw);
 // inverse.
 cudaError_t launch_cholesky_inverse(int n, int bw, double* Kb, double* invL, double* Lsc, double* Kinv,
                                     int* err_flag, cudaStream_t s, int num_sms);
+// Explicit inverse of the block tridiagonal coarsest matrix (m DOFs per node
+// row) by nested dissection (mto_coarsest.cu).  Used for rows of at most
+// MAX_BLOCK_ROW DOFs, whose separator blocks fit one block's shared memory.
+// work: 3 n m doubles; *launches counts the kernels.
+constexpr int MAX_BLOCK_ROW = 80;
+bool block_inverse_fits(int n, int m);
+cudaError_t prepare_block_inverse(int m);  // once per size, outside any stream capture
+cudaError_t launch_block_inverse(int n, int m, int bw, const double* Kb, double* work, double* Kinv, int* err_flag,
+                                 cudaStream_t s, long long* launches);
 // dcdx (+)= -penal x^(penal-1) E_i w_e, w_e = u_e^T KE u_e (dense user layouts),
 // on element rows [j0, j1) (j1 < 0: to the last row).
 cudaError_t launch_sensitivity(int nelx, int nely, int n_phase, const double* x, PhaseTable ph,

@@ -253,60 +253,80 @@ __global__ void kmom_kernel(Grid g, const double* __restrict__ mom, double nu, f
 }
 
 // Row r of the coarsest matrix K_0 (free DOF (node (i, j), component c)) in
-// lower band storage: Kb[r * (bw + 1) + d] = K_0[r][r - d], d = 0..bw.
+// lower band storage: Kb[r * (bw + 1) + d] = K_0[r][r - d], d = 0..bw.  Four
+// lanes per row, one for each element around the node: a lane forms its
+// element's row (the row's DOF against the four nodes), and each of the ten
+// entries of the lower triangle is summed over the lanes in a fixed order (one
+// thread per row spent 9 us of FP64 issue on its four elements).
 __global__ void band_assemble_kernel(Grid g, const double* __restrict__ coef,
                                      const int* __restrict__ dof_index, int n, int bw,
                                      double* __restrict__ Kb) {
   const long long s = g.size();
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-    // Find the node of row r: scan is avoided by storing the inverse map in
-    // dof_index's second half (2 * g.size() .. + n).
+  const int lanes = 4 * n;
+  for (int q0 = blockIdx.x * blockDim.x; q0 < lanes; q0 += gridDim.x * blockDim.x) {  // uniform over the block
+    const int q = q0 + threadIdx.x;
+    const bool active = q < lanes;
+    const int r = active ? q >> 2 : n - 1, t = q & 3;
+    // The inverse map of the free DOFs is stored in dof_index's second half.
     const int sidx = dof_index[2 * s + r];
-    const long long k = sidx >> 1;
     const int c = sidx & 1;
+    const long long k = sidx >> 1;
     const int j = (int)(k / g.pitch) - 1, i = (int)(k % g.pitch) - OFFX;
-    double* row = Kb + (long long)r * (bw + 1);
-    const int ei[4] = {i - 1, i, i - 1, i}, ej[4] = {j - 1, j - 1, j, j}, eq[4] = {2, 3, 1, 0};
-    for (int t = 0; t < 4; ++t) {
-      if (ei[t] < 0 || ei[t] >= g.nx || ej[t] < 0 || ej[t] >= g.ny) continue;
-      const long long ke = g.at(ei[t], ej[t]);
-      double A[5][5] = {};
-      A[0][0] = coef[ke];
-      A[0][1] = A[1][0] = coef[s + ke];
-      A[1][1] = coef[2 * s + ke];
-      A[2][2] = coef[3 * s + ke];
-      A[2][3] = A[3][2] = coef[4 * s + ke];
-      A[3][3] = coef[5 * s + ke];
-      A[0][2] = A[2][0] = coef[6 * s + ke];
-      A[0][3] = A[3][0] = coef[7 * s + ke];
-      A[1][2] = A[2][1] = coef[8 * s + ke];
-      A[1][3] = A[3][1] = coef[9 * s + ke];
-      A[4][4] = coef[10 * s + ke];
-      A[1][4] = A[4][1] = coef[11 * s + ke];
-      A[3][4] = A[4][3] = coef[12 * s + ke];
-      // J column of this row's DOF.
-      const int q = eq[t];
-      const double s1 = (q == 1 || q == 2) ? 1.0 : -1.0, s2 = (q >= 2) ? 1.0 : -1.0;
-      const double s3 = s1 * s2;  // s1 s2 = s3 (see elem_diag)
-      double ja[5];
-      if (c == 0) { ja[0] = s1; ja[1] = s3; ja[2] = 0; ja[3] = 0; ja[4] = s2; }
-      else { ja[0] = 0; ja[1] = 0; ja[2] = s2; ja[3] = s3; ja[4] = s1; }
-      double Aj[5];
-      for (int m = 0; m < 5; ++m) {
-        Aj[m] = 0.0;
-        for (int l = 0; l < 5; ++l) Aj[m] += A[m][l] * ja[l];
+    // Element t: (i - 1, j - 1), (i, j - 1), (i - 1, j), (i, j), where the node is TR, TL, BR, BL.
+    const int ei = i - 1 + (t & 1), ej = j - 1 + (t >> 1);
+    double e[4][2] = {};  // against the element's nodes BL, BR, TR, TL
+    if (active && ei >= 0 && ei < g.nx && ej >= 0 && ej < g.ny) {
+      double A[NCOEF];
+#pragma unroll
+      for (int m = 0; m < NCOEF; ++m) A[m] = coef[m * s + g.at(ei, ej)];
+      // A times the J column of this row's DOF (s1, s2, s3 of elem_diag).
+      const double s1 = (t & 1) ? -1.0 : 1.0, s2 = (t >> 1) ? -1.0 : 1.0, s3 = s1 * s2;
+      double a1, a3, b2, b3, ss;
+      if (c == 0) {  // (s1, s3, 0, 0, s2)
+        a1 = s1 * A[0] + s3 * A[1];
+        a3 = s1 * A[1] + s3 * A[2] + s2 * A[11];
+        b2 = s1 * A[6] + s3 * A[8];
+        b3 = s1 * A[7] + s3 * A[9] + s2 * A[12];
+        ss = s3 * A[11] + s2 * A[10];
+      } else {  // (0, 0, s2, s3, s1)
+        a1 = s2 * A[6] + s3 * A[7];
+        a3 = s2 * A[8] + s3 * A[9] + s1 * A[11];
+        b2 = s2 * A[3] + s3 * A[4];
+        b3 = s2 * A[4] + s3 * A[5] + s1 * A[12];
+        ss = s3 * A[12] + s1 * A[10];
       }
-      // Element nodes: BL (ei, ej), BR, TR, TL.
-      const int ni[4] = {ei[t], ei[t] + 1, ei[t] + 1, ei[t]}, nj[4] = {ej[t], ej[t], ej[t] + 1, ej[t] + 1};
+#pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const double t1 = (m == 1 || m == 2) ? 1.0 : -1.0, t2 = (m >= 2) ? 1.0 : -1.0;
-        const double t3 = t1 * t2;
-        const long long kn = g.at(ni[m], nj[m]);
-        const double ex = Aj[0] * t1 + Aj[1] * t3 + Aj[4] * t2;  // u_x column of node m
-        const double ey = Aj[2] * t2 + Aj[3] * t3 + Aj[4] * t1;  // u_y column
+        const double t1 = (m == 1 || m == 2) ? 1.0 : -1.0, t2 = (m >= 2) ? 1.0 : -1.0, t3 = t1 * t2;
+        e[m][0] = t1 * a1 + t3 * a3 + t2 * ss;
+        e[m][1] = t2 * b2 + t3 * b3 + t1 * ss;
+      }
+    }
+    // Nodes (i + di, j + dj) of the row and the row below, first the own one.
+    double* row = Kb + (long long)r * (bw + 1);
+#pragma unroll
+    for (int w = 0; w < 5; ++w) {
+      const int di = w == 0 ? 0 : (w == 1 ? -1 : w - 3), dj = w < 2 ? 0 : -1;
+      // The node's corner in this lane's element: column di + 1 - (t & 1), row dj + 1 - (t >> 1).
+      const int col = di + 1 - (t & 1), rw = dj + 1 - (t >> 1);
+      const bool in = col >= 0 && col <= 1 && rw >= 0 && rw <= 1;
+      double x = 0.0, y = 0.0;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const bool hit = in && m == (rw ? 3 - col : col);
+        x = hit ? e[m][0] : x;
+        y = hit ? e[m][1] : y;
+      }
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, o);
+        y += __shfl_xor_sync(0xffffffffu, y, o);
+      }
+      if (active && t == 0 && i + di >= 0 && i + di <= g.nx && j + dj >= 0) {
+        const long long kn = g.at(i + di, j + dj);
         const int cx = dof_index[2 * kn], cy = dof_index[2 * kn + 1];
-        if (cx >= 0 && cx <= r && r - cx <= bw) row[r - cx] += ex;
-        if (cy >= 0 && cy <= r && r - cy <= bw) row[r - cy] += ey;
+        if (cx >= 0 && cx <= r && r - cx <= bw) row[r - cx] = x;
+        if (cy >= 0 && cy <= r && r - cy <= bw) row[r - cy] = y;
       }
     }
   }
@@ -576,7 +596,7 @@ cudaError_t launch_kmom(const Grid& g, const double* mom, double nu, float* out,
 
 cudaError_t launch_band_assemble(const Grid& g, const double* coef64, const int* dof_index, int n,
                                  int bw, double* Kb, cudaStream_t s) {
-  band_assemble_kernel<<<(n + 127) / 128, 128, 0, s>>>(g, coef64, dof_index, n, bw, Kb);
+  band_assemble_kernel<<<(4 * n + 127) / 128, 128, 0, s>>>(g, coef64, dof_index, n, bw, Kb);
   return cudaGetLastError();
 }
 
