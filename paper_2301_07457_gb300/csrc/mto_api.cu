@@ -1546,16 +1546,31 @@ mto_status mto_apply_operator(mto_ctx* c, int level, int use_vcycle_operator, co
   LevelBuf& B = c->lv[level];
   const int tw = target_warps(c, level);
   const bool fine = level == c->L;
-  if (fine && (!c->mixed || !use_vcycle_operator)) {
-    KL(launch_pack(B.g, v_dev, c->tmp, c->cs, c->num_sms));
+  if (!c->mixed || level == 0 || (fine && !use_vcycle_operator)) {
+    // float64 operators (the mixed cycle's coarsest level is float64 too):
+    // one sweep between the caller's arrays, without copies into the padded
+    // layout (at 2048^2 those were a quarter of the call), unless the arrays
+    // overlap.
     SweepParams<double> p = base_params<double>(c, B.g);
-    p.v = c->tmp;
-    p.out = c->q;
-    p.E = c->Efx;
-    KL(launch_sweep<double>(SRC_FINE64, MODE_APPLY, false, false, p,
-                            tw, c->num_sms, c->cs));
-    KL(launch_unpack(B.g, c->q, y_dev, c->cs, c->num_sms));
-  } else if (c->mixed && level > 0) {
+    const size_t bytes = sizeof(double2) * (size_t)(B.g.nx + 1) * (B.g.ny + 1);
+    const uintptr_t va = reinterpret_cast<uintptr_t>(v_dev), ya = reinterpret_cast<uintptr_t>(y_dev);
+    const bool direct = va + bytes <= ya || ya + bytes <= va;
+    if (direct) {
+      p.dense = 1;
+      p.v = reinterpret_cast<const double2*>(v_dev);
+      p.out = reinterpret_cast<double2*>(y_dev);
+    } else {
+      // Float32 level vectors: the finest level's float64 scratch vectors
+      // (larger than any coarse grid) hold the operands.
+      p.out = fine || c->mixed ? c->q : (double2*)B.z[1];
+      double2* vin = fine || c->mixed ? c->tmp : (double2*)B.z[0];
+      KL(launch_pack(B.g, v_dev, vin, c->cs, c->num_sms));
+      p.v = vin;
+    }
+    p.E = fine ? c->Efx : B.fx;
+    KL(launch_sweep<double>(fine ? SRC_FINE64 : SRC_COARSE, MODE_APPLY, false, false, p, tw, c->num_sms, c->cs));
+    if (!direct) KL(launch_unpack(B.g, p.out, y_dev, c->cs, c->num_sms));
+  } else {
     KL(launch_pack_f32(B.g, v_dev, (float2*)B.z[0], c->cs, c->num_sms));
     SweepParams<float> p = base_params<float>(c, B.g);
     p.v = (const float2*)B.z[0];
@@ -1569,20 +1584,6 @@ mto_status mto_apply_operator(mto_ctx* c, int level, int use_vcycle_operator, co
     KL(launch_sweep<float>(fine ? SRC_FINEBF : (cfine ? SRC_CFINE : SRC_CMOM), MODE_APPLY, false,
                            false, p, tw, c->num_sms, c->cs));
     KL(launch_unpack_f32(B.g, (const float2*)B.z[1], y_dev, c->cs, c->num_sms));
-  } else {
-    // float64 coarse levels.  The mixed cycle's coarsest level is float64
-    // too; its level vectors are float2, so the finest level's float64
-    // scratch vectors (larger than any coarse grid) hold the operands.
-    double2* vin = c->mixed ? c->tmp : (double2*)B.z[0];
-    double2* vout = c->mixed ? c->q : (double2*)B.z[1];
-    KL(launch_pack(B.g, v_dev, vin, c->cs, c->num_sms));
-    SweepParams<double> p = base_params<double>(c, B.g);
-    p.v = vin;
-    p.out = vout;
-    p.E = B.fx;
-    KL(launch_sweep<double>(SRC_COARSE, MODE_APPLY, false, false, p,
-                            tw, c->num_sms, c->cs));
-    KL(launch_unpack(B.g, vout, y_dev, c->cs, c->num_sms));
   }
   return leave(c);
 }
@@ -1592,13 +1593,13 @@ mto_status mto_apply_preconditioner(mto_ctx* c, const double* r_dev, double* z_d
   if (!c->has_design) return MTO_ERR_STATE;
   ST(enter(c));
   LevelBuf& B = c->lv[c->L];
-  KL(launch_pack(B.g, r_dev, c->r, c->cs, c->num_sms));
   int zi = 0;
-  if (c->mixed) {
+  if (c->mixed) {  // the float32 cycle reads r32 alone
     KL(launch_pack_f32(B.g, r_dev, c->r32, c->cs, c->num_sms));
     ST(fine_cycle<float>(c, nullptr, false, &zi));
     KL(launch_unpack_f32(B.g, (const float2*)B.z[zi], z_dev, c->cs, c->num_sms));
   } else {
+    KL(launch_pack(B.g, r_dev, c->r, c->cs, c->num_sms));
     ST(fine_cycle<double>(c, nullptr, false, &zi));
     KL(launch_unpack(B.g, (const double2*)B.z[zi], z_dev, c->cs, c->num_sms));
   }

@@ -183,6 +183,13 @@ template <int SRC, int MODE, bool DOT, typename ZT> struct FSweep {
     } else if constexpr (MODE == MODE_RESID) {
       r.v = a.v[k];
       if (lag) r.z = a.xdir[k];
+    } else if constexpr (MODE == MODE_APPLY) {
+      if (a.dense) {  // the caller's vector: clamped nodes are read as zero, ghosts do not exist
+        r.v = make_double2(0.0, 0.0);
+        if (a.g.active(i, jj)) r.v = a.v[(long long)jj * (a.g.nx + 1) + i];
+      } else {
+        r.v = a.v[k];
+      }
     } else {
       r.v = a.v[k];
     }
@@ -408,7 +415,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         const bool inb = je > je0 && own_col && je >= 0 && je <= g.ny;
         const bool act = inb && !col_fixed && !(((g.fixed & 1u) && je == 0) || ((g.fixed & 8u) && je == g.ny));
         if constexpr (MODE == MODE_APPLY) {
-          if (inb) a.out[k] = act ? kv : zero2;
+          if (inb) a.out[a.dense ? (long long)je * (g.nx + 1) + i : k] = act ? kv : zero2;
         } else if constexpr (MODE == MODE_RESID) {
           double2 r = zero2;
           if (act) r = sub2(cur.b, kv);

@@ -15,8 +15,8 @@ namespace mto {
 
 __device__ __forceinline__ double xpow(double x, double p, int ip) {
   if (ip >= 0) {
-    double r = 1.0;
-    for (int k = 0; k < ip; ++k) r *= x;
+    double r = ip > 0 ? x : 1.0;
+    for (int k = 1; k < ip; ++k) r *= x;
     return r;
   }
   return pow(x, p);

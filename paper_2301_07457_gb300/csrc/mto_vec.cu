@@ -158,68 +158,61 @@ __global__ void __launch_bounds__(VEC_NT)
   block_reduce_finish<VEC_NT>(acc0 + acc1, 0.0, partials, ticket, sc, finish, out_value);
 }
 
+// Layout conversions between the caller's arrays and the padded grids: each
+// block walks whole rows, so that no thread divides by a row length (the
+// 64-bit divisions of a linear index cost more than the copy).
+template <typename F> __device__ __forceinline__ void for_row_entries(int j0, int j1, int i0, int i1, F fn) {
+  for (int j = j0 + (int)blockIdx.x; j < j1; j += (int)gridDim.x)
+    for (int i = i0 + (int)threadIdx.x; i < i1; i += (int)blockDim.x) fn(i, j);
+}
+
 __global__ void pack_kernel(Grid g, const double* __restrict__ src, double2* __restrict__ dst,
                             int* nonzero) {
-  const long long n = g.size();
   bool nz = false;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-       k += (long long)gridDim.x * blockDim.x) {
-    int i, j;
-    node_of(g, k, i, j);
+  for_row_entries(-1, g.rows - 1, -OFFX, g.pitch - OFFX, [&](int i, int j) {
     double2 v = make_double2(0.0, 0.0);
     if (g.active(i, j)) {
       const long long s = 2 * ((long long)j * (g.nx + 1) + i);
       v = make_double2(src[s], src[s + 1]);
-      nz = nz || v.x != 0.0 || v.y != 0.0;
+      // Bits other than the sign: no comparison on the FP64 pipe (NaN counts as non-zero).
+      nz = nz || ((bits_of(v.x) | bits_of(v.y)) << 1) != 0ull;
     }
-    dst[k] = v;
-  }
+    dst[g.at(i, j)] = v;
+  });
   if (nonzero != nullptr && __any_sync(0xffffffffu, nz) && (threadIdx.x & 31) == 0) atomicOr(nonzero, 1);
 }
 
 __global__ void unpack_kernel(Grid g, const double2* __restrict__ src, double* __restrict__ dst) {
-  const long long n = (long long)(g.nx + 1) * (g.ny + 1);
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-       k += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(k % (g.nx + 1)), j = (int)(k / (g.nx + 1));
+  for_row_entries(0, g.ny + 1, 0, g.nx + 1, [&](int i, int j) {
     const double2 v = src[g.at(i, j)];
-    dst[2 * k] = v.x;
-    dst[2 * k + 1] = v.y;
-  }
+    const long long k = 2 * ((long long)j * (g.nx + 1) + i);
+    dst[k] = v.x;
+    dst[k + 1] = v.y;
+  });
 }
 
 __global__ void pack_f32_kernel(Grid g, const double* __restrict__ src, float2* __restrict__ dst) {
-  const long long n = g.size();
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-       k += (long long)gridDim.x * blockDim.x) {
-    int i, j;
-    node_of(g, k, i, j);
+  for_row_entries(-1, g.rows - 1, -OFFX, g.pitch - OFFX, [&](int i, int j) {
     float2 v = make_float2(0.f, 0.f);
     if (g.active(i, j)) {
       const long long s = 2 * ((long long)j * (g.nx + 1) + i);
       v = make_float2((float)src[s], (float)src[s + 1]);
     }
-    dst[k] = v;
-  }
+    dst[g.at(i, j)] = v;
+  });
 }
 
 __global__ void unpack_f32_kernel(Grid g, const float2* __restrict__ src, double* __restrict__ dst) {
-  const long long n = (long long)(g.nx + 1) * (g.ny + 1);
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-       k += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(k % (g.nx + 1)), j = (int)(k / (g.nx + 1));
+  for_row_entries(0, g.ny + 1, 0, g.nx + 1, [&](int i, int j) {
     const float2 v = src[g.at(i, j)];
-    dst[2 * k] = v.x;
-    dst[2 * k + 1] = v.y;
-  }
+    const long long k = 2 * ((long long)j * (g.nx + 1) + i);
+    dst[k] = v.x;
+    dst[k + 1] = v.y;
+  });
 }
 
 __global__ void unpack_elems_kernel(Grid g, const double* __restrict__ src, double* __restrict__ dst) {
-  const long long n = (long long)g.nx * g.ny;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n;
-       k += (long long)gridDim.x * blockDim.x) {
-    dst[k] = src[g.at((int)(k % g.nx), (int)(k / g.nx))];
-  }
+  for_row_entries(0, g.ny, 0, g.nx, [&](int i, int j) { dst[(long long)j * g.nx + i] = src[g.at(i, j)]; });
 }
 
 // One warp per row of K_0^-1; every block stages the free coarse right-hand
@@ -332,25 +325,30 @@ cudaError_t launch_dot(long long n, const double2* a, const double2* b, double* 
 
 cudaError_t launch_pack(const Grid& g, const double* src, double2* dst, cudaStream_t s, int num_sms,
                         int* nonzero) {
-  pack_kernel<<<vec_blocks(g.size(), num_sms), VEC_NT, 0, s>>>(g, src, dst, nonzero);
+  (void)num_sms;
+  pack_kernel<<<g.rows, VEC_NT, 0, s>>>(g, src, dst, nonzero);
   return cudaGetLastError();
 }
 cudaError_t launch_unpack(const Grid& g, const double2* src, double* dst, cudaStream_t s, int num_sms) {
-  unpack_kernel<<<vec_blocks((long long)(g.nx + 1) * (g.ny + 1), num_sms), VEC_NT, 0, s>>>(g, src, dst);
+  (void)num_sms;
+  unpack_kernel<<<g.ny + 1, VEC_NT, 0, s>>>(g, src, dst);
   return cudaGetLastError();
 }
 cudaError_t launch_pack_f32(const Grid& g, const double* src, float2* dst, cudaStream_t s, int num_sms) {
-  pack_f32_kernel<<<vec_blocks(g.size(), num_sms), VEC_NT, 0, s>>>(g, src, dst);
+  (void)num_sms;
+  pack_f32_kernel<<<g.rows, VEC_NT, 0, s>>>(g, src, dst);
   return cudaGetLastError();
 }
 cudaError_t launch_unpack_f32(const Grid& g, const float2* src, double* dst, cudaStream_t s, int num_sms) {
-  unpack_f32_kernel<<<vec_blocks((long long)(g.nx + 1) * (g.ny + 1), num_sms), VEC_NT, 0, s>>>(g, src, dst);
+  (void)num_sms;
+  unpack_f32_kernel<<<g.ny + 1, VEC_NT, 0, s>>>(g, src, dst);
   return cudaGetLastError();
 }
 
 cudaError_t launch_unpack_elems(const Grid& g, const double* src, double* dst, cudaStream_t s,
                                 int num_sms) {
-  unpack_elems_kernel<<<vec_blocks((long long)g.nx * g.ny, num_sms), VEC_NT, 0, s>>>(g, src, dst);
+  (void)num_sms;
+  unpack_elems_kernel<<<g.ny, VEC_NT, 0, s>>>(g, src, dst);
   return cudaGetLastError();
 }
 
