@@ -8,6 +8,7 @@
 // host round trip happens inside a solve.  With kernel timing on, the loop is
 // driven from the host instead (graph of two iterations, polled), because
 // event records cannot live inside a conditional body.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -755,7 +756,13 @@ mto_status set_design_sync(mto_ctx* c, int n_phase, const double* x_dev, const d
 size_t partials_count(const mto_ctx* c) {
   const Grid& gf = c->lv[c->L].g;
   int maxb = vec_blocks(gf.size(), c->num_sms);
-  if (maxb < c->num_sms) maxb = c->num_sms;  // small launches: up to one block per SM
+  // Small launches take up to one block per SM, or the row-per-warp kernel in
+  // blocks of eight warps (where a marching task would have at most two rows
+  // of 30 columns, so at most 4.3 of its tasks per target warp).
+  if (maxb < c->num_sms) maxb = c->num_sms;
+  const long long strips = (gf.nx + 1 + SPLIT_STRIDE - 1) / SPLIT_STRIDE;
+  const long long most = std::max(5LL * MAX_TARGET_WARPS_PER_SM * c->num_sms, 2 * strips);
+  maxb = (int)std::max<long long>(maxb, std::min(strips * (gf.ny + 1), most) / (SWEEP_NT / 32) + 1);
   for (int mode = 0; mode <= MODE_RESTRICT; ++mode) {
     for (int cols = 1; cols <= 2; ++cols) {
       const SweepShape s = sweep_shape(gf, mode, MAX_TARGET_WARPS_PER_SM * c->num_sms, cols, c->num_sms);

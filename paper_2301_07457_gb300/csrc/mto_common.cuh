@@ -72,6 +72,11 @@ __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
 
+// The same in two parts, for kernels that first load what no kernel of the
+// chain writes (design data).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <typename T> struct V2;
 template <> struct V2<double> { using t = double2; };
 template <> struct V2<float> { using t = float2; };
@@ -400,7 +405,9 @@ __device__ __forceinline__ void finish_scalars(DevScalars* sc, int kind, double 
 // of the block (any number of warps up to NT / 32) must call it.  Block partials go to partials[2*blockIdx.x + k];
 // the last block to arrive (ticket) adds them in block order, runs the
 // finishing action and re-arms the ticket.  No floating-point atomics.
-template <int NT>
+// TWO = false: v1 is not summed (the FP64 additions and shuffles of the tail
+// are a chain that small launches wait for).
+template <int NT, bool TWO = true>
 __device__ __forceinline__ void block_reduce_finish(double v0, double v1, double* partials,
                                                     unsigned* ticket, DevScalars* sc, int kind,
                                                     double* out_value, int tag = 0) {
@@ -408,24 +415,33 @@ __device__ __forceinline__ void block_reduce_finish(double v0, double v1, double
   __shared__ bool last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nwarps = (int)(blockDim.x >> 5);
+  // Sum over the block's threads, valid in thread 0.
+  auto block_sum = [&](double& a, double& b) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-    v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-  }
-  if (lane == 0) {
-    red[0][wid] = v0;
-    red[1][wid] = v1;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int w = 0; w < nwarps; ++w) {
-      a += red[0][w];
-      b += red[1][w];
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (TWO) b += __shfl_xor_sync(0xffffffffu, b, o);
     }
-    partials[2 * blockIdx.x] = a;
-    partials[2 * blockIdx.x + 1] = b;
+    if (nwarps == 1) return;
+    if (lane == 0) {
+      red[0][wid] = a;
+      if (TWO) red[1][wid] = b;
+    }
+    __syncthreads();
+    if (wid == 0) {
+      a = lane < nwarps ? red[0][lane] : 0.0;
+      if (TWO) b = lane < nwarps ? red[1][lane] : 0.0;
+#pragma unroll
+      for (int o = NT / 64; o > 0; o >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (TWO) b += __shfl_xor_sync(0xffffffffu, b, o);
+      }
+    }
+  };
+  block_sum(v0, v1);
+  if (threadIdx.x == 0) {
+    partials[2 * blockIdx.x] = v0;
+    if (TWO) partials[2 * blockIdx.x + 1] = v1;
     __threadfence();
     const unsigned t = atomicAdd(ticket, 1u);
     last = (t == gridDim.x - 1);
@@ -437,28 +453,13 @@ __device__ __forceinline__ void block_reduce_finish(double v0, double v1, double
   double a = 0.0, b = 0.0;
   for (int k = threadIdx.x; k < (int)gridDim.x; k += (int)blockDim.x) {
     a += ((volatile double*)partials)[2 * k];
-    b += ((volatile double*)partials)[2 * k + 1];
+    if (TWO) b += ((volatile double*)partials)[2 * k + 1];
   }
-  // Fixed-order tree over the block's threads.
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(0xffffffffu, a, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
-  __syncthreads();
-  if (lane == 0) {
-    red[0][wid] = a;
-    red[1][wid] = b;
-  }
-  __syncthreads();
+  __syncthreads();  // red is reused
+  block_sum(a, b);
   if (threadIdx.x == 0) {
-    double s0 = 0.0, s1 = 0.0;
-    for (int w = 0; w < nwarps; ++w) {
-      s0 += red[0][w];
-      s1 += red[1][w];
-    }
-    if (sc) finish_scalars(sc, kind, s0, s1, tag);
-    if (out_value) out_value[0] = s0;
+    if (sc) finish_scalars(sc, kind, a, b, tag);
+    if (out_value) out_value[0] = a;
     *ticket = 0u;
     __threadfence();
   }

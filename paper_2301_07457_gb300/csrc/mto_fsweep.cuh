@@ -478,8 +478,194 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
     }
   }
   if constexpr (REDUCE) {
-    block_reduce_finish<SWEEP_NT>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
+    block_reduce_finish<SWEEP_NT, DOT>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
   }
+}
+
+// ---------------------------------------------------------------------------
+// Small grids: one node row per warp, its two element rows side by side.
+//
+// Where a grid gives every warp one or two rows, a marching sweep is a chain
+// of two or three element rows of about 600 instructions each, issued by one
+// warp per scheduler at five clocks apiece: 3 us of a launch's 7, whatever the
+// grid.  Here a warp completes one node row je of 14 columns: lanes 0-15
+// evaluate the element row below it, lanes 16-31 the one above, both at once;
+// the halves exchange their parts of K v, and the lower one finishes u_x, the
+// upper one u_y.  The restriction uses a block of three warps for the three
+// fine rows of a coarse row.  Element data and diagonals, which no kernel of
+// the chain writes, are loaded before the wait for the previous kernel.
+// ---------------------------------------------------------------------------
+constexpr int SPLIT_STRIDE = 14;   // columns per warp
+constexpr int SPLIT_RSTRIDE = 12;  // fine columns per warp of the restriction (6 coarse ones)
+constexpr int SPLIT_RWARPS = 3;
+
+template <int SRC, int MODE, bool DOT, typename ZT>
+__global__ void __launch_bounds__(SWEEP_NT, 2) fsplit_kernel(const SweepParams<double> a) {
+  using F = FSweep<SRC, MODE, DOT, ZT>;
+  using Pack = typename F::Pack;
+  constexpr bool REDUCE = DOT || MODE == MODE_RESID || MODE == MODE_KP;
+  constexpr bool RESTRICT = MODE == MODE_RESTRICT;
+  pdl_trigger();
+  const Grid g = a.g;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int half = lane >> 4, hl = lane & 15;
+  // Task: a strip and a node row (restriction: a strip and a coarse row).
+  const int wg = RESTRICT ? (int)blockIdx.x : blockIdx.x * (int)(blockDim.x >> 5) + warp;
+  const int strip = wg % a.nstrips, row = wg / a.nstrips;
+  const int i = strip * (RESTRICT ? SPLIT_RSTRIDE : SPLIT_STRIDE) - (RESTRICT ? 2 : 1) + hl;
+  const int je = RESTRICT ? 2 * row - 1 + warp : row;
+  const bool task = row < a.nchunks && je >= 0 && je <= g.ny;  // uniform over the warp
+  const int jr = (task ? je : 0) - 1 + half;                   // this half's element row
+  const long long ke = g.at(task ? i : 0, jr);                 // element (i, jr), node (i, jr)
+  const long long kn = g.at(task ? i : 0, task ? je : 0);      // node (i, je)
+  const int c = half;                                          // component this lane finishes
+  const bool own = task && hl >= 1 && hl <= 14 && i >= 0 && i <= g.nx;
+  const bool act = own && !g.is_fixed(i, je);
+
+  Pack lo, hi;  // node rows jr and jr + 1
+  {
+    const unsigned long long* E = static_cast<const unsigned long long*>(a.E) + ke;
+#pragma unroll
+    for (int n = 0; n < F::Elem::N; ++n) lo.k[n] = __ldg(E + n * a.cstride);
+  }
+  double d = 0.0;
+  if constexpr (F::SMOOTHING)
+    d = SRC == SRC_FINE64 ? __ldg(a.invd1 + kn) : __ldg(reinterpret_cast<const double*>(a.invd2 + kn) + c);
+  pdl_wait_prior();
+
+  double beta = 0.0, alag = 0.0;
+  bool lag = false, vzero = false, done = false;
+  if (a.sc != nullptr) {
+    if (a.gate) {
+      done = a.sc->done != RUNNING;
+      if (a.replace_gate) done = done || a.sc->rr_every <= 0 || (a.sc->iter % a.sc->rr_every) != 0;
+    }
+    if constexpr (MODE == MODE_KP) {
+      beta = a.sc->beta;
+      lag = a.sc->x_lag != 0;
+      alag = a.sc->alpha;
+    }
+    if constexpr (MODE == MODE_RESID) {
+      vzero = a.zero_gate && a.sc->x_nonzero == 0;
+      lag = a.xlag && a.sc->x_lag != 0;
+      alag = a.sc->alpha;
+    }
+  }
+  // Without the pending step its operands are read all the same (unused).
+  F::load_top(a, ke, task ? i : 0, jr, MODE == MODE_RESID && a.xlag, lo);
+  F::load_top(a, ke + g.pitch, task ? i : 0, jr + 1, MODE == MODE_RESID && a.xlag, hi);
+  double b = 0.0, rd = 0.0, qd = 0.0, x = 0.0;
+  if constexpr (F::S::NEEDS_B) b = reinterpret_cast<const double*>(a.b + kn)[c];
+  if constexpr (DOT) {
+    rd = reinterpret_cast<const double*>(a.rdot + kn)[c];
+    if (a.qdot != nullptr) qd = reinterpret_cast<const double*>(a.qdot + kn)[c];
+  }
+  if constexpr (MODE == MODE_KP) x = reinterpret_cast<const double*>(a.xvec + kn)[c];
+  if (done) return;  // uniform over the grid
+
+  double dot0 = 0.0, dot1 = 0.0;
+  double res = 0.0;  // RESTRICT: b - K v of this lane's component
+  if (task) {
+    const double2 vlo = F::value(a, lo, i, jr, beta, lag, alag), vhi = F::value(a, hi, i, jr + 1, beta, lag, alag);
+    // Scales of the warp.
+    auto expo = [](double v) { return fx_exponent((unsigned)__double2hiint(v)); };
+    const int e0 = max(expo(vlo.x), expo(vlo.y)), e1 = max(expo(vhi.x), expo(vhi.y));
+    const bool bad0 = e0 == 0x7ff, bad1 = e1 == 0x7ff;
+    const int B = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(max(bad0 ? 0 : e0, bad1 ? 0 : e1), 1));
+    const unsigned bad = __ballot_sync(0xffffffffu, bad0 || bad1);
+    const double2 zero2 = make_double2(0.0, 0.0);
+    const Fx2 vb = fx2_from(bad0 ? zero2 : vlo, B), vt = fx2_from(bad1 ? zero2 : vhi, B);
+    auto right = [](const Fx2& v) -> Fx2 {  // next column of the half (its last lane: its own value, halo only)
+      return {{__shfl_down_sync(0xffffffffu, v.x.lo, 1, 16), __shfl_down_sync(0xffffffffu, v.x.mid, 1, 16),
+               __shfl_down_sync(0xffffffffu, v.x.hi, 1, 16)},
+              {__shfl_down_sync(0xffffffffu, v.y.lo, 1, 16), __shfl_down_sync(0xffffffffu, v.y.mid, 1, 16),
+               __shfl_down_sync(0xffffffffu, v.y.hi, 1, 16)}};
+    };
+    const Fx2 vbr = right(vb), vtr = right(vt);
+    const Fx2 ac = fsub(vbr, vb), bt = fsub(vtr, vt), up = fsub(fadd(vtr, vt), fadd(vbr, vb));
+    const FxStrain w = {fx_add(ac.x, bt.x), fx_sub(bt.x, ac.x), up.y, fx_sub(bt.y, ac.y),
+                        fx_add(up.x, fx_add(ac.y, bt.y))};
+    const unsigned tag = fx_tag(lo.k);
+    const int X = (int)(tag & 0x7ffu);
+    const int Xm = (int)__reduce_max_sync(0xffffffffu, (unsigned)X);
+    const int sh = Xm - X;
+    const bool rare = __any_sync(0xffffffffu, tag != 0u && (sh >= 32 || (tag & FX_TAG_NEG)));
+    FxStrain t = F::Elem::core(a, w, lo.k, rare);
+    if (rare)
+      t = {fx_sar_limbs(t.c1, sh), fx_sar_limbs(t.c3, sh), fx_sar_limbs(t.d2, sh), fx_sar_limbs(t.d3, sh),
+           fx_sar_limbs(t.s, sh)};
+    t = {fx_sar31(t.c1, sh & 31), fx_sar31(t.c3, sh & 31), fx_sar31(t.d2, sh & 31), fx_sar31(t.d3, sh & 31),
+         fx_sar31(t.s, sh & 31)};
+    // The node row is the top edge of the element row below (forces t_c1 + t_c3,
+    // vertical forces +) and the bottom edge of the one above (t_c1 - t_c3, -).
+    const int above = -half;
+    const Fx2 h = {fx_add(t.c1, fx_flip(t.c3, above)), fx_add(t.s, fx_flip(t.d3, above))};
+    const Fx2 v = {fx_flip(t.s, above), fx_flip(t.d2, above)};
+    const Fx2 from_left = fadd(v, h);
+    auto left = [](const Fx& f) -> Fx {
+      return {__shfl_up_sync(0xffffffffu, f.lo, 1, 16), __shfl_up_sync(0xffffffffu, f.mid, 1, 16),
+              __shfl_up_sync(0xffffffffu, f.hi, 1, 16)};
+    };
+    const Fx2 part = fadd(Fx2{left(from_left.x), left(from_left.y)}, fsub(v, h));
+    // Each half sends the component that the other finishes.
+    const Fx send = half ? part.x : part.y, keep = half ? part.y : part.x;
+    const Fx got = {__shfl_xor_sync(0xffffffffu, send.lo, 16), __shfl_xor_sync(0xffffffffu, send.mid, 16),
+                    __shfl_xor_sync(0xffffffffu, send.hi, 16)};
+    const Fx sum = fx_add(keep, got);
+    const int unit = B + Xm + F::Elem::UNIT;
+    double kv = fx_to_double<false>(sum, unit);
+    if (unit < FX_UNIT_MIN || unit > FX_UNIT_MAX) kv = fx_to_double(sum, unit);  // uniform over the warp
+    if (bad != 0u || Xm == 0x7ff) {  // neighbours of non-finite values
+      const unsigned m = (bad | (bad >> 16)) & 0xffffu;
+      if (Xm == 0x7ff || (((m | (m << 1) | (m >> 1)) >> hl) & 1u)) kv = NAN;
+    }
+
+    const double2 mid = half ? vlo : vhi;  // node row je
+    const double vc = c ? mid.y : mid.x;
+    if constexpr (MODE == MODE_APPLY) {
+      double* out = reinterpret_cast<double*>(a.out + (a.dense ? (long long)je * (g.nx + 1) + i : kn));
+      if (own) out[c] = act ? kv : 0.0;
+    } else if constexpr (MODE == MODE_RESID) {
+      const double r = act ? b - (vzero ? 0.0 : kv) : 0.0;
+      if (own) {
+        reinterpret_cast<double*>(a.out + kn)[c] = r;
+        if (a.out32 != nullptr) reinterpret_cast<float*>(a.out32 + kn)[c] = float(r);
+      }
+      dot0 = r * r;
+    } else if constexpr (MODE == MODE_KP) {
+      const double q = act ? kv : 0.0;
+      if (own) {
+        reinterpret_cast<double*>(a.p_out + kn)[c] = vc;
+        reinterpret_cast<double*>(a.out + kn)[c] = q;
+        dot0 = vc * q;
+        const double2 old = half ? lo.v : hi.v;
+        if (lag) reinterpret_cast<double*>(a.xvec + kn)[c] = fma(alag, c ? old.y : old.x, x);
+      }
+    } else if constexpr (F::SMOOTHING) {
+      const double z = act ? fma(d, b - kv, vc) : 0.0;
+      if (own) reinterpret_cast<double*>(a.out + kn)[c] = z;
+      if constexpr (DOT) {
+        dot0 = z * rd;
+        if (a.qdot != nullptr) dot1 = z * qd;
+      }
+    } else if constexpr (RESTRICT) {
+      res = act ? b - kv : 0.0;
+    }
+  }
+  if constexpr (RESTRICT) {
+    // Full weighting of the three rows, each column first.
+    __shared__ double rows[SPLIT_RWARPS][32];
+    rows[warp][lane] = res;
+    __syncthreads();
+    const int I = i >> 1;
+    if (warp == 0 && row < a.nchunks && (hl & 1) == 0 && hl >= 2 && hl <= 12 && I >= 0 && I <= a.gc.nx) {
+      auto column = [&](int l) { return fma(0.5, rows[2][l], fma(0.5, rows[0][l], rows[1][l])); };
+      const double val = fma(0.5, column(lane - 1) + column(lane + 1), column(lane));
+      reinterpret_cast<double*>(a.bc + a.gc.at(I, row))[c] = a.gc.is_fixed(I, row) ? 0.0 : val;
+    }
+  }
+  if constexpr (REDUCE)
+    block_reduce_finish<SWEEP_NT, DOT>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
 }
 
 }  // namespace mto

@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(NA_NT)
     }
   }
   unsigned* ticket = reinterpret_cast<unsigned*>(scratch + 2 * NA_MAX_BLOCKS);
-  block_reduce_finish<NA_NT>(acc, 0.0, scratch, ticket, nullptr, FIN_NONE, out);
+  block_reduce_finish<NA_NT, false>(acc, 0.0, scratch, ticket, nullptr, FIN_NONE, out);
 }
 
 // The device address of the scratch array on `device`, looked up once per

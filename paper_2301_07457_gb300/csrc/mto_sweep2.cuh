@@ -774,7 +774,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) sweep2_kernel(const SweepParams<T
   double dot0 = 0.0, dot1 = 0.0;
   sweep2_warp<T, SRC, MODE, DOT, ZT, PF>(a, wg, lane, dot0, dot1);
   if constexpr (REDUCE) {
-    block_reduce_finish<SWEEP_NT>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value,
+    block_reduce_finish<SWEEP_NT, DOT && MODE != MODE_SMOOTH0>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value,
                                   a.tag);
   }
 }

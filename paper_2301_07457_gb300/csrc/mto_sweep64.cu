@@ -59,21 +59,38 @@ SweepShape sweep_shape(const Grid& g, int mode, int target_warps, int cols, int 
 
 int sweep_cols(bool f64, int src, int mode) { return sweep_cols_of(f64, src, mode); }
 
+// Small grids, where a marching task would have one or two rows, take the
+// kernel that completes a row per warp (its two element rows side by side):
+// per node it costs what two-row tasks do, and its chain is a third as long.
+// PCG iterations: 256^2 168 -> 115 us, 1024^2 (coarse levels only) 446 -> 391
+// us; a 64^2 solve 3.00 -> 1.92 ms.
+constexpr int SPLIT_MAX_H = 2;
+
 template <int SRC, int MODE, bool DOT, typename ZT>
 static cudaError_t go(SweepParams<double> p, int tw, int num_sms, cudaStream_t s) {
-  constexpr int COLS = sweep_cols_of(true, SRC, MODE);
-  void (*kernel)(SweepParams<double>);
-  static_assert(COLS == 1, "one column per lane");
-  kernel = fsweep_kernel<SRC, MODE, DOT, ZT, 1>;
+  void (*kernel)(SweepParams<double>) = fsweep_kernel<SRC, MODE, DOT, ZT, 1>;
   if (tw <= 0) {
     static const int wave = full_wave_warps(kernel, num_sms);  // same for every device of a run
     tw = wave;
   }
-  const SweepShape sh = sweep_shape(p.g, MODE, tw, COLS, num_sms);
+  const SweepShape sh = sweep_shape(p.g, MODE, tw, sweep_cols_of(true, SRC, MODE), num_sms);
   p.nstrips = sh.nstrips;
   p.nchunks = sh.nchunks;
   p.H = sh.H;
-  return launch_pdl(kernel, sh.nblocks, sh.nthreads, 0, s, p);
+  int nblocks = sh.nblocks, nthreads = sh.nthreads;
+  if (sh.H <= SPLIT_MAX_H) {
+    const bool restrict = MODE == MODE_RESTRICT;
+    const int stride = restrict ? SPLIT_RSTRIDE : SPLIT_STRIDE;
+    kernel = fsplit_kernel<SRC, MODE, DOT, ZT>;
+    p.nstrips = (p.g.nx + 1 + stride - 1) / stride;
+    p.nchunks = restrict ? p.gc.ny + 1 : p.g.ny + 1;
+    const int tasks = p.nstrips * p.nchunks;
+    int per_block = (tasks + num_sms - 1) / num_sms;
+    per_block = per_block > SWEEP_NT / 32 ? SWEEP_NT / 32 : per_block;
+    nblocks = restrict ? tasks : (tasks + per_block - 1) / per_block;
+    nthreads = 32 * (restrict ? SPLIT_RWARPS : per_block);
+  }
+  return launch_pdl(kernel, nblocks, nthreads, 0, s, p);
 }
 
 template <>

@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(VEC_NT)
     one(k + stride, q1, r1);
   }
   if (k < n) one(k, q[k], r[k]);
-  block_reduce_finish<VEC_NT>(acc, 0.0, partials, ticket, sc, FIN_UPDATE, nullptr);
+  block_reduce_finish<VEC_NT, false>(acc, 0.0, partials, ticket, sc, FIN_UPDATE, nullptr);
 }
 
 // The pending x step after the loop: x += alpha p[p_par] when x_lag.
@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(VEC_NT)
     const double2 x = a[k], y = b[k];
     acc0 = fma(x.x, y.x, fma(x.y, y.y, acc0));
   }
-  block_reduce_finish<VEC_NT>(acc0 + acc1, 0.0, partials, ticket, sc, finish, out_value);
+  block_reduce_finish<VEC_NT, false>(acc0 + acc1, 0.0, partials, ticket, sc, finish, out_value);
 }
 
 // Layout conversions between the caller's arrays and the padded grids: each
