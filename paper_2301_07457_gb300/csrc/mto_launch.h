@@ -8,6 +8,7 @@
 #include "mto_fused.cuh"
 #include "mto_gemv.cuh"
 #include "mto_sweep2.cuh"
+#include "mto_tile.cuh"
 
 namespace mto {
 

@@ -16,11 +16,28 @@ template <int SRC, int MODE, bool DOT> constexpr int lookahead() {
   return 3;
 }
 
+// Two-stage passes of levels with at most this many tiles per SM run by tiles
+// (mto_tile.cuh): one V-cycle takes 60 -> 41 us at 256^2, 110 -> 90 us at
+// 1024^2, 236 -> 216 us at 2048^2 (all levels up to 256^2), 160 -> 141 us at
+// 1856 x 1216 (up to 464 x 304: 7.7 tiles per SM).  A 512^2 level (14 tiles per
+// SM) takes 1-4 us longer by tiles, a 1024^2 level 30 us: there the recomputed
+// halo counts.  Launch shapes below one warp per SM ask for marching tasks.
+constexpr int TILES_PER_SM = 8;
+
 template <int SRC, int MODE, bool DOT>
 static cudaError_t go(SweepParams<float> p, int tw, int num_sms, cudaStream_t s) {
   constexpr int COLS = sweep_cols_of(false, SRC, MODE);
   constexpr int PF = lookahead<SRC, MODE, DOT>();
   void (*kernel)(SweepParams<float>);
+  if constexpr (MODE == MODE_PRE2 || MODE == MODE_POST2) {
+    const int across = p.g.nx / TILE_X + 1;  // tiles of nx + 1 nodes
+    const long long tiles = (long long)across * (p.g.ny / TILE_Y + 1);
+    if (tiles <= TILES_PER_SM * num_sms && (tw <= 0 || tw >= num_sms)) {
+      kernel = MODE == MODE_PRE2 ? tile_pre2_kernel<SRC> : tile_post2_kernel<SRC>;
+      p.nstrips = across;
+      return launch_pdl(kernel, (int)tiles, SWEEP_NT, 0, s, p);
+    }
+  }
   if constexpr (MODE == MODE_POST2) kernel = post2_kernel<SRC, 2>;
   else if constexpr (MODE == MODE_PRE2) kernel = pre2_kernel<SRC, 2>;
   else if constexpr (COLS == 2) kernel = sweep2_kernel<float, SRC, MODE, DOT, float2, PF>;

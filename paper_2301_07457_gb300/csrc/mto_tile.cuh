@@ -1,0 +1,203 @@
+// The two-stage passes of the small float32 coarse levels (Alg. 1), one tile
+// of nodes per block.
+//
+// Same passes as the marching kernels of mto_fused.cuh: PRE2 (two smoothing
+// sweeps from zero, residual, restriction) and POST2 (prolongation, two
+// sweeps).  On a small grid a marching task has one or two rows of output but
+// marches five to seven, 300 instructions each, in one warp: 4.6 us of a
+// launch's 7.5.  Here a block holds the tile and its halo in shared memory and
+// takes one thread per element or node, so that a pass is a chain of two
+// element evaluations and two node sums; the halo (about the tile again) is
+// recomputed, which costs nothing while the grid does not fill the chip.
+// Element data and diagonals are loaded before the wait for the previous
+// kernel.
+//
+// Every value is formed by the same operations in the same order as there, so
+// the results are those of the marching kernels bit for bit.
+#pragma once
+
+#include "mto_fused.cuh"
+
+namespace mto {
+
+constexpr int TILE_CX = 8, TILE_CY = 4;             // PRE2: coarse nodes per block
+constexpr int TILE_X = 2 * TILE_CX, TILE_Y = 2 * TILE_CY;  // fine nodes per block (POST2: its output)
+
+// Element forces in shared memory: bottom edge ga, top edge gb, vertical gs
+// (the edge bookkeeping of mto_sweep.cuh), EW x EH elements.
+template <int EW, int EH> struct TileForces {
+  float2 ga[EW * EH], gb[EW * EH], gs[EW * EH];
+
+  // Forces of element e from its corner values.
+  template <int SRC>
+  __device__ __forceinline__ void put(const SweepParams<float>& a, const ERaw<float, SRC>& er, int e, float2 bl,
+                                      float2 br, float2 tl, float2 tr) {
+    const float2 ac = sub2(br, bl), bt = sub2(tr, tl), dl = sub2(tl, bl), dr = sub2(tr, br);
+    const float2 cd1 = add2(ac, bt), cd3 = sub2(bt, ac), cd2 = add2(dl, dr);
+    Strain<float> w;
+    w.c1 = cd1.x;
+    w.c3 = cd3.x;
+    w.d3 = cd3.y;
+    w.d2 = cd2.y;
+    w.s = cd2.x + cd1.y;
+    float dummy;
+    const Strain<float> t = Sweep<float, SRC, MODE_SMOOTH, false, float2>::core(a, er, w, dummy);
+    const float2 p = make_float2(t.c1, t.s), m = make_float2(t.c3, t.d3);
+    ga[e] = sub2(p, m);
+    gb[e] = add2(p, m);
+    gs[e] = make_float2(t.s, t.d2);
+  }
+  // K v at the node whose upper right element is e.
+  __device__ __forceinline__ float2 at_node(int e) const {
+    const float2 gh = add2(ga[e], gb[e - EW]), ghl = add2(ga[e - 1], gb[e - EW - 1]);
+    const float2 gv = add2(gs[e], gs[e - 1]), gvp = add2(gs[e - EW], gs[e - EW - 1]);
+    return add2(sub2(ghl, gh), sub2(gvp, gv));
+  }
+};
+
+// Element (ei, ej), zero outside the mesh.
+template <int SRC>
+__device__ __forceinline__ ERaw<float, SRC> tile_element(const SweepParams<float>& a, int ei, int ej) {
+  ERaw<float, SRC> er{};
+  if (ei >= 0 && ei < a.g.nx && ej >= 0 && ej < a.g.ny)
+    Sweep<float, SRC, MODE_SMOOTH, false, float2>::load_e(a, a.g.at(ei, ej), ei, ej, er);
+  return er;
+}
+
+template <int SRC> __global__ void __launch_bounds__(SWEEP_NT) tile_pre2_kernel(const SweepParams<float> a) {
+  pdl_trigger();
+  // z0 on NW x NH nodes from (x0, y0), elements one less each way; z1 inside.
+  constexpr int NW = TILE_X + 5, NH = TILE_Y + 5, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
+  static_assert(EW * EH <= SWEEP_NT && ZW * ZH <= SWEEP_NT, "one element and one node per thread");
+  __shared__ TileForces<EW, EH> f;
+  __shared__ float2 z[NW * NH], r[ZW * ZH];
+  const Grid g = a.g, gc = a.gc;
+  const int t = threadIdx.x;
+  const int I0 = ((int)blockIdx.x % a.nstrips) * TILE_CX, J0 = ((int)blockIdx.x / a.nstrips) * TILE_CY;
+  const int x0 = 2 * I0 - 3, y0 = 2 * J0 - 3;
+  const int ex = t % EW, ey = t / EW;
+  const bool elem = t < EW * EH;
+  ERaw<float, SRC> er{};
+  if (elem) er = tile_element<SRC>(a, x0 + ex, y0 + ey);
+  // The thread's z1 node.
+  const int zx = 1 + t % ZW, zy = 1 + t / ZW, i = x0 + zx, j = y0 + zy;
+  const bool node = t < ZW * ZH, valid = node && g.valid(i, j);
+  const float2 zero2 = make_float2(0.f, 0.f);
+  float2 d = zero2, b = zero2;
+  if (valid) d = __ldg(a.invd2 + g.at(i, j));
+  float2 dh[2], bh[2];  // of the z0 nodes t and t + SWEEP_NT
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int n = t + u * SWEEP_NT, ii = x0 + n % NW, jj = y0 + n / NW;
+    dh[u] = n < NW * NH && g.valid(ii, jj) ? __ldg(a.invd2 + g.at(ii, jj)) : zero2;
+  }
+  pdl_wait_prior();
+  const bool done = a.sc != nullptr && a.gate && a.sc->done != RUNNING;
+  if (valid) b = a.b[g.at(i, j)];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int n = t + u * SWEEP_NT, ii = x0 + n % NW, jj = y0 + n / NW;
+    bh[u] = n < NW * NH && g.valid(ii, jj) ? a.b[g.at(ii, jj)] : zero2;
+  }
+  if (done) return;  // uniform over the grid
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int n = t + u * SWEEP_NT;
+    if (n < NW * NH) z[n] = mul2(dh[u], bh[u]);
+  }
+  __syncthreads();
+  // z1 = z0 + w/D (b - K z0).
+  const int c = ey * NW + ex;
+  if (elem) f.template put<SRC>(a, er, t, z[c], z[c + 1], z[c + NW], z[c + NW + 1]);
+  __syncthreads();
+  const int zn = zy * NW + zx, en = zy * EW + zx;  // node and its upper right element
+  if (node) {
+    const float2 z1 = fma2(d, sub2(b, f.at_node(en)), z[zn]);
+    z[zn] = z1;
+    if (valid && zx >= 3 && zx < 3 + TILE_X && zy >= 3 && zy < 3 + TILE_Y) a.out[g.at(i, j)] = z1;
+  }
+  __syncthreads();
+  // Residual.
+  if (elem && ex >= 1 && ex < EW - 1 && ey >= 1 && ey < EH - 1)
+    f.template put<SRC>(a, er, t, z[c], z[c + 1], z[c + NW], z[c + NW + 1]);
+  __syncthreads();
+  if (node && zx >= 2 && zx < NW - 2 && zy >= 2 && zy < NH - 2) {
+    const float m = g.active(i, j) ? 1.f : 0.f;
+    r[t] = mul2(sub2(b, f.at_node(en)), make_float2(m, m));
+  }
+  __syncthreads();
+  // Full weighting: across, then over the three rows.
+  if (t < TILE_CX * TILE_CY) {
+    const int p = t % TILE_CX, q = t / TILE_CX, I = I0 + p, J = J0 + q;
+    if (I <= gc.nx && J <= gc.ny) {
+      const int n = (2 + 2 * q) * ZW + 2 + 2 * p;  // r at fine node (2 I, 2 J)
+      auto across = [&](int k) {
+        const float2 r0 = r[k], r1 = r[k + 1], rl = r[k - 1];
+        return make_float2(r0.x + 0.5f * (r1.x + rl.x), r0.y + 0.5f * (r1.y + rl.y));
+      };
+      const float2 lo = across(n - ZW), mid = across(n), hi = across(n + ZW);
+      const float2 acc = add2(make_float2(0.5f * lo.x, 0.5f * lo.y), mid);
+      const float2 val = make_float2(acc.x + 0.5f * hi.x, acc.y + 0.5f * hi.y);
+      a.bc[gc.at(I, J)] = gc.is_fixed(I, J) ? zero2 : val;
+    }
+  }
+}
+
+template <int SRC> __global__ void __launch_bounds__(SWEEP_NT) tile_post2_kernel(const SweepParams<float> a) {
+  pdl_trigger();
+  constexpr int NW = TILE_X + 4, NH = TILE_Y + 4, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
+  static_assert(EW * EH <= SWEEP_NT && NW * NH <= SWEEP_NT, "one element and one node per thread");
+  __shared__ TileForces<EW, EH> f;
+  __shared__ float2 z[NW * NH];
+  const Grid g = a.g, gc = a.gc;
+  const int t = threadIdx.x;
+  const int x0 = ((int)blockIdx.x % a.nstrips) * TILE_X - 2, y0 = ((int)blockIdx.x / a.nstrips) * TILE_Y - 2;
+  const int ex = t % EW, ey = t / EW;
+  const bool elem = t < EW * EH;
+  ERaw<float, SRC> er{};
+  if (elem) er = tile_element<SRC>(a, x0 + ex, y0 + ey);
+  // The thread's z2 (and z3) node.
+  const int zx = 1 + t % ZW, zy = 1 + t / ZW, i = x0 + zx, j = y0 + zy;
+  const bool node = t < ZW * ZH, valid = node && g.valid(i, j);
+  const float2 zero2 = make_float2(0.f, 0.f);
+  float2 d = zero2, b = zero2;
+  if (valid) d = __ldg(a.invd2 + g.at(i, j));
+  pdl_wait_prior();
+  const bool done = a.sc != nullptr && a.gate && a.sc->done != RUNNING;
+  if (valid) b = a.b[g.at(i, j)];
+  // z = v + P z_c at node t (mto_sweep2.cuh's interpolation).
+  float2 v = zero2;
+  {
+    const int ii = x0 + t % NW, jj = y0 + t / NW;
+    if (t < NW * NH && g.valid(ii, jj)) {
+      v = a.v[g.at(ii, jj)];
+      const long long kc = gc.at(ii >> 1, jj >> 1);
+      const long long up = (jj & 1) ? gc.pitch : 0;
+      const float2 c00 = a.zc[kc], c01 = a.zc[kc + up], c10 = a.zc[kc + 1], c11 = a.zc[kc + 1 + up];
+      const float2 cy0 = make_float2(0.5f * (c00.x + c01.x), 0.5f * (c00.y + c01.y));
+      const float2 cy1 = make_float2(0.5f * (c10.x + c11.x), 0.5f * (c10.y + c11.y));
+      v = (ii & 1) ? make_float2(v.x + 0.5f * (cy0.x + cy1.x), v.y + 0.5f * (cy0.y + cy1.y))
+                   : make_float2(v.x + cy0.x, v.y + cy0.y);
+    }
+  }
+  if (done) return;  // uniform over the grid
+  if (t < NW * NH) z[t] = v;
+  __syncthreads();
+  const int c = ey * NW + ex;
+  if (elem) f.template put<SRC>(a, er, t, z[c], z[c + 1], z[c + NW], z[c + NW + 1]);
+  __syncthreads();
+  const int zn = zy * NW + zx, en = zy * EW + zx;
+  float2 z2 = zero2;
+  if (node) {
+    z2 = fma2(d, sub2(b, f.at_node(en)), z[zn]);
+    z[zn] = z2;
+  }
+  __syncthreads();
+  if (elem && ex >= 1 && ex < EW - 1 && ey >= 1 && ey < EH - 1)
+    f.template put<SRC>(a, er, t, z[c], z[c + 1], z[c + NW], z[c + NW + 1]);
+  __syncthreads();
+  if (valid && zx >= 2 && zx < 2 + TILE_X && zy >= 2 && zy < 2 + TILE_Y)
+    a.out[g.at(i, j)] = fma2(d, sub2(b, f.at_node(en)), z2);
+}
+
+}  // namespace mto

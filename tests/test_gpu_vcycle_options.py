@@ -123,3 +123,22 @@ def test_w_cycle_solve(mto, prec):
         ref = solver.solve_pcgmg(nelx, nely, x, EP, 3.0, f, n_coarsen=4, tol=1e-8, gamma=2)
         assert abs(st["iters"] - ref["iters"]) <= 1, (st["iters"], ref["iters"])
     mesh.close()
+
+
+@pytest.mark.parametrize("kind", ["galerkin", "rediscretize"])
+@pytest.mark.parametrize("nx,ny,nc", [(32, 32, 3), (48, 40, 3), (136, 72, 3), (264, 136, 2), (96, 264, 3)])
+def test_tiled_coarse_passes_equal_marching_ones(mto, nx, ny, nc, kind):
+    """The small float32 levels run by tiles (a block per tile); a launch shape of one warp makes
+    them march instead.  Both form every value by the same operations: equal bit for bit."""
+    x = torch.from_numpy(dirichlet_design(nx, ny, 4, seed=nx)).cuda()
+    r = torch.from_numpy(np.random.default_rng(ny).standard_normal((ny + 1, nx + 1, 2))).cuda()
+    z = []
+    for warps in (0, 1):
+        m = mto.Mesh(nx, ny, n_coarsen=nc, precision="mixed", fixed_edges=mto.EDGE_BOTTOM | mto.EDGE_LEFT,
+                     coarse_kind=kind)
+        for l in range(1, nc):
+            m.set_launch_shape(l, warps)
+        m.set_design(x, [1.0, 0.5, 0.25, 1e-9], 3.0)
+        z.append(m.apply_preconditioner(r))
+        m.close()
+    assert torch.equal(z[0], z[1])
