@@ -24,6 +24,7 @@
 // kept.  Per depth, deepest first, three launches: (1) one block per range
 // forms S and inverts it while other blocks form V, (2) W, (3) the update of
 // K_0^-1 by 16 x 16 tiles of its lower triangle, mirrored.
+#include "mto_fixed.cuh"
 #include "mto_launch.h"
 
 namespace mto {
@@ -83,7 +84,8 @@ __device__ __forceinline__ double couple(const BlockRows& a, int q, int s, int b
 }
 __device__ __forceinline__ int couple_at(int m, int b, int e) { return min(max(couple_first(b) + e, 0), m - 1); }
 
-constexpr int SEP_NT = 256;   // threads of the separator blocks (and the V blocks)
+constexpr int SEP_NT = 224;   // threads that hold S: seven warps, so that with the
+constexpr int SEP_BLOCK = SEP_NT + 32;  // diagonal's every scheduler has two (V blocks use them all)
 constexpr int V_ROWS = 8;     // rows per V block
 constexpr int W_ROWS = 2;     // rows per W block
 constexpr int W_NT = 64 * W_ROWS;
@@ -93,7 +95,7 @@ constexpr int TILE_NT = 128;  // 2 x 2 entries per thread, even and odd columns 
 // V rows [r0, r0 + V_ROWS) of the ranges of this depth.
 __device__ __forceinline__ void form_v(const BlockRows& a, int depth, int r0) {
   const int m = a.m;
-  for (int t = threadIdx.x; t < V_ROWS * m; t += SEP_NT) {
+  for (int t = threadIdx.x; t < V_ROWS * m; t += SEP_BLOCK) {
     const int r = r0 + t / m, b = t % m;
     if (r >= a.n) return;
     const int j = r / m;
@@ -113,51 +115,43 @@ __device__ __forceinline__ void form_v(const BlockRows& a, int depth, int r0) {
   }
 }
 
-// 1 / d for d > 0: Newton's iteration of third order from the float32
-// reciprocal, y + y (e + e^2) with e = 1 - d y (|e| < 2^-22, so the error is
-// that of the last rounding or two): three dependent FP64 operations where the
-// division takes about ten, which matters as it stands on the chain of pivots.
-__device__ __forceinline__ double reciprocal(double d) {
-  if (d < 1.0e-30 || d > 1.0e30) return 1.0 / d;
-  const double y = (double)__frcp_rn(__double2float_rn(d));
-  const double e = fma(-d, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
-
 // S of the range, inverted in place by symmetric sweeps on its lower triangle
 // (S -> -S^-1): pivot p = a_kk turns a_ij into a_ij - a_ik a_jk / p, column k
-// into a_ik / p and a_kk into -1 / p.  Thread 0 updates the next pivot first
-// and forms its reciprocal while the other warps update the rest; two barriers
-// per pivot.
+// into a_ik / p and a_kk into -1 / p.  The triangle lives in the registers of
+// SEP_NT threads (E entries each); per pivot the column and its quotients pass
+// through shared memory.  An extra warp keeps a second copy of the diagonal,
+// so that the next pivot's reciprocal is formed while the others update.  Two
+// barriers per pivot; the FP64 pipe bounds a pivot (three to six FMAs of two
+// warps per scheduler at 64 clocks, and a latency of about 140): 25 -> 19 us
+// for m = 34 against the triangle in shared memory.
+template <int E>
 __device__ __forceinline__ void form_s(const BlockRows& a, const Range& g, double* sm) {
   const int m = a.m, tid = threadIdx.x;
   double* G1 = sm;               // last diagonal block of the left part's inverse
   double* G2 = G1 + m * m;       // first one of the right part's
   double* X1 = G2 + m * m;       // G1 B_s^T
   double* X2 = X1 + m * m;       // G2 B_{s+1}
-  double* A = G1;                // S, lower triangle in full storage (G1 is done by then)
   double* C1 = X2 + m * m;       // couplings [b][e] to the left and the right
   double* C2 = C1 + NCOUPLE * m;
-  double* u = C2 + NCOUPLE * m;  // pivot column
-  double* v = u + m;             // and the same over the pivot
-  short2* pairs = reinterpret_cast<short2*>(v + m);
-  __shared__ double rec;
+  double* u = C2 + NCOUPLE * m;  // pivot column, two buffers
+  double* v = u + 2 * m;         // the same over the pivot
+  double* diag = v + m;
+  __shared__ double rec[2];
   const bool left = g.s > g.lo, right = g.s + 1 < g.hi;
   const int base = g.s * m;
-  for (int t = tid; t < m * m; t += SEP_NT) {
+  for (int t = tid; t < m * m; t += SEP_BLOCK) {
     const int i = t / m, b = t % m;
     G1[t] = left ? a.Kinv[(size_t)(base - m + i) * a.n + base - m + b] : 0.0;
     G2[t] = right ? a.Kinv[(size_t)(base + m + i) * a.n + base + m + b] : 0.0;
-    if (b <= i) pairs[i * (i + 1) / 2 + b] = make_short2((short)i, (short)b);
   }
-  for (int t = tid; t < NCOUPLE * m; t += SEP_NT) {
+  for (int t = tid; t < NCOUPLE * m; t += SEP_BLOCK) {
     const int b = t / NCOUPLE, e = t % NCOUPLE;
     C1[t] = left ? couple(a, g.s - 1, g.s, b, e) : 0.0;
     C2[t] = right ? couple(a, g.s + 1, g.s, b, e) : 0.0;
   }
   __syncthreads();
   if (left || right)
-    for (int t = tid; t < m * m; t += SEP_NT) {
+    for (int t = tid; t < m * m; t += SEP_BLOCK) {
       const int i = t / m, b = t % m;
       double x = 0.0, y = 0.0;
 #pragma unroll
@@ -171,72 +165,108 @@ __device__ __forceinline__ void form_s(const BlockRows& a, const Range& g, doubl
     }
   __syncthreads();
   const int np = m * (m + 1) / 2;
-  for (int t = tid; t < np; t += SEP_NT) {
-    const int i = pairs[t].x, j = pairs[t].y;
+  const bool worker = tid < SEP_NT;
+  double A[E];
+  int ij[E];  // i << 16 | j, i >= j
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int t = tid + e * SEP_NT;
+    A[e] = 0.0;
+    ij[e] = -1;
+    if (!worker || t >= np) continue;
+    int i = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+    while ((i + 1) * (i + 2) / 2 <= t) ++i;
+    while (i * (i + 1) / 2 > t) --i;
+    const int j = t - i * (i + 1) / 2;
+    ij[e] = i << 16 | j;
     double x = k0(a, base + i, base + j), y = 0.0;
     if (left || right) {
 #pragma unroll
-      for (int e = 0; e < NCOUPLE; ++e) {
-        const int l = couple_at(m, i, e) * m + j;
-        x = fma(-C1[i * NCOUPLE + e], X1[l], x);
-        y = fma(-C2[i * NCOUPLE + e], X2[l], y);
+      for (int c = 0; c < NCOUPLE; ++c) {
+        const int l = couple_at(m, i, c) * m + j;
+        x = fma(-C1[i * NCOUPLE + c], X1[l], x);
+        y = fma(-C2[i * NCOUPLE + c], X2[l], y);
       }
     }
-    A[i * m + j] = x + y;
+    A[e] = x + y;
+    if (j == 0) u[i] = A[e];
+    if (i == j) diag[i] = A[e];
   }
   __syncthreads();
-  auto pivot = [&](double d) {
+  auto pivot = [&](double d, int k) {
+    // Positive and between 2^-996 and 2^996, by the exponent (no comparison on
+    // the FP64 pipe, whose latency the chain of pivots would see).
+    if ((unsigned)(__double2hiint(d) - 0x01b00000) < 0x7c800000u) {
+      rec[k & 1] = fx_reciprocal(d);
+      return;
+    }
     if (!(d > 0.0) || !(d < 1.0e300)) {
       *a.err = 1;
       d = 1.0;
     }
-    rec = reciprocal(d);
+    rec[k & 1] = 1.0 / d;
   };
-  if (tid == 0) pivot(A[0]);
+  constexpr int ND = (MAX_BLOCK_ROW + 31) / 32;
+  double dg[ND];  // the extra warp's diagonal: entries lane, lane + 32, ...
+  const int lane = tid & 31;
+#pragma unroll
+  for (int q = 0; q < ND; ++q) dg[q] = lane + 32 * q < m ? diag[lane + 32 * q] : 1.0;
+  if (tid == SEP_NT) pivot(dg[0], 0);
   __syncthreads();
   for (int k = 0; k < m; ++k) {
-    const double r = rec;
+    const double r = rec[k & 1];
+    double* uk = u + (k & 1) * m;
+    double* un = u + ((k + 1) & 1) * m;
     // With u_k = -1 and v_k = -r the pivot row, column and entry are -u_i v_j
     // (or its mirror image) too.
-    for (int i = tid; i < m; i += SEP_NT) {
-      const double x = i >= k ? A[i * m + k] : A[k * m + i];
-      u[i] = i == k ? -1.0 : x;
-      v[i] = i == k ? -r : x * r;
+    if (tid < m) {
+      v[tid] = tid == k ? -r : uk[tid] * r;
+      if (tid == k) uk[tid] = -1.0;
     }
     __syncthreads();
-    if (tid < 32) {
-      if (tid == 0 && k + 1 < m) {
-        const double d = fma(-u[k + 1], v[k + 1], A[(k + 1) * m + k + 1]);
-        A[(k + 1) * m + k + 1] = d;
-        pivot(d);
+    if (worker) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        if (ij[e] < 0) continue;
+        const int i = ij[e] >> 16, j = ij[e] & 0xffff;
+        // i >= j: in the pivot row (i = k) the -1 is in u_i, in the pivot
+        // column (j = k) the -r in v_j.
+        A[e] = fma(-uk[i], v[j], i == k || j == k ? 0.0 : A[e]);
+        if (i == k + 1) un[j] = A[e];
+        else if (j == k + 1) un[i] = A[e];
       }
     } else {
-      for (int t = tid - 32; t < np; t += SEP_NT - 32) {
-        const int i = pairs[t].x, j = pairs[t].y;
-        if (i == k + 1 && j == k + 1) continue;
-        // i >= j: in the pivot row (i = k) u_i v_j would be -a_jk / p with the
-        // pivot's -1 in u_i, in the pivot column (j = k) the -r in v_j.
-        A[i * m + j] = fma(-u[i], v[j], i == k || j == k ? 0.0 : A[i * m + j]);
+#pragma unroll
+      for (int q = 0; q < ND; ++q) {
+        const int d = lane + 32 * q;
+        if (32 * q < m && d > k && d < m) {
+          dg[q] = fma(-uk[d], v[d], dg[q]);
+          if (d == k + 1) pivot(dg[q], k + 1);
+        }
       }
     }
     __syncthreads();
   }
+#pragma unroll
+  for (int e = 0; e < E; ++e)
+    if (ij[e] >= 0) X1[(ij[e] >> 16) * m + (ij[e] & 0xffff)] = A[e];
+  __syncthreads();
   const bool leaf = g.hi - g.lo == 1;
-  for (int t = tid; t < m * m; t += SEP_NT) {
+  for (int t = tid; t < m * m; t += SEP_BLOCK) {
     const int i = t / m, j = t % m;
-    const double x = -(i >= j ? A[i * m + j] : A[j * m + i]);
+    const double x = -(i >= j ? X1[i * m + j] : X1[j * m + i]);
     a.S[(size_t)(base + i) * m + j] = x;
     if (leaf) a.Kinv[(size_t)(base + i) * a.n + base + j] = x;
   }
 }
 
-__global__ void __launch_bounds__(SEP_NT) separator_kernel(BlockRows a, int depth) {
+template <int E> __global__ void __launch_bounds__(SEP_BLOCK) separator_kernel(BlockRows a, int depth) {
   pdl_wait();
   extern __shared__ double dyn[];
   const int nranges = 1 << depth;
   if ((int)blockIdx.x < nranges) {
     Range g;
-    if (range_of(a.J, depth, -1, blockIdx.x, g)) form_s(a, g, dyn);
+    if (range_of(a.J, depth, -1, blockIdx.x, g)) form_s<E>(a, g, dyn);
   } else {
     form_v(a, depth, ((int)blockIdx.x - nranges) * V_ROWS);
   }
@@ -305,29 +335,31 @@ __global__ void __launch_bounds__(TILE_NT) range_update_kernel(BlockRows a, int 
 #pragma unroll
     for (int w = 0; w < 2; ++w) any = any || (lo_r[u] >= 0 && lo_r[u] == lo_c[w]);
   if (!__syncthreads_or(any)) return;
-  // W of the tile's rows and V of its columns, staged 32 columns at a time.
-  __shared__ double ws[TILE][33], vs[TILE][33];
-  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-  for (int k0c = 0; k0c < m; k0c += 32) {
-    const int kn = min(32, m - k0c);
-    for (int q = threadIdx.x; q < TILE * 32; q += TILE_NT) {
-      const int i = q >> 5, k = q & 31;
-      const int ri = I * TILE + i, ci = K * TILE + i;
-      ws[i][k] = k < kn && ri < n ? a.W[(size_t)ri * m + k0c + k] : 0.0;
-      vs[i][k] = k < kn && ci < n ? a.V[(size_t)ci * m + k0c + k] : 0.0;
-    }
-    __syncthreads();
-    for (int k = half; k < kn; k += 2) {
-      const double w0 = ws[ty][k], w1 = ws[ty + 8][k], v0 = vs[tx][k], v1 = vs[tx + 8][k];
-      acc[0][0] = fma(-w0, v0, acc[0][0]);
-      acc[0][1] = fma(-w0, v1, acc[0][1]);
-      acc[1][0] = fma(-w1, v0, acc[1][0]);
-      acc[1][1] = fma(-w1, v1, acc[1][1]);
-    }
-    __syncthreads();
+  // W of the tile's rows and V of its columns (row pitch odd: no bank conflicts
+  // down a column of the tile).
+  extern __shared__ double dyn[];
+  const int pitch = m + 1;
+  double *ws = dyn, *vs = dyn + TILE * pitch;
+  for (int q = threadIdx.x; q < TILE * m; q += TILE_NT) {
+    const int i = q / m, k = q - i * m;
+    const int ri = I * TILE + i, ci = K * TILE + i;
+    ws[i * pitch + k] = ri < n ? a.W[(size_t)ri * m + k] : 0.0;
+    vs[i * pitch + k] = ci < n ? a.V[(size_t)ci * m + k] : 0.0;
   }
+  __syncthreads();
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  const double *w0p = ws + ty * pitch, *w1p = w0p + 8 * pitch, *v0p = vs + tx * pitch, *v1p = v0p + 8 * pitch;
+#pragma unroll 4
+  for (int k = half; k < m; k += 2) {
+    const double w0 = w0p[k], w1 = w1p[k], v0 = v0p[k], v1 = v1p[k];
+    acc[0][0] = fma(-w0, v0, acc[0][0]);
+    acc[0][1] = fma(-w0, v1, acc[0][1]);
+    acc[1][0] = fma(-w1, v0, acc[1][0]);
+    acc[1][1] = fma(-w1, v1, acc[1][1]);
+  }
+  __syncthreads();
   // The odd columns' sums join the even ones'.
-  double* odd = &ws[0][0];
+  double* odd = dyn;
   if (half == 1) {
 #pragma unroll
     for (int u = 0; u < 2; ++u)
@@ -353,8 +385,21 @@ __global__ void __launch_bounds__(TILE_NT) range_update_kernel(BlockRows a, int 
     }
 }
 
+size_t update_smem(int m) { return sizeof(double) * (size_t)(2 * TILE * (m + 1) > 256 ? 2 * TILE * (m + 1) : 256); }
+
 size_t separator_smem(int m) {
-  return sizeof(double) * (4 * (size_t)m * m + (2 * NCOUPLE + 2) * m) + sizeof(short2) * ((size_t)m * (m + 1) / 2);
+  return sizeof(double) * (4 * (size_t)m * m + (2 * NCOUPLE + 4) * m);
+}
+
+// Entries of S per thread: the fewest that hold m (m + 1) / 2 of them.
+using SeparatorKernel = void (*)(BlockRows, int);
+SeparatorKernel separator_for(int m) {
+  const int np = m * (m + 1) / 2;
+  if (np <= 3 * SEP_NT) return separator_kernel<3>;
+  if (np <= 6 * SEP_NT) return separator_kernel<6>;
+  if (np <= 10 * SEP_NT) return separator_kernel<10>;
+  static_assert(MAX_BLOCK_ROW * (MAX_BLOCK_ROW + 1) / 2 <= 15 * SEP_NT, "widest block row");
+  return separator_kernel<15>;
 }
 
 }  // namespace
@@ -362,7 +407,7 @@ size_t separator_smem(int m) {
 bool block_inverse_fits(int n, int m) { return m >= 2 && m <= MAX_BLOCK_ROW && n >= m && n % m == 0; }
 
 cudaError_t prepare_block_inverse(int m) {
-  return raise_max_dynamic_smem((const void*)separator_kernel, separator_smem(m));
+  return raise_max_dynamic_smem((const void*)separator_for(m), separator_smem(m));
 }
 
 cudaError_t launch_block_inverse(int n, int m, int bw, const double* Kb, double* work, double* Kinv, int* err_flag,
@@ -374,13 +419,13 @@ cudaError_t launch_block_inverse(int n, int m, int bw, const double* Kb, double*
   for (int d = depth; d >= 0; --d) {
     // Ranges of the deepest level are single rows: no V.
     const int vblocks = d == depth ? 0 : (n + V_ROWS - 1) / V_ROWS;
-    cudaError_t e = launch_pdl(separator_kernel, (1 << d) + vblocks, SEP_NT, separator_smem(m), s, a, d);
+    cudaError_t e = launch_pdl(separator_for(m), (1 << d) + vblocks, SEP_BLOCK, separator_smem(m), s, a, d);
     if (e != cudaSuccess) return e;
     *launches += 1;
     if (d == depth) continue;
     e = launch_pdl(separator_column_kernel, (n + W_ROWS - 1) / W_ROWS, W_NT, 0, s, a, d);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(range_update_kernel, ntiles, TILE_NT, 0, s, a, d);
+    e = launch_pdl(range_update_kernel, ntiles, TILE_NT, update_smem(m), s, a, d);
     if (e != cudaSuccess) return e;
     *launches += 2;
   }

@@ -105,6 +105,10 @@ int main() {
       if (q[i] >> 63) back = -back;
       if (std::fabs(back - c6[i]) > std::fabs(p) * 1.2e-16) return fail("coarse factor", n);
     }
+    // Reciprocal: within an ulp.
+    const double rd = make(0, 30 + (int)(next_u64() % 1980), t % 5 ? next_u64() : (t % 3 ? 0 : ~0ull));
+    const double rq = fx_reciprocal(rd), rw = 1.0 / rd;
+    if (rq != rw && rq != std::nextafter(rw, INFINITY) && rq != std::nextafter(rw, 0.0)) return fail("reciprocal", n);
     if (fx_wide(fx_flip(a, -1)) != -fx_wide(a) || fx_wide(fx_flip(a, 0)) != fx_wide(a)) return fail("flip", n);
   }
   unsigned long long z[FX_NCOARSE];
