@@ -106,9 +106,6 @@ __host__ __device__ __forceinline__ Fx fx_sar(const Fx& a, int s) {
   return fx_sar31(fx_sar_limbs(a, s), s & 31);
 }
 
-// Biased exponent of a float64 from its upper word (0: zero or subnormal).
-__host__ __device__ __forceinline__ int fx_exponent(unsigned hi) { return (int)((hi >> 20) & 0x7ffu); }
-
 // The significand of a finite float64 before the shift to the common scale
 // (by B - max(exponent, 1)): times 2^38, upper two limbs (the lowest is zero),
 // with sign.  With FLUSH subnormals give zero: where B > FX_FLUSH_B they lie
@@ -222,41 +219,6 @@ template <bool CHECKED = true> __host__ __device__ __forceinline__ double fx_to_
   }
   const double r = double_of(((m >> 11) + ((m >> 10) & 1u) + ((unsigned long long)(unsigned)ex << 52)) | sign);
   return a2 != 0u ? r : 0.0;
-}
-
-// 1 / d to within an ulp for normal d > 0 whose reciprocal is normal, on the
-// integer pipe: a dependent FP64 operation costs about 140 clocks here, the
-// division a chain of ten, this about 150 in all.  Newton's iteration of third
-// order, R + R (e + e^2) with e = 1 - D R, on the significand D in [1, 2) from
-// the float32 reciprocal R (|e| < 2^-21, so what is left is below 2^-62).
-__host__ __device__ __forceinline__ double fx_reciprocal(double d) {
-  const unsigned long long bits = bits_of(d);
-  const unsigned hi = (unsigned)(bits >> 32);
-  const int k = fx_exponent(hi) - 1023;
-  const unsigned long long D = ((bits & 0xfffffffffffffull) | 0x10000000000000ull) << 11;  // D 2^63
-  // The leading 24 bits of D as a float32, truncated.
-  const float df = float_of(0x3f800000u | (unsigned)((bits >> 29) & 0x7fffffu));
-#ifdef __CUDA_ARCH__
-  const float y = __frcp_rn(df);  // in (1/2, 1]
-#else
-  const float y = 1.0f / df;
-#endif
-  // R 2^32, below 2^32: the float32's 24 bits one place up, less one unit of 2^-32.
-  const unsigned yb = bits_of(y);
-  const unsigned R = y < 1.0f ? ((yb & 0x7fffffu) | 0x800000u) << 8 : 0xffffffffu;
-  // e 2^63 = 2^63 - D R 2^-32 2^... : D R 2^95 from two 32 x 32 products.
-  const unsigned long long lo = (unsigned long long)(unsigned)D * R, up = (unsigned long long)(unsigned)(D >> 32) * R;
-  const unsigned long long p = up + (lo >> 32);  // D R 2^63 (floor)
-  const long long e = (long long)(0x8000000000000000ull - p);
-  const long long es = e >> 20;                 // e 2^43
-  const long long c = e + ((es * es) >> 23);    // e + e^2, scaled by 2^63
-  // R (1 + c) 2^63 = R 2^32 2^31 + (R 2^32) (c 2^63) 2^-32.
-  const long long ch = c >> 32;
-  const unsigned long long cl = (unsigned long long)c & 0xffffffffull;
-  const unsigned long long q =
-      ((unsigned long long)R << 31) + (unsigned long long)(ch * (long long)R) + ((cl * R) >> 32);
-  const unsigned long long m = (q + 0x200ull) >> 10;  // 53 bits (2^53 for d a power of two)
-  return double_of(((unsigned long long)(unsigned)(1021 - k) << 52) + m);
 }
 
 // (m << lift) aligned to exponent X, for a factor f of magnitude m 2^(e - 1075).

@@ -50,6 +50,7 @@ struct PLevel {
   int nx, ny;       // elements; nodes (nx + 1) x (ny + 1), row pitch nx + 1
   void* z[2];       // iterates (ping-pong) in the V-cycle's type; boundary entries stay zero
   void* b;          // right-hand side (coarse levels), same type
+  unsigned magic;   // ceil(2^32 / (nx - 1)) where it divides every node index exactly, else 0
 };
 
 struct PStats {
@@ -87,13 +88,36 @@ __device__ __forceinline__ void rows_of(int ny, Part pt, int& j0, int& j1) {
   j1 = min(ny, j0 + per);
 }
 
+// t / w by the level's multiplier (the division by a run-time width took as
+// long as the stencil's loads).
+__device__ __forceinline__ int div_width(int t, int w, unsigned magic) {
+  return magic ? (int)__umulhi((unsigned)t, magic) : t / w;
+}
+
+// float <-> double on the integer pipe (the FP64 pipe also runs the hardware
+// conversions, at 64 clocks a warp); subnormal and out-of-range values take
+// the hardware path, so that every value is converted as by a cast.
+__device__ __forceinline__ double wide(double v) { return v; }
+__device__ __forceinline__ double wide(float v) {
+  const unsigned b = __float_as_uint(v);
+  if ((b & 0x7f800000u) == 0u && (b << 1) != 0u) return (double)v;
+  return mto::f2d_exact(v);
+}
+template <typename VT> __device__ __forceinline__ VT narrow(double v);
+template <> __device__ __forceinline__ double narrow<double>(double v) { return v; }
+template <> __device__ __forceinline__ float narrow<float>(double v) {
+  const unsigned e = ((unsigned)__double2hiint(v) >> 20) & 0x7ffu;
+  if (e != 0u && e - 897u >= 253u) return (float)v;
+  return mto::d2f_rn(v);
+}
+
 // For every interior node of this CTA's rows: v = ld(i, j, k), then st(k, v).
 // Each thread takes NB nodes at a time and evaluates ld (loads and
 // arithmetic, no stores) for all of them before the first st, so that the
 // loads of the NB nodes are in flight together: a phase then costs about
 // nodes / (NB * threads) memory round trips instead of nodes / threads.
 template <int NB, typename Ld, typename St>
-__device__ __forceinline__ void for_nodes_nb(int nx, int ny, Part pt, Ld ld, St st) {
+__device__ __forceinline__ void for_nodes_nb(int nx, int ny, unsigned magic, Part pt, Ld ld, St st) {
   int j0, j1;
   rows_of(ny, pt, j0, j1);
   const int w = nx - 1;
@@ -106,8 +130,9 @@ __device__ __forceinline__ void for_nodes_nb(int nx, int ny, Part pt, Ld ld, St 
       const int t = t0 + u * PNT;
       ks[u] = -1;
       if (t < count) {
-        const int j = j0 + t / w;
-        const int i = 1 + t % w;
+        const int row = div_width(t, w, magic);
+        const int j = j0 + row;
+        const int i = 1 + t - row * w;
         ks[u] = j * (nx + 1) + i;
         v[u] = ld(i, j, ks[u]);
       }
@@ -119,14 +144,15 @@ __device__ __forceinline__ void for_nodes_nb(int nx, int ny, Part pt, Ld ld, St 
 }
 
 // Calls fn(i, j, k) for every interior node of this CTA's rows.
-template <typename F> __device__ __forceinline__ void for_nodes(int nx, int ny, Part pt, F fn) {
+template <typename F> __device__ __forceinline__ void for_nodes(int nx, int ny, unsigned magic, Part pt, F fn) {
   int j0, j1;
   rows_of(ny, pt, j0, j1);
   const int w = nx - 1;
   const int count = (j1 - j0) * w;
   for (int t = threadIdx.x; t < count; t += PNT) {
-    const int j = j0 + t / w;
-    const int i = 1 + t % w;
+    const int row = div_width(t, w, magic);
+    const int j = j0 + row;
+    const int i = 1 + t - row * w;
     fn(i, j, j * (nx + 1) + i);
   }
 }
@@ -146,7 +172,7 @@ enum { SLOT_RHO = 0, SLOT_PQ = 1, SLOT_RR = 2, SLOT_FF = 3, SLOT_TRUE = 3, SLOT_
 
 // The 9-point stencil on a vector of type T, evaluated in float64.
 template <typename T> __device__ __forceinline__ double apply_k64(const T* z, int k, int pitch) {
-  auto v = [&](int o) { return (double)z[k + o]; };
+  auto v = [&](int o) { return wide(z[k + o]); };
   const double s = (v(-pitch - 1) + v(-pitch) + v(-pitch + 1)) + (v(-1) + v(1)) +
                    (v(pitch - 1) + v(pitch) + v(pitch + 1));
   return (8.0 * v(0) - s) * (1.0 / 3.0);
@@ -181,51 +207,62 @@ template <typename VT, bool MANY> struct Solver {
   }
   __device__ VT* Z(int l, int i) const { return static_cast<VT*>(d.lv[l].z[i]); }
   __device__ VT* B(int l) const { return static_cast<VT*>(d.lv[l].b); }
+  // A right-hand side entry in the V-cycle's type.
+  __device__ static VT narrow_b(double v) { return narrow<VT>(v); }
+  __device__ static VT narrow_b(float v) { return v; }
   // Iterate buffers: the pre-smoothed iterate and the final one of level l.
   __device__ int pre_buf() const { return (d.nu1 - 1) & 1; }
   __device__ int final_buf(int l) const { return l == 0 ? 0 : (d.nu1 - 1 + d.nu2) & 1; }
 
-  // Sum of a (and b) over the cluster, in rank order; every thread of every
-  // CTA gets the same result.  Includes the phase barrier.
-  __device__ void allreduce(double& a, double& b, int slot_a, int slot_b) {
+  // Sum of a (and, with TWO, b) over the cluster; every thread of every CTA
+  // gets the same result (the same tree over the CTAs' sums everywhere).
+  // Includes the phase barrier.  A warp's float64 instruction holds its
+  // scheduler's pipe for 64 clocks, so no thread sums in series what lanes can.
+  template <bool TWO> __device__ void allreduce_n(double& a, double& b, int slot_a, int slot_b) {
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       a += __shfl_xor_sync(0xffffffffu, a, o);
-      b += __shfl_xor_sync(0xffffffffu, b, o);
+      if (TWO) b += __shfl_xor_sync(0xffffffffu, b, o);
     }
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) {
+    if (lane == 0) {
       sh.warp[0][w] = a;
-      sh.warp[1][w] = b;
+      if (TWO) sh.warp[1][w] = b;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      double sa = 0.0, sb = 0.0;
-      for (int i = 0; i < PWARPS; ++i) {
-        sa += sh.warp[0][i];
-        sb += sh.warp[1][i];
+    if (w == 0) {
+      double sa = lane < PWARPS ? sh.warp[0][lane] : 0.0, sb = TWO && lane < PWARPS ? sh.warp[1][lane] : 0.0;
+#pragma unroll
+      for (int o = PWARPS / 2; o > 0; o >>= 1) {
+        sa += __shfl_xor_sync(0xffffffffu, sa, o);
+        if (TWO) sb += __shfl_xor_sync(0xffffffffu, sb, o);
       }
-      if (C > 1) {
-        for (int dst = 0; dst < C; ++dst) {
-          cl.map_shared_rank(&sh.red[slot_a][0], dst)[rank] = sa;
-          if (slot_b >= 0) cl.map_shared_rank(&sh.red[slot_b][0], dst)[rank] = sb;
-        }
-      } else {
-        sh.red[slot_a][0] = sa;
-        if (slot_b >= 0) sh.red[slot_b][0] = sb;
+      sa = __shfl_sync(0xffffffffu, sa, 0);
+      if (TWO) sb = __shfl_sync(0xffffffffu, sb, 0);
+      if (lane < C) {
+        PShared* dst = C > 1 ? cl.map_shared_rank(&sh, lane) : &sh;
+        dst->red[slot_a][rank] = sa;
+        if (TWO) dst->red[slot_b][rank] = sb;
       }
     }
     sync(C > 1);
-    a = 0.0;
-    b = 0.0;
-    for (int i = 0; i < C; ++i) {
-      a += sh.red[slot_a][i];
-      if (slot_b >= 0) b += sh.red[slot_b][i];
+    a = lane < C ? sh.red[slot_a][lane] : 0.0;
+    if (TWO) b = lane < C ? sh.red[slot_b][lane] : 0.0;
+#pragma unroll
+    for (int o = PMAXC / 2; o > 0; o >>= 1) {
+      if (o >= C) continue;  // the lanes beyond hold zeros
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (TWO) b += __shfl_xor_sync(0xffffffffu, b, o);
     }
+    a = __shfl_sync(0xffffffffu, a, 0);
+    if (TWO) b = __shfl_sync(0xffffffffu, b, 0);
+  }
+  __device__ void allreduce(double& a, double& b, int slot_a, int slot_b) {
+    allreduce_n<true>(a, b, slot_a, slot_b);
   }
   __device__ double allreduce1(double a, int slot) {
     double b = 0.0;
-    allreduce(a, b, slot, -1);
+    allreduce_n<false>(a, b, slot, slot);
     return a;
   }
 
@@ -241,16 +278,16 @@ template <typename VT, bool MANY> struct Solver {
     const int pitch = lv.nx + 1;
     const VT wd = VT(d.wd), cz = VT(1.0 - 8.0 * d.wd / 3.0), cs = VT(d.wd / 3.0);
     // Nodes in flight per thread: as many as the 255-register budget holds.
-    constexpr int NB = (sizeof(VT) == 8 ? 4 : 8) / (MANY ? 2 : 1);
+    constexpr int NB = (sizeof(VT) == 8 ? 4 : 8) / (MANY ? 4 : 1);
     for_nodes_nb<NB>(
-        lv.nx, lv.ny, part(cluster),
+        lv.nx, lv.ny, lv.magic, part(cluster),
         [&](int, int, int k) {
-          return fma(cz, src[k], fma(wd, VT(b[k]), cs * nbsum_t(src, k, pitch)));
+          return fma(cz, src[k], fma(wd, narrow_b(b[k]), cs * nbsum_t(src, k, pitch)));
         },
         [&](int k, VT v) {
           dst[k] = v;
-          if (dotv) acc = fma((double)v, dotv[k], acc);
-          if (dotq) accq = fma((double)v, dotq[k], accq);
+          if (dotv) acc = fma(wide(v), dotv[k], acc);
+          if (dotq) accq = fma(wide(v), dotq[k], accq);
         });
   }
 
@@ -259,8 +296,8 @@ template <typename VT, bool MANY> struct Solver {
   __device__ void prolong_add(int l, VT* z, const VT* zc, bool cluster) {
     const PLevel& lv = d.lv[l];
     const int pc = d.lv[l - 1].nx + 1;
-    for_nodes_nb<MANY ? 2 : 4>(
-        lv.nx, lv.ny, part(cluster),
+    for_nodes_nb<MANY ? 1 : 4>(
+        lv.nx, lv.ny, lv.magic, part(cluster),
         [&](int i, int j, int k) { return z[k] + prolong_t(zc, pc, i, j); },
         [&](int k, VT v) { z[k] = v; });
   }
@@ -271,9 +308,9 @@ template <typename VT, bool MANY> struct Solver {
     const PLevel& lv = d.lv[l];
     const int pitch = lv.nx + 1;
     const VT third = VT(1.0 / 3.0);
-    for_nodes_nb<MANY ? 2 : 4>(
-        lv.nx, lv.ny, part(cluster),
-        [&](int, int, int k) { return VT(b[k]) - (VT(8) * zpre[k] - nbsum_t(zpre, k, pitch)) * third; },
+    for_nodes_nb<MANY ? 1 : 4>(
+        lv.nx, lv.ny, lv.magic, part(cluster),
+        [&](int, int, int k) { return narrow_b(b[k]) - (VT(8) * zpre[k] - nbsum_t(zpre, k, pitch)) * third; },
         [&](int k, VT v) { res[k] = v; });
   }
 
@@ -287,8 +324,8 @@ template <typename VT, bool MANY> struct Solver {
     VT* z0 = Z(l - 1, 0);
     const VT wd = VT(d.wd), h = VT(0.5), qt = VT(0.25);
     const bool first = l - 1 >= 1;
-    for_nodes_nb<MANY ? 2 : 4>(
-        c.nx, c.ny, part(cluster),
+    for_nodes_nb<MANY ? 1 : 4>(
+        c.nx, c.ny, c.magic, part(cluster),
         [&](int I, int J, int) {
           const int k = 2 * J * pf + 2 * I;
           return res[k] + h * ((res[k - 1] + res[k + 1]) + (res[k - pf] + res[k + pf])) +
@@ -313,11 +350,11 @@ template <typename VT, bool MANY> struct Solver {
     VT* z0 = Z(l - 1, 0);
     const VT wd = VT(d.wd), h = VT(0.5), qt = VT(0.25), third = VT(1.0 / 3.0);
     const bool first = l - 1 >= 1;
-    for_nodes_nb<2>(
-        c.nx, c.ny, part(cluster),
+    for_nodes_nb<MANY ? 1 : 2>(
+        c.nx, c.ny, c.magic, part(cluster),
         [&](int I, int J, int) {
           const int k = 2 * J * pf + 2 * I;
-          auto res = [&](int kk) { return VT(b[kk]) - (VT(8) * zpre[kk] - nbsum_t(zpre, kk, pf)) * third; };
+          auto res = [&](int kk) { return narrow_b(b[kk]) - (VT(8) * zpre[kk] - nbsum_t(zpre, kk, pf)) * third; };
           return res(k) + h * ((res(k - 1) + res(k + 1)) + (res(k - pf) + res(k + pf))) +
                  qt * ((res(k - pf - 1) + res(k - pf + 1)) + (res(k + pf - 1) + res(k + pf + 1)));
         },
@@ -333,20 +370,20 @@ template <typename VT, bool MANY> struct Solver {
     const PLevel& lv = d.lv[l];
     const int pitch = lv.nx + 1, pc = d.lv[l - 1].nx + 1;
     const VT wd = VT(d.wd), cz = VT(1.0 - 8.0 * d.wd / 3.0), cs = VT(d.wd / 3.0);
-    for_nodes_nb<2>(
-        lv.nx, lv.ny, part(cluster),
+    for_nodes_nb<MANY ? 1 : 2>(
+        lv.nx, lv.ny, lv.magic, part(cluster),
         [&](int i, int j, int k) {
           auto zf = [&](int di, int dj) {
             return zpre[k + dj * pitch + di] + prolong_t(zc, pc, i + di, j + dj);
           };
           const VT s = (zf(-1, -1) + zf(0, -1) + zf(1, -1)) + (zf(-1, 0) + zf(1, 0)) +
                        (zf(-1, 1) + zf(0, 1) + zf(1, 1));
-          return fma(cz, zf(0, 0), fma(wd, VT(b[k]), cs * s));
+          return fma(cz, zf(0, 0), fma(wd, narrow_b(b[k]), cs * s));
         },
         [&](int k, VT v) {
           dst[k] = v;
-          if (dotv) acc = fma((double)v, dotv[k], acc);
-          if (dotq) accq = fma((double)v, dotq[k], accq);
+          if (dotv) acc = fma(wide(v), dotv[k], acc);
+          if (dotq) accq = fma(wide(v), dotq[k], accq);
         });
   }
 
@@ -360,10 +397,10 @@ template <typename VT, bool MANY> struct Solver {
     for (int a = warp; a < n; a += PWARPS) {
       double s = 0.0;
       for (int bb = lane; bb < n; bb += 32)
-        s = fma(d.Kinv[(size_t)a * n + bb], (double)b0[(1 + bb / w) * pitch + 1 + bb % w], s);
+        s = fma(d.Kinv[(size_t)a * n + bb], wide(b0[(1 + bb / w) * pitch + 1 + bb % w]), s);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) z0[(1 + a / w) * pitch + 1 + a % w] = VT(s);
+      if (lane == 0) z0[(1 + a / w) * pitch + 1 + a % w] = narrow<VT>(s);
     }
   }
 
@@ -478,10 +515,10 @@ template <typename VT, bool MANY> struct Solver {
     }
     sync(cl_on);
     double rr = 0.0, ff = 0.0;
-    for_nodes(nx, ny, pt, [&](int, int, int k) {
+    for_nodes(nx, ny, F.magic, pt, [&](int, int, int k) {
       const double rk = f[k] - apply_k64(x, k, pitch);
       r[k] = rk;
-      z0[k] = VT(wd * rk);
+      z0[k] = narrow<VT>(wd * rk);
       rr = fma(rk, rk, rr);
       ff = fma(f[k], f[k], ff);
     });
@@ -489,7 +526,7 @@ template <typename VT, bool MANY> struct Solver {
     int it = 0, status = PST_RUNNING;
     double rho_old = 1.0, alpha_old = 0.0;
     const VT* z = Z(d.L, final_buf(d.L));
-    constexpr int NBC = (sizeof(VT) == 8 ? 4 : 8) / (MANY ? 2 : 1);  // nodes in flight per thread (registers)
+    constexpr int NBC = (sizeof(VT) == 8 ? 4 : 8) / (MANY ? 4 : 1);  // nodes in flight per thread (registers)
     for (;;) {
       if (!isfinite(rr)) {
         status = PST_BREAKDOWN;
@@ -520,13 +557,13 @@ template <typename VT, bool MANY> struct Solver {
         status = PST_BREAKDOWN;
         break;
       }
-      const double beta = it == 0 ? 0.0 : (flex ? -alpha_old * zq / rho_old : rho / rho_old);
+      const double beta = it == 0 ? 0.0 : (flex ? mto::quotient(-alpha_old * zq, rho_old) : mto::quotient(rho, rho_old));
       double pq = 0.0;
       for_nodes_nb<NBC>(
-          nx, ny, pt,
+          nx, ny, F.magic, pt,
           [&](int, int, int k) {
             const double kz = apply_k64(z, k, pitch);
-            const double zk = (double)z[k];
+            const double zk = wide(z[k]);
             const double pk = it == 0 ? zk : fma(beta, p[k], zk);
             const double qk = it == 0 ? kz : fma(beta, q[k], kz);
             return double2{pk, qk};
@@ -541,15 +578,15 @@ template <typename VT, bool MANY> struct Solver {
         status = PST_BREAKDOWN;
         break;
       }
-      const double alpha = rho / pq;
+      const double alpha = mto::quotient(rho, pq);
       double rn = 0.0;
       for_nodes_nb<NBC>(
-          nx, ny, pt,
+          nx, ny, F.magic, pt,
           [&](int, int, int k) { return double2{fma(alpha, p[k], x[k]), fma(-alpha, q[k], r[k])}; },
           [&](int k, double2 v) {
             x[k] = v.x;
             r[k] = v.y;
-            z0[k] = VT(wd * v.y);  // the next V-cycle's first smoothing step from zero
+            z0[k] = narrow<VT>(wd * v.y);  // the next V-cycle's first smoothing step from zero
             rn = fma(v.y, v.y, rn);
           });
       rr = allreduce1(rn, SLOT_RR);
@@ -559,7 +596,7 @@ template <typename VT, bool MANY> struct Solver {
     }
     // True residual of the returned iterate.
     double rt = 0.0;
-    for_nodes(nx, ny, pt, [&](int, int, int k) {
+    for_nodes(nx, ny, F.magic, pt, [&](int, int, int k) {
       const double rk = f[k] - apply_k64(x, k, pitch);
       rt = fma(rk, rk, rt);
     });
@@ -580,7 +617,7 @@ template <typename VT, bool MANY> struct Solver {
     const double wd = d.wd;
     const double* v = d.f;
     VT* z0 = Z(d.L, 0);
-    for_nodes(F.nx, F.ny, part(cl_on), [&](int, int, int k) { z0[k] = VT(wd * v[k]); });
+    for_nodes(F.nx, F.ny, F.magic, part(cl_on), [&](int, int, int k) { z0[k] = VT(wd * v[k]); });
     sync(cl_on);
     double u = 0.0, w = 0.0;
     vcycle(v, nullptr, nullptr, u, w);
@@ -598,7 +635,7 @@ template <typename VT, bool MANY> struct Solver {
     const int nx = F.nx, ny = F.ny, pitch = nx + 1;
     const double* v = d.f;
     double* y = d.x;
-    for_nodes(nx, ny, part(C > 1), [&](int i, int j, int k) {
+    for_nodes(nx, ny, F.magic, part(C > 1), [&](int i, int j, int k) {
       auto vv = [&](int di, int dj) {
         const int ii = i + di, jj = j + dj;
         return (ii == 0 || ii == nx || jj == 0 || jj == ny) ? 0.0 : v[k + dj * pitch + di];
@@ -623,12 +660,13 @@ template <typename VT, bool MANY> struct Solver {
 
 // One cluster of C CTAs per descriptor (right-hand side); VT is the V-cycle's
 // value type.  MANY: more clusters than the chip holds at one CTA per SM, so
-// two share each SM (128 registers, half the nodes in flight per thread) and
-// run while the other waits; the arithmetic and its order are the same.  64
-// right-hand sides at 256^2: 12.2 -> 8.8 ms (float64 V-cycle), 10.4 -> 6.7 ms
-// (float32).
+// four share each SM (64 registers, a quarter of the nodes in flight per
+// thread) and run while the others wait; the arithmetic and its order are the
+// same.  64 right-hand sides at 256^2: 12.2 -> 6.8 ms (float64 V-cycle), 10.4 ->
+// 4.0 ms (float32); two to a SM took 8.7 and 6.7 ms, three 7.7 and 5.5, six 6.9
+// and 4.2 (spills).
 template <typename VT, bool MANY>
-__global__ void __launch_bounds__(PNT, MANY ? 2 : 1) poisson_cluster_kernel(const PDesc* __restrict__ descs, int C) {
+__global__ void __launch_bounds__(PNT, MANY ? 4 : 1) poisson_cluster_kernel(const PDesc* __restrict__ descs, int C) {
   __shared__ PDesc sd;
   __shared__ PShared sh;
   cg::cluster_group cl = cg::this_cluster();
@@ -863,6 +901,9 @@ PDesc make_desc(const mto_poisson* c, int k, int mode, const double* in, double*
     const int sh = c->L - l;
     d.lv[l].nx = c->nelx >> sh;
     d.lv[l].ny = c->nely >> sh;
+    // Exact for every index t with t width < 2^32.
+    const unsigned long long width = d.lv[l].nx - 1, nodes = width * (d.lv[l].ny - 1);
+    d.lv[l].magic = width > 1 && nodes * width < (1ull << 32) ? (unsigned)(((1ull << 32) + width - 1) / width) : 0u;
     d.lv[l].z[0] = base + w.z0[l];
     d.lv[l].z[1] = base + w.z1[l];
     d.lv[l].b = base + w.b[l];
