@@ -191,9 +191,10 @@ mto_status coarse_cycle(mto_ctx* c, int l, DevScalars* sc, int start, int* final
   };
   // Pre-smoothing from U = 0: the first sweep (U = w D^-1 F) is formed on the
   // fly inside the second when there are two or more.  With exactly two on a
-  // float32 level, the residual and its restriction run in the same pass
-  // (mto_fused.cuh).
-  const bool fused_pre = (src == SRC_CMOM || src == SRC_CFINE) && c->o.nu1 == 2;
+  // float32 level or a small float64 one, the residual and its restriction run
+  // in the same pass (mto_fused.cuh, mto_tile.cuh, mto_ftile.cuh).
+  const bool two_stage = sizeof(T) == 4 || float64_tiles(L.g, tw, c->num_sms);
+  const bool fused_pre = two_stage && c->o.nu1 == 2;
   if (start >= 0) {
     cur = start;
     for (int s = 0; s < c->o.nu1; ++s) {
@@ -218,10 +219,9 @@ mto_status coarse_cycle(mto_ctx* c, int l, DevScalars* sc, int start, int* final
   }
   int cidx = 0;
   ST(coarse_calls<T>(c, l - 1, c->o.gamma, sc, &cidx));
-  // Post-smoothing; on the float32 levels the prolongation sweep and the
-  // next one run fused (mto_fused.cuh).
+  // Post-smoothing; there the prolongation sweep and the next one run fused.
   int s = 1;
-  if ((src == SRC_CMOM || src == SRC_CFINE) && c->o.nu2 >= 2) {
+  if (two_stage && c->o.nu2 >= 2) {
     KL(sweep(MODE_POST2, (const T2*)L.z[cur], (T2*)L.z[cur ^ 1], (const T2*)C.z[cidx]));
     s = 2;
   } else {
@@ -332,26 +332,42 @@ mto_status fine_cycle(mto_ctx* c, DevScalars* sc, bool with_dot, int* final_idx)
               : cudaSuccess;
   };
   int first = 1;
-  if (fused0) {
+  // Small float64 grids: both pre-smoothing sweeps with the restriction, and
+  // the prolongation with the next sweep, in one pass each (mto_ftile.cuh).
+  const bool two_stage = !MIX && float64_tiles(L.g, tw, c->num_sms);
+  if (two_stage && c->o.nu1 == 2) {
     CK(t0());
-    KL(sweep(MODE_SMOOTH0, nullptr, (T2*)L.z[0], nullptr, fuse_update(c) && with_dot));
+    KL(sweep(MODE_PRE2, nullptr, (T2*)L.z[0], nullptr, false));
     CK(t1());
-    first = 2;
+  } else {
+    if (fused0) {
+      CK(t0());
+      KL(sweep(MODE_SMOOTH0, nullptr, (T2*)L.z[0], nullptr, fuse_update(c) && with_dot));
+      CK(t1());
+      first = 2;
+    }
+    for (int s = first; s < c->o.nu1; ++s) {
+      if (s == 1) CK(t0());
+      KL(sweep(MODE_SMOOTH, (const T2*)L.z[cur], (T2*)L.z[cur ^ 1], nullptr, false));
+      if (s == 1) CK(t1());
+      cur ^= 1;
+    }
+    KL(sweep(MODE_RESTRICT, (const T2*)L.z[cur], nullptr, nullptr, false));
   }
-  for (int s = first; s < c->o.nu1; ++s) {
-    if (s == 1) CK(t0());
-    KL(sweep(MODE_SMOOTH, (const T2*)L.z[cur], (T2*)L.z[cur ^ 1], nullptr, false));
-    if (s == 1) CK(t1());
-    cur ^= 1;
-  }
-  KL(sweep(MODE_RESTRICT, (const T2*)L.z[cur], nullptr, nullptr, false));
   // Alg. 1 calls the next coarser grid once from the finest grid.
   int cidx = 0;
   ST(coarse_calls<T>(c, c->L - 1, 1, sc, &cidx));
-  KL(sweep(MODE_PSMOOTH, (const T2*)L.z[cur], (T2*)L.z[cur ^ 1], (const T2*)C.z[cidx],
-           with_dot && c->o.nu2 == 1));
+  int post = 1;
+  if (two_stage && c->o.nu2 >= 2) {
+    post = 2;
+    KL(sweep(MODE_POST2, (const T2*)L.z[cur], (T2*)L.z[cur ^ 1], (const T2*)C.z[cidx],
+             with_dot && c->o.nu2 == 2));
+  } else {
+    KL(sweep(MODE_PSMOOTH, (const T2*)L.z[cur], (T2*)L.z[cur ^ 1], (const T2*)C.z[cidx],
+             with_dot && c->o.nu2 == 1));
+  }
   cur ^= 1;
-  for (int s = 1; s < c->o.nu2; ++s) {
+  for (int s = post; s < c->o.nu2; ++s) {
     KL(sweep(MODE_SMOOTH, (const T2*)L.z[cur], (T2*)L.z[cur ^ 1], nullptr,
              with_dot && s == c->o.nu2 - 1));
     cur ^= 1;
@@ -759,7 +775,7 @@ size_t partials_count(const mto_ctx* c) {
   // Small launches take up to one block per SM, or the row-per-warp kernel in
   // blocks of eight warps (where a marching task would have at most two rows
   // of 30 columns, so at most 4.3 of its tasks per target warp).
-  if (maxb < c->num_sms) maxb = c->num_sms;
+  maxb = std::max(maxb, FTILES_PER_SM * c->num_sms);  // tiles of the two-stage passes, or a block per SM
   const long long strips = (gf.nx + 1 + SPLIT_STRIDE - 1) / SPLIT_STRIDE;
   const long long most = std::max(5LL * MAX_TARGET_WARPS_PER_SM * c->num_sms, 2 * strips);
   maxb = (int)std::max<long long>(maxb, std::min(strips * (gf.ny + 1), most) / (SWEEP_NT / 32) + 1);

@@ -5,6 +5,7 @@
 #include <utility>
 
 #include "mto_fsweep.cuh"
+#include "mto_ftile.cuh"
 #include "mto_fused.cuh"
 #include "mto_gemv.cuh"
 #include "mto_sweep2.cuh"
@@ -70,6 +71,13 @@ int sweep_cols(bool f64, int src, int mode);
 template <typename T>
 cudaError_t launch_sweep(int src, int mode, bool dot, bool zfloat, SweepParams<T> p,
                          int target_warps, int num_sms, cudaStream_t s);
+
+// Whether the two-stage passes PRE2 / POST2 of a float64 level run by tiles
+// (mto_ftile.cuh; its sweeps run one by one otherwise): at most
+// FTILES_PER_SM tiles per SM, and no launch shape that asks for marching tasks
+// (below one warp per SM).
+constexpr int FTILES_PER_SM = 4;
+bool float64_tiles(const Grid& g, int target_warps, int num_sms);
 
 // Warps of one full wave of a sweep kernel: resident blocks per SM (from its
 // registers) times the SM count.

@@ -93,6 +93,18 @@ static cudaError_t go(SweepParams<double> p, int tw, int num_sms, cudaStream_t s
   return launch_pdl(kernel, nblocks, nthreads, 0, s, p);
 }
 
+static int tiles_across(const Grid& g) { return g.nx / TILE_X + 1; }
+static long long tile_count(const Grid& g) { return (long long)tiles_across(g) * (g.ny / TILE_Y + 1); }
+
+bool float64_tiles(const Grid& g, int target_warps, int num_sms) {
+  return tile_count(g) <= FTILES_PER_SM * num_sms && (target_warps <= 0 || target_warps >= num_sms);
+}
+
+static cudaError_t go_tiles(void (*kernel)(SweepParams<double>), SweepParams<double> p, cudaStream_t s) {
+  p.nstrips = tiles_across(p.g);
+  return launch_pdl(kernel, (int)tile_count(p.g), SWEEP_NT, 0, s, p);
+}
+
 template <>
 cudaError_t launch_sweep<double>(int src, int mode, bool dot, bool zfloat, SweepParams<double> p,
                                  int tw, int num_sms, cudaStream_t s) {
@@ -111,6 +123,9 @@ cudaError_t launch_sweep<double>(int src, int mode, bool dot, bool zfloat, Sweep
         return dot ? go<SRC_FINE64, MODE_PSMOOTH, true, double2>(p, tw, num_sms, s)
                    : go<SRC_FINE64, MODE_PSMOOTH, false, double2>(p, tw, num_sms, s);
       case MODE_RESTRICT: return go<SRC_FINE64, MODE_RESTRICT, false, double2>(p, tw, num_sms, s);
+      case MODE_PRE2: return go_tiles(ftile_pre2_kernel<SRC_FINE64>, p, s);
+      case MODE_POST2:
+        return go_tiles(dot ? ftile_post2_kernel<SRC_FINE64, true> : ftile_post2_kernel<SRC_FINE64, false>, p, s);
       default: return cudaErrorInvalidValue;
     }
   }
@@ -121,6 +136,8 @@ cudaError_t launch_sweep<double>(int src, int mode, bool dot, bool zfloat, Sweep
       case MODE_SMOOTH0: return go<SRC_COARSE, MODE_SMOOTH0, false, double2>(p, tw, num_sms, s);
       case MODE_PSMOOTH: return go<SRC_COARSE, MODE_PSMOOTH, false, double2>(p, tw, num_sms, s);
       case MODE_RESTRICT: return go<SRC_COARSE, MODE_RESTRICT, false, double2>(p, tw, num_sms, s);
+      case MODE_PRE2: return go_tiles(ftile_pre2_kernel<SRC_COARSE>, p, s);
+      case MODE_POST2: return go_tiles(ftile_post2_kernel<SRC_COARSE, false>, p, s);
       default: return cudaErrorInvalidValue;
     }
   }

@@ -118,3 +118,28 @@ def test_non_finite_values_reach_their_neighbours_only(mto, warps, value):
         assert np.isfinite(y[~near]).all()
         assert np.allclose(y[~near], good[~near], rtol=1e-12, atol=1e-12)
     m.close()
+
+
+@pytest.mark.parametrize("warps", [MARCH, ROWS])
+@pytest.mark.parametrize("nc", [1, 3])
+def test_cycle_is_linear_in_scale_and_passes_nan_on(mto, warps, nc):
+    """Small levels run their two-stage passes by tiles (ROWS) or sweep by sweep in marching tasks.
+    A power of two on the input comes out on the output up to the rounding of each scale's last
+    bits; a non-finite residual reaches every free node through the coarsest solve."""
+    nx, ny, fixed = 72, 40, BOTTOM
+    m = mto.Mesh(nx, ny, n_coarsen=nc, fixed_edges=fixed)
+    for l in range(-1, nc + 1):
+        m.set_launch_shape(l, warps)
+    m.set_design(dev(dirichlet_design(nx, ny, 4, seed=5)), EP, 3.0)
+    r = np.random.default_rng(8).standard_normal((ny + 1, nx + 1, 2))
+    r[0] = 0.0
+    z = m.apply_preconditioner(dev(r)).cpu().numpy()
+    for s in (2.0 ** -900, 2.0 ** 900):
+        zs = m.apply_preconditioner(dev(r * s)).cpu().numpy() / s
+        assert np.linalg.norm(zs - z) <= 1e-12 * np.linalg.norm(z)
+    for value in (np.nan, np.inf):
+        bad = r.copy()
+        bad[17, 33, 1] = value
+        zb = m.apply_preconditioner(dev(bad)).cpu().numpy()
+        assert not np.isfinite(zb[1:]).any() and np.all(zb[0] == 0.0)
+    m.close()
