@@ -217,23 +217,32 @@ __global__ void unpack_elems_kernel(Grid g, const double* __restrict__ src, doub
 
 // One warp per row of K_0^-1; every block stages the free coarse right-hand
 // side in shared memory first (mto_gemv.cuh).
-constexpr int GEMV_NT = 256;
+// A block of 128 threads spreads a system of 16 x 16 elements (544 DOFs) over
+// every SM, as long as its threads can hold the indices of b they stage; larger
+// systems take 256 (iteration of a 64^2 float64 solve: 54.2 -> 53.0 us, 256^2 105.2
+// -> 101.5; at 850 DOFs 128 threads would cost 3 us, 512 cost 2 us anywhere).
+constexpr int GEMV_NT = 256, GEMV_SMALL_NT = 128;
+static int gemv_threads(int n) { return n <= GEMV_IDX * GEMV_SMALL_NT ? GEMV_SMALL_NT : GEMV_NT; }
 
 template <typename T>
 __global__ void __launch_bounds__(GEMV_NT)
     coarsest_gemv_kernel(int n, const int* __restrict__ free_idx, const double* __restrict__ Kinv,
                          const T* __restrict__ b, T* __restrict__ z, const DevScalars* sc) {
-  // K_0^-1 and the DOF map are set up once per design: load this warp's row
-  // before waiting for the previous kernel (programmatic dependent launch).
-  const int row = blockIdx.x * (GEMV_NT / 32) + (threadIdx.x >> 5);
+  // K_0^-1 and the DOF map are set up once per design: load this warp's row and
+  // the indices of b before waiting for the previous kernel (programmatic
+  // dependent launch).
+  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   double kreg[GEMV_REG_COLS];
   int zidx = 0;
+  int idx[GEMV_IDX];
+  pdl_trigger();
+  gemv_indices(n, free_idx, idx);
   if (row < n) gemv_prefetch(n, row, lane, free_idx, Kinv, kreg, zidx);
-  pdl_wait();
+  pdl_wait_prior();
   if (stop_now(sc)) return;
   extern __shared__ double bs[];
-  gemv_stage<T>(n, free_idx, b, bs);
+  gemv_stage<T>(n, free_idx, idx, b, bs);
   if (row < n) gemv_row<T>(n, row, lane, free_idx, Kinv, bs, z, kreg, zidx);
 }
 
@@ -358,8 +367,8 @@ cudaError_t launch_coarsest_gemv(const Grid& g, int n, const int* free_idx, cons
                                  DevScalars* sc, cudaStream_t s) {
   (void)g;
   if (n > GEMV_MAXN) return cudaErrorInvalidValue;
-  const int blocks = (n + GEMV_NT / 32 - 1) / (GEMV_NT / 32);
-  return launch_pdl(coarsest_gemv_kernel<T>, blocks, GEMV_NT, n * sizeof(double), s, n, free_idx, Kinv,
+  const int nt = gemv_threads(n), blocks = (n + nt / 32 - 1) / (nt / 32);
+  return launch_pdl(coarsest_gemv_kernel<T>, blocks, nt, n * sizeof(double), s, n, free_idx, Kinv,
                     reinterpret_cast<const T*>(b), reinterpret_cast<T*>(z),
                     static_cast<const DevScalars*>(sc));
 }
