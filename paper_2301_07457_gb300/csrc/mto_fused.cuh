@@ -120,7 +120,7 @@ __device__ __forceinline__ void post2_warp(const SweepParams<float>& a, int wg, 
   {
     VR r;
     S2::load_v(a, k0, i0, je0, r);
-    S2::finish_v(a, r, i0, je0, T(0), vb0, vb1);
+    S2::finish_v(a, r, i0, je0, vb0, vb1);
   }
   T2 vb2 = shfl_down2(vb0);
   T2 ac0 = sub2(vb1, vb0), ac1 = sub2(vb2, vb1);
@@ -149,7 +149,7 @@ __device__ __forceinline__ void post2_warp(const SweepParams<float>& a, int wg, 
 
       // ---- stage A: z2 at node row je ----
       T2 vt0, vt1;
-      S2::finish_v(a, cur.vt, i0, je + 1, T(0), vt0, vt1);
+      S2::finish_v(a, cur.vt, i0, je + 1, vt0, vt1);
       T2 kv0, kv1;
       element_row2<S2>(a, cur.e, vb0, vb1, vb2, vt0, vt1, ac0, ac1, gbp0, gbp1, gvp0, gvp1, kv0, kv1);
       // D^-1 and v vanish on clamped and ghost nodes, so z2 does too.  The

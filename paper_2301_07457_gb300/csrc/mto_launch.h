@@ -64,7 +64,6 @@ constexpr int sweep_cols_of(bool f64, int src, int mode) {
   (void)mode;
   return f64 ? 1 : 2;
 }
-int sweep_cols(bool f64, int src, int mode);
 
 // Launch one sweep over p.g; the launch shape follows from target_warps
 // (0: one full wave of the kernel on num_sms SMs).

@@ -1,9 +1,8 @@
-// Measurement of the float64 pipe: the peak that the float64 sweeps are
-// reported against.  Every thread runs PROBE_CHAINS independent chains of
+// Measurement of the float64 pipe, the rate of every kernel that computes in
+// float64 (the sweeps' stencils run on the integer pipe instead).  Every thread runs PROBE_CHAINS independent chains of
 // dependent fused multiply-adds, so the SM always has float64 instructions
 // ready to issue; the rate is the number of FMA instructions per second (one
-// FMA = one float64 pipe operation, the unit in which the sweeps' work is
-// counted), timed with CUDA events on the caller's stream.
+// FMA = one float64 pipe operation), timed with CUDA events on the caller's stream.
 #include <cuda_runtime.h>
 
 #include "mto_ctx.cuh"

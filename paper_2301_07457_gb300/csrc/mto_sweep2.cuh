@@ -59,15 +59,9 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
 
 // Element data of the pair (i0, j), (i1, j).
 template <typename T, int SRC> struct ERaw2;
-template <typename T> struct ERaw2<T, SRC_FINE64> {
-  double2 k[4];  // element i0: k[0], k[1]; element i1: k[2], k[3]
-};
 template <typename T> struct ERaw2<T, SRC_FINEBF> {
   __nv_bfloat162 E;
   __nv_bfloat162 El;  // SMOOTH0: elements i0 - 2, i0 - 1
-};
-template <typename T> struct ERaw2<T, SRC_COARSE> {
-  typename V2<T>::t A[NCOEF];
 };
 template <typename T> struct ERaw2<T, SRC_CFINE> {
   __nv_bfloat162 lo[2], hi[2];  // fine moduli of rows 2J, 2J+1; [w] = coarse element i0 + w
@@ -76,20 +70,6 @@ template <typename T> struct ERaw2<T, SRC_CMOM> {
   typename V2<T>::t m[NMOM];
 };
 
-template <typename T>
-__device__ __forceinline__ ERaw<T, SRC_FINE64> pick(const ERaw2<T, SRC_FINE64>& r, int w) {
-  ERaw<T, SRC_FINE64> e;
-  e.k01 = w ? r.k[2] : r.k[0];
-  e.k23 = w ? r.k[3] : r.k[1];
-  return e;
-}
-template <typename T>
-__device__ __forceinline__ ERaw<T, SRC_COARSE> pick(const ERaw2<T, SRC_COARSE>& r, int w) {
-  ERaw<T, SRC_COARSE> e;
-#pragma unroll
-  for (int c = 0; c < NCOEF; ++c) e.A[c] = w ? r.A[c].y : r.A[c].x;
-  return e;
-}
 template <typename T>
 __device__ __forceinline__ ERaw<T, SRC_CMOM> pick(const ERaw2<T, SRC_CMOM>& r, int w) {
   ERaw<T, SRC_CMOM> e;
@@ -106,12 +86,10 @@ __device__ __forceinline__ ERaw<T, SRC_CFINE> pick(const ERaw2<T, SRC_CFINE>& r,
 }
 
 // Top-row loads of the marched vector for the pair.
-template <typename T, typename ZT> struct VRaw2 {
+template <typename T> struct VRaw2 {
   using T2 = typename V2<T>::t;
-  T2 v0, v1;              // z, p_old, x, or b (SMOOTH0)
-  ZT z0, z1;              // KP: z
+  T2 v0, v1;              // z, or b (SMOOTH0)
   T2 c00, c10, c01, c11;  // PSMOOTH: coarse nodes (I, Jlo), (I+1, Jlo), (I, Jhi), (I+1, Jhi)
-  double2 d1;             // SMOOTH0, float64 finest level: w / D of the pair
   T2 d20, d21;            // SMOOTH0, coarse levels: w / D per DOF
   double2 r0, r1, q0, q1;  // SMOOTH0 with the CG update: float64 r and q of the pair
 };
@@ -134,7 +112,7 @@ struct DRaw2 {
 template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep2 {
   using T2 = typename V2<T>::t;
   using S = Sweep<T, SRC, MODE, DOT, ZT>;
-  using VR = VRaw2<T, ZT>;
+  using VR = VRaw2<T>;
   using ER = ERaw2<T, SRC>;
   using NR = NRaw2<T>;
   static constexpr bool SMOOTHING = S::SMOOTHING;
@@ -143,18 +121,11 @@ template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep2 {
   // bf16 finest moduli run one row ahead of the elements.
   static constexpr bool E_AHEAD = SRC == SRC_FINEBF;
 
-  // k: offset of node (i0, jj); i0 even.  lag (RESID): also load the
-  // direction of the pending x step; (bf16 SMOOTH0 with the CG update): the
-  // update is pending, load the last step's r.
+  // k: offset of node (i0, jj); i0 even.  lag (bf16 SMOOTH0 with the CG
+  // update): the update is pending, load the last step's r.
   __device__ __forceinline__ static void load_v(const SweepParams<T>& a, long long k, int i0, int jj,
                                                 VR& r, bool lag = false) {
-    if constexpr (MODE == MODE_RESID) {
-      ld_pair(a.v, k, r.v0, r.v1);
-      if (lag) ld_pair(a.xdir, k, r.z0, r.z1);
-    } else if constexpr (MODE == MODE_KP) {
-      ld_pair(static_cast<const ZT*>(a.zkp), k, r.z0, r.z1);
-      ld_pair(a.v, k, r.v0, r.v1);
-    } else if constexpr (MODE == MODE_PSMOOTH) {
+    if constexpr (MODE == MODE_PSMOOTH) {
       ld_pair(a.v, k, r.v0, r.v1);
       // Node i0 sits on coarse column I = i0 / 2, node i1 halfway to I + 1;
       // row jj on coarse row jj / 2, or halfway between Jlo and Jhi when odd
@@ -178,8 +149,7 @@ template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep2 {
       } else {
         ld_pair(a.b, k, r.v0, r.v1);
       }
-      if constexpr (SRC == SRC_FINE64) r.d1 = reinterpret_cast<const double2*>(a.invd1)[k >> 1];
-      else if constexpr (SRC != SRC_FINEBF) ld_pair(a.invd2, k, r.d20, r.d21);
+      if constexpr (SRC != SRC_FINEBF) ld_pair(a.invd2, k, r.d20, r.d21);
     } else {
       ld_pair(a.v, k, r.v0, r.v1);
     }
@@ -188,24 +158,8 @@ template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep2 {
   // Marched values of the pair at row jj (SMOOTH0 on the bf16 level is formed
   // in the kernel, where the top-row D is known).
   __device__ __forceinline__ static void finish_v(const SweepParams<T>& a, const VR& r, int i0, int jj,
-                                                  T beta, T2& o0, T2& o1, bool lag = false,
-                                                  T alag = T(0)) {
-    if constexpr (MODE == MODE_RESID) {
-      o0 = r.v0;
-      o1 = r.v1;
-      if (lag) {  // x + alpha p: the iterate the pending step leads to
-        o0 = mk2<T>(fma(alag, T(r.z0.x), o0.x), fma(alag, T(r.z0.y), o0.y));
-        o1 = mk2<T>(fma(alag, T(r.z1.x), o1.x), fma(alag, T(r.z1.y), o1.y));
-      }
-    } else if constexpr (MODE == MODE_KP) {
-      if constexpr (sizeof(T) == 8) {
-        o0 = mk2<T>(to_f64(r.z0.x) + beta * r.v0.x, to_f64(r.z0.y) + beta * r.v0.y);
-        o1 = mk2<T>(to_f64(r.z1.x) + beta * r.v1.x, to_f64(r.z1.y) + beta * r.v1.y);
-      } else {
-        o0 = mk2<T>(T(r.z0.x) + beta * r.v0.x, T(r.z0.y) + beta * r.v0.y);
-        o1 = mk2<T>(T(r.z1.x) + beta * r.v1.x, T(r.z1.y) + beta * r.v1.y);
-      }
-    } else if constexpr (MODE == MODE_PSMOOTH) {
+                                                  T2& o0, T2& o1) {
+    if constexpr (MODE == MODE_PSMOOTH) {
       const T h = T(0.5);
       const T2 cy0 = mk2<T>(h * (r.c00.x + r.c01.x), h * (r.c00.y + r.c01.y));
       const T2 cy1 = mk2<T>(h * (r.c10.x + r.c11.x), h * (r.c10.y + r.c11.y));
@@ -215,13 +169,8 @@ template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep2 {
                : mk2<T>(T(0), T(0));
     } else if constexpr (MODE == MODE_SMOOTH0) {
       // w D^-1 is zero on clamped and ghost nodes, so no mask is needed.
-      if constexpr (SRC == SRC_FINE64) {
-        o0 = mk2<T>(T(r.d1.x) * r.v0.x, T(r.d1.x) * r.v0.y);
-        o1 = mk2<T>(T(r.d1.y) * r.v1.x, T(r.d1.y) * r.v1.y);
-      } else {
-        o0 = mk2<T>(r.d20.x * r.v0.x, r.d20.y * r.v0.y);
-        o1 = mk2<T>(r.d21.x * r.v1.x, r.d21.y * r.v1.y);
-      }
+      o0 = mk2<T>(r.d20.x * r.v0.x, r.d20.y * r.v0.y);
+      o1 = mk2<T>(r.d21.x * r.v1.x, r.d21.y * r.v1.y);
     } else {
       o0 = r.v0;
       o1 = r.v1;
@@ -247,34 +196,23 @@ template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep2 {
       } else {
         r.lo[0] = r.lo[1] = r.hi[0] = r.hi[1] = __floats2bfloat162_rn(0.f, 0.f);
       }
-    } else if constexpr (SRC == SRC_FINE64) {
-      const double2* p = static_cast<const double2*>(a.E) + 2 * e;
-      r.k[0] = __ldg(p);
-      r.k[1] = __ldg(p + 1);
-      r.k[2] = __ldg(p + 2);
-      r.k[3] = __ldg(p + 3);
     } else if constexpr (SRC == SRC_FINEBF) {
       const __nv_bfloat16* Eb = static_cast<const __nv_bfloat16*>(a.E);
       r.E = *reinterpret_cast<const __nv_bfloat162*>(Eb + e);
       // SMOOTH0 forms D at both columns of the top row, so every lane needs
       // the modulus of element i0 - 1 itself (lane 0 has no left lane).
       if constexpr (MODE == MODE_SMOOTH0) r.El = *reinterpret_cast<const __nv_bfloat162*>(Eb + e - 2);
-    } else if constexpr (SRC == SRC_CMOM) {
-      using T2c = typename V2<T>::t;
-#pragma unroll
-      for (int c = 0; c < NMOM; ++c) r.m[c] = *reinterpret_cast<const T2c*>(a.coef + c * a.cstride + e);
     } else {
       using T2c = typename V2<T>::t;
 #pragma unroll
-      for (int c = 0; c < NCOEF; ++c) r.A[c] = *reinterpret_cast<const T2c*>(a.coef + c * a.cstride + e);
+      for (int c = 0; c < NMOM; ++c) r.m[c] = *reinterpret_cast<const T2c*>(a.coef + c * a.cstride + e);
     }
   }
 
   __device__ __forceinline__ static void load_n(const SweepParams<T>& a, long long k, NR& r) {
     if constexpr (NEEDS_B) ld_pair(a.b, k, r.b0, r.b1);
     if constexpr (SMOOTHING && MODE != MODE_SMOOTH0) {
-      if constexpr (SRC == SRC_FINE64) r.d1 = reinterpret_cast<const double2*>(a.invd1)[k >> 1];
-      else if constexpr (SRC == SRC_COARSE || SRC == SRC_CFINE || SRC == SRC_CMOM) ld_pair(a.invd2, k, r.d20, r.d21);
+      if constexpr (SRC == SRC_CFINE || SRC == SRC_CMOM) ld_pair(a.invd2, k, r.d20, r.d21);
     }
   }
 
@@ -289,8 +227,7 @@ template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep2 {
     if constexpr (SRC == SRC_FINEBF) {
       return fine_core<T>(s, E, a.kf);
     } else {
-      T dummy;
-      return S::core(a, pick(er, w), s, dummy);
+      return S::core(a, pick(er, w), s);
     }
   }
 };
@@ -346,24 +283,7 @@ __device__ __forceinline__ void sweep2_warp(const SweepParams<T>& a, int wg, int
   }
   const int strip = wg % a.nstrips;
   const int chunk = wg / a.nstrips;
-  T beta = T(0);
-  if constexpr (MODE == MODE_KP) beta = T(a.sc->beta);
-  bool vzero = false;
-  if constexpr (MODE == MODE_RESID) vzero = a.zero_gate && a.sc->x_nonzero == 0;
-  // Pending x step (x_lag): K p advances x at its owned nodes, the residual
-  // replacement works on x + alpha p.
   bool lag = false;
-  T alag = T(0);
-  if constexpr (MODE == MODE_KP) {
-    lag = a.sc->x_lag != 0;
-    alag = T(a.sc->alpha);
-  }
-  if constexpr (MODE == MODE_RESID) {
-    if (a.xlag && a.sc != nullptr && a.sc->x_lag != 0) {
-      lag = true;
-      alag = T(a.sc->alpha);
-    }
-  }
   if constexpr (UPD) lag = upd;  // read the last step's r
 
   constexpr int STRIDE = MODE == MODE_RESTRICT ? SWEEP2_RSTRIDE : SWEEP2_STRIDE;
@@ -372,26 +292,7 @@ __device__ __forceinline__ void sweep2_warp(const SweepParams<T>& a, int wg, int
   const bool own0 = lane >= 1 && i0 >= 0 && i0 <= g.nx;
   const bool own1 = lane <= 30 && i0 + 1 >= 0 && i0 + 1 <= g.nx;
 
-  if (vzero) {
-    // Residual of a zero iterate: r = b on the free DOFs, no operator needed.
-    if (chunk < a.nchunks) {
-      const int r0 = chunk * a.H, r1 = min(r0 + a.H - 1, g.ny);
-      for (int j = r0; j <= r1; ++j) {
-        const long long k = g.at(i0, j);
-        T2 b0, b1;
-        ld_pair(a.b, k, b0, b1);
-        const T2 zero = mk2<T>(T(0), T(0));
-        const T2 q0 = own0 && !g.is_fixed(i0, j) ? b0 : zero;
-        const T2 q1 = own1 && !g.is_fixed(i0 + 1, j) ? b1 : zero;
-        st_pair(a.out, k, q0, q1, own0, own1);
-        if (a.out32 != nullptr)
-          st_pair(a.out32, k, make_float2(float(q0.x), float(q0.y)), make_float2(float(q1.x), float(q1.y)),
-                  own0, own1);
-        dot0 += double(q0.x) * double(q0.x) + double(q0.y) * double(q0.y) +
-                double(q1.x) * double(q1.x) + double(q1.y) * double(q1.y);
-      }
-    }
-  } else if (chunk < a.nchunks) {
+  if (chunk < a.nchunks) {
     int je0, je1, Jb = 0, Je = 0;
     if constexpr (MODE == MODE_RESTRICT) {
       Jb = chunk * (a.H >> 1);
@@ -484,15 +385,12 @@ __device__ __forceinline__ void sweep2_warp(const SweepParams<T>& a, int wg, int
         vb0 = mk2<T>(wc0.x * b0r.x, wc0.y * b0r.y);
         vb1 = mk2<T>(wc1.x * b1r.x, wc1.y * b1r.y);
       } else {
-        S2::finish_v(a, r0, i0, je0, beta, vb0, vb1, lag, alag);
+        S2::finish_v(a, r0, i0, je0, vb0, vb1);
       }
       if constexpr (MODE == MODE_SMOOTH0) {
         bc0 = b0r;
         bc1 = b1r;
-        if constexpr (SRC == SRC_FINE64) {
-          wc0 = mk2<T>(T(r0.d1.x), T(r0.d1.x));
-          wc1 = mk2<T>(T(r0.d1.y), T(r0.d1.y));
-        } else if constexpr (!FBF) {
+        if constexpr (!FBF) {
           wc0 = r0.d20;
           wc1 = r0.d21;
         }
@@ -522,18 +420,6 @@ __device__ __forceinline__ void sweep2_warp(const SweepParams<T>& a, int wg, int
         if (je > je1) break;
         const Pack cur = ring[u];
         if (je + PF <= je1) load_pack(ring[u], je + PF, k + PF * pitch);
-        if constexpr (MODE == MODE_KP) {
-          // Pending x step at the top row (owned rows only): x += alpha p_old.
-          // Done at once, so that x occupies registers only briefly; other
-          // warps cover the load with FP64 work.
-          if (lag && je + 1 <= je1) {  // uniform over the warp
-            T2 x0, x1;
-            ld_pair(a.xvec, k + pitch, x0, x1);
-            x0 = mk2<T>(fma(alag, cur.vt.v0.x, x0.x), fma(alag, cur.vt.v0.y, x0.y));
-            x1 = mk2<T>(fma(alag, cur.vt.v1.x, x1.x), fma(alag, cur.vt.v1.y, x1.y));
-            st_pair(a.xvec, k + pitch, x0, x1, own0, own1);
-          }
-        }
         DRaw2 dcur;
         if constexpr (DOT && !UPD) {
           if (je > je0) S2::load_d(a, k, dcur);
@@ -583,15 +469,13 @@ __device__ __forceinline__ void sweep2_warp(const SweepParams<T>& a, int wg, int
           vt0 = mul2(wt0, btop0);
           vt1 = mul2(wt1, btop1);
         } else {
-          S2::finish_v(a, cur.vt, i0, je + 1, beta, vt0, vt1, lag, alag);
+          S2::finish_v(a, cur.vt, i0, je + 1, vt0, vt1);
         }
 
         const T2 vt2 = shfl_down2(vt0);  // lane 31: its own value, used only for halo output
         const T2 bt0 = sub2(vt1, vt0), bt1 = sub2(vt2, vt1);  // top edges
         const T2 dl0 = sub2(vt0, vb0), dl1 = sub2(vt1, vb1);  // vertical edges at i0, i1
-        T2 dl2;                                               // vertical edge at i0 + 2
-        if constexpr (sizeof(T) == 8) dl2 = shfl_down2(dl0);  // a shuffle is cheaper than FP64
-        else dl2 = sub2(vt2, vb2);
+        const T2 dl2 = sub2(vt2, vb2);                        // vertical edge at i0 + 2
         // Strain coordinates as component pairs: (c1, d1) = a + b,
         // (c3, d3) = b - a, (c2, d2) = dl + dr, s = c2 + d1.
         Strain<T> w0, w1;
@@ -635,27 +519,9 @@ __device__ __forceinline__ void sweep2_warp(const SweepParams<T>& a, int wg, int
         const bool act0 = inb0 && !cfix0 && !rfix, act1 = inb1 && !cfix1 && !rfix;
 
         if constexpr (MODE == MODE_APPLY) {
-          if constexpr (sizeof(T) == 4) {  // mask by multiplication (FMA pipe, values finite)
-            const T m0 = act0 ? T(1) : T(0), m1 = act1 ? T(1) : T(0);
-            st_pair(a.out, k, mk2<T>(kv0.x * m0, kv0.y * m0), mk2<T>(kv1.x * m1, kv1.y * m1), inb0, inb1);
-          } else {
-            st_pair(a.out, k, act0 ? kv0 : zero2, act1 ? kv1 : zero2, inb0, inb1);
-          }
-        } else if constexpr (MODE == MODE_RESID) {
-          const T2 r0 = act0 ? sub2(cur.n.b0, kv0) : zero2;
-          const T2 r1 = act1 ? sub2(cur.n.b1, kv1) : zero2;
-          st_pair(a.out, k, r0, r1, inb0, inb1);
-          if (a.out32 != nullptr)
-            st_pair(a.out32, k, make_float2(float(r0.x), float(r0.y)),
-                    make_float2(float(r1.x), float(r1.y)), inb0, inb1);
-          dot0 = fma(double(r0.x), double(r0.x), fma(double(r0.y), double(r0.y), dot0));
-          dot0 = fma(double(r1.x), double(r1.x), fma(double(r1.y), double(r1.y), dot0));
-        } else if constexpr (MODE == MODE_KP) {
-          const T2 q0 = act0 ? kv0 : zero2, q1 = act1 ? kv1 : zero2;
-          st_pair(a.p_out, k, vb0, vb1, inb0, inb1);
-          st_pair(a.out, k, q0, q1, inb0, inb1);
-          if (inb0) dot0 = fma(double(vb0.x), double(q0.x), fma(double(vb0.y), double(q0.y), dot0));
-          if (inb1) dot0 = fma(double(vb1.x), double(q1.x), fma(double(vb1.y), double(q1.y), dot0));
+          // Mask by multiplication (FMA pipe, values finite).
+          const T m0 = act0 ? T(1) : T(0), m1 = act1 ? T(1) : T(0);
+          st_pair(a.out, k, mk2<T>(kv0.x * m0, kv0.y * m0), mk2<T>(kv1.x * m1, kv1.y * m1), inb0, inb1);
         } else if constexpr (S2::SMOOTHING) {
           T2 b0, b1, d0, d1;
           if constexpr (MODE == MODE_SMOOTH0) {
@@ -666,10 +532,7 @@ __device__ __forceinline__ void sweep2_warp(const SweepParams<T>& a, int wg, int
           } else {
             b0 = cur.n.b0;
             b1 = cur.n.b1;
-            if constexpr (SRC == SRC_FINE64) {
-              d0 = mk2<T>(T(cur.n.d1.x), T(cur.n.d1.x));
-              d1 = mk2<T>(T(cur.n.d1.y), T(cur.n.d1.y));
-            } else if constexpr (FBF) {
+            if constexpr (FBF) {
               // D from the moduli is zero on ghost nodes: mask w / D itself.
               float w0f, w1f;
               fbf_winv(ep0, ep1, ec0, ec1, float(a.wdiag), w0f, w1f);
@@ -729,9 +592,6 @@ __device__ __forceinline__ void sweep2_warp(const SweepParams<T>& a, int wg, int
           if constexpr (FBF0) {
             wc0 = wt0;
             wc1 = wt1;
-          } else if constexpr (SRC == SRC_FINE64) {
-            wc0 = mk2<T>(T(cur.vt.d1.x), T(cur.vt.d1.x));
-            wc1 = mk2<T>(T(cur.vt.d1.y), T(cur.vt.d1.y));
           } else {
             wc0 = cur.vt.d20;
             wc1 = cur.vt.d21;
@@ -763,12 +623,9 @@ __device__ __forceinline__ void sweep2_warp(const SweepParams<T>& a, int wg, int
 // wave is then 16 warps per SM, which the launch shapes assume.
 template <typename T, int SRC, int MODE, bool DOT, typename ZT, int PF>
 __global__ void __launch_bounds__(SWEEP_NT, 2) sweep2_kernel(const SweepParams<T> a) {
-  constexpr bool REDUCE = DOT || MODE == MODE_RESID || MODE == MODE_KP;
+  constexpr bool REDUCE = DOT;
   pdl_wait();
-  if (a.sc != nullptr && a.gate) {
-    if (a.sc->done != RUNNING) return;  // uniform over the grid
-    if (a.replace_gate && (a.sc->rr_every <= 0 || (a.sc->iter % a.sc->rr_every) != 0)) return;
-  }
+  if (a.sc != nullptr && a.gate && a.sc->done != RUNNING) return;  // uniform over the grid
   const int lane = threadIdx.x & 31;
   const int wg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   double dot0 = 0.0, dot1 = 0.0;

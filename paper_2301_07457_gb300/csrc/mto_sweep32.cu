@@ -40,8 +40,7 @@ static cudaError_t go(SweepParams<float> p, int tw, int num_sms, cudaStream_t s)
   }
   if constexpr (MODE == MODE_POST2) kernel = post2_kernel<SRC, 2>;
   else if constexpr (MODE == MODE_PRE2) kernel = pre2_kernel<SRC, 2>;
-  else if constexpr (COLS == 2) kernel = sweep2_kernel<float, SRC, MODE, DOT, float2, PF>;
-  else kernel = sweep_kernel<float, SRC, MODE, DOT, float2, PF>;
+  else kernel = sweep2_kernel<float, SRC, MODE, DOT, float2, PF>;
   if (tw <= 0) {
     static const int wave = full_wave_warps(kernel, num_sms);  // same for every device of a run
     tw = wave;

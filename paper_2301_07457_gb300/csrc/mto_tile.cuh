@@ -40,8 +40,7 @@ template <int EW, int EH> struct TileForces {
     w.d3 = cd3.y;
     w.d2 = cd2.y;
     w.s = cd2.x + cd1.y;
-    float dummy;
-    const Strain<float> t = Sweep<float, SRC, MODE_SMOOTH, false, float2>::core(a, er, w, dummy);
+    const Strain<float> t = Sweep<float, SRC, MODE_SMOOTH, false, float2>::core(a, er, w);
     const float2 p = make_float2(t.c1, t.s), m = make_float2(t.c3, t.d3);
     ga[e] = sub2(p, m);
     gb[e] = add2(p, m);
