@@ -269,9 +269,12 @@ double2* rbuf(const mto_ctx* c, int par) { return (fuse_update(c) && par == 1) ?
 // V-cycle on the finest level with right-hand side r (float64).  With
 // with_dot (inside the PCG loop), the last post-smoothing sweep also forms
 // z.r (and z.q) and finishes beta (FIN_RHO), and with fuse_update the first
-// sweep applies the pending CG update of r.
+// sweep applies the pending CG update of r.  Without with_dot, the mixed cycle
+// takes its right-hand side from din (first sweep fused, nu1 >= 2; else from
+// r32) and may leave its result in dout (nu2 >= 2), both in the caller's layout.
 template <typename T>
-mto_status fine_cycle(mto_ctx* c, DevScalars* sc, bool with_dot, int* final_idx) {
+mto_status fine_cycle(mto_ctx* c, DevScalars* sc, bool with_dot, int* final_idx,
+                      const double2* din = nullptr, double2* dout = nullptr) {
   using T2 = typename V2<T>::t;
   constexpr bool MIX = sizeof(T) == 4;
   LevelBuf& L = c->lv[c->L];
@@ -293,7 +296,8 @@ mto_status fine_cycle(mto_ctx* c, DevScalars* sc, bool with_dot, int* final_idx)
     }
   }
   int cur = 0;
-  auto sweep = [&](int mode, const T2* v, T2* out, const T2* zc, bool dot) -> cudaError_t {
+  auto sweep = [&](int mode, const T2* v, T2* out, const T2* zc, bool dot,
+                   double2* dense = nullptr) -> cudaError_t {
     SweepParams<T> p = base_params<T>(c, L.g);
     p.gc = C.g;
     p.gate = 1;
@@ -307,6 +311,11 @@ mto_status fine_cycle(mto_ctx* c, DevScalars* sc, bool with_dot, int* final_idx)
     p.kf = fine_const<T>(c);
     p.invd1 = c->invd1;
     p.wdiag = T(c->w_over_kdiag);
+    if (MIX && !dot && mode == MODE_SMOOTH0) {
+      p.din = din;
+      p.out32 = c->r32;
+    }
+    p.dout = dense;
     if (dot && mode == MODE_SMOOTH0) {
       // The CG update r -= alpha q of the last step (mixed precision).
       p.r64 = rbuf(c, c->cur_par);
@@ -369,7 +378,7 @@ mto_status fine_cycle(mto_ctx* c, DevScalars* sc, bool with_dot, int* final_idx)
   cur ^= 1;
   for (int s = post; s < c->o.nu2; ++s) {
     KL(sweep(MODE_SMOOTH, (const T2*)L.z[cur], (T2*)L.z[cur ^ 1], nullptr,
-             with_dot && s == c->o.nu2 - 1));
+             with_dot && s == c->o.nu2 - 1, s == c->o.nu2 - 1 ? dout : nullptr));
     cur ^= 1;
   }
   *final_idx = cur;
@@ -1617,10 +1626,16 @@ mto_status mto_apply_preconditioner(mto_ctx* c, const double* r_dev, double* z_d
   ST(enter(c));
   LevelBuf& B = c->lv[c->L];
   int zi = 0;
-  if (c->mixed) {  // the float32 cycle reads r32 alone
-    KL(launch_pack_f32(B.g, r_dev, c->r32, c->cs, c->num_sms));
-    ST(fine_cycle<float>(c, nullptr, false, &zi));
-    KL(launch_unpack_f32(B.g, (const float2*)B.z[zi], z_dev, c->cs, c->num_sms));
+  if (c->mixed) {
+    // The first and last finest-level sweeps read and write the caller's
+    // arrays themselves where they are the fused SMOOTH0 and a SMOOTH (the
+    // arrays may overlap: the last kernel writes, only the first one reads);
+    // the float32 cycle otherwise reads r32 alone.
+    const double2* din = c->o.nu1 >= 2 ? reinterpret_cast<const double2*>(r_dev) : nullptr;
+    double2* dout = c->o.nu2 >= 2 ? reinterpret_cast<double2*>(z_dev) : nullptr;
+    if (din == nullptr) KL(launch_pack_f32(B.g, r_dev, c->r32, c->cs, c->num_sms));
+    ST(fine_cycle<float>(c, nullptr, false, &zi, din, dout));
+    if (dout == nullptr) KL(launch_unpack_f32(B.g, (const float2*)B.z[zi], z_dev, c->cs, c->num_sms));
   } else {
     KL(launch_pack(B.g, r_dev, c->r, c->cs, c->num_sms));
     ST(fine_cycle<double>(c, nullptr, false, &zi));

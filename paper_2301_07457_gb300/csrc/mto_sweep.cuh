@@ -101,6 +101,8 @@ template <typename T> struct SweepParams {
   const double2* rdot;  // dot partner for z.r
   const double2* qdot;  // dot partner for z.q (flexible beta), may be null
   int dense;               // float64 APPLY: v and out in the caller's layout [ny + 1][nx + 1] (no padding)
+  const double2* din;      // bf16 SMOOTH0 of a V-cycle called alone: b in the caller's layout
+  double2* dout;           // bf16 SMOOTH: output in the caller's layout instead of out (may be null)
   double2* r64;            // bf16 SMOOTH0 with the CG update: r of this step (written)
   const double2* r64_prev;  // ... r of the last step, read while the update is pending
   const double2* q64;       // ... and q = K p of the last step

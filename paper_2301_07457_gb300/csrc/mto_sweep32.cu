@@ -11,7 +11,7 @@ namespace mto {
 // loads takes.
 template <int SRC, int MODE, bool DOT> constexpr int lookahead() {
   if (SRC == SRC_CMOM && MODE == MODE_PSMOOTH) return 1;
-  if (SRC == SRC_FINEBF && MODE == MODE_SMOOTH0 && DOT) return 1;  // float64 r and q per row
+  if (SRC == SRC_FINEBF && MODE == MODE_SMOOTH0) return DOT ? 1 : 2;  // float64 r (and q) per row
   if (DOT || MODE == MODE_PSMOOTH || SRC == SRC_CFINE || SRC == SRC_CMOM) return 2;
   return 3;
 }

@@ -14,6 +14,8 @@ V-cycle 2e-5 against the oracle's float64 V-cycle on the same bf16-rounded
 moduli; solves reach the requested float64 true residual.
 """
 
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -142,3 +144,34 @@ def test_tiled_coarse_passes_equal_marching_ones(mto, nx, ny, nc, kind):
         z.append(m.apply_preconditioner(r))
         m.close()
     assert torch.equal(z[0], z[1])
+
+
+@pytest.mark.parametrize("nu1,nu2", [(2, 2), (3, 3), (1, 2), (2, 1)])
+@pytest.mark.parametrize("nx,ny,nc", [(8, 8, 1), (32, 24, 3), (62, 34, 1), (136, 72, 3)])
+def test_mixed_cycle_between_the_callers_arrays(mto, nx, ny, nc, nu1, nu2):
+    """With two sweeps or more, the first and last finest sweeps read and write the caller's
+    float64 arrays.  The cycle is a float32 function of the rounded right-hand side on the free
+    nodes, so rounding r first, non-finite values on clamped nodes, and an output that is the
+    input (or overlaps it) change no bit."""
+    x = torch.from_numpy(dirichlet_design(nx, ny, 4, seed=nx)).cuda()
+    r = torch.from_numpy(np.random.default_rng(ny).standard_normal((ny + 1, nx + 1, 2))).cuda()
+    m = mto.Mesh(nx, ny, n_coarsen=nc, precision="mixed", fixed_edges=mto.EDGE_BOTTOM | mto.EDGE_RIGHT,
+                 nu1=nu1, nu2=nu2)
+    m.set_design(x, EP, 3.0)
+    z = m.apply_preconditioner(r)
+    assert torch.equal(z, z.float().double()) and z.abs().max() > 0
+    assert not z[0].any() and not z[:, -1].any()
+    assert torch.equal(m.apply_preconditioner(r.float().double()), z)
+    bad = r.clone()
+    bad[0] = float("nan")
+    bad[:, -1] = float("inf")
+    assert torch.equal(m.apply_preconditioner(bad), z)
+    for shift in (0, 2, 2 * (nx + 1) + 2):  # doubles from the input's start to the output's
+        buf = torch.zeros(r.numel() + shift, dtype=torch.float64, device=DEV)
+        buf[:r.numel()] = r.reshape(-1)
+        st = m._lib.mto_apply_preconditioner(m._h, ctypes.c_void_p(buf.data_ptr()),
+                                             ctypes.c_void_p(buf.data_ptr() + 8 * shift))
+        assert st == 0
+        torch.cuda.synchronize()
+        assert torch.equal(buf[shift:], z.reshape(-1)), shift
+    m.close()
