@@ -375,7 +375,7 @@ void mto_poisson_destroy(mto_poisson* p);
  * inside the solver's CUDA graph) around two hot kernels of every PCG
  * iteration: [0] the finest-level outer sweep p = z + beta p, q = K p (float64)
  * and [1] the first finest-level kernel of the V-cycle (in its precision): the
- * damped-Jacobi sweeps from zero, on small float64 meshes together with the
+ * damped-Jacobi sweeps from zero, on small meshes together with the
  * residual and its restriction.  mto_get_kernel_times returns their mean duration in
  * ms over the iterations sampled since timing was enabled (host arrays of 2).
  * mto_get_launch_count returns the number of kernels this context has

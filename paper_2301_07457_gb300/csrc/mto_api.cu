@@ -311,12 +311,13 @@ mto_status fine_cycle(mto_ctx* c, DevScalars* sc, bool with_dot, int* final_idx,
     p.kf = fine_const<T>(c);
     p.invd1 = c->invd1;
     p.wdiag = T(c->w_over_kdiag);
-    if (MIX && !dot && mode == MODE_SMOOTH0) {
+    const bool from_b = mode == MODE_SMOOTH0 || mode == MODE_PRE2;  // first kernel, b alone
+    if (MIX && !dot && from_b) {
       p.din = din;
       p.out32 = c->r32;
     }
     p.dout = dense;
-    if (dot && mode == MODE_SMOOTH0) {
+    if (dot && from_b) {
       // The CG update r -= alpha q of the last step (mixed precision).
       p.r64 = rbuf(c, c->cur_par);
       p.r64_prev = rbuf(c, c->cur_par ^ 1);
@@ -341,12 +342,14 @@ mto_status fine_cycle(mto_ctx* c, DevScalars* sc, bool with_dot, int* final_idx,
               : cudaSuccess;
   };
   int first = 1;
-  // Small float64 grids: both pre-smoothing sweeps with the restriction, and
-  // the prolongation with the next sweep, in one pass each (mto_ftile.cuh).
-  const bool two_stage = !MIX && float64_tiles(L.g, tw, c->num_sms);
+  // Small grids: both pre-smoothing sweeps with the restriction, and
+  // the prolongation with the next sweep, in one pass each (mto_tile.cuh,
+  // mto_ftile.cuh).
+  const bool two_stage =
+      MIX ? float32_tiles(true, L.g, tw, c->num_sms) : float64_tiles(L.g, tw, c->num_sms);
   if (two_stage && c->o.nu1 == 2) {
     CK(t0());
-    KL(sweep(MODE_PRE2, nullptr, (T2*)L.z[0], nullptr, false));
+    KL(sweep(MODE_PRE2, nullptr, (T2*)L.z[0], nullptr, fuse_update(c) && with_dot));
     CK(t1());
   } else {
     if (fused0) {
@@ -370,7 +373,7 @@ mto_status fine_cycle(mto_ctx* c, DevScalars* sc, bool with_dot, int* final_idx,
   if (two_stage && c->o.nu2 >= 2) {
     post = 2;
     KL(sweep(MODE_POST2, (const T2*)L.z[cur], (T2*)L.z[cur ^ 1], (const T2*)C.z[cidx],
-             with_dot && c->o.nu2 == 2));
+             with_dot && c->o.nu2 == 2, c->o.nu2 == 2 ? dout : nullptr));
   } else {
     KL(sweep(MODE_PSMOOTH, (const T2*)L.z[cur], (T2*)L.z[cur ^ 1], (const T2*)C.z[cidx],
              with_dot && c->o.nu2 == 1));
@@ -784,7 +787,7 @@ size_t partials_count(const mto_ctx* c) {
   // Small launches take up to one block per SM, or the row-per-warp kernel in
   // blocks of eight warps (where a marching task would have at most two rows
   // of 30 columns, so at most 4.3 of its tasks per target warp).
-  maxb = std::max(maxb, FTILES_PER_SM * c->num_sms);  // tiles of the two-stage passes, or a block per SM
+  maxb = std::max(maxb, std::max(FTILES_PER_SM, FINE_TILES_PER_SM) * c->num_sms);  // tiles of the two-stage passes, or a block per SM
   const long long strips = (gf.nx + 1 + SPLIT_STRIDE - 1) / SPLIT_STRIDE;
   const long long most = std::max(5LL * MAX_TARGET_WARPS_PER_SM * c->num_sms, 2 * strips);
   maxb = (int)std::max<long long>(maxb, std::min(strips * (gf.ny + 1), most) / (SWEEP_NT / 32) + 1);

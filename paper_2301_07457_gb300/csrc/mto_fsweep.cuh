@@ -12,13 +12,14 @@
 // which takes five products of three factors per element instead of seven of
 // four (24 bytes of element data instead of 32).
 //
-// Measured at 2048^2: K p 0.318 -> 0.125 ms (bound before by the FP64 pipe at
-// 36 operations per node; now the ALU pipe is busy 55-65% of the time, the
-// FP64 pipe 40% with the 6 operations of the CG recurrence, DRAM 3 TB/s: 16
-// warps of 128 registers per SM do not fill any of them), the operator alone
-// 0.323 -> 0.152 ms with its layout conversions, relative error against exact
-// arithmetic 2.3e-16 -> 1.8e-16.  A float64 4096^2 solve takes 196 instead of
-// 373 ms, a mixed 2048^2 solve 14.9 instead of 20.9 ms.
+// Measured at 2048^2: K p 0.318 -> 0.115 ms (bound before by the FP64 pipe at
+// 36 operations per node; now the ALU pipe is busy 67% of the time, instruction
+// issue 63%, the FP64 pipe 43% with the 6 operations of the CG recurrence, DRAM
+// 3.5 TB/s: 16 warps of 128 registers per SM do not fill any of them), the
+// operator alone 0.325 -> 0.108 ms, relative error against exact arithmetic
+// 2.3e-16 -> 1.8e-16.  With the coarse levels in fixed point too, a float64
+// 4096^2 step takes 128 instead of 362 ms, a mixed 2048^2 step 13.1 instead of
+// 21.7 ms.
 //
 // Bounds (mto_fixed.cuh; |F| < 2^91): edge differences < 2^92, c1, c3, c2, d1,
 // d2, d3 < 2^93, s and c1 +- d2 < 2^94; factors < 2^61, so every product

@@ -77,6 +77,17 @@ cudaError_t launch_sweep(int src, int mode, bool dot, bool zfloat, SweepParams<T
 // (below one warp per SM).
 constexpr int FTILES_PER_SM = 4;
 bool float64_tiles(const Grid& g, int target_warps, int num_sms);
+// The same for a float32 level (mto_tile.cuh).  Coarse levels: at most
+// TILES_PER_SM tiles per SM: one V-cycle takes 60 -> 41 us at 256^2, 110 -> 90 us
+// at 1024^2, 236 -> 216 us at 2048^2 (all levels up to 256^2), 160 -> 141 us at
+// 1856 x 1216 (up to 464 x 304: 7.7 tiles per SM); a 512^2 level (14 tiles per
+// SM) takes 1-4 us longer by tiles, a 1024^2 level 30 us: there the recomputed
+// halo counts.  The bf16 finest level recomputes the float64 CG update in its
+// halo too and stops at FINE_TILES_PER_SM: a mixed PCG iteration takes 42.5 ->
+// 33.8 us at 64^2, 56.1 -> 47.0 us at 200 x 136, 64.2 -> 55.2 us at 256^2 (3.7
+// tiles per SM), but 74.0 -> 77.5 us at 368^2 (7.4) and 77.0 -> 94.5 us at 512^2.
+constexpr int TILES_PER_SM = 8, FINE_TILES_PER_SM = 5;
+bool float32_tiles(bool finest, const Grid& g, int target_warps, int num_sms);
 
 // Warps of one full wave of a sweep kernel: resident blocks per SM (from its
 // registers) times the SM count.

@@ -61,8 +61,8 @@ enum Mode {
   MODE_PSMOOTH,
   MODE_RESTRICT,
   MODE_SMOOTH0,
-  // Two-stage passes of the float32 coarse levels (mto_fused.cuh, mto_tile.cuh)
-  // and of small float64 levels (mto_ftile.cuh):
+  // Two-stage passes of the float32 coarse levels (mto_fused.cuh, mto_tile.cuh),
+  // of small bf16 finest levels and small float64 levels (mto_tile.cuh, mto_ftile.cuh):
   MODE_POST2,  // prolongation + two sweeps, fused
   MODE_PRE2    // two sweeps from zero + residual + restriction, fused
 };
@@ -179,6 +179,9 @@ template <> __device__ __forceinline__ float2 mul2<float2>(float2 a, float2 b) {
 }
 
 template <typename T, int SRC> struct ERaw;
+template <typename T> struct ERaw<T, SRC_FINEBF> {
+  T E;
+};
 template <typename T> struct ERaw<T, SRC_CFINE> {
   __nv_bfloat162 lo, hi;  // fine moduli of rows 2J and 2J+1, columns 2I and 2I+1
 };
@@ -197,7 +200,9 @@ template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep {
 
   __device__ __forceinline__ static void load_e(const SweepParams<T>& a, long long e, int ii, int jj,
                                                 ER& r) {
-    if constexpr (SRC == SRC_CFINE) {
+    if constexpr (SRC == SRC_FINEBF) {
+      r.E = __bfloat162float(static_cast<const __nv_bfloat16*>(a.E)[e]);
+    } else if constexpr (SRC == SRC_CFINE) {
       // Ghost and padding elements have no children: zero operator.
       if ((unsigned)ii < (unsigned)a.g.nx && (unsigned)jj < (unsigned)a.g.ny) {
         const __nv_bfloat162* Ef = static_cast<const __nv_bfloat162*>(a.E);
@@ -208,7 +213,7 @@ template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep {
         r.lo = r.hi = __floats2bfloat162_rn(0.f, 0.f);
       }
     } else {
-      static_assert(SRC == SRC_CMOM, "elements read one by one: the float32 coarse levels");
+      static_assert(SRC == SRC_CMOM, "elements read one by one: the float32 levels");
 #pragma unroll
       for (int c = 0; c < NMOM; ++c) r.m[c] = a.coef[c * a.cstride + e];
     }
@@ -218,7 +223,9 @@ template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep {
   __device__ __forceinline__ static Strain<T> core(const SweepParams<T>& a, const ER& er,
                                                    const Strain<T>& w) {
     Strain<T> t;
-    if constexpr (SRC == SRC_CFINE) {
+    if constexpr (SRC == SRC_FINEBF) {
+      t = fine_core<T>(w, er.E, a.kf);
+    } else if constexpr (SRC == SRC_CFINE) {
       // Moments of the four child moduli (children at xi, eta = +-1/2 of the
       // parent): M00 = S/4, M10 = X/8, M01 = Y/8, M20 = M02 = M00/3,
       // M11 = Z/16, then the 13 coefficients of mto_common.cuh.

@@ -16,13 +16,12 @@ template <int SRC, int MODE, bool DOT> constexpr int lookahead() {
   return 3;
 }
 
-// Two-stage passes of levels with at most this many tiles per SM run by tiles
-// (mto_tile.cuh): one V-cycle takes 60 -> 41 us at 256^2, 110 -> 90 us at
-// 1024^2, 236 -> 216 us at 2048^2 (all levels up to 256^2), 160 -> 141 us at
-// 1856 x 1216 (up to 464 x 304: 7.7 tiles per SM).  A 512^2 level (14 tiles per
-// SM) takes 1-4 us longer by tiles, a 1024^2 level 30 us: there the recomputed
-// halo counts.  Launch shapes below one warp per SM ask for marching tasks.
-constexpr int TILES_PER_SM = 8;
+static int tiles_across(const Grid& g) { return g.nx / TILE_X + 1; }  // tiles of nx + 1 nodes
+static long long tile_count(const Grid& g) { return (long long)tiles_across(g) * (g.ny / TILE_Y + 1); }
+
+bool float32_tiles(bool finest, const Grid& g, int tw, int num_sms) {
+  return tile_count(g) <= (finest ? FINE_TILES_PER_SM : TILES_PER_SM) * num_sms && (tw <= 0 || tw >= num_sms);
+}
 
 template <int SRC, int MODE, bool DOT>
 static cudaError_t go(SweepParams<float> p, int tw, int num_sms, cudaStream_t s) {
@@ -30,15 +29,15 @@ static cudaError_t go(SweepParams<float> p, int tw, int num_sms, cudaStream_t s)
   constexpr int PF = lookahead<SRC, MODE, DOT>();
   void (*kernel)(SweepParams<float>);
   if constexpr (MODE == MODE_PRE2 || MODE == MODE_POST2) {
-    const int across = p.g.nx / TILE_X + 1;  // tiles of nx + 1 nodes
-    const long long tiles = (long long)across * (p.g.ny / TILE_Y + 1);
-    if (tiles <= TILES_PER_SM * num_sms && (tw <= 0 || tw >= num_sms)) {
-      kernel = MODE == MODE_PRE2 ? tile_pre2_kernel<SRC> : tile_post2_kernel<SRC>;
-      p.nstrips = across;
-      return launch_pdl(kernel, (int)tiles, SWEEP_NT, 0, s, p);
+    if (float32_tiles(SRC == SRC_FINEBF, p.g, tw, num_sms)) {
+      kernel = MODE == MODE_PRE2 ? tile_pre2_kernel<SRC, DOT> : tile_post2_kernel<SRC, DOT>;
+      p.nstrips = tiles_across(p.g);
+      return launch_pdl(kernel, (int)tile_count(p.g), SWEEP_NT, 0, s, p);
     }
+    if constexpr (SRC == SRC_FINEBF) return cudaErrorInvalidValue;  // two kernels there (fine_cycle)
   }
-  if constexpr (MODE == MODE_POST2) kernel = post2_kernel<SRC, 2>;
+  if constexpr (SRC == SRC_FINEBF && (MODE == MODE_PRE2 || MODE == MODE_POST2)) kernel = nullptr;
+  else if constexpr (MODE == MODE_POST2) kernel = post2_kernel<SRC, 2>;
   else if constexpr (MODE == MODE_PRE2) kernel = pre2_kernel<SRC, 2>;
   else kernel = sweep2_kernel<float, SRC, MODE, DOT, float2, PF>;
   if (tw <= 0) {
@@ -69,6 +68,12 @@ cudaError_t launch_sweep<float>(int src, int mode, bool dot, bool zfloat, SweepP
         return dot ? go<SRC_FINEBF, MODE_PSMOOTH, true>(p, tw, num_sms, s)
                    : go<SRC_FINEBF, MODE_PSMOOTH, false>(p, tw, num_sms, s);
       case MODE_RESTRICT: return go<SRC_FINEBF, MODE_RESTRICT, false>(p, tw, num_sms, s);
+      case MODE_PRE2:  // with dot: carrying the CG update
+        return dot ? go<SRC_FINEBF, MODE_PRE2, true>(p, tw, num_sms, s)
+                   : go<SRC_FINEBF, MODE_PRE2, false>(p, tw, num_sms, s);
+      case MODE_POST2:
+        return dot ? go<SRC_FINEBF, MODE_POST2, true>(p, tw, num_sms, s)
+                   : go<SRC_FINEBF, MODE_POST2, false>(p, tw, num_sms, s);
       default: return cudaErrorInvalidValue;
     }
   }

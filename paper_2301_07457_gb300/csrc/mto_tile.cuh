@@ -1,5 +1,5 @@
-// The two-stage passes of the small float32 coarse levels (Alg. 1), one tile
-// of nodes per block.
+// The two-stage passes of the small float32 levels (Alg. 1), one tile of nodes
+// per block.
 //
 // Same passes as the marching kernels of mto_fused.cuh: PRE2 (two smoothing
 // sweeps from zero, residual, restriction) and POST2 (prolongation, two
@@ -14,6 +14,12 @@
 //
 // Every value is formed by the same operations in the same order as there, so
 // the results are those of the marching kernels bit for bit.
+//
+// On the bf16 finest level the passes replace two marching kernels each
+// (mto_sweep2.cuh): PRE2 with DOT also carries the CG update of the outer
+// iteration, POST2 with DOT forms the dot products (their partial sums are per
+// tile, so these differ in the last bits).  Two launches and a trip through
+// memory less per cycle at each end: a mixed iteration 56 -> 47 us at 200 x 136.
 #pragma once
 
 #include "mto_fused.cuh"
@@ -63,8 +69,24 @@ __device__ __forceinline__ ERaw<float, SRC> tile_element(const SweepParams<float
   return er;
 }
 
-template <int SRC> __global__ void __launch_bounds__(SWEEP_NT) tile_pre2_kernel(const SweepParams<float> a) {
+// w/D at node (i, j) of the bf16 finest level, zero on clamped and ghost nodes.
+__device__ __forceinline__ float2 tile_winv(const SweepParams<float>& a, int i, int j) {
+  if (!a.g.active(i, j)) return make_float2(0.f, 0.f);
+  const __nv_bfloat16* E = static_cast<const __nv_bfloat16*>(a.E) + a.g.at(i, j);
+  const float own = __bfloat162float(E[-a.g.pitch]) + __bfloat162float(E[0]);
+  const float left = __bfloat162float(E[-a.g.pitch - 1]) + __bfloat162float(E[-1]);
+  const float w = __fdividef(a.wdiag, own + left);
+  return make_float2(w, w);
+}
+template <int SRC> __device__ __forceinline__ float2 tile_d(const SweepParams<float>& a, int i, int j) {
+  if constexpr (SRC == SRC_FINEBF) return tile_winv(a, i, j);
+  else return __ldg(a.invd2 + a.g.at(i, j));
+}
+
+template <int SRC, bool DOT>
+__global__ void __launch_bounds__(SWEEP_NT) tile_pre2_kernel(const SweepParams<float> a) {
   pdl_trigger();
+  constexpr bool FBF = SRC == SRC_FINEBF;
   // z0 on NW x NH nodes from (x0, y0), elements one less each way; z1 inside.
   constexpr int NW = TILE_X + 5, NH = TILE_Y + 5, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
   static_assert(EW * EH <= SWEEP_NT && ZW * ZH <= SWEEP_NT, "one element and one node per thread");
@@ -83,28 +105,79 @@ template <int SRC> __global__ void __launch_bounds__(SWEEP_NT) tile_pre2_kernel(
   const bool node = t < ZW * ZH, valid = node && g.valid(i, j);
   const float2 zero2 = make_float2(0.f, 0.f);
   float2 d = zero2, b = zero2;
-  if (valid) d = __ldg(a.invd2 + g.at(i, j));
+  if (valid) d = tile_d<SRC>(a, i, j);
   float2 dh[2], bh[2];  // of the z0 nodes t and t + SWEEP_NT
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const int n = t + u * SWEEP_NT, ii = x0 + n % NW, jj = y0 + n / NW;
-    dh[u] = n < NW * NH && g.valid(ii, jj) ? __ldg(a.invd2 + g.at(ii, jj)) : zero2;
+    dh[u] = n < NW * NH && g.valid(ii, jj) ? tile_d<SRC>(a, ii, jj) : zero2;
   }
   pdl_wait_prior();
   const bool done = a.sc != nullptr && a.gate && a.sc->done != RUNNING;
-  if (valid) b = a.b[g.at(i, j)];
+  double dot0 = 0.0;
+  if constexpr (FBF) {
+    // Right-hand side from float64, into shared memory for the z1 nodes: r
+    // after the CG update (as in mto_sweep2.cuh), or the caller's vector.
+    __shared__ float2 bs[NW * NH];
+    bool upd = false;
+    double aupd = 0.0;
+    if constexpr (DOT) {
+      upd = a.sc->upd_pending != 0;
+      aupd = upd ? a.sc->alpha : 0.0;
+    }
+    if (done) return;  // uniform over the grid
+    double2 rv[2], qv[2];
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int n = t + u * SWEEP_NT, ii = x0 + n % NW, jj = y0 + n / NW;
-    bh[u] = n < NW * NH && g.valid(ii, jj) ? a.b[g.at(ii, jj)] : zero2;
-  }
-  if (done) return;  // uniform over the grid
+    for (int u = 0; u < 2; ++u) {
+      const int n = t + u * SWEEP_NT, ii = x0 + n % NW, jj = y0 + n / NW;
+      rv[u] = qv[u] = make_double2(0.0, 0.0);
+      if constexpr (DOT) {
+        if (n < NW * NH && g.valid(ii, jj)) {
+          rv[u] = upd ? a.r64_prev[g.at(ii, jj)] : static_cast<const double2*>(a.r64)[g.at(ii, jj)];
+          qv[u] = a.q64[g.at(ii, jj)];
+        }
+      } else {
+        if (n < NW * NH && g.active(ii, jj)) rv[u] = a.din[(long long)jj * (g.nx + 1) + ii];
+      }
+    }
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int n = t + u * SWEEP_NT;
-    if (n < NW * NH) z[n] = mul2(dh[u], bh[u]);
+    for (int u = 0; u < 2; ++u) {
+      const int n = t + u * SWEEP_NT, nx = n % NW, ny = n / NW;
+      const bool own = nx >= 3 && nx < 3 + TILE_X && ny >= 3 && ny < 3 + TILE_Y && g.valid(x0 + nx, y0 + ny);
+      if constexpr (DOT) {
+        const double2 rn = make_double2(fma(-aupd, qv[u].x, rv[u].x), fma(-aupd, qv[u].y, rv[u].y));
+        bh[u] = make_float2(d2f_rn(rn.x), d2f_rn(rn.y));
+        if (upd && own) {
+          a.r64[g.at(x0 + nx, y0 + ny)] = rn;
+          a.out32[g.at(x0 + nx, y0 + ny)] = bh[u];
+          dot0 = fma(rn.x, rn.x, fma(rn.y, rn.y, dot0));
+        }
+      } else {
+        bh[u] = make_float2((float)rv[u].x, (float)rv[u].y);
+        if (own) a.out32[g.at(x0 + nx, y0 + ny)] = bh[u];
+      }
+      if (n < NW * NH) {
+        z[n] = mul2(dh[u], bh[u]);
+        bs[n] = bh[u];
+      }
+    }
+    __syncthreads();
+    if (node) b = bs[zy * NW + zx];
+  } else {
+    if (valid) b = a.b[g.at(i, j)];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int n = t + u * SWEEP_NT, ii = x0 + n % NW, jj = y0 + n / NW;
+      bh[u] = n < NW * NH && g.valid(ii, jj) ? a.b[g.at(ii, jj)] : zero2;
+    }
+    if (done) return;  // uniform over the grid
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int n = t + u * SWEEP_NT;
+      if (n < NW * NH) z[n] = mul2(dh[u], bh[u]);
+    }
+    __syncthreads();
   }
-  __syncthreads();
   // z1 = z0 + w/D (b - K z0).
   const int c = ey * NW + ex;
   if (elem) f.template put<SRC>(a, er, t, z[c], z[c + 1], z[c + NW], z[c + NW + 1]);
@@ -140,9 +213,12 @@ template <int SRC> __global__ void __launch_bounds__(SWEEP_NT) tile_pre2_kernel(
       a.bc[gc.at(I, J)] = gc.is_fixed(I, J) ? zero2 : val;
     }
   }
+  if constexpr (DOT)
+    block_reduce_finish<SWEEP_NT, false>(dot0, 0.0, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
 }
 
-template <int SRC> __global__ void __launch_bounds__(SWEEP_NT) tile_post2_kernel(const SweepParams<float> a) {
+template <int SRC, bool DOT>
+__global__ void __launch_bounds__(SWEEP_NT) tile_post2_kernel(const SweepParams<float> a) {
   pdl_trigger();
   constexpr int NW = TILE_X + 4, NH = TILE_Y + 4, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
   static_assert(EW * EH <= SWEEP_NT && NW * NH <= SWEEP_NT, "one element and one node per thread");
@@ -160,10 +236,18 @@ template <int SRC> __global__ void __launch_bounds__(SWEEP_NT) tile_post2_kernel
   const bool node = t < ZW * ZH, valid = node && g.valid(i, j);
   const float2 zero2 = make_float2(0.f, 0.f);
   float2 d = zero2, b = zero2;
-  if (valid) d = __ldg(a.invd2 + g.at(i, j));
+  if (valid) d = tile_d<SRC>(a, i, j);
+  const bool own = valid && zx >= 2 && zx < 2 + TILE_X && zy >= 2 && zy < 2 + TILE_Y;
+  double2 rd = make_double2(0.0, 0.0), qd = rd;
   pdl_wait_prior();
   const bool done = a.sc != nullptr && a.gate && a.sc->done != RUNNING;
   if (valid) b = a.b[g.at(i, j)];
+  if constexpr (DOT) {
+    if (own) {
+      rd = a.rdot[g.at(i, j)];
+      if (a.qdot != nullptr) qd = a.qdot[g.at(i, j)];
+    }
+  }
   // z = v + P z_c at node t (mto_sweep2.cuh's interpolation).
   float2 v = zero2;
   {
@@ -195,8 +279,21 @@ template <int SRC> __global__ void __launch_bounds__(SWEEP_NT) tile_post2_kernel
   if (elem && ex >= 1 && ex < EW - 1 && ey >= 1 && ey < EH - 1)
     f.template put<SRC>(a, er, t, z[c], z[c + 1], z[c + NW], z[c + NW + 1]);
   __syncthreads();
-  if (valid && zx >= 2 && zx < 2 + TILE_X && zy >= 2 && zy < 2 + TILE_Y)
-    a.out[g.at(i, j)] = fma2(d, sub2(b, f.at_node(en)), z2);
+  double dot0 = 0.0, dot1 = 0.0;
+  if (own) {
+    const float2 z3 = fma2(d, sub2(b, f.at_node(en)), z2);
+    if (SRC == SRC_FINEBF && !DOT && a.dout != nullptr)
+      a.dout[(long long)j * (g.nx + 1) + i] = make_double2(z3.x, z3.y);
+    else
+      a.out[g.at(i, j)] = z3;
+    if constexpr (DOT) {
+      const double zx64 = to_f64(z3.x), zy64 = to_f64(z3.y);
+      dot0 = fma(zx64, rd.x, zy64 * rd.y);
+      if (a.qdot != nullptr) dot1 = fma(zx64, qd.x, zy64 * qd.y);
+    }
+  }
+  if constexpr (DOT)
+    block_reduce_finish<SWEEP_NT>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
 }
 
 }  // namespace mto

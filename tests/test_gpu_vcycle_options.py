@@ -175,3 +175,27 @@ def test_mixed_cycle_between_the_callers_arrays(mto, nx, ny, nc, nu1, nu2):
         torch.cuda.synchronize()
         assert torch.equal(buf[shift:], z.reshape(-1)), shift
     m.close()
+
+
+@pytest.mark.parametrize("nu1,nu2", [(2, 2), (2, 3), (3, 2)])
+@pytest.mark.parametrize("nx,ny,nc", [(8, 8, 1), (32, 24, 2), (62, 34, 1), (264, 136, 3)])
+def test_tiled_finest_mixed_passes_equal_marching_ones(mto, nx, ny, nc, nu1, nu2):
+    """The same for the bf16 finest level; its dot products and |r|^2 are summed by tiles, so a
+    solve follows the bars of the mixed solves (iterations +- 2, u to 1e-6)."""
+    x = torch.from_numpy(dirichlet_design(nx, ny, 4, seed=nx)).cuda()
+    r = torch.from_numpy(np.random.default_rng(ny).standard_normal((ny + 1, nx + 1, 2))).cuda()
+    f = torch.from_numpy(load_top_edge(nx, ny)).cuda()
+    z, u, it = [], [], []
+    for warps in (0, 1):
+        m = mto.Mesh(nx, ny, n_coarsen=nc, precision="mixed", tol=1e-10, nu1=nu1, nu2=nu2, rr_every=5)
+        m.set_launch_shape(nc, warps)
+        m.set_design(x, EP, 3.0)
+        z.append(m.apply_preconditioner(r))
+        uu, st = m.solve(f)
+        assert st["status"] == "MTO_OK" and st["rel_res_true"] <= 1e-10, st
+        u.append(uu)
+        it.append(st["iters"])
+        m.close()
+    assert torch.equal(z[0], z[1])
+    assert abs(it[0] - it[1]) <= 2, it
+    assert rel(u[0].cpu().numpy(), u[1].cpu().numpy()) < 1e-6
