@@ -19,7 +19,15 @@
 // (mto_sweep2.cuh): PRE2 with DOT also carries the CG update of the outer
 // iteration, POST2 with DOT forms the dot products (their partial sums are per
 // tile, so these differ in the last bits).  Two launches and a trip through
-// memory less per cycle at each end: a mixed iteration 56 -> 47 us at 200 x 136.
+// memory less per cycle at each end: a mixed iteration 56 -> 45 us at 200 x 136.
+//
+// The finest-level passes do not let the next kernel launch early: its blocks
+// would wait in the registers and shared memory that this kernel's own tiles
+// (one to five per SM, with a reduction at their end) and another load case's
+// kernels still want.  With and without the early launch: mixed iteration at
+// 200 x 136 47.4 -> 45.4 us, its two load cases at once 1590 -> 1316 us, 256^2
+// 2115 -> 1980 us, one 64^2 solve 734 -> 748 us.  Coarse levels gain from it
+// (mixed iteration at 2048^2 366.6 -> 363.6 us, at 1024^2 144.7 -> 142.2 us).
 #pragma once
 
 #include "mto_fused.cuh"
@@ -85,7 +93,7 @@ template <int SRC> __device__ __forceinline__ float2 tile_d(const SweepParams<fl
 
 template <int SRC, bool DOT>
 __global__ void __launch_bounds__(SWEEP_NT) tile_pre2_kernel(const SweepParams<float> a) {
-  pdl_trigger();
+  if constexpr (SRC != SRC_FINEBF) pdl_trigger();  // see the top of the file
   constexpr bool FBF = SRC == SRC_FINEBF;
   // z0 on NW x NH nodes from (x0, y0), elements one less each way; z1 inside.
   constexpr int NW = TILE_X + 5, NH = TILE_Y + 5, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
@@ -219,7 +227,7 @@ __global__ void __launch_bounds__(SWEEP_NT) tile_pre2_kernel(const SweepParams<f
 
 template <int SRC, bool DOT>
 __global__ void __launch_bounds__(SWEEP_NT) tile_post2_kernel(const SweepParams<float> a) {
-  pdl_trigger();
+  if constexpr (SRC != SRC_FINEBF) pdl_trigger();  // see the top of the file
   constexpr int NW = TILE_X + 4, NH = TILE_Y + 4, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
   static_assert(EW * EH <= SWEEP_NT && NW * NH <= SWEEP_NT, "one element and one node per thread");
   __shared__ TileForces<EW, EH> f;
