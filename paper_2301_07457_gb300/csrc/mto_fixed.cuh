@@ -16,13 +16,15 @@
 // 2^-90 of the warp's largest value under that.  Element coefficients are
 // 61-bit integers with one exponent X per element; a product keeps the upper
 // 96 of its 157 bits, so forces are  T 2^(B + Xm - 2132)  with Xm the largest X
-// met so far, with the same relation between the largest force and the last
-// bit (coarse elements: 59-bit integers, T 2^(B + Xm - 2130)).  Every sum of
-// the operator fits: |K v| < 2^95 (bounds at the kernel).
-// The results are more accurate than the float64 evaluation, whose every sum
-// rounds at 2^-53 of its own terms, as long as a node's terms are not more
-// than about 2^30 below the largest of the warp's window (30 columns by the
-// rows of the task).
+// met so far (coarse elements: 59-bit integers, T 2^(B + Xm - 2130)): the last
+// bit relates to the largest coefficient times the largest value of the window,
+// not to the largest force.  Every sum of the operator fits: |K v| < 2^95
+// (bounds at the kernel).
+//
+// A window (30 columns by the rows of a task, 14 columns by three rows, or a
+// tile) shares its scales, so the error of a node's K v is absolute, whatever
+// the size of its own terms: FX_SPAN below says from where on they are
+// evaluated in float64 instead.
 //
 // The functions also compile as host code (checked against 128-bit
 // arithmetic there).
@@ -252,6 +254,39 @@ __host__ __device__ __forceinline__ void fx_put_tag(unsigned long long* w, unsig
 __host__ __device__ __forceinline__ unsigned fx_tag(const unsigned long long* w) {
   return ((unsigned)w[0] & 15u) | (((unsigned)w[1] & 15u) << 4) | (((unsigned)w[2] & 15u) << 8);
 }
+
+// Factor c 2^(X - bias) of an element with tag `tag`.
+__host__ __device__ __forceinline__ double fx_factor(unsigned long long c, unsigned tag, int bias) {
+#ifdef __CUDA_ARCH__
+  return ldexp((double)c, (int)(tag & 0x7ffu) - bias);
+#else
+  return __builtin_ldexp((double)c, (int)(tag & 0x7ffu) - bias);
+#endif
+}
+
+// Upper word of the larger magnitude of a pair.
+__host__ __device__ __forceinline__ unsigned fx_magnitude(double x, double y) {
+  const unsigned a = (unsigned)(bits_of(x) >> 32) & 0x7fffffffu, b = (unsigned)(bits_of(y) >> 32) & 0x7fffffffu;
+  return a > b ? a : b;
+}
+// Whether scales of weight Q = B + Xm lose too much of an element of weight q,
+// the sum of the (biased) exponents of its largest factor and of its largest
+// nodal value: the window is then done in float64.
+//
+// The terms |K||v| of a node next to the element are at least about 2^(q - 2046).
+// Its error is at most 18 units of the last place, so 2^(Q - q - 82) of them,
+// and usually 2^-6 of that.  Measured on a soft block beside solids, random values
+// of one size: error over the row's terms (largest / root mean square) 2.1e-16 /
+// 5.7e-17 up to Q - q = 34, 2.9e-16 / 6.5e-17 at 36, 3.0e-16 / 7.7e-17 at 37,
+// 3.5e-16 / 7.8e-17 at 38, against 4.1e-16 / 7.7e-17 in float64: the line lies at the
+// last one that is better than float64 in both.  A void of 1e-9 (2^-30) beside
+// solids stays within it for values down to 1/64 of the window's largest; a
+// float64 iteration on a smooth two-phase design with that void takes 64 us at
+// 64^2 (78 with the line at 34, 57 with none), 105 at 256^2 (114, 104).
+// Float64 subnormals count as zeros here, next to values above 2^-926.
+constexpr int FX_SPAN = 36;
+__host__ __device__ __forceinline__ bool fx_beyond(int Q, int q) { return Q - q > FX_SPAN; }
+constexpr int FX_NEVER = -(1 << 20);  // a weight that no scales hold
 
 // A fine element: its three factors (p, c, g of mto_fsweep.cuh) as integers
 // below 2^61, factor = c 2^(X - 1083); all of one sign (that of the modulus).

@@ -1,5 +1,5 @@
-// Marching sweeps of the float64 finest level with the element operator in
-// 96-bit fixed point (mto_fixed.cuh).
+// Sweeps of the float64 levels with the element operator in 96-bit fixed
+// point (mto_fixed.cuh): marching, and a row per warp on small grids.
 //
 // Same strips, chunks, modes and edge-force bookkeeping as mto_sweep.cuh, one
 // node column per lane.  The marched vector, its update (p = z + beta p_old,
@@ -27,9 +27,19 @@
 //
 // Scales are uniform over the warp.  A row whose largest exponent is above B
 // (or an element above Xm) raises it and shifts the carried state; this
-// happens in the first rows of a task and hardly ever after.  A non-finite
-// nodal value enters as zero and marks its row, and every node next to it gets
-// a NaN; a non-finite modulus makes the task's results NaN.
+// happens in the first rows of a task and hardly ever after.
+//
+// Where an element's terms lie too far below the scales (fx_beyond in
+// mto_fixed.cuh) the task is done again in float64 (rows_f64).  The
+// fixed-point loop only keeps the smallest weight of its elements, four or five
+// integer instructions a row, and compares it with the scales at its end: a vote
+// and a call in every row took K p at 2048^2 from 113 to 119 us, an early exit
+// from the loop to 117, this to 115.  A non-finite nodal value or modulus takes
+// the task to float64 too, and so reaches the nodes next to it alone.  Normal
+// work hardly ever gets there (designs with a void of 1e-9, 64^2 to 1024^2: no
+// marching row that was counted, up to 1% of the tiles); with a void of 1e-12 in
+// half of a smooth design an iteration takes 169 instead of 104 us at 256^2 and
+// 442 instead of 371 us at 1024^2 (278 and 992 us where all was in float64).
 #pragma once
 
 #include "mto_fixed.cuh"
@@ -88,6 +98,14 @@ template <> struct FxElem<SRC_FINE64> {
     const Fx p = fx_mul(fx_add(w.c1, w.d2), k[0]), g = fx_mul(fx_sub(w.c1, w.d2), k[2]);
     return {fx_add(p, g), fx_mul(w.c3, k[1]), fx_sub(p, g), fx_mul(w.d3, k[1]), fx_mul(w.s, k[2])};
   }
+  // The same in float64.
+  __device__ __forceinline__ static Strain<double> core64(const SweepParams<double>&, const Strain<double>& w,
+                                                          const unsigned long long* k) {
+    const unsigned tag = fx_tag(k);
+    const double P = fx_factor(k[0], tag, 1083), C = fx_factor(k[1], tag, 1083), G = fx_factor(k[2], tag, 1083);
+    const double p = P * (w.c1 + w.d2), g = G * (w.c1 - w.d2), sg = tag & FX_TAG_NEG ? -1.0 : 1.0;
+    return {sg * (p + g), sg * (C * w.c3), sg * (p - g), sg * (C * w.d3), sg * (G * w.s)};
+  }
 };
 template <> struct FxElem<SRC_COARSE> {
   static constexpr int N = FX_NCOARSE, UNIT = -2130;
@@ -134,6 +152,38 @@ template <> struct FxElem<SRC_COARSE> {
     t.s = fx_flip(fx_add(ts, fx_add(fx_mul(c3, g1), fx_mul(d3, g2))), s12);
     return t;
   }
+  // The same in float64.
+  __device__ __forceinline__ static Strain<double> core64(const SweepParams<double>& a, const Strain<double>& w,
+                                                          const unsigned long long* k) {
+    const unsigned tag = fx_tag(k);
+    double f[FX_NCOARSE];
+#pragma unroll
+    for (int n = 0; n < FX_NCOARSE; ++n) {
+      const double m = fx_factor(k[n] & 0x7fffffffffffffffull, tag, 1081);
+      f[n] = (k[n] >> 63) ? -m : m;
+    }
+    const double g = ldexp((double)a.gfix, -64), nu = 1.0 - 2.0 * g;
+    const double m0 = f[FXC_M00], m1 = f[FXC_M10], m2 = f[FXC_M01], k9 = f[FXC_C3D3];
+    Strain<double> t;
+    t.c1 = m0 * (w.c1 + nu * w.d2) + (m2 * w.c3 + nu * (m1 * w.d3));
+    t.d2 = m0 * (w.d2 + nu * w.c1) + (m1 * w.d3 + nu * (m2 * w.c3));
+    t.c3 = f[FXC_C3C3] * w.c3 + m2 * (w.c1 + nu * w.d2) + (k9 * w.d3 + g * (m1 * w.s));
+    t.d3 = f[FXC_D3D3] * w.d3 + m1 * (w.d2 + nu * w.c1) + (k9 * w.c3 + g * (m2 * w.s));
+    t.s = g * (m0 * w.s + (m1 * w.c3 + m2 * w.d3));
+    return t;
+  }
+};
+
+// A warp's columns: lane `lane` has column i; rows from je0, coarse rows Jb .. Je
+// of a restriction.
+struct FTask {
+  int i, lane, je0, Jb, Je;
+  bool own_col;
+};
+// What a task sums: dot products, the coarse row in progress (RESTRICT).
+struct FSums {
+  double dot0, dot1;
+  double2 racc;
 };
 
 template <int SRC, int MODE, bool DOT, typename ZT> struct FSweep {
@@ -236,11 +286,120 @@ template <int SRC, int MODE, bool DOT, typename ZT> struct FSweep {
       return r.v;
     }
   }
+
+  // What a mode does with K v of node (i, je); k: its offset, v: its marched
+  // value, b, d: its right-hand side and w/D (all lanes of the warp).
+  __device__ __forceinline__ static void finish_row(const SweepParams<double>& a, const FTask& t, long long k, int je,
+                                                    bool inb, bool act, const double2& v, const double2& kv,
+                                                    const double2& b, const double2& d, const Pack& cur,
+                                                    FSums& sums) {
+    const double2 zero2 = make_double2(0.0, 0.0);
+    if constexpr (MODE == MODE_APPLY) {
+      if (inb) a.out[a.dense ? (long long)je * (a.g.nx + 1) + t.i : k] = act ? kv : zero2;
+    } else if constexpr (MODE == MODE_RESID) {
+      double2 r = zero2;
+      if (act) r = sub2(b, kv);
+      if (inb) a.out[k] = r;
+      if (inb && a.out32 != nullptr) a.out32[k] = make_float2(float(r.x), float(r.y));
+      sums.dot0 = fma(r.x, r.x, fma(r.y, r.y, sums.dot0));
+    } else if constexpr (MODE == MODE_KP) {
+      const double2 q = act ? kv : zero2;
+      if (inb) {
+        a.p_out[k] = v;
+        a.out[k] = q;
+        sums.dot0 = fma(v.x, q.x, fma(v.y, q.y, sums.dot0));
+      }
+    } else if constexpr (SMOOTHING) {
+      double2 zn = zero2;
+      if (act) zn = make_double2(fma(d.x, b.x - kv.x, v.x), fma(d.y, b.y - kv.y, v.y));
+      if (inb) a.out[k] = zn;
+      if constexpr (DOT) {
+        if (act) {
+          sums.dot0 = fma(zn.x, cur.rd.x, fma(zn.y, cur.rd.y, sums.dot0));
+          if (a.qdot != nullptr) sums.dot1 = fma(zn.x, cur.qd.x, fma(zn.y, cur.qd.y, sums.dot1));
+        }
+      }
+    } else if constexpr (MODE == MODE_RESTRICT) {
+      double2 r = zero2;
+      if (act) r = sub2(b, kv);
+      // Full weighting, vertically along the march (1/2, 1, 1/2 over fine
+      // rows 2J - 1, 2J, 2J + 1), then horizontally once per coarse row.
+      if (je > t.je0) {
+        if (je & 1) {
+          const int Jlo = (je - 1) / 2;
+          const double2 col = make_double2(fma(0.5, r.x, sums.racc.x), fma(0.5, r.y, sums.racc.y));
+          const double2 cu = shfl_up2(col), cd = shfl_down2(col);
+          const double2 val = make_double2(fma(0.5, cu.x + cd.x, col.x), fma(0.5, cu.y + cd.y, col.y));
+          const bool producer = (t.lane & 1) == 0 && t.lane >= 2 && t.lane <= 28;
+          const int I = t.i >> 1;
+          if (producer && Jlo >= t.Jb && Jlo <= t.Je && I >= 0 && I <= a.gc.nx)
+            a.bc[a.gc.at(I, Jlo)] = a.gc.is_fixed(I, Jlo) ? zero2 : val;
+          sums.racc = make_double2(0.5 * r.x, 0.5 * r.y);
+        } else {
+          sums.racc = add2(sums.racc, r);
+        }
+      }
+    }
+  }
 };
+
+// Rows je0 + 1 .. je1 of a warp's columns in float64 (all lanes of the warp):
+// the marching sweep with the element operator on the FP64 pipe, at about three
+// times the cost.  x has had its pending step (KP).  Without FINISH nothing is
+// written and racc is K v of the last row.  A call of its own, so that its
+// registers do not weigh on the kernels.
+template <int SRC, int MODE, bool DOT, typename ZT, bool FINISH>
+__device__ __noinline__ FSums rows_f64(const SweepParams<double>& a, FTask t0, int je1, double beta, bool lag,
+                                       double alag) {
+  using F = FSweep<SRC, MODE, DOT, ZT>;
+  const Grid& g = a.g;
+  const double2 zero2 = make_double2(0.0, 0.0);
+  const int je0 = t0.je0;
+  FSums sums = {0.0, 0.0, zero2};
+  long long k = g.at(t0.i, je0);
+  typename F::Pack cur;
+  F::load_top(a, k, t0.i, je0, lag, cur);
+  double2 vb = F::value(a, cur, t0.i, je0, beta, lag, alag), below = zero2, bc = zero2, dc = zero2, kv = zero2;
+  if constexpr (MODE == MODE_SMOOTH0) {
+    bc = cur.v;
+    dc = cur.dt;
+  }
+#pragma unroll 1
+  for (int je = je0; je <= je1; ++je, k += g.pitch) {
+    F::load(a, k, t0.i, je, lag, cur);
+    const double2 vt = F::value(a, cur, t0.i, je + 1, beta, lag, alag);
+    const double2 ac = sub2(shfl_down2(vb), vb), bt = sub2(shfl_down2(vt), vt), dl = sub2(vt, vb);
+    const double2 up = add2(dl, shfl_down2(dl));
+    Strain<double> w;
+    w.c1 = ac.x + bt.x;
+    w.c3 = bt.x - ac.x;
+    w.d2 = up.y;
+    w.d3 = bt.y - ac.y;
+    w.s = up.x + (ac.y + bt.y);
+    const Strain<double> t = F::Elem::core64(a, w, cur.k);
+    // Forces of the element row on the nodes of its bottom and of its top edge.
+    auto edge = [&](double2 h, double2 v) { return add2(shfl_up2(add2(v, h)), sub2(v, h)); };
+    kv = add2(below, edge(make_double2(t.c1 - t.c3, t.s - t.d3), make_double2(-t.s, -t.d2)));
+    if constexpr (FINISH) {
+      const bool inb = je > je0 && t0.own_col && je >= 0 && je <= g.ny;
+      const bool act = inb && !g.is_fixed(t0.i, je);
+      const double2 b = MODE == MODE_SMOOTH0 ? bc : cur.b, d = MODE == MODE_SMOOTH0 ? dc : cur.d;
+      F::finish_row(a, t0, k, je, inb, act, vb, kv, b, d, cur, sums);
+    }
+    below = edge(make_double2(t.c1 + t.c3, t.s + t.d3), make_double2(t.s, t.d2));
+    vb = vt;
+    if constexpr (MODE == MODE_SMOOTH0) {
+      bc = cur.v;
+      dc = cur.dt;
+    }
+  }
+  if constexpr (!FINISH) sums.racc = kv;
+  return sums;
+}
 
 // Two resident blocks per SM, as sweep2_kernel.
 template <int SRC, int MODE, bool DOT, typename ZT, int PF>
-__global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<double> a) {
+__global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const __grid_constant__ SweepParams<double> a) {
   using F = FSweep<SRC, MODE, DOT, ZT>;
   using Pack = typename F::Pack;
   constexpr bool REDUCE = DOT || MODE == MODE_RESID || MODE == MODE_KP;
@@ -254,7 +413,8 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
   const int wg = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int strip = wg % a.nstrips;
   const int chunk = wg / a.nstrips;
-  double dot0 = 0.0, dot1 = 0.0;
+  const double2 zero2 = make_double2(0.0, 0.0);
+  FSums sums = {0.0, 0.0, zero2};
   double beta = 0.0, alag = 0.0;
   bool vzero = false, lag = false;
   if constexpr (MODE == MODE_KP) {
@@ -269,7 +429,6 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
       alag = a.sc->alpha;
     }
   }
-  const double2 zero2 = make_double2(0.0, 0.0);
 
   if (vzero) {
     // Residual of a zero iterate: r = b on the free DOFs, no operator needed.
@@ -281,7 +440,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         const double2 r = g.is_fixed(i, j) ? zero2 : a.b[k];
         a.out[k] = r;
         if (a.out32 != nullptr) a.out32[k] = make_float2(float(r.x), float(r.y));
-        dot0 = fma(r.x, r.x, fma(r.y, r.y, dot0));
+        sums.dot0 = fma(r.x, r.x, fma(r.y, r.y, sums.dot0));
       }
     }
   } else if (chunk < a.nchunks) {
@@ -304,20 +463,22 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
     const long long pitch = g.pitch;
 
     int B = 1, Xm = 0;             // scales of the nodal values and of the coefficients
-    unsigned bad0 = 0, badp = 0;   // lanes with a non-finite value: node rows je, je - 1
+    int eb = 0;                    // exponent of node (i, je)
+    int low = 1 << 20;             // smallest weight of the column's elements
+    const FTask t0 = {i, lane, je0, Jb, Je, own_col};
     // Carried from the row below: edge differences and sums (i + 1 minus / plus
     // i) of node row je, and the forces of element row je - 1 on its top and
     // left edges.
     Fx2 ac = {fx_zero(), fx_zero()}, sc = ac, gbp = ac, gsp = ac;
     // Marched values of a row at scale B, which the row raises if it has to;
-    // bad: the lanes whose value is not finite (taken as zero).
-    auto to_fixed = [&](double2 v, unsigned& bad) -> Fx2 {
-      bad = 0;
-      const int e = max(fx_exponent((unsigned)__double2hiint(v.x)), fx_exponent((unsigned)__double2hiint(v.y)));
+    // e: the pair's larger exponent.
+    auto to_fixed = [&](double2 v, int& e) -> Fx2 {
+      e = max(fx_exponent((unsigned)__double2hiint(v.x)), fx_exponent((unsigned)__double2hiint(v.y)));
       if (__any_sync(0xffffffffu, e > B)) {
-        bad = __ballot_sync(0xffffffffu, e == 0x7ff);
-        if (e == 0x7ff) v = zero2;
-        const int Bn = (int)__reduce_max_sync(0xffffffffu, e == 0x7ff ? 0u : (unsigned)e);
+        const bool finite = e != 0x7ff;
+        if (!finite) v = zero2;
+        if (!__all_sync(0xffffffffu, finite)) low = FX_NEVER;
+        const int Bn = (int)__reduce_max_sync(0xffffffffu, finite ? (unsigned)e : 0u);
         if (Bn > B) {
           ac = fsar(ac, Bn - B);
           sc = fsar(sc, Bn - B);
@@ -337,7 +498,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
       Pack r0;
       F::load_top(a, k0, i, je0, lag, r0);
       vbd = F::value(a, r0, i, je0, beta, lag, alag);
-      const Fx2 vb = to_fixed(vbd, bad0);
+      const Fx2 vb = to_fixed(vbd, eb);
       const Fx2 vr = fshfl_down(vb);
       ac = fsub(vr, vb);
       sc = fadd(vr, vb);
@@ -346,8 +507,6 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         dc = r0.dt;
       }
     }
-    double2 racc = zero2;  // RESTRICT: partial coarse row of this column
-
     Pack ring[PF];
 #pragma unroll
     for (int u = 0; u < PF; ++u)
@@ -370,8 +529,8 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         }
         // ---- element (i, je) from rows je (vb) and je + 1 (vt) ----
         const double2 vtd = F::value(a, cur, i, je + 1, beta, lag, alag);
-        unsigned badt;
-        const Fx2 vt = to_fixed(vtd, badt);
+        int et;
+        const Fx2 vt = to_fixed(vtd, et);
         const Fx2 vr = fshfl_down(vt);  // lane 31: its own value, used only for halo output
         const Fx2 bt = fsub(vr, vt), st = fadd(vr, vt);
         const Fx2 up = fsub(st, sc);  // (c2, d2): left plus right edge
@@ -383,7 +542,8 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         const bool rare = __any_sync(0xffffffffu, tag != 0u && (unsigned)(Xm - (int)tag) >= 32u);
         const int X = (int)(tag & 0x7ffu);
         if (rare) {
-          const int Xn = max(Xm, (int)__reduce_max_sync(0xffffffffu, (unsigned)X));
+          if (__any_sync(0xffffffffu, X == 0x7ff)) low = FX_NEVER;
+          const int Xn = max(Xm, (int)__reduce_max_sync(0xffffffffu, X == 0x7ff ? 0u : (unsigned)X));
           gbp = fsar(gbp, Xn - Xm);
           gsp = fsar(gsp, Xn - Xm);
           Xm = Xn;
@@ -407,62 +567,16 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         double2 kv = make_double2(fx_to_double<false>(kvf.x, unit), fx_to_double<false>(kvf.y, unit));
         if (unit < FX_UNIT_MIN || unit > FX_UNIT_MAX)  // uniform over the warp
           kv = make_double2(fx_to_double(kvf.x, unit), fx_to_double(kvf.y, unit));
-        const unsigned badn = badp | bad0 | badt;
-        if (badn != 0u || Xm == 0x7ff) {  // uniform over the warp; neighbours of non-finite values
-          const bool near = ((badn | (badn << 1) | (badn >> 1)) >> lane) & 1u;
-          if (near || Xm == 0x7ff) kv = make_double2(NAN, NAN);
-        }
 
+        // Weight of the element, where it is not zero on all corners (as most
+        // are in the first cycle of a solve) and has material.
+        const int ec = max(eb, et), e4 = max(ec, __shfl_down_sync(0xffffffffu, ec, 1));
+        if (min(e4, X) != 0) low = min(low, e4 + X);
+        eb = et;
         const bool inb = je > je0 && own_col && je >= 0 && je <= g.ny;
         const bool act = inb && !col_fixed && !(((g.fixed & 1u) && je == 0) || ((g.fixed & 8u) && je == g.ny));
-        if constexpr (MODE == MODE_APPLY) {
-          if (inb) a.out[a.dense ? (long long)je * (g.nx + 1) + i : k] = act ? kv : zero2;
-        } else if constexpr (MODE == MODE_RESID) {
-          double2 r = zero2;
-          if (act) r = sub2(cur.b, kv);
-          if (inb) a.out[k] = r;
-          if (inb && a.out32 != nullptr) a.out32[k] = make_float2(float(r.x), float(r.y));
-          dot0 = fma(r.x, r.x, fma(r.y, r.y, dot0));
-        } else if constexpr (MODE == MODE_KP) {
-          const double2 q = act ? kv : zero2;
-          if (inb) {
-            a.p_out[k] = vbd;
-            a.out[k] = q;
-            dot0 = fma(vbd.x, q.x, fma(vbd.y, q.y, dot0));
-          }
-        } else if constexpr (F::SMOOTHING) {
-          const double2 b = MODE == MODE_SMOOTH0 ? bc : cur.b;
-          const double2 d = MODE == MODE_SMOOTH0 ? dc : cur.d;
-          double2 zn = zero2;
-          if (act) zn = make_double2(fma(d.x, b.x - kv.x, vbd.x), fma(d.y, b.y - kv.y, vbd.y));
-          if (inb) a.out[k] = zn;
-          if constexpr (DOT) {
-            if (act) {
-              dot0 = fma(zn.x, cur.rd.x, fma(zn.y, cur.rd.y, dot0));
-              if (a.qdot != nullptr) dot1 = fma(zn.x, cur.qd.x, fma(zn.y, cur.qd.y, dot1));
-            }
-          }
-        } else if constexpr (MODE == MODE_RESTRICT) {
-          double2 r = zero2;
-          if (act) r = sub2(cur.b, kv);
-          // Full weighting, vertically along the march (1/2, 1, 1/2 over fine
-          // rows 2J - 1, 2J, 2J + 1), then horizontally once per coarse row.
-          if (je > je0) {
-            if (je & 1) {
-              const int Jlo = (je - 1) / 2;
-              const double2 col = make_double2(fma(0.5, r.x, racc.x), fma(0.5, r.y, racc.y));
-              const double2 cu = shfl_up2(col), cd = shfl_down2(col);
-              const double2 val = make_double2(fma(0.5, cu.x + cd.x, col.x), fma(0.5, cu.y + cd.y, col.y));
-              const bool producer = (lane & 1) == 0 && lane >= 2 && lane <= 28;
-              const int I = i >> 1;
-              if (producer && Jlo >= Jb && Jlo <= Je && I >= 0 && I <= a.gc.nx)
-                a.bc[a.gc.at(I, Jlo)] = a.gc.is_fixed(I, Jlo) ? zero2 : val;
-              racc = make_double2(0.5 * r.x, 0.5 * r.y);
-            } else {
-              racc = add2(racc, r);
-            }
-          }
-        }
+        const double2 b = MODE == MODE_SMOOTH0 ? bc : cur.b, d = MODE == MODE_SMOOTH0 ? dc : cur.d;
+        F::finish_row(a, t0, k, je, inb, act, vbd, kv, b, d, cur, sums);
         if constexpr (MODE == MODE_SMOOTH0) {
           bc = cur.v;
           dc = cur.dt;
@@ -472,14 +586,14 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const SweepParams<d
         gsp = gs;
         sc = st;
         vbd = vtd;
-        badp = bad0;
-        bad0 = badt;
         k += pitch;
       }
     }
+    if (__any_sync(0xffffffffu, lane <= 30 && fx_beyond(B + Xm, low)))
+      sums = rows_f64<SRC, MODE, DOT, ZT, true>(a, t0, je1, beta, lag, alag);
   }
   if constexpr (REDUCE) {
-    block_reduce_finish<SWEEP_NT, DOT>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
+    block_reduce_finish<SWEEP_NT, DOT>(sums.dot0, sums.dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
   }
 }
 
@@ -500,8 +614,16 @@ constexpr int SPLIT_STRIDE = 14;   // columns per warp
 constexpr int SPLIT_RSTRIDE = 12;  // fine columns per warp of the restriction (6 coarse ones)
 constexpr int SPLIT_RWARPS = 3;
 
+// Resident blocks per SM that the fixed-point path's registers allow; rows_f64
+// would take a few more (here and in the tiles together a float64 iteration at
+// 256^2 99.1 -> 100.7 us, at 64^2, which does not fill the chip, 52.7 -> 52.3).
+template <int SRC, int MODE, bool DOT> constexpr int split_blocks() {
+  return SRC == SRC_COARSE ? 2 : (MODE == MODE_KP || DOT ? 3 : 4);
+}
+
 template <int SRC, int MODE, bool DOT, typename ZT>
-__global__ void __launch_bounds__(SWEEP_NT, 2) fsplit_kernel(const SweepParams<double> a) {
+__global__ void __launch_bounds__(SWEEP_NT, (split_blocks<SRC, MODE, DOT>()))
+    fsplit_kernel(const __grid_constant__ SweepParams<double> a) {
   using F = FSweep<SRC, MODE, DOT, ZT>;
   using Pack = typename F::Pack;
   constexpr bool REDUCE = DOT || MODE == MODE_RESID || MODE == MODE_KP;
@@ -564,18 +686,17 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsplit_kernel(const SweepParams<d
   if constexpr (MODE == MODE_KP) x = reinterpret_cast<const double*>(a.xvec + kn)[c];
   if (done) return;  // uniform over the grid
 
-  double dot0 = 0.0, dot1 = 0.0;
+  FSums sums = {0.0, 0.0, make_double2(0.0, 0.0)};
   double res = 0.0;  // RESTRICT: b - K v of this lane's component
   if (task) {
     const double2 vlo = F::value(a, lo, i, jr, beta, lag, alag), vhi = F::value(a, hi, i, jr + 1, beta, lag, alag);
     // Scales of the warp.
     auto expo = [](double v) { return fx_exponent((unsigned)__double2hiint(v)); };
     const int e0 = max(expo(vlo.x), expo(vlo.y)), e1 = max(expo(vhi.x), expo(vhi.y));
-    const bool bad0 = e0 == 0x7ff, bad1 = e1 == 0x7ff;
-    const int B = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(max(bad0 ? 0 : e0, bad1 ? 0 : e1), 1));
-    const unsigned bad = __ballot_sync(0xffffffffu, bad0 || bad1);
+    const int ec = max(e0, e1);
+    const int B = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(ec, 1));
     const double2 zero2 = make_double2(0.0, 0.0);
-    const Fx2 vb = fx2_from(bad0 ? zero2 : vlo, B), vt = fx2_from(bad1 ? zero2 : vhi, B);
+    const Fx2 vb = fx2_from(vlo, B), vt = fx2_from(vhi, B);
     auto right = [](const Fx2& v) -> Fx2 {  // next column of the half (its last lane: its own value, halo only)
       return {{__shfl_down_sync(0xffffffffu, v.x.lo, 1, 16), __shfl_down_sync(0xffffffffu, v.x.mid, 1, 16),
                __shfl_down_sync(0xffffffffu, v.x.hi, 1, 16)},
@@ -616,14 +737,24 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsplit_kernel(const SweepParams<d
     const int unit = B + Xm + F::Elem::UNIT;
     double kv = fx_to_double<false>(sum, unit);
     if (unit < FX_UNIT_MIN || unit > FX_UNIT_MAX) kv = fx_to_double(sum, unit);  // uniform over the warp
-    if (bad != 0u || Xm == 0x7ff) {  // neighbours of non-finite values
-      const unsigned m = (bad | (bad >> 16)) & 0xffffu;
-      if (Xm == 0x7ff || (((m | (m << 1) | (m >> 1)) >> hl) & 1u)) kv = NAN;
-    }
-
+    // Whether the scales hold the terms of the elements, as in the marching
+    // kernel; a non-finite value or modulus has made a scale non-finite.
+    const int e4 = max(ec, __shfl_down_sync(0xffffffffu, ec, 1, 16));
+    const bool again = (__any_sync(0xffffffffu, hl <= 14 && min(e4, X) != 0 && fx_beyond(B + Xm, e4 + X)) ||
+                        B == 0x7ff || Xm == 0x7ff) && !vzero;
     const double2 mid = half ? vlo : vhi;  // node row je
     const double vc = c ? mid.y : mid.x;
-    if constexpr (MODE == MODE_APPLY) {
+    if constexpr (MODE == MODE_KP) {
+      const double2 old = half ? lo.v : hi.v;
+      if (own && lag) reinterpret_cast<double*>(a.xvec + kn)[c] = fma(alag, c ? old.y : old.x, x);
+    }
+    if (again) {  // uniform over the warp: in float64, written from the lower half
+      const FTask t0 = {i, lane, je - 1, 0, 0, own && half == 0};
+      sums = rows_f64<SRC, MODE, DOT, ZT, !RESTRICT>(a, t0, je, beta, lag, alag);
+      if constexpr (RESTRICT) kv = c ? sums.racc.y : sums.racc.x;
+    }
+    if (again && !RESTRICT) {
+    } else if constexpr (MODE == MODE_APPLY) {
       double* out = reinterpret_cast<double*>(a.out + (a.dense ? (long long)je * (g.nx + 1) + i : kn));
       if (own) out[c] = act ? kv : 0.0;
     } else if constexpr (MODE == MODE_RESID) {
@@ -632,22 +763,20 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsplit_kernel(const SweepParams<d
         reinterpret_cast<double*>(a.out + kn)[c] = r;
         if (a.out32 != nullptr) reinterpret_cast<float*>(a.out32 + kn)[c] = float(r);
       }
-      dot0 = r * r;
+      sums.dot0 = r * r;
     } else if constexpr (MODE == MODE_KP) {
       const double q = act ? kv : 0.0;
       if (own) {
         reinterpret_cast<double*>(a.p_out + kn)[c] = vc;
         reinterpret_cast<double*>(a.out + kn)[c] = q;
-        dot0 = vc * q;
-        const double2 old = half ? lo.v : hi.v;
-        if (lag) reinterpret_cast<double*>(a.xvec + kn)[c] = fma(alag, c ? old.y : old.x, x);
+        sums.dot0 = vc * q;
       }
     } else if constexpr (F::SMOOTHING) {
       const double z = act ? fma(d, b - kv, vc) : 0.0;
       if (own) reinterpret_cast<double*>(a.out + kn)[c] = z;
       if constexpr (DOT) {
-        dot0 = z * rd;
-        if (a.qdot != nullptr) dot1 = z * qd;
+        sums.dot0 = z * rd;
+        if (a.qdot != nullptr) sums.dot1 = z * qd;
       }
     } else if constexpr (RESTRICT) {
       res = act ? b - kv : 0.0;
@@ -666,7 +795,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsplit_kernel(const SweepParams<d
     }
   }
   if constexpr (REDUCE)
-    block_reduce_finish<SWEEP_NT, DOT>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
+    block_reduce_finish<SWEEP_NT, DOT>(sums.dot0, sums.dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
 }
 
 }  // namespace mto

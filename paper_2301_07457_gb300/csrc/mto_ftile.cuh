@@ -6,10 +6,16 @@
 // The tiles, stages and halos are those of mto_tile.cuh, the arithmetic is that
 // of mto_fsweep.cuh: one thread per element or node, the marched values and the
 // corner forces of the elements as 96-bit integers in shared memory, one scale
-// per tile and stage.  Against two launches of the row-per-warp kernel a pass
-// saves a launch and a trip through memory (a coarse level 10.4 -> 9.6 us, the
-// finest 256^2 one with its dot products 25 -> 22 us; a float64 PCG iteration
-// 114 -> 108 us at 256^2, 391 -> 375 us at 1024^2).
+// per tile and stage.  A tile whose scales do not hold the terms of one of its
+// elements (fx_beyond in mto_fixed.cuh) is done again in float64, by the same
+// stages on DTile in the same shared memory.
+//
+// Against two launches of the row-per-warp kernel a pass saves a launch and a
+// trip through memory (a coarse level 10.4 -> 9.6 us, the finest 256^2 one with
+// its dot products 25 -> 22 us; a float64 PCG iteration 114 -> 108 us at 256^2,
+// 391 -> 375 us at 1024^2).  Both stages run the same copy of the operator's code:
+// a block executes it once each, and fetching it is a good part of the kernel's
+// time (a float64 iteration 57.9 -> 54.0 us at 64^2, 105.3 -> 99.7 us at 256^2).
 #pragma once
 
 #include "mto_fsweep.cuh"
@@ -31,26 +37,25 @@ template <int N> struct FxArray {
 
 // One operator evaluation per stage over a tile of NW x NH nodes.
 template <int SRC, int NW, int NH> struct FTile {
+  static constexpr bool FIXED = true;
   static constexpr int N = NW * NH, EW = NW - 1, EH = NH - 1, NE = EW * EH;
   FxArray<N> vx, vy;             // nodal values at the stage's scale
   FxArray<NE> fx[4], fy[4];      // forces of element e on its corners BL, BR, TR, TL
   int B[2], X;                   // scales: nodal values of the two stages, coefficients
-  int any_bad, any_rare;
-  unsigned char bad[N];          // non-finite nodal values (taken as zero)
+  int lost;                      // an element's terms lie beyond the scales, or are not finite
+  unsigned mag[N];               // magnitudes of the nodal values
 
-  __device__ __forceinline__ static int exponent(const double2& v) {
-    return max(fx_exponent((unsigned)__double2hiint(v.x)), fx_exponent((unsigned)__double2hiint(v.y)));
-  }
+  __device__ __forceinline__ static int exponent(const double2& v) { return (int)(fx_magnitude(v.x, v.y) >> 20); }
   // All threads, before the first raise() (with a barrier between).
   __device__ __forceinline__ void init() {
     if (threadIdx.x < 2) B[threadIdx.x] = 1;
     if (threadIdx.x == 2) X = 0;
-    if (threadIdx.x == 3) any_bad = any_rare = 0;
+    if (threadIdx.x == 3) lost = 0;
   }
   // Raises the scale of stage s to the exponent e of a thread's value (0: none).
   __device__ __forceinline__ void raise(int s, int e) {
     if (e == 0x7ff) {
-      any_bad = 1;
+      lost = 1;
       e = 0;
     }
     const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
@@ -62,17 +67,20 @@ template <int SRC, int NW, int NH> struct FTile {
   }
   // Node n gets value v at the scale of stage s (whole warps).
   __device__ __forceinline__ void put(int s, int n, bool in, double2 v) {
-    const bool bd = exponent(v) == 0x7ff;
-    if (bd) v = make_double2(0.0, 0.0);
+    const unsigned m = fx_magnitude(v.x, v.y);
+    if ((m >> 20) == 0x7ffu) v = make_double2(0.0, 0.0);
     const Fx2 f = fx2_from(v, B[s]);
     if (!in) return;
+    mag[n] = m;
     vx.put(n, f.x);
     vy.put(n, f.y);
-    bad[n] = bd;
   }
-  // Forces of the thread's element e, whose BL node is c; tag, k: its factors.
-  __device__ __forceinline__ void element(const SweepParams<double>& a, int e, int c, unsigned tag,
+  // Forces of the thread's element e at stage s, whose BL node is c; tag, k: its factors.
+  __device__ __forceinline__ void element(const SweepParams<double>& a, int s, int e, int c, unsigned tag,
                                           const unsigned long long* k, bool rare) {
+    const unsigned m = max(max(mag[c], mag[c + 1]), max(mag[c + NW], mag[c + NW + 1]));
+    const int x = (int)(tag & 0x7ffu);
+    if (x == 0x7ff || (m != 0u && tag != 0u && fx_beyond(B[s] + X, (int)(m >> 20) + x))) lost = 1;
     const Fx2 bl = {vx.get(c), vy.get(c)}, br = {vx.get(c + 1), vy.get(c + 1)};
     const Fx2 tl = {vx.get(c + NW), vy.get(c + NW)}, tr = {vx.get(c + NW + 1), vy.get(c + NW + 1)};
     const Fx2 ac = fsub(br, bl), bt = fsub(tr, tl), up = fsub(fadd(tr, tl), fadd(br, bl));
@@ -103,13 +111,41 @@ template <int SRC, int NW, int NH> struct FTile {
     double2 kv = make_double2(fx_to_double<false>(x, unit), fx_to_double<false>(y, unit));
     if (unit < FX_UNIT_MIN || unit > FX_UNIT_MAX)  // uniform over the block
       kv = make_double2(fx_to_double(x, unit), fx_to_double(y, unit));
-    if (any_bad || X == 0x7ff) {
-      bool near = X == 0x7ff;
-      for (int dy = -NW; dy <= NW; dy += NW)
-        for (int dx = -1; dx <= 1; ++dx) near = near || bad[n + dy + dx];
-      if (near) kv = make_double2(NAN, NAN);
-    }
     return kv;
+  }
+};
+
+// The same in float64.
+template <int SRC, int NW, int NH> struct DTile {
+  static constexpr bool FIXED = false;
+  static constexpr int N = NW * NH, EW = NW - 1, EH = NH - 1, NE = EW * EH;
+  double vx[N], vy[N], fx[4][NE], fy[4][NE];
+  static constexpr int X = 0, lost = 0;
+
+  __device__ __forceinline__ static int exponent(const double2&) { return 0; }
+  __device__ __forceinline__ void init() {}
+  __device__ __forceinline__ void raise(int, int) {}
+  __device__ __forceinline__ void raise_elements(unsigned) {}
+  __device__ __forceinline__ void put(int, int n, bool in, double2 v) {
+    if (!in) return;
+    vx[n] = v.x;
+    vy[n] = v.y;
+  }
+  __device__ __forceinline__ double2 get(int n) const { return make_double2(vx[n], vy[n]); }
+  __device__ __forceinline__ void element(const SweepParams<double>& a, int, int e, int c, unsigned,
+                                          const unsigned long long* k, bool) {
+    const Strain<double> w = strain_coords<double, double2>(get(c), get(c + 1), get(c + NW + 1), get(c + NW));
+    double2 f[4];
+    strain_forces<double, double2>(FxElem<SRC>::core64(a, w, k), f[0], f[1], f[2], f[3]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      fx[q][e] = f[q].x;
+      fy[q][e] = f[q].y;
+    }
+  }
+  __device__ __forceinline__ double2 at_node(int, int, int e) const {
+    return make_double2((fx[0][e] + fx[1][e - 1]) + (fx[2][e - EW - 1] + fx[3][e - EW]),
+                        (fy[0][e] + fy[1][e - 1]) + (fy[2][e - EW - 1] + fy[3][e - EW]));
   }
 };
 
@@ -139,12 +175,13 @@ template <int SRC> __device__ __forceinline__ double2 ftile_d(const SweepParams<
   }
 }
 
-template <int SRC> __global__ void __launch_bounds__(SWEEP_NT, 2) ftile_pre2_kernel(const SweepParams<double> a) {
-  pdl_trigger();
-  constexpr int NW = TILE_X + 5, NH = TILE_Y + 5, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
+constexpr int PRE2_W = TILE_X + 5, PRE2_H = TILE_Y + 5, POST2_W = TILE_X + 4, POST2_H = TILE_Y + 4;
+
+// A tile of PRE2.  False: its scales do not hold it (uniform over the block).
+template <int SRC, typename Tile>
+__device__ __forceinline__ bool pre2_tile(const SweepParams<double>& a, Tile& f, double2* r) {
+  constexpr int NW = PRE2_W, NH = PRE2_H, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
   static_assert(EW * EH <= SWEEP_NT && ZW * ZH <= SWEEP_NT && NW * NH <= 2 * SWEEP_NT, "threads");
-  __shared__ FTile<SRC, NW, NH> f;
-  __shared__ double2 r[ZW * ZH];
   const Grid g = a.g, gc = a.gc;
   const int t = threadIdx.x;
   f.init();
@@ -175,7 +212,7 @@ template <int SRC> __global__ void __launch_bounds__(SWEEP_NT, 2) ftile_pre2_ker
     const int n = t + u * SWEEP_NT, ii = x0 + n % NW, jj = y0 + n / NW;
     bh[u] = n < NW * NH && g.valid(ii, jj) ? a.b[g.at(ii, jj)] : zero2;
   }
-  if (done) return;  // uniform over the grid
+  if (done) return true;  // uniform over the grid
 #pragma unroll
   for (int u = 0; u < 2; ++u) z0[u] = make_double2(z0[u].x * bh[u].x, z0[u].y * bh[u].y);
   __syncthreads();
@@ -187,34 +224,30 @@ template <int SRC> __global__ void __launch_bounds__(SWEEP_NT, 2) ftile_pre2_ker
   if (t < ((NW * NH - SWEEP_NT + 31) / 32) * 32) f.put(0, t + SWEEP_NT, t + SWEEP_NT < NW * NH, z0[1]);
   const bool rare = er.rare(f.X);
   __syncthreads();
-  // z1 = z0 + w/D (b - K z0).
+  // Stage 0: z1 = z0 + w/D (b - K z0); stage 1: the residual.
   const int c = ey * NW + ex;
-  if (elem) f.element(a, t, c, er.tag, er.k, rare);
-  __syncthreads();
   const int zn = zy * NW + zx, en = zy * EW + zx;  // node and its upper right element
-  double2 z1 = zero2;
-  if (node) {
-    const double2 kv = f.at_node(0, zn, en);
-    z1 = make_double2(fma(d.x, b.x - kv.x, d.x * b.x), fma(d.y, b.y - kv.y, d.y * b.y));
-    if (!g.active(i, j)) z1 = zero2;
+  const bool act = node && g.active(i, j);
+  const bool inner = node && zx >= 2 && zx < NW - 2 && zy >= 2 && zy < NH - 2;
+  const bool inner_elem = elem && ex >= 1 && ex < EW - 1 && ey >= 1 && ey < EH - 1;
+  double2 kv = zero2;
+#pragma unroll 1
+  for (int s = 0;; ++s) {
+    if (s == 0 ? elem : inner_elem) f.element(a, s, t, c, er.tag, er.k, rare);
+    __syncthreads();
+    if (s == 0 ? act : inner && act) kv = f.at_node(s, zn, en);
+    if (s == 1) break;
+    double2 z1 = zero2;
+    if (act) z1 = make_double2(fma(d.x, b.x - kv.x, d.x * b.x), fma(d.y, b.y - kv.y, d.y * b.y));
     if (valid && zx >= 3 && zx < 3 + TILE_X && zy >= 3 && zy < 3 + TILE_Y) a.out[g.at(i, j)] = z1;
+    f.raise(1, f.exponent(z1));
+    __syncthreads();
+    f.put(1, zn, node, z1);
+    __syncthreads();
   }
-  f.raise(1, f.exponent(z1));
+  if (inner) r[t] = act ? make_double2(b.x - kv.x, b.y - kv.y) : zero2;
   __syncthreads();
-  f.put(1, zn, node, z1);
-  __syncthreads();
-  // Residual.
-  if (elem && ex >= 1 && ex < EW - 1 && ey >= 1 && ey < EH - 1) f.element(a, t, c, er.tag, er.k, rare);
-  __syncthreads();
-  if (node && zx >= 2 && zx < NW - 2 && zy >= 2 && zy < NH - 2) {
-    double2 res = zero2;
-    if (g.active(i, j)) {
-      const double2 kv = f.at_node(1, zn, en);
-      res = make_double2(b.x - kv.x, b.y - kv.y);
-    }
-    r[t] = res;
-  }
-  __syncthreads();
+  if (f.lost) return false;
   // Full weighting, over the three rows of each column first; one component per thread.
   if (t < 2 * TILE_CX * TILE_CY) {
     const int cc = t & 1, p = (t >> 1) % TILE_CX, q = (t >> 1) / TILE_CX, I = I0 + p, J = J0 + q;
@@ -226,14 +259,38 @@ template <int SRC> __global__ void __launch_bounds__(SWEEP_NT, 2) ftile_pre2_ker
       reinterpret_cast<double*>(a.bc + gc.at(I, J))[cc] = gc.is_fixed(I, J) ? 0.0 : val;
     }
   }
+  return true;
 }
 
-template <int SRC, bool DOT>
-__global__ void __launch_bounds__(SWEEP_NT, 2) ftile_post2_kernel(const SweepParams<double> a) {
+// Shared memory of a tile, of whichever kind is running.
+template <typename F, typename D> union TileMemory {
+  F fixed;
+  D wide;
+};
+
+template <int SRC>
+__device__ __noinline__ void pre2_tile_f64(const SweepParams<double>& a, DTile<SRC, PRE2_W, PRE2_H>& f, double2* r) {
+  pre2_tile<SRC>(a, f, r);
+}
+
+// Blocks per SM that the fixed-point path's registers allow.
+template <int SRC>
+__global__ void __launch_bounds__(SWEEP_NT, SRC == SRC_FINE64 ? 4 : 2)
+    ftile_pre2_kernel(const __grid_constant__ SweepParams<double> a) {
   pdl_trigger();
-  constexpr int NW = TILE_X + 4, NH = TILE_Y + 4, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
+  __shared__ TileMemory<FTile<SRC, PRE2_W, PRE2_H>, DTile<SRC, PRE2_W, PRE2_H>> m;
+  __shared__ double2 r[(PRE2_W - 2) * (PRE2_H - 2)];
+  if (pre2_tile<SRC>(a, m.fixed, r)) return;
+  __syncthreads();  // every thread has read `lost`
+  pre2_tile_f64<SRC>(a, m.wide, r);
+}
+
+// A tile of POST2, its dot products in dots.
+enum TileResult { TILE_OK, TILE_LOST, TILE_STOPPED };
+template <int SRC, bool DOT, typename Tile>
+__device__ __forceinline__ TileResult post2_tile(const SweepParams<double>& a, Tile& f, double2* zs, double2& dots) {
+  constexpr int NW = POST2_W, NH = POST2_H, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
   static_assert(EW * EH <= SWEEP_NT && NW * NH <= SWEEP_NT, "threads");
-  __shared__ FTile<SRC, NW, NH> f;
   const Grid g = a.g, gc = a.gc;
   const int t = threadIdx.x;
   f.init();
@@ -277,7 +334,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) ftile_post2_kernel(const SweepPar
       v = make_double2(fma(w, t0.x + t1.x, v.x), fma(w, t0.y + t1.y, v.y));
     }
   }
-  if (done) return;  // uniform over the grid
+  if (done) return TILE_STOPPED;  // uniform over the grid
   __syncthreads();
   f.raise(0, f.exponent(v));
   f.raise_elements(er.tag);
@@ -285,39 +342,62 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) ftile_post2_kernel(const SweepPar
   f.put(0, t, t < NW * NH, v);
   const bool rare = er.rare(f.X);
   // The value at the thread's own z2 node, by way of shared memory.
-  __shared__ double2 zs[NW * NH];
   if (t < NW * NH) zs[t] = v;
   __syncthreads();
   const int c = ey * NW + ex;
-  if (elem) f.element(a, t, c, er.tag, er.k, rare);
-  __syncthreads();
   const int zn = zy * NW + zx, en = zy * EW + zx;
-  double2 z2 = zero2;
-  if (node && g.active(i, j)) {
-    const double2 kv = f.at_node(0, zn, en), z = zs[zn];
-    z2 = make_double2(fma(d.x, b.x - kv.x, z.x), fma(d.y, b.y - kv.y, z.y));
+  const bool act = node && g.active(i, j);
+  const bool inner_elem = elem && ex >= 1 && ex < EW - 1 && ey >= 1 && ey < EH - 1;
+  double2 z = act ? zs[zn] : zero2;
+#pragma unroll 1
+  for (int s = 0; s < 2; ++s) {
+    if (s == 0 ? elem : inner_elem) f.element(a, s, t, c, er.tag, er.k, rare);
+    __syncthreads();
+    if (s == 0 ? act : own && act) {
+      const double2 kv = f.at_node(s, zn, en);
+      z = make_double2(fma(d.x, b.x - kv.x, z.x), fma(d.y, b.y - kv.y, z.y));
+    }
+    if (s == 1) break;
+    f.raise(1, f.exponent(z));
+    __syncthreads();
+    f.put(1, zn, node, z);
+    __syncthreads();
   }
-  f.raise(1, f.exponent(z2));
-  __syncthreads();
-  f.put(1, zn, node, z2);
-  __syncthreads();
-  if (elem && ex >= 1 && ex < EW - 1 && ey >= 1 && ey < EH - 1) f.element(a, t, c, er.tag, er.k, rare);
-  __syncthreads();
-  double dot0 = 0.0, dot1 = 0.0;
+  dots = zero2;
+  if (f.lost) return TILE_LOST;  // uniform over the block
   if (own) {
-    double2 z3 = zero2;
-    if (g.active(i, j)) {
-      const double2 kv = f.at_node(1, zn, en);
-      z3 = make_double2(fma(d.x, b.x - kv.x, z2.x), fma(d.y, b.y - kv.y, z2.y));
-    }
-    a.out[k] = z3;
+    a.out[k] = z;
     if constexpr (DOT) {
-      dot0 = fma(z3.x, rd.x, z3.y * rd.y);
-      if (a.qdot != nullptr) dot1 = fma(z3.x, qd.x, z3.y * qd.y);
+      dots.x = fma(z.x, rd.x, z.y * rd.y);
+      if (a.qdot != nullptr) dots.y = fma(z.x, qd.x, z.y * qd.y);
     }
+  }
+  return TILE_OK;
+}
+
+template <int SRC, bool DOT>
+__device__ __noinline__ double2 post2_tile_f64(const SweepParams<double>& a, DTile<SRC, POST2_W, POST2_H>& f,
+                                               double2* zs) {
+  double2 dots;
+  post2_tile<SRC, DOT>(a, f, zs, dots);
+  return dots;
+}
+
+template <int SRC, bool DOT>
+__global__ void __launch_bounds__(SWEEP_NT, SRC == SRC_FINE64 ? (DOT ? 3 : 4) : 2)
+    ftile_post2_kernel(const __grid_constant__ SweepParams<double> a) {
+  pdl_trigger();
+  __shared__ TileMemory<FTile<SRC, POST2_W, POST2_H>, DTile<SRC, POST2_W, POST2_H>> m;
+  __shared__ double2 zs[POST2_W * POST2_H];
+  double2 dots;
+  const TileResult res = post2_tile<SRC, DOT>(a, m.fixed, zs, dots);
+  if (res == TILE_STOPPED) return;
+  if (res == TILE_LOST) {
+    __syncthreads();  // every thread has read `lost`
+    dots = post2_tile_f64<SRC, DOT>(a, m.wide, zs);
   }
   if constexpr (DOT)
-    block_reduce_finish<SWEEP_NT>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
+    block_reduce_finish<SWEEP_NT>(dots.x, dots.y, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
 }
 
 }  // namespace mto
