@@ -145,7 +145,8 @@ template <typename T, int SRC, int MODE, bool DOT, typename ZT> struct Sweep2 {
     } else if constexpr (MODE == MODE_SMOOTH0) {
       if constexpr (SRC == SRC_FINEBF && DOT) {  // the CG update forms b from r and q
         ld_pair(lag ? a.r64_prev : static_cast<const double2*>(a.r64), k, r.r0, r.r1);
-        ld_pair(a.q64, k, r.q0, r.q1);
+        r.q0 = r.q1 = make_double2(0.0, 0.0);
+        if (lag) ld_pair(a.q64, k, r.q0, r.q1);  // else q is a leftover, perhaps not finite
       } else if constexpr (SRC == SRC_FINEBF) {  // the caller's vector: clamped nodes are read as zero
         const Grid& g = a.g;
         const double2* row = a.din + (long long)jj * (g.nx + 1);

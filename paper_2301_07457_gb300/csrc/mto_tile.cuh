@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(SWEEP_NT) tile_pre2_kernel(const SweepParams<f
       if constexpr (DOT) {
         if (n < NW * NH && g.valid(ii, jj)) {
           rv[u] = upd ? a.r64_prev[g.at(ii, jj)] : static_cast<const double2*>(a.r64)[g.at(ii, jj)];
-          qv[u] = a.q64[g.at(ii, jj)];
+          if (upd) qv[u] = a.q64[g.at(ii, jj)];  // else q is a leftover, perhaps not finite
         }
       } else {
         if (n < NW * NH && g.active(ii, jj)) rv[u] = a.din[(long long)jj * (g.nx + 1) + ii];
