@@ -255,13 +255,12 @@ __host__ __device__ __forceinline__ unsigned fx_tag(const unsigned long long* w)
   return ((unsigned)w[0] & 15u) | (((unsigned)w[1] & 15u) << 4) | (((unsigned)w[2] & 15u) << 8);
 }
 
-// Factor c 2^(X - bias) of an element with tag `tag`.
-__host__ __device__ __forceinline__ double fx_factor(unsigned long long c, unsigned tag, int bias) {
-#ifdef __CUDA_ARCH__
-  return ldexp((double)c, (int)(tag & 0x7ffu) - bias);
-#else
-  return __builtin_ldexp((double)c, (int)(tag & 0x7ffu) - bias);
-#endif
+// Factor c 2^(X - bias) of an element with tag `tag`, NaN where the element is
+// not finite (formed on the integer pipe).
+__host__ __device__ __forceinline__ double fx_factor(unsigned long long c, bool neg, unsigned tag, int bias) {
+  const int X = (int)(tag & 0x7ffu);
+  const double f = fx_to_double(Fx{(unsigned)c, (unsigned)(c >> 32), 0}, X - bias);
+  return double_of(X == 0x7ff ? 0x7ff8000000000000ull : bits_of(f) | (neg ? 0x8000000000000000ull : 0ull));
 }
 
 // Upper word of the larger magnitude of a pair.

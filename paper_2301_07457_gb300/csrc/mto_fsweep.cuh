@@ -38,8 +38,10 @@
 // the task to float64 too, and so reaches the nodes next to it alone.  Normal
 // work hardly ever gets there (designs with a void of 1e-9, 64^2 to 1024^2: no
 // marching row that was counted, up to 1% of the tiles); with a void of 1e-12 in
-// half of a smooth design an iteration takes 169 instead of 104 us at 256^2 and
-// 442 instead of 371 us at 1024^2 (278 and 992 us where all was in float64).
+// half of a smooth design an iteration takes 160 instead of 104 us at 256^2 and
+// 433 instead of 371 us at 1024^2 (278 and 992 us where all was in float64), and
+// with factors some 2^-60 apart everywhere the operator at 2048^2 takes 407 us and a
+// V-cycle 2.61 ms (318 us and 2.41 ms).
 #pragma once
 
 #include "mto_fixed.cuh"
@@ -102,9 +104,11 @@ template <> struct FxElem<SRC_FINE64> {
   __device__ __forceinline__ static Strain<double> core64(const SweepParams<double>&, const Strain<double>& w,
                                                           const unsigned long long* k) {
     const unsigned tag = fx_tag(k);
-    const double P = fx_factor(k[0], tag, 1083), C = fx_factor(k[1], tag, 1083), G = fx_factor(k[2], tag, 1083);
-    const double p = P * (w.c1 + w.d2), g = G * (w.c1 - w.d2), sg = tag & FX_TAG_NEG ? -1.0 : 1.0;
-    return {sg * (p + g), sg * (C * w.c3), sg * (p - g), sg * (C * w.d3), sg * (G * w.s)};
+    const bool neg = tag & FX_TAG_NEG;
+    const double P = fx_factor(k[0], neg, tag, 1083), C = fx_factor(k[1], neg, tag, 1083),
+                 G = fx_factor(k[2], neg, tag, 1083);
+    const double p = P * (w.c1 + w.d2), g = G * (w.c1 - w.d2);
+    return {p + g, C * w.c3, p - g, C * w.d3, G * w.s};
   }
 };
 template <> struct FxElem<SRC_COARSE> {
@@ -158,10 +162,7 @@ template <> struct FxElem<SRC_COARSE> {
     const unsigned tag = fx_tag(k);
     double f[FX_NCOARSE];
 #pragma unroll
-    for (int n = 0; n < FX_NCOARSE; ++n) {
-      const double m = fx_factor(k[n] & 0x7fffffffffffffffull, tag, 1081);
-      f[n] = (k[n] >> 63) ? -m : m;
-    }
+    for (int n = 0; n < FX_NCOARSE; ++n) f[n] = fx_factor(k[n] & 0x7fffffffffffffffull, k[n] >> 63, tag, 1081);
     const double g = ldexp((double)a.gfix, -64), nu = 1.0 - 2.0 * g;
     const double m0 = f[FXC_M00], m1 = f[FXC_M10], m2 = f[FXC_M01], k9 = f[FXC_C3D3];
     Strain<double> t;
@@ -359,7 +360,7 @@ __device__ __noinline__ FSums rows_f64(const SweepParams<double>& a, FTask t0, i
   long long k = g.at(t0.i, je0);
   typename F::Pack cur;
   F::load_top(a, k, t0.i, je0, lag, cur);
-  double2 vb = F::value(a, cur, t0.i, je0, beta, lag, alag), below = zero2, bc = zero2, dc = zero2, kv = zero2;
+  double2 vb = F::value(a, cur, t0.i, je0, beta, lag, alag), gbp = zero2, gsp = zero2, bc = zero2, dc = zero2, kv = zero2;
   if constexpr (MODE == MODE_SMOOTH0) {
     bc = cur.v;
     dc = cur.dt;
@@ -377,16 +378,17 @@ __device__ __noinline__ FSums rows_f64(const SweepParams<double>& a, FTask t0, i
     w.d3 = bt.y - ac.y;
     w.s = up.x + (ac.y + bt.y);
     const Strain<double> t = F::Elem::core64(a, w, cur.k);
-    // Forces of the element row on the nodes of its bottom and of its top edge.
-    auto edge = [&](double2 h, double2 v) { return add2(shfl_up2(add2(v, h)), sub2(v, h)); };
-    kv = add2(below, edge(make_double2(t.c1 - t.c3, t.s - t.d3), make_double2(-t.s, -t.d2)));
+    // Edge forces and node row je, as in the fixed-point loop.
+    const double2 gh = add2(make_double2(t.c1 - t.c3, t.s - t.d3), gbp), gd = sub2(gsp, make_double2(t.s, t.d2));
+    kv = add2(shfl_up2(add2(gd, gh)), sub2(gd, gh));
     if constexpr (FINISH) {
       const bool inb = je > je0 && t0.own_col && je >= 0 && je <= g.ny;
       const bool act = inb && !g.is_fixed(t0.i, je);
       const double2 b = MODE == MODE_SMOOTH0 ? bc : cur.b, d = MODE == MODE_SMOOTH0 ? dc : cur.d;
       F::finish_row(a, t0, k, je, inb, act, vb, kv, b, d, cur, sums);
     }
-    below = edge(make_double2(t.c1 + t.c3, t.s + t.d3), make_double2(t.s, t.d2));
+    gbp = make_double2(t.c1 + t.c3, t.s + t.d3);
+    gsp = make_double2(t.s, t.d2);
     vb = vt;
     if constexpr (MODE == MODE_SMOOTH0) {
       bc = cur.v;
