@@ -74,8 +74,14 @@ cudaError_t launch_sweep(int src, int mode, bool dot, bool zfloat, SweepParams<T
 // Whether the two-stage passes PRE2 / POST2 of a float64 level run by tiles
 // (mto_ftile.cuh; its sweeps run one by one otherwise): at most
 // FTILES_PER_SM tiles per SM, and no launch shape that asks for marching tasks
-// (below one warp per SM).
-constexpr int FTILES_PER_SM = 4;
+// (below one warp per SM).  A float64 iteration without any tiles / with them:
+// 56.5 / 53.2 us at 64^2 (0.3 tiles per SM on the finest grid), 114 / 100 at 256^2
+// (3.7), 120 / 110 at 288^2 (4.6), 131 / 115 at 320^2 (5.7; with the limit at 4, which
+// leaves the finest grid out, 124); a solve at 352^2 (6.8) 3.84 ms with the limit at 4,
+// 3.60 here.  Beyond it: 384^2 (8.1) 3.77 ms, with its finest grid tiled 3.82;
+// 416^2 (9.6) 4.10 and 4.36; 512^2 (14.1) 4.87 and 5.53.  Two load cases at
+// 320^2 5.68 -> 5.55 ms.
+constexpr int FTILES_PER_SM = 8;
 bool float64_tiles(const Grid& g, int target_warps, int num_sms);
 // The same for a float32 level (mto_tile.cuh).  Coarse levels: at most
 // TILES_PER_SM tiles per SM: one V-cycle takes 60 -> 41 us at 256^2, 110 -> 90 us
