@@ -88,6 +88,8 @@ template <typename P> mto_status dalloc_t(mto_ctx* c, P** out, size_t count) {
 mto_status enter(mto_ctx* c) {
   CK(cudaSetDevice(c->device));
   CK(cudaEventRecord(c->ev_in, c->user_stream));
+  // Orders the caller's work, and the design data of an earlier call that a
+  // call's first kernel may load early (launch_pdl).
   CK(cudaStreamWaitEvent(c->stream, c->ev_in, 0));
   c->cs = c->stream;
   return MTO_OK;
@@ -703,7 +705,7 @@ mto_status enqueue_hierarchy(mto_ctx* c) {
   // run on a side stream while this one prepares the smoothers and the
   // element data of the other levels, which they do not depend on.
   LevelBuf& B0 = c->lv[0];
-  KL(launch_coefs<double>(B0.g, B0.mom, c->nu, B0.coef64, c->cs, c->num_sms));
+  KL(launch_coefs(B0.g, B0.mom, c->nu, B0.coef64, c->cs, c->num_sms));
   CK(cudaMemsetAsync(c->Kd, 0, sizeof(double) * c->n0 * (c->bw0 + 1), c->cs));
   CK(cudaMemsetAsync(c->err_flag, 0, sizeof(int), c->cs));
   KL(launch_band_assemble(B0.g, B0.coef64, c->dof_index, c->n0, c->bw0, c->Kd, c->cs));
@@ -734,6 +736,7 @@ mto_status enqueue_hierarchy(mto_ctx* c) {
   }
   // The coarsest level's factors (apply_operator).
   KL(launch_fx_coefs(B0.g, B0.mom, c->nu, B0.fx, c->cs, c->num_sms));
+  // Also what the kernels that load design data early rely on (launch_pdl).
   CK(cudaStreamWaitEvent(c->cs, c->ev_join, 0));
   return MTO_OK;
 }

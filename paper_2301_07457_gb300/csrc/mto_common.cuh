@@ -63,17 +63,22 @@ inline Grid make_grid(int nx, int ny, unsigned fixed) {
 
 // Programmatic dependent launch.  The kernels of the PCG iteration are
 // launched with launch_pdl (mto_launch.h): the next kernel on the stream may
-// be scheduled while this one runs, and each of them calls pdl_wait() before
-// its first global memory access, which returns once the previous grid has
+// be scheduled while this one runs, and each of them waits, before it touches
+// anything that a kernel of the chain writes, until the previous grid has
 // completed and its writes are visible.  The early trigger lets the next
 // kernel's blocks take SM slots as this kernel's blocks retire, which hides
-// the launch latency between the many short kernels of a V-cycle.
+// the launch latency between the many short kernels of a V-cycle.  pdl_wait()
+// triggers and waits at once; most kernels begin with it.  The tiles of the
+// bf16 finest level never trigger (mto_tile.cuh).
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
 }
 
-// The same in two parts, for kernels that first load what no kernel of the
-// chain writes (design data).
+// The same in two parts, for the kernels that first load design data (moduli,
+// factors, diagonals, K_0^-1: fsplit, the tiles, the coarsest GEMV).  A kernel
+// that triggers before it waits does not order such loads of the next kernel
+// behind its own predecessor, so design data must be complete before the
+// last ordinary launch or event wait in front of the chain: see launch_pdl.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

@@ -19,9 +19,16 @@ namespace mto {
 // problems' concurrent branches.
 extern thread_local bool g_pdl;
 
-// Launch a kernel that calls pdl_wait() first, allowing programmatic
-// dependent launch after the previous kernel on the stream (captured into
-// graphs as a programmatic edge) while g_pdl is set.
+// Launch a kernel that waits for the previous one (mto_common.cuh), allowing
+// programmatic dependent launch after the previous kernel on the stream
+// (captured into graphs as a programmatic edge) while g_pdl is set.
+//
+// Some of these kernels load design data before that wait.  What holds these
+// loads back is the last ordinary launch, event wait or graph launch on the
+// stream before the chain: every kernel that writes design data is in front of
+// one (enqueue_hierarchy ends with an event wait, enter() begins each call with
+// one).  A set-up kernel turned into launch_pdl, or one of those waits left out,
+// would make the early loads a race.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t s,
                        Args&&... args) {
@@ -54,16 +61,10 @@ struct SweepShape {
 };
 SweepShape sweep_shape(const Grid& g, int mode, int target_warps, int cols, int spread = 0);
 
-// Node columns per lane of the instantiation that launch_sweep uses for a
-// float64 (f64) or float32 sweep of source src in mode `mode`.  Two for every
-// float32 sweep (issue- and latency-bound), one for the float64 sweeps, where
-// a pair of elements (13 float64 coefficients each on coarse levels, 96-bit
-// values on the finest) needs too many registers.
-constexpr int sweep_cols_of(bool f64, int src, int mode) {
-  (void)src;
-  (void)mode;
-  return f64 ? 1 : 2;
-}
+// Node columns per lane: two in the float32 sweeps (issue- and latency-bound),
+// one in the float64 sweeps, where the 96-bit values and the factors of a pair
+// of elements need too many registers.
+constexpr int SWEEP_COLS_F32 = 2, SWEEP_COLS_F64 = 1;
 
 // Launch one sweep over p.g; the launch shape follows from target_warps
 // (0: one full wave of the kernel on num_sms SMs).
@@ -188,8 +189,7 @@ cudaError_t launch_moments_from_fine(const Grid& gc, const Grid& gf, const doubl
 // Moments of level l-1 from those of level l.
 cudaError_t launch_moments_from_coarse(const Grid& gc, const Grid& gf, const double* momf,
                                        int rediscretize, double* momc, cudaStream_t s, int num_sms);
-template <typename T>
-cudaError_t launch_coefs(const Grid& g, const double* mom, double nu, T* coef, cudaStream_t s,
+cudaError_t launch_coefs(const Grid& g, const double* mom, double nu, double* coef, cudaStream_t s,
                          int num_sms);
 // Fixed-point factors (FX_NCOARSE arrays of g.size() words) of a float64 coarse level.
 cudaError_t launch_fx_coefs(const Grid& g, const double* mom, double nu, unsigned long long* out,

@@ -14,8 +14,9 @@
 // solved by one thread-block cluster of C CTAs (C = 1 for small meshes, up to
 // 16): the CTAs own blocks of node rows of every large level and separate
 // dependent phases with the hardware cluster barrier; scalar reductions are
-// all-gathered through distributed shared memory and summed in rank order,
-// so every CTA holds the same scalars and takes the same branches.  Levels
+// all-gathered through distributed shared memory and summed by the same tree of
+// lanes in every CTA, so every CTA holds the same scalars and takes the same
+// branches.  Levels
 // with at most LOCAL_MAX_NODES (256) interior nodes (and the coarsest solve)
 // run inside CTA 0 alone with block barriers, on vectors in its shared memory
 // (2-3% of a solve up to 128^2); the other vectors live in global memory
@@ -664,7 +665,9 @@ template <typename VT, bool MANY> struct Solver {
 // thread) and run while the others wait; the arithmetic and its order are the
 // same.  64 right-hand sides at 256^2: 12.2 -> 6.8 ms (float64 V-cycle), 10.4 ->
 // 4.0 ms (float32); two to a SM took 8.7 and 6.7 ms, three 7.7 and 5.5, six 6.9
-// and 4.2 (spills).
+// and 4.2.  At 64 registers the float32 kernel spills (812 bytes stored, 968
+// loaded per thread, the float64 one 16 and 40) and is still the faster choice;
+// of the kernels with 255 registers only the float64 one does (84 and 144).
 template <typename VT, bool MANY>
 __global__ void __launch_bounds__(PNT, MANY ? 4 : 1) poisson_cluster_kernel(const PDesc* __restrict__ descs, int C) {
   __shared__ PDesc sd;

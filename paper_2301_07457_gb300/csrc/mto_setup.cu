@@ -137,8 +137,7 @@ __global__ void moments_from_coarse_kernel(Grid gc, Grid gf, const double* __res
   }
 }
 
-template <typename T>
-__global__ void coefs_kernel(Grid g, const double* __restrict__ mom, double nu, T* __restrict__ coef) {
+__global__ void coefs_kernel(Grid g, const double* __restrict__ mom, double nu, double* __restrict__ coef) {
   const long long n = (long long)g.nx * g.ny;
   const long long s = g.size();
   const double kap = 1.0 / (4.0 * (1.0 - nu * nu)), gs = 0.5 * (1.0 - nu);
@@ -154,7 +153,7 @@ __global__ void coefs_kernel(Grid g, const double* __restrict__ mom, double nu, 
                              kap * (nu + gs) * M11, kap * gs * M00, kap * gs * M10,
                              kap * gs * M01};
 #pragma unroll
-    for (int c = 0; c < NCOEF; ++c) coef[c * s + k] = (T)A[c];
+    for (int c = 0; c < NCOEF; ++c) coef[c * s + k] = A[c];
   }
 }
 
@@ -561,14 +560,11 @@ cudaError_t launch_moments_from_coarse(const Grid& gc, const Grid& gf, const dou
   return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_coefs(const Grid& g, const double* mom, double nu, T* coef, cudaStream_t s,
+cudaError_t launch_coefs(const Grid& g, const double* mom, double nu, double* coef, cudaStream_t s,
                          int num_sms) {
-  coefs_kernel<T><<<blocks_for((long long)g.nx * g.ny, num_sms), 256, 0, s>>>(g, mom, nu, coef);
+  coefs_kernel<<<blocks_for((long long)g.nx * g.ny, num_sms), 256, 0, s>>>(g, mom, nu, coef);
   return cudaGetLastError();
 }
-template cudaError_t launch_coefs<double>(const Grid&, const double*, double, double*, cudaStream_t, int);
-template cudaError_t launch_coefs<float>(const Grid&, const double*, double, float*, cudaStream_t, int);
 
 cudaError_t launch_fx_coefs(const Grid& g, const double* mom, double nu, unsigned long long* out,
                             cudaStream_t s, int num_sms) {

@@ -99,7 +99,6 @@ template <typename T> struct NRaw2 {
   using T2 = typename V2<T>::t;
   T2 b0, b1;
   T2 d20, d21;
-  double2 d1;
 };
 
 // float64 dot partners of the pair (z.r, z.q), loaded one row ahead outside

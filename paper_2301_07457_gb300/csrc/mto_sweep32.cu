@@ -25,7 +25,6 @@ bool float32_tiles(bool finest, const Grid& g, int tw, int num_sms) {
 
 template <int SRC, int MODE, bool DOT>
 static cudaError_t go(SweepParams<float> p, int tw, int num_sms, cudaStream_t s) {
-  constexpr int COLS = sweep_cols_of(false, SRC, MODE);
   constexpr int PF = lookahead<SRC, MODE, DOT>();
   void (*kernel)(SweepParams<float>);
   if constexpr (MODE == MODE_PRE2 || MODE == MODE_POST2) {
@@ -44,7 +43,7 @@ static cudaError_t go(SweepParams<float> p, int tw, int num_sms, cudaStream_t s)
     static const int wave = full_wave_warps(kernel, num_sms);  // same for every device of a run
     tw = wave;
   }
-  const SweepShape sh = sweep_shape(p.g, MODE, tw, COLS);
+  const SweepShape sh = sweep_shape(p.g, MODE, tw, SWEEP_COLS_F32);
   p.nstrips = sh.nstrips;
   p.nchunks = sh.nchunks;
   p.H = sh.H;

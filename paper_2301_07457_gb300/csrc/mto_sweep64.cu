@@ -72,7 +72,7 @@ static cudaError_t go(SweepParams<double> p, int tw, int num_sms, cudaStream_t s
     static const int wave = full_wave_warps(kernel, num_sms);  // same for every device of a run
     tw = wave;
   }
-  const SweepShape sh = sweep_shape(p.g, MODE, tw, sweep_cols_of(true, SRC, MODE), num_sms);
+  const SweepShape sh = sweep_shape(p.g, MODE, tw, SWEEP_COLS_F64, num_sms);
   p.nstrips = sh.nstrips;
   p.nchunks = sh.nchunks;
   p.H = sh.H;
