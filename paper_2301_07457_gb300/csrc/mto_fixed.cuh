@@ -279,10 +279,11 @@ __host__ __device__ __forceinline__ unsigned fx_magnitude(double x, double y) {
 // 5.7e-17 up to Q - q = 34, 2.9e-16 / 6.5e-17 at 36, 3.0e-16 / 7.7e-17 at 37,
 // 3.5e-16 / 7.8e-17 at 38, against 4.1e-16 / 7.7e-17 in float64: the line lies at the
 // last one that is better than float64 in both.  A void of 1e-9 (2^-30) beside
-// solids stays within it for values down to 1/64 of the window's largest; a
-// float64 iteration on a smooth two-phase design with that void takes 64 us at
-// 64^2 (78 with the line at 34, 57 with none), 105 at 256^2 (114, 104).
-// Float64 subnormals count as zeros here, next to values above 2^-926.
+// solids stays within it for values down to 1/64 of the window's largest: a
+// float64 iteration on a smooth two-phase design with that void takes 58 us at
+// 64^2 (57 without the check) and 103 at 256^2 (104).
+// Float64 subnormals have no exponent of their own: next to values above 2^-986
+// they may be lost.
 constexpr int FX_SPAN = 36;
 __host__ __device__ __forceinline__ bool fx_beyond(int Q, int q) { return Q - q > FX_SPAN; }
 constexpr int FX_NEVER = -(1 << 20);  // a weight that no scales hold

@@ -35,11 +35,12 @@
 // integer instructions a row, and compares it with the scales at its end: a vote
 // and a call in every row took K p at 2048^2 from 113 to 119 us, an early exit
 // from the loop to 117, this to 115.  A non-finite nodal value or modulus takes
-// the task to float64 too, and so reaches the nodes next to it alone.  Normal
-// work hardly ever gets there (designs with a void of 1e-9, 64^2 to 1024^2: no
-// marching row that was counted, up to 1% of the tiles); with a void of 1e-12 in
-// half of a smooth design an iteration takes 160 instead of 104 us at 256^2 and
-// 433 instead of 371 us at 1024^2 (278 and 992 us where all was in float64), and
+// the task to float64 too, and so reaches the nodes next to it alone.  With a
+// void of 1e-9 the sweeps of a random or a smooth design do not get there, on an
+// optimised one a task in a thousand of the first sweep of a cycle and of its
+// residual does (w/D b spans more than a vector of the iteration); with a void of
+// 1e-12 in half of a smooth design an iteration takes 136 instead of 104 us at
+// 256^2 and 414 instead of 371 us at 1024^2 (278 and 992 us where all was in float64), and
 // with factors some 2^-60 apart everywhere the operator at 2048^2 takes 407 us and a
 // V-cycle 2.61 ms (318 us and 2.41 ms).
 #pragma once

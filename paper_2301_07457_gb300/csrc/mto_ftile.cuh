@@ -6,9 +6,12 @@
 // The tiles, stages and halos are those of mto_tile.cuh, the arithmetic is that
 // of mto_fsweep.cuh: one thread per element or node, the marched values and the
 // corner forces of the elements as 96-bit integers in shared memory, one scale
-// per tile and stage.  A tile whose scales do not hold the terms of one of its
-// elements (fx_beyond in mto_fixed.cuh) is done again in float64, by the same
-// stages on DTile in the same shared memory.
+// per tile and stage.  An element whose terms the scales do not hold (fx_beyond
+// in mto_fixed.cuh) is evaluated in float64, and a node next to one sums the two
+// kinds apart.  Most launches of a first sweep on an optimised design hold a few
+// such elements in the void, and wait for the tile that does: a float64 iteration
+// of the optimiser's loop at 512^2 takes 169 us with fixed point alone, 190 with the
+// whole tile done again, 183 so (1024^2 366, 414, 410).
 //
 // Against two launches of the row-per-warp kernel a pass saves a launch and a
 // trip through memory (a coarse level 10.4 -> 9.6 us, the finest 256^2 one with
@@ -33,60 +36,89 @@ template <int N> struct FxArray {
     mid[i] = v.mid;
     hi[i] = v.hi;
   }
+  // A float64 in the place of one, marked by an upper limb that no value has.
+  static constexpr int WIDE = 0x7fffffff;
+  __device__ __forceinline__ bool is64(int i) const { return hi[i] == WIDE; }
+  __device__ __forceinline__ double get64(int i) const { return __hiloint2double((int)mid[i], (int)lo[i]); }
+  __device__ __forceinline__ void put64(int i, double v) {
+    lo[i] = (unsigned)__double2loint(v);
+    mid[i] = (unsigned)__double2hiint(v);
+    hi[i] = WIDE;
+  }
+};
+
+// An element's words, passed by value.
+template <int SRC> struct FxWords {
+  unsigned long long k[FxElem<SRC>::N];
 };
 
 // One operator evaluation per stage over a tile of NW x NH nodes.
 template <int SRC, int NW, int NH> struct FTile {
-  static constexpr bool FIXED = true;
   static constexpr int N = NW * NH, EW = NW - 1, EH = NH - 1, NE = EW * EH;
   FxArray<N> vx, vy;             // nodal values at the stage's scale
   FxArray<NE> fx[4], fy[4];      // forces of element e on its corners BL, BR, TR, TL
   int B[2], X;                   // scales: nodal values of the two stages, coefficients
-  int lost;                      // an element's terms lie beyond the scales, or are not finite
-  unsigned mag[N];               // magnitudes of the nodal values
+  double2 value[N];              // the nodal values themselves
+  unsigned mag[N];               // their magnitudes
+  int any_wide;                  // some element of the tile is evaluated in float64 (of either stage)
 
   __device__ __forceinline__ static int exponent(const double2& v) { return (int)(fx_magnitude(v.x, v.y) >> 20); }
   // All threads, before the first raise() (with a barrier between).
   __device__ __forceinline__ void init() {
     if (threadIdx.x < 2) B[threadIdx.x] = 1;
     if (threadIdx.x == 2) X = 0;
-    if (threadIdx.x == 3) lost = 0;
+    if (threadIdx.x == 3) any_wide = 0;
   }
   // Raises the scale of stage s to the exponent e of a thread's value (0: none).
   __device__ __forceinline__ void raise(int s, int e) {
-    if (e == 0x7ff) {
-      lost = 1;
-      e = 0;
-    }
+    if (e == 0x7ff) e = 0;
     const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
     if ((threadIdx.x & 31) == 0) atomicMax(&B[s], m);
   }
   __device__ __forceinline__ void raise_elements(unsigned tag) {
-    const int m = (int)__reduce_max_sync(0xffffffffu, tag & 0x7ffu);
+    const unsigned x = tag & 0x7ffu;
+    const int m = (int)__reduce_max_sync(0xffffffffu, x == 0x7ffu ? 0u : x);
     if ((threadIdx.x & 31) == 0) atomicMax(&X, m);
   }
   // Node n gets value v at the scale of stage s (whole warps).
   __device__ __forceinline__ void put(int s, int n, bool in, double2 v) {
     const unsigned m = fx_magnitude(v.x, v.y);
-    if ((m >> 20) == 0x7ffu) v = make_double2(0.0, 0.0);
-    const Fx2 f = fx2_from(v, B[s]);
+    const Fx2 f = fx2_from((m >> 20) == 0x7ffu ? make_double2(0.0, 0.0) : v, B[s]);
     if (!in) return;
+    value[n] = v;
     mag[n] = m;
     vx.put(n, f.x);
     vy.put(n, f.y);
   }
-  // Forces of the thread's element e at stage s, whose BL node is c; tag, k: its factors.
+  // The forces in float64.  A call of its own, so that its registers do not weigh on the kernels.
+  __device__ __noinline__ void element_f64(const SweepParams<double>& a, int e, int c, FxWords<SRC> words) {
+    const Strain<double> w =
+        strain_coords<double, double2>(value[c], value[c + 1], value[c + NW + 1], value[c + NW]);
+    double2 f[4];
+    strain_forces<double, double2>(FxElem<SRC>::core64(a, w, words.k), f[0], f[1], f[2], f[3]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      fx[q].put64(e, f[q].x);
+      fy[q].put64(e, f[q].y);
+    }
+  }
+  // Forces of the thread's element e at stage s, whose BL node is c; tag, words: its factors.
   __device__ __forceinline__ void element(const SweepParams<double>& a, int s, int e, int c, unsigned tag,
-                                          const unsigned long long* k, bool rare) {
+                                          const FxWords<SRC>& words, bool rare) {
     const unsigned m = max(max(mag[c], mag[c + 1]), max(mag[c + NW], mag[c + NW + 1]));
     const int x = (int)(tag & 0x7ffu);
-    if (x == 0x7ff || (m != 0u && tag != 0u && fx_beyond(B[s] + X, (int)(m >> 20) + x))) lost = 1;
+    const bool w64 = (m >> 20) == 0x7ffu || x == 0x7ff || (m != 0u && x != 0 && fx_beyond(B[s] + X, (int)(m >> 20) + x));
+    if (w64) {
+      any_wide = 1;
+      element_f64(a, e, c, words);
+      return;
+    }
     const Fx2 bl = {vx.get(c), vy.get(c)}, br = {vx.get(c + 1), vy.get(c + 1)};
     const Fx2 tl = {vx.get(c + NW), vy.get(c + NW)}, tr = {vx.get(c + NW + 1), vy.get(c + NW + 1)};
     const Fx2 ac = fsub(br, bl), bt = fsub(tr, tl), up = fsub(fadd(tr, tl), fadd(br, bl));
     const FxStrain w = {fx_add(ac.x, bt.x), fx_sub(bt.x, ac.x), up.y, fx_sub(bt.y, ac.y),
                         fx_add(up.x, fx_add(ac.y, bt.y))};
-    FxStrain t = FxElem<SRC>::core(a, w, k, rare);
+    FxStrain t = FxElem<SRC>::core(a, w, words.k, rare);
     const int sh = X - (int)(tag & 0x7ffu);
     if (rare)
       t = {fx_sar_limbs(t.c1, sh), fx_sar_limbs(t.c3, sh), fx_sar_limbs(t.d2, sh), fx_sar_limbs(t.d3, sh),
@@ -103,61 +135,46 @@ template <int SRC, int NW, int NH> struct FTile {
     fy[2].put(e, fx_add(hb, t.d2));
     fy[3].put(e, fx_sub(t.d2, hb));
   }
-  // K v at node n, whose upper right element is e.
-  __device__ __forceinline__ double2 at_node(int s, int n, int e) const {
+  // K v at the node whose upper right element is e.
+  __device__ __forceinline__ double2 at_node(int s, int e) const {
+    const int unit = B[s] + X + FxElem<SRC>::UNIT;
+    if (any_wide) return at_node_mixed(unit, e);  // uniform over the block
     const Fx x = fx_add(fx_add(fx[0].get(e), fx[1].get(e - 1)), fx_add(fx[2].get(e - EW - 1), fx[3].get(e - EW)));
     const Fx y = fx_add(fx_add(fy[0].get(e), fy[1].get(e - 1)), fx_add(fy[2].get(e - EW - 1), fy[3].get(e - EW)));
-    const int unit = B[s] + X + FxElem<SRC>::UNIT;
     double2 kv = make_double2(fx_to_double<false>(x, unit), fx_to_double<false>(y, unit));
     if (unit < FX_UNIT_MIN || unit > FX_UNIT_MAX)  // uniform over the block
       kv = make_double2(fx_to_double(x, unit), fx_to_double(y, unit));
     return kv;
   }
-};
-
-// The same in float64.
-template <int SRC, int NW, int NH> struct DTile {
-  static constexpr bool FIXED = false;
-  static constexpr int N = NW * NH, EW = NW - 1, EH = NH - 1, NE = EW * EH;
-  double vx[N], vy[N], fx[4][NE], fy[4][NE];
-  static constexpr int X = 0, lost = 0;
-
-  __device__ __forceinline__ static int exponent(const double2&) { return 0; }
-  __device__ __forceinline__ void init() {}
-  __device__ __forceinline__ void raise(int, int) {}
-  __device__ __forceinline__ void raise_elements(unsigned) {}
-  __device__ __forceinline__ void put(int, int n, bool in, double2 v) {
-    if (!in) return;
-    vx[n] = v.x;
-    vy[n] = v.y;
-  }
-  __device__ __forceinline__ double2 get(int n) const { return make_double2(vx[n], vy[n]); }
-  __device__ __forceinline__ void element(const SweepParams<double>& a, int, int e, int c, unsigned,
-                                          const unsigned long long* k, bool) {
-    const Strain<double> w = strain_coords<double, double2>(get(c), get(c + 1), get(c + NW + 1), get(c + NW));
-    double2 f[4];
-    strain_forces<double, double2>(FxElem<SRC>::core64(a, w, k), f[0], f[1], f[2], f[3]);
+  // The same where an element may be in float64.
+  __device__ __noinline__ double2 at_node_mixed(int unit, int e) const {
+    const int at[4] = {e, e - 1, e - EW - 1, e - EW};
+    Fx x = fx_zero(), y = x;
+    double2 w[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      fx[q][e] = f[q].x;
-      fy[q][e] = f[q].y;
+      w[q] = make_double2(0.0, 0.0);
+      if (fx[q].is64(at[q])) {
+        w[q] = make_double2(fx[q].get64(at[q]), fy[q].get64(at[q]));
+      } else {
+        x = fx_add(x, fx[q].get(at[q]));
+        y = fx_add(y, fy[q].get(at[q]));
+      }
     }
-  }
-  __device__ __forceinline__ double2 at_node(int, int, int e) const {
-    return make_double2((fx[0][e] + fx[1][e - 1]) + (fx[2][e - EW - 1] + fx[3][e - EW]),
-                        (fy[0][e] + fy[1][e - 1]) + (fy[2][e - EW - 1] + fy[3][e - EW]));
+    return make_double2(((w[0].x + w[1].x) + (w[2].x + w[3].x)) + fx_to_double(x, unit),
+                        ((w[0].y + w[1].y) + (w[2].y + w[3].y)) + fx_to_double(y, unit));
   }
 };
 
 template <int SRC> struct FTileElem {
-  unsigned long long k[FxElem<SRC>::N];
+  FxWords<SRC> words;
   unsigned tag;
   __device__ __forceinline__ void load(const SweepParams<double>& a, bool in, int ei, int ej) {
     const bool valid = in && ei >= 0 && ei < a.g.nx && ej >= 0 && ej < a.g.ny;
     const unsigned long long* E = static_cast<const unsigned long long*>(a.E) + (valid ? a.g.at(ei, ej) : 0);
 #pragma unroll
-    for (int n = 0; n < FxElem<SRC>::N; ++n) k[n] = valid ? __ldg(E + n * a.cstride) : 0ull;
-    tag = fx_tag(k);
+    for (int n = 0; n < FxElem<SRC>::N; ++n) words.k[n] = valid ? __ldg(E + n * a.cstride) : 0ull;
+    tag = fx_tag(words.k);
   }
   // A scale far below the tile's or an unexpected sign (whole warps; once X is final).
   __device__ __forceinline__ bool rare(int X) const {
@@ -175,12 +192,14 @@ template <int SRC> __device__ __forceinline__ double2 ftile_d(const SweepParams<
   }
 }
 
-constexpr int PRE2_W = TILE_X + 5, PRE2_H = TILE_Y + 5, POST2_W = TILE_X + 4, POST2_H = TILE_Y + 4;
-
-// A tile of PRE2.  False: its scales do not hold it (uniform over the block).
-template <int SRC, typename Tile>
-__device__ __forceinline__ bool pre2_tile(const SweepParams<double>& a, Tile& f, double2* r) {
-  constexpr int NW = PRE2_W, NH = PRE2_H, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
+// Blocks per SM that the fixed-point path's registers allow (as split_blocks()).
+template <int SRC>
+__global__ void __launch_bounds__(SWEEP_NT, SRC == SRC_FINE64 ? 4 : 2)
+    ftile_pre2_kernel(const __grid_constant__ SweepParams<double> a) {
+  pdl_trigger();
+  constexpr int NW = TILE_X + 5, NH = TILE_Y + 5, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
+  __shared__ FTile<SRC, NW, NH> f;
+  __shared__ double2 r[ZW * ZH];
   static_assert(EW * EH <= SWEEP_NT && ZW * ZH <= SWEEP_NT && NW * NH <= 2 * SWEEP_NT, "threads");
   const Grid g = a.g, gc = a.gc;
   const int t = threadIdx.x;
@@ -212,7 +231,7 @@ __device__ __forceinline__ bool pre2_tile(const SweepParams<double>& a, Tile& f,
     const int n = t + u * SWEEP_NT, ii = x0 + n % NW, jj = y0 + n / NW;
     bh[u] = n < NW * NH && g.valid(ii, jj) ? a.b[g.at(ii, jj)] : zero2;
   }
-  if (done) return true;  // uniform over the grid
+  if (done) return;  // uniform over the grid
 #pragma unroll
   for (int u = 0; u < 2; ++u) z0[u] = make_double2(z0[u].x * bh[u].x, z0[u].y * bh[u].y);
   __syncthreads();
@@ -233,9 +252,9 @@ __device__ __forceinline__ bool pre2_tile(const SweepParams<double>& a, Tile& f,
   double2 kv = zero2;
 #pragma unroll 1
   for (int s = 0;; ++s) {
-    if (s == 0 ? elem : inner_elem) f.element(a, s, t, c, er.tag, er.k, rare);
+    if (s == 0 ? elem : inner_elem) f.element(a, s, t, c, er.tag, er.words, rare);
     __syncthreads();
-    if (s == 0 ? act : inner && act) kv = f.at_node(s, zn, en);
+    if (s == 0 ? act : inner && act) kv = f.at_node(s, en);
     if (s == 1) break;
     double2 z1 = zero2;
     if (act) z1 = make_double2(fma(d.x, b.x - kv.x, d.x * b.x), fma(d.y, b.y - kv.y, d.y * b.y));
@@ -247,7 +266,6 @@ __device__ __forceinline__ bool pre2_tile(const SweepParams<double>& a, Tile& f,
   }
   if (inner) r[t] = act ? make_double2(b.x - kv.x, b.y - kv.y) : zero2;
   __syncthreads();
-  if (f.lost) return false;
   // Full weighting, over the three rows of each column first; one component per thread.
   if (t < 2 * TILE_CX * TILE_CY) {
     const int cc = t & 1, p = (t >> 1) % TILE_CX, q = (t >> 1) / TILE_CX, I = I0 + p, J = J0 + q;
@@ -259,37 +277,14 @@ __device__ __forceinline__ bool pre2_tile(const SweepParams<double>& a, Tile& f,
       reinterpret_cast<double*>(a.bc + gc.at(I, J))[cc] = gc.is_fixed(I, J) ? 0.0 : val;
     }
   }
-  return true;
 }
 
-// Shared memory of a tile, of whichever kind is running.
-template <typename F, typename D> union TileMemory {
-  F fixed;
-  D wide;
-};
-
-template <int SRC>
-__device__ __noinline__ void pre2_tile_f64(const SweepParams<double>& a, DTile<SRC, PRE2_W, PRE2_H>& f, double2* r) {
-  pre2_tile<SRC>(a, f, r);
-}
-
-// Blocks per SM that the fixed-point path's registers allow.
-template <int SRC>
-__global__ void __launch_bounds__(SWEEP_NT, SRC == SRC_FINE64 ? 4 : 2)
-    ftile_pre2_kernel(const __grid_constant__ SweepParams<double> a) {
+template <int SRC, bool DOT>
+__global__ void __launch_bounds__(SWEEP_NT, SRC == SRC_FINE64 ? (DOT ? 3 : 4) : 2)
+    ftile_post2_kernel(const __grid_constant__ SweepParams<double> a) {
   pdl_trigger();
-  __shared__ TileMemory<FTile<SRC, PRE2_W, PRE2_H>, DTile<SRC, PRE2_W, PRE2_H>> m;
-  __shared__ double2 r[(PRE2_W - 2) * (PRE2_H - 2)];
-  if (pre2_tile<SRC>(a, m.fixed, r)) return;
-  __syncthreads();  // every thread has read `lost`
-  pre2_tile_f64<SRC>(a, m.wide, r);
-}
-
-// A tile of POST2, its dot products in dots.
-enum TileResult { TILE_OK, TILE_LOST, TILE_STOPPED };
-template <int SRC, bool DOT, typename Tile>
-__device__ __forceinline__ TileResult post2_tile(const SweepParams<double>& a, Tile& f, double2* zs, double2& dots) {
-  constexpr int NW = POST2_W, NH = POST2_H, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
+  constexpr int NW = TILE_X + 4, NH = TILE_Y + 4, EW = NW - 1, EH = NH - 1, ZW = NW - 2, ZH = NH - 2;
+  __shared__ FTile<SRC, NW, NH> f;
   static_assert(EW * EH <= SWEEP_NT && NW * NH <= SWEEP_NT, "threads");
   const Grid g = a.g, gc = a.gc;
   const int t = threadIdx.x;
@@ -334,27 +329,25 @@ __device__ __forceinline__ TileResult post2_tile(const SweepParams<double>& a, T
       v = make_double2(fma(w, t0.x + t1.x, v.x), fma(w, t0.y + t1.y, v.y));
     }
   }
-  if (done) return TILE_STOPPED;  // uniform over the grid
+  if (done) return;  // uniform over the grid
   __syncthreads();
   f.raise(0, f.exponent(v));
   f.raise_elements(er.tag);
   __syncthreads();
   f.put(0, t, t < NW * NH, v);
   const bool rare = er.rare(f.X);
-  // The value at the thread's own z2 node, by way of shared memory.
-  if (t < NW * NH) zs[t] = v;
   __syncthreads();
   const int c = ey * NW + ex;
   const int zn = zy * NW + zx, en = zy * EW + zx;
   const bool act = node && g.active(i, j);
   const bool inner_elem = elem && ex >= 1 && ex < EW - 1 && ey >= 1 && ey < EH - 1;
-  double2 z = act ? zs[zn] : zero2;
+  double2 z = act ? f.value[zn] : zero2;
 #pragma unroll 1
   for (int s = 0; s < 2; ++s) {
-    if (s == 0 ? elem : inner_elem) f.element(a, s, t, c, er.tag, er.k, rare);
+    if (s == 0 ? elem : inner_elem) f.element(a, s, t, c, er.tag, er.words, rare);
     __syncthreads();
     if (s == 0 ? act : own && act) {
-      const double2 kv = f.at_node(s, zn, en);
+      const double2 kv = f.at_node(s, en);
       z = make_double2(fma(d.x, b.x - kv.x, z.x), fma(d.y, b.y - kv.y, z.y));
     }
     if (s == 1) break;
@@ -363,41 +356,16 @@ __device__ __forceinline__ TileResult post2_tile(const SweepParams<double>& a, T
     f.put(1, zn, node, z);
     __syncthreads();
   }
-  dots = zero2;
-  if (f.lost) return TILE_LOST;  // uniform over the block
+  double dot0 = 0.0, dot1 = 0.0;
   if (own) {
     a.out[k] = z;
     if constexpr (DOT) {
-      dots.x = fma(z.x, rd.x, z.y * rd.y);
-      if (a.qdot != nullptr) dots.y = fma(z.x, qd.x, z.y * qd.y);
+      dot0 = fma(z.x, rd.x, z.y * rd.y);
+      if (a.qdot != nullptr) dot1 = fma(z.x, qd.x, z.y * qd.y);
     }
   }
-  return TILE_OK;
-}
-
-template <int SRC, bool DOT>
-__device__ __noinline__ double2 post2_tile_f64(const SweepParams<double>& a, DTile<SRC, POST2_W, POST2_H>& f,
-                                               double2* zs) {
-  double2 dots;
-  post2_tile<SRC, DOT>(a, f, zs, dots);
-  return dots;
-}
-
-template <int SRC, bool DOT>
-__global__ void __launch_bounds__(SWEEP_NT, SRC == SRC_FINE64 ? (DOT ? 3 : 4) : 2)
-    ftile_post2_kernel(const __grid_constant__ SweepParams<double> a) {
-  pdl_trigger();
-  __shared__ TileMemory<FTile<SRC, POST2_W, POST2_H>, DTile<SRC, POST2_W, POST2_H>> m;
-  __shared__ double2 zs[POST2_W * POST2_H];
-  double2 dots;
-  const TileResult res = post2_tile<SRC, DOT>(a, m.fixed, zs, dots);
-  if (res == TILE_STOPPED) return;
-  if (res == TILE_LOST) {
-    __syncthreads();  // every thread has read `lost`
-    dots = post2_tile_f64<SRC, DOT>(a, m.wide, zs);
-  }
   if constexpr (DOT)
-    block_reduce_finish<SWEEP_NT>(dots.x, dots.y, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
+    block_reduce_finish<SWEEP_NT>(dot0, dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);
 }
 
 }  // namespace mto
