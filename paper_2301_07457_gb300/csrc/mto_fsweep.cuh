@@ -400,6 +400,33 @@ __device__ __noinline__ FSums rows_f64(const SweepParams<double>& a, FTask t0, i
   return sums;
 }
 
+// The restriction's tasks of a block that are to be done again in float64
+// (`lost`: this warp's is), their rows by all its warps: a row takes one warp about
+// a microsecond of its FP64 pipe, and on an optimised design one or two tasks of
+// a launch are waited for (a float64 iteration at 1024^2 433 -> 422 us).  In the
+// other sweeps the barrier at the end costs what this gains.
+template <int SRC, bool DOT, typename ZT>
+__device__ __noinline__ void restrict_f64(const SweepParams<double>& a, bool lost) {
+  __shared__ unsigned mask;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  if (threadIdx.x == 0) mask = 0;
+  __syncthreads();
+  if (lost && lane == 0) atomicOr(&mask, 1u << warp);
+  __syncthreads();
+  // Each lost task is shared by `parts` warps, this warp has part `part` of the
+  // one that is `mine`.
+  unsigned m = mask;
+  const int parts = nwarps / __popc(m), mine = warp / parts, part = warp % parts;
+  for (int q = 0; q < mine; ++q) m &= m - 1;
+  if (m == 0u) return;
+  const int wg = blockIdx.x * nwarps + __ffs((int)m) - 1, strip = wg % a.nstrips, chunk = wg / a.nstrips;
+  const int Jb = chunk * (a.H >> 1), n = min(a.H >> 1, a.gc.ny + 1 - Jb), per = (n + parts - 1) / parts;
+  const int i = strip * SWEEP_RSTRIDE - 2 + lane, J0 = Jb + part * per, J1 = min(Jb + n, J0 + per) - 1;
+  if (J0 > J1) return;
+  const FTask t = {i, lane, max(2 * J0 - 2, -1), J0, J1, lane >= 1 && lane <= 30 && i >= 0 && i <= a.g.nx};
+  rows_f64<SRC, MODE_RESTRICT, DOT, ZT, true>(a, t, 2 * J1 + 1, 0.0, false, 0.0);
+}
+
 // Two resident blocks per SM, as sweep2_kernel.
 template <int SRC, int MODE, bool DOT, typename ZT, int PF>
 __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const __grid_constant__ SweepParams<double> a) {
@@ -419,7 +446,7 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const __grid_consta
   const double2 zero2 = make_double2(0.0, 0.0);
   FSums sums = {0.0, 0.0, zero2};
   double beta = 0.0, alag = 0.0;
-  bool vzero = false, lag = false;
+  bool vzero = false, lag = false, lost = false;
   if constexpr (MODE == MODE_KP) {
     beta = a.sc->beta;
     lag = a.sc->x_lag != 0;  // K p advances x by the pending step at its owned nodes
@@ -592,8 +619,15 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const __grid_consta
         k += pitch;
       }
     }
-    if (__any_sync(0xffffffffu, lane <= 30 && fx_beyond(B + Xm, low)))
-      sums = rows_f64<SRC, MODE, DOT, ZT, true>(a, t0, je1, beta, lag, alag);
+    if constexpr (MODE == MODE_RESTRICT) {
+      lost = __any_sync(0xffffffffu, lane <= 30 && fx_beyond(B + Xm, low));
+    } else {
+      if (__any_sync(0xffffffffu, lane <= 30 && fx_beyond(B + Xm, low)))
+        sums = rows_f64<SRC, MODE, DOT, ZT, true>(a, t0, je1, beta, lag, alag);
+    }
+  }
+  if constexpr (MODE == MODE_RESTRICT) {
+    if (__syncthreads_or(lost)) restrict_f64<SRC, DOT, ZT>(a, lost);
   }
   if constexpr (REDUCE) {
     block_reduce_finish<SWEEP_NT, DOT>(sums.dot0, sums.dot1, a.partials, a.ticket, a.sc, a.finish, a.out_value, a.tag);

@@ -84,6 +84,33 @@ def test_soft_beside_stiff(mto, ratio, kind, warps):
     m.close()
 
 
+@pytest.mark.parametrize("ratio", [1e-9, 1e-12, 1e-24])
+def test_soft_parts_of_a_large_mesh(mto, ratio):
+    """Marching tasks in full blocks on the finest grid, tiles below it, soft patches of several sizes.
+    Here a cycle in float64 instructions throughout is within 1.0e-13 of the oracle's (on the stiff nodes
+    4.1e-11, also at ratio 1: the large smooth response to a random residual), so 20 times that is allowed."""
+    nx, ny, nc, fixed = 512, 480, 5, BOTTOM
+    x = np.zeros((2, ny, nx))
+    for j, i, h, w in ((30, 40, 3, 5), (100, 200, 17, 31), (250, 20, 64, 130), (301, 300, 150, 90), (470, 500, 10, 12)):
+        x[1, j:j + h, i:i + w] = 1.0
+    x[0] = 1.0 - x[1]
+    Es = [1.0, ratio]
+    lv = multigrid.build_hierarchy(nx, ny, fem.simp_moduli(x, Es, 3.0), fem.element_stiffness(0.3), fixed, nc)
+    m = build(mto, nx, ny, nc, x, Es, fixed)
+    rng = np.random.default_rng(6)
+    for l in (nc, nc - 1):
+        v = rng.choice([-1.0, 1.0], m.level_shape(l)) * rng.uniform(0.5, 1.0, m.level_shape(l))
+        check_rows(m, lv, l, v * 2.0 ** rng.integers(-20, 21, v.shape[:2] + (1,)))
+    r = rng.standard_normal((ny + 1, nx + 1, 2))
+    r[0] = 0.0
+    z = m.apply_preconditioner(dev(r)).cpu().numpy().ravel()[lv[nc].free]
+    ref = multigrid.vcycle_preconditioner(lv, 0.6, 2, 2)(r.ravel()[lv[nc].free])
+    assert np.linalg.norm(z - ref) <= 2e-12 * np.linalg.norm(ref)
+    stiff = lv[nc].diag > 0.1
+    assert np.linalg.norm((z - ref)[stiff]) <= 8e-10 * np.linalg.norm(ref[stiff])
+    m.close()
+
+
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 @pytest.mark.parametrize("warps", [MARCH, ROWS])
 @pytest.mark.parametrize("at", [(3, 5), (20, 31), (23, 44)])
