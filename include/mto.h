@@ -263,6 +263,9 @@ mto_status mto_run_host_wait(mto_ctx* ctx, mto_solve_stats* stats);
  * context's precision (float32 levels compute in float32; the finest level
  * of the mixed path offers both: use_vcycle_operator = 1 selects the
  * bfloat16/float32 smoother operator, 0 the float64 outer operator).
+ * Float64 operators are accurate row by row: y_i is within a few units of
+ * 2^-53 of sum_j |K_ij| |v_j|, however far apart moduli and values lie (but
+ * subnormal values beside normal ones may count as zero).
  * mto_apply_preconditioner: z = one V-cycle applied to r on the finest level
  * (Alg. 1 from U = 0, as inside PCG). */
 mto_status mto_apply_operator(mto_ctx* ctx, int level, int use_vcycle_operator, const double* v_dev,
