@@ -49,8 +49,8 @@ def build(mto, nx, ny, nc, x, Es, fixed=BOTTOM, warps=ROWS, **kw):
     return m
 
 
-def check_rows(m, lv, l, v):
-    y = m.apply_operator(l, dev(v)).cpu().numpy().ravel()
+def check_rows(m, lv, l, v, scale=1.0):
+    y = m.apply_operator(l, dev(v * scale)).cpu().numpy().ravel() / scale
     free, K = lv[l].free, lv[l].K
     ref, bar = np.zeros(y.size), np.zeros(y.size)
     ref[free], bar[free] = K @ v.ravel()[free], abs(K) @ abs(v.ravel()[free])
@@ -81,6 +81,23 @@ def test_soft_beside_stiff(mto, ratio, kind, warps):
     assert np.linalg.norm(z - ref) <= 1e-13 * np.linalg.norm(ref)
     stiff = lv[2].diag > 0.1
     assert np.linalg.norm((z - ref)[stiff]) <= 1e-12 * np.linalg.norm(ref[stiff])
+    m.close()
+
+
+@pytest.mark.parametrize("power", [-960, 0, 1000])
+@pytest.mark.parametrize("warps", [MARCH, ROWS])
+def test_void_block_at_extreme_sizes(mto, warps, power):
+    """The usual void beside solids, values near both ends of float64, each row by its own terms."""
+    nx, ny = 40, 22
+    x = dirichlet_design(nx, ny, 4, seed=4)
+    x[:, 5:9, 3:30] = 0.0
+    x[3, 5:9, 3:30] = 1.0
+    Es = [1.0, 0.5, 0.25, 1e-9]
+    lv = multigrid.build_hierarchy(nx, ny, fem.simp_moduli(x, Es, 3.0), fem.element_stiffness(0.3), BOTTOM, 1)
+    m = build(mto, nx, ny, 1, x, Es, warps=warps)
+    for l in range(2):
+        v = np.random.default_rng(l).standard_normal(m.level_shape(l))
+        check_rows(m, lv, l, v, 2.0 ** power)  # a power of two: exact in the reference too
     m.close()
 
 
