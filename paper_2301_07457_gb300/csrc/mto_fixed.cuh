@@ -23,7 +23,7 @@
 //
 // A window (30 columns by the rows of a task, 14 columns by three rows, or a
 // tile) shares its scales, so the error of a node's K v is absolute, whatever
-// the size of its own terms: FX_SPAN below says from where on they are
+// the size of its own terms: FX_SPAN_* below says from where on they are
 // evaluated in float64 instead.
 //
 // The functions also compile as host code (checked against 128-bit
@@ -270,7 +270,7 @@ __host__ __device__ __forceinline__ unsigned fx_magnitude(double x, double y) {
 }
 // Whether scales of weight Q = B + Xm lose too much of an element of weight q,
 // the sum of the (biased) exponents of its largest factor and of its largest
-// nodal value: the window is then done in float64.
+// nodal value: beyond span places the element is done in float64.
 //
 // The terms |K||v| of a node next to the element are at least about 2^(q - 2046).
 // Its error is at most 18 units of the last place, so 2^(Q - q - 82) of them,
@@ -278,14 +278,21 @@ __host__ __device__ __forceinline__ unsigned fx_magnitude(double x, double y) {
 // of one size: error over the row's terms (largest / root mean square) 2.1e-16 /
 // 5.7e-17 up to Q - q = 34, 2.9e-16 / 6.5e-17 at 36, 3.0e-16 / 7.7e-17 at 37,
 // 3.5e-16 / 7.8e-17 at 38, against 4.1e-16 / 7.7e-17 in float64: the line lies at the
-// last one that is better than float64 in both.  A void of 1e-9 (2^-30) beside
-// solids stays within it for values down to 1/64 of the window's largest: a
-// float64 iteration on a smooth two-phase design with that void takes 58 us at
-// 64^2 (57 without the check) and 103 at 256^2 (104).
+// last one that is better than float64 in both.  A coarse element's factors have
+// two bits fewer and its terms are cut off more often: 3.6e-16 / 9.3e-17 at 33,
+// 4.8e-16 / 1.0e-16 at 34, 5.7e-16 / 1.4e-16 at 35, 1.3e-15 / 2.3e-16 at 36, against
+// 4.8e-16 / 9.0e-17 in float64.  With the line at 34 the whole sweep (elements on
+// both sides of it) shows at most 4.8e-16 / 9.1e-17, at 36 5.2e-16 / 1.1e-16.
+// A void of 1e-9 (2^-30) beside solids stays within it for values down to 1/64 of
+// the window's largest on the finest level, 1/16 on a coarse one: a float64
+// iteration on a smooth two-phase design with that void takes 61 us at 64^2 (57
+// without the check) and 107 at 256^2 (104); with 36 on the coarse levels too 58 and
+// 104, and on late designs of an optimiser's loop 184 / 421 at 512^2 / 1024^2 against
+// 204 / 478.
 // Float64 subnormals have no exponent of their own: next to values above 2^-986
 // they may be lost.
-constexpr int FX_SPAN = 36;
-__host__ __device__ __forceinline__ bool fx_beyond(int Q, int q) { return Q - q > FX_SPAN; }
+constexpr int FX_SPAN_FINE = 36, FX_SPAN_COARSE = 34;
+__host__ __device__ __forceinline__ bool fx_beyond(int Q, int q, int span) { return Q - q > span; }
 constexpr int FX_NEVER = -(1 << 20);  // a weight that no scales hold
 
 // A fine element: its three factors (p, c, g of mto_fsweep.cuh) as integers

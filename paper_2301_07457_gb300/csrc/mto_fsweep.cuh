@@ -39,8 +39,8 @@
 // void of 1e-9 the sweeps of a random or a smooth design do not get there, on an
 // optimised one a task in a thousand of the first sweep of a cycle and of its
 // residual does (w/D b spans more than a vector of the iteration); with a void of
-// 1e-12 in half of a smooth design an iteration takes 136 instead of 104 us at
-// 256^2 and 414 instead of 371 us at 1024^2 (278 and 992 us where all was in float64), and
+// 1e-12 in half of a smooth design an iteration takes 141 instead of 104 us at
+// 256^2 and 420 instead of 371 us at 1024^2 (278 and 992 us where all was in float64), and
 // with factors some 2^-60 apart everywhere the operator at 2048^2 takes 407 us and a
 // V-cycle 2.61 ms (318 us and 2.41 ms).
 #pragma once
@@ -93,7 +93,7 @@ struct FxStrain {
 // factor may be negative that is positive for every positive modulus.
 template <int SRC> struct FxElem;
 template <> struct FxElem<SRC_FINE64> {
-  static constexpr int N = FX_NFINE, UNIT = -2132;
+  static constexpr int N = FX_NFINE, UNIT = -2132, SPAN = FX_SPAN_FINE;
   __device__ __forceinline__ static FxStrain core(const SweepParams<double>&, FxStrain w, const unsigned long long* k,
                                                   bool neg) {
     if (neg && (fx_tag(k) & FX_TAG_NEG))
@@ -113,7 +113,7 @@ template <> struct FxElem<SRC_FINE64> {
   }
 };
 template <> struct FxElem<SRC_COARSE> {
-  static constexpr int N = FX_NCOARSE, UNIT = -2130;
+  static constexpr int N = FX_NCOARSE, UNIT = -2130, SPAN = FX_SPAN_COARSE;
   __device__ __forceinline__ static FxStrain core(const SweepParams<double>& a, FxStrain w,
                                                   const unsigned long long* k, bool neg) {
     constexpr unsigned long long MAG = 0x7fffffffffffffffull;
@@ -403,7 +403,8 @@ __device__ __noinline__ FSums rows_f64(const SweepParams<double>& a, FTask t0, i
 // The restriction's tasks of a block that are to be done again in float64
 // (`lost`: this warp's is), their rows by all its warps: a row takes one warp about
 // a microsecond of its FP64 pipe, and on an optimised design one or two tasks of
-// a launch are waited for (a float64 iteration at 1024^2 433 -> 422 us).  In the
+// a launch are waited for (a float64 iteration at 1024^2 433 -> 422 us, with
+// FX_SPAN_COARSE at 36).  In the
 // other sweeps the barrier at the end costs what this gains.
 template <int SRC, bool DOT, typename ZT>
 __device__ __noinline__ void restrict_f64(const SweepParams<double>& a, bool lost) {
@@ -620,9 +621,9 @@ __global__ void __launch_bounds__(SWEEP_NT, 2) fsweep_kernel(const __grid_consta
       }
     }
     if constexpr (MODE == MODE_RESTRICT) {
-      lost = __any_sync(0xffffffffu, lane <= 30 && fx_beyond(B + Xm, low));
+      lost = __any_sync(0xffffffffu, lane <= 30 && fx_beyond(B + Xm, low, F::Elem::SPAN));
     } else {
-      if (__any_sync(0xffffffffu, lane <= 30 && fx_beyond(B + Xm, low)))
+      if (__any_sync(0xffffffffu, lane <= 30 && fx_beyond(B + Xm, low, F::Elem::SPAN)))
         sums = rows_f64<SRC, MODE, DOT, ZT, true>(a, t0, je1, beta, lag, alag);
     }
   }
@@ -777,7 +778,7 @@ __global__ void __launch_bounds__(SWEEP_NT, (split_blocks<SRC, MODE, DOT>()))
     // Whether the scales hold the terms of the elements, as in the marching
     // kernel; a non-finite value or modulus has made a scale non-finite.
     const int e4 = max(ec, __shfl_down_sync(0xffffffffu, ec, 1, 16));
-    const bool again = (__any_sync(0xffffffffu, hl <= 14 && min(e4, X) != 0 && fx_beyond(B + Xm, e4 + X)) ||
+    const bool again = (__any_sync(0xffffffffu, hl <= 14 && min(e4, X) != 0 && fx_beyond(B + Xm, e4 + X, F::Elem::SPAN)) ||
                         B == 0x7ff || Xm == 0x7ff) && !vzero;
     const double2 mid = half ? vlo : vhi;  // node row je
     const double vc = c ? mid.y : mid.x;

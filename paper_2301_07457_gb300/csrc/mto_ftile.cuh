@@ -11,7 +11,7 @@
 // kinds apart.  Most launches of a first sweep on an optimised design hold a few
 // such elements in the void, and wait for the tile that does: a float64 iteration
 // of the optimiser's loop at 512^2 takes 169 us with fixed point alone, 190 with the
-// whole tile done again, 183 so (1024^2 366, 414, 410).
+// whole tile done again, 183 so (1024^2 366, 414, 410; all with FX_SPAN_COARSE at 36).
 //
 // Against two launches of the row-per-warp kernel a pass saves a launch and a
 // trip through memory (a coarse level 10.4 -> 9.6 us, the finest 256^2 one with
@@ -107,7 +107,7 @@ template <int SRC, int NW, int NH> struct FTile {
                                           const FxWords<SRC>& words, bool rare) {
     const unsigned m = max(max(mag[c], mag[c + 1]), max(mag[c + NW], mag[c + NW + 1]));
     const int x = (int)(tag & 0x7ffu);
-    const bool w64 = (m >> 20) == 0x7ffu || x == 0x7ff || (m != 0u && x != 0 && fx_beyond(B[s] + X, (int)(m >> 20) + x));
+    const bool w64 = (m >> 20) == 0x7ffu || x == 0x7ff || (m != 0u && x != 0 && fx_beyond(B[s] + X, (int)(m >> 20) + x, FxElem<SRC>::SPAN));
     if (w64) {
       any_wide = 1;
       element_f64(a, e, c, words);
